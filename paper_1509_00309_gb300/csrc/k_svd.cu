@@ -42,78 +42,256 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
+// Sum over the CTA, returned to every thread.  The 16 warps' partial sums are added by one warp:
+// an FP64 instruction holds its sub-partition's FP64 pipe for 64 cycles whatever its lanes do, so
+// the same 16 additions made by every warp took 4.9k cycles a call, these four take 0.4k.
 __device__ double block_sum(double v, double* sh) {
   v = warp_sum(v);
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
   __syncthreads();
   if (l == 0) sh[w] = v;
   __syncthreads();
-  double s = 0.0;
-  for (int i = 0; i < kWarps; ++i) s += sh[i];
+  if (w == 0) {
+    double s = l < kWarps ? sh[l] : 0.0;
+#pragma unroll
+    for (int o = kWarps / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (l == 0) sh[0] = s;
+  }
+  __syncthreads();
+  const double s = sh[0];
   __syncthreads();
   return s;
 }
 
-// In-place Householder QR of the p x q column-major matrix a (ld lda), p >= q.  R is left in
-// the upper triangle, the reflector vectors (without their unit first entry) below it.
-__device__ void householder_qr(double* a, int p, int q, int64_t lda, double* tau, double* sh) {
-  const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int j = 0; j < q; ++j) {
-    double* col = a + (int64_t)j * lda;
-    double part = 0.0;
-    for (int i = j + 1 + threadIdx.x; i < p; i += kThreads) part += col[i] * col[i];
-    const double s = block_sum(part, sh);
-    const double x0 = col[j];
-    double t = 0.0, beta = x0, v0 = 1.0;
-    if (s > 0.0) {
-      beta = -copysign(sqrt(x0 * x0 + s), x0);
-      v0 = x0 - beta;
-      t = (beta - x0) / beta;
+// ---------------------------------------------------------------------------------------------
+// Householder steps.  What bounds them is the FP64 pipe: one warp-instruction per 19 cycles and
+// SM, an addition in a reduction as dear as a fused multiply-add, and a scalar square root or
+// division (9 such instructions) repeated by 16 warps dearer than the column work of a small
+// step.  So:
+//  - a warp takes four columns at a time and sums their four inner products together
+//    (warp_sum4: 6 additions instead of 20); the scalars that follow (the multiplier, the new
+//    entry of R, the downdated norm) are then formed for the four columns by one instruction
+//    each, in the lanes that hold their sums; the columns stay in registers from the inner
+//    product to the update;
+//  - the reflector is not scaled: v = (v_0, x_{j+1}, ...) with x the column as it is, and
+//    H y = y - v (v.y) rn rv with rn = 1 / ||x_j..||, rv = 1 / |v_0| (v.v / 2 = ||x|| |v_0|; two
+//    factors, so that neither over- nor underflows before ||x||^2 does).  One warp forms these
+//    while the others already take their columns' inner products with x, which need no scalar.
+// Measured: the two 16-column QRs of a 164 x 132 tile took 580k SM cycles before, 18k a step;
+// recompression of the 1D-chain product (N = 512) 757 -> 485 us, the build of the 3D lattice at
+// N = 4096 (pivoted QR of every block) 28.5 -> 24.5 ms.
+// ---------------------------------------------------------------------------------------------
+constexpr int kRowsPerLane = CLR_MAX_CLUSTER / 32;
+constexpr int kGroup = 4;   // columns a warp takes together
+
+// The warp's sums of s[0..3]: lane l receives the sum of s[l / 8].
+__device__ __forceinline__ double warp_sum4(const double (&s)[kGroup]) {
+  const int l = threadIdx.x % 32;
+  const bool h16 = (l & 16) != 0, h8 = (l & 8) != 0;
+  double a0 = h16 ? s[2] : s[0], a1 = h16 ? s[3] : s[1];
+  a0 += __shfl_xor_sync(0xffffffffu, h16 ? s[0] : s[2], 16);
+  a1 += __shfl_xor_sync(0xffffffffu, h16 ? s[1] : s[3], 16);
+  double a = h8 ? a1 : a0;
+  a += __shfl_xor_sync(0xffffffffu, h8 ? a0 : a1, 8);
+  a += __shfl_xor_sync(0xffffffffu, a, 4);
+  a += __shfl_xor_sync(0xffffffffu, a, 2);
+  a += __shfl_xor_sync(0xffffffffu, a, 1);
+  return a;
+}
+
+__device__ __forceinline__ void group_sync(int bar, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(threads) : "memory");
+}
+
+// Up to four columns held by a warp (rows l, l + 32, ... of n; nt = ceil(n / 32)).  The reflector
+// x is read again where it is used: the registers hold the four columns.
+struct ColGroup {
+  double y[kGroup][kRowsPerLane];
+  template <class Col>
+  __device__ __forceinline__ double load_dot(const double* x, int n, int nt, int c0, int ncol,
+                                             Col col) {
+    const int l = threadIdx.x % 32;
+    const double* yc[kGroup];
+    double s[kGroup];
+#pragma unroll
+    for (int c = 0; c < kGroup; ++c) {
+      s[c] = 0.0;
+      yc[c] = col(c0 + c < ncol ? c0 + c : c0);
     }
-    __syncthreads();
-    if (s > 0.0) {
-      const double inv = 1.0 / v0;
-      for (int i = j + 1 + threadIdx.x; i < p; i += kThreads) col[i] *= inv;
+#pragma unroll
+    for (int t = 0; t < kRowsPerLane; ++t)
+      if (t < nt) {
+        const bool in = l + 32 * t < n;
+#pragma unroll
+        for (int c = 0; c < kGroup; ++c) y[c][t] = in ? yc[c][l + 32 * t] : 0.0;
+      }
+#pragma unroll
+    for (int t = 0; t < kRowsPerLane; ++t)
+      if (t < nt) {
+        const double xv = l + 32 * t < n ? x[l + 32 * t] : 0.0;
+#pragma unroll
+        for (int c = 0; c < kGroup; ++c)
+          if (c0 + c < ncol) s[c] = fma(xv, y[c][t], s[c]);
+      }
+    return warp_sum4(s);
+  }
+  // y_c -= f_c x, f_c in the lanes 8 c .. 8 c + 7
+  template <class Col>
+  __device__ __forceinline__ void update_store(const double* x, double f, int n, int nt, int c0,
+                                               int ncol, Col col) {
+    const int l = threadIdx.x % 32;
+    double fc[kGroup];
+    double* yc[kGroup];
+#pragma unroll
+    for (int c = 0; c < kGroup; ++c) {
+      fc[c] = __shfl_sync(0xffffffffu, f, 8 * c);
+      yc[c] = col(c0 + c < ncol ? c0 + c : c0);
     }
-    if (threadIdx.x == 0) {
-      col[j] = beta;
-      tau[j] = t;
-    }
-    __syncthreads();
-    if (t != 0.0) {
-      for (int c = j + 1 + w; c < q; c += kWarps) {
-        double* y = a + (int64_t)c * lda;
-        double d = 0.0;
-        for (int i = j + 1 + l; i < p; i += 32) d += col[i] * y[i];
-        d = warp_sum(d) + y[j];
-        const double f = t * d;
-        if (l == 0) y[j] -= f;
-        for (int i = j + 1 + l; i < p; i += 32) y[i] -= f * col[i];
+#pragma unroll
+    for (int t = 0; t < kRowsPerLane; ++t)
+      if (t < nt) {
+        const bool in = l + 32 * t < n;
+        const double xv = in ? x[l + 32 * t] : 0.0;
+#pragma unroll
+        for (int c = 0; c < kGroup; ++c)
+          if (c0 + c < ncol) {
+            y[c][t] = fma(-fc[c], xv, y[c][t]);
+            if (in) yc[c][l + 32 * t] = y[c][t];
+          }
+      }
+  }
+  __device__ __forceinline__ double sum_squares(int nt, int c0, int ncol) const {
+    double s[kGroup];
+#pragma unroll
+    for (int c = 0; c < kGroup; ++c) {
+      s[c] = 0.0;
+      if (c0 + c < ncol) {
+#pragma unroll
+        for (int t = 0; t < kRowsPerLane; ++t)
+          if (t < nt) s[c] = fma(y[c][t], y[c][t], s[c]);
       }
     }
-    __syncthreads();
+    return warp_sum4(s);
+  }
+};
+
+// The reflector of a column (x0 above the n rows x), by one warp: *v0, *rn, *rv as above (rn =
+// 0 and H = I when the rows below are zero) and the new diagonal entry (returned).
+__device__ __forceinline__ double make_reflector(const double* x, int n, double x0, double* v0,
+                                                 double* rn, double* rv) {
+  double s = 0.0;
+  for (int i = threadIdx.x % 32; i < n; i += 32) s = fma(x[i], x[i], s);
+  s = warp_sum(s);
+  double beta = x0, a = 0.0, b = 0.0, c = 0.0;
+  if (s > 0.0) {
+    const double nrm = sqrt(fma(x0, x0, s));
+    a = x0 + copysign(nrm, x0);
+    b = 1.0 / nrm;
+    c = 1.0 / fabs(a);
+    beta = -copysign(nrm, x0);
+  }
+  *v0 = a;
+  *rn = b;
+  *rv = c;
+  return beta;
+}
+
+// The reflectors of one QR in shared memory: H_j = I - v v^T rn[j] rv[j], v = (v0[j], rows
+// below the diagonal of column j).
+struct Reflectors {
+  double v0[CLR_MAX_CLUSTER], rn[CLR_MAX_CLUSTER], rv[CLR_MAX_CLUSTER];
+};
+
+// In-place Householder QR of the p x q column-major matrix a (ld p), p >= q, by the nw warps of
+// a group (warp w of it; bar: the group's named barrier).  R is left in the upper triangle, the
+// reflector rows below it.
+__device__ __noinline__ void householder_qr(double* a, int p, int q, Reflectors& h, int w, int nw,
+                                            int bar) {
+  const int l = threadIdx.x % 32;
+  for (int j = 0; j < q; ++j) {
+    double* cj = a + (int64_t)j * p;
+    const int n = p - j - 1, nt = (n + 31) / 32, ncol = q - j - 1;
+    auto col = [&](int c) { return a + (int64_t)(j + 1 + c) * p + j + 1; };
+    const double* x = cj + j + 1;
+    ColGroup g;
+    double d = 0.0;
+    if (w == 0) {
+      double v0, rn, rv;
+      const double beta = make_reflector(x, n, cj[j], &v0, &rn, &rv);
+      __syncwarp();
+      if (l == 0) {
+        cj[j] = beta;
+        h.v0[j] = v0;
+        h.rn[j] = rn;
+        h.rv[j] = rv;
+      }
+    } else if (kGroup * (w - 1) < ncol) {
+      d = g.load_dot(x, n, nt, kGroup * (w - 1), ncol, col);
+    }
+    group_sync(bar, 32 * nw);
+    const double v0 = h.v0[j], rn = h.rn[j], rv = h.rv[j];
+    // the groups taken above, then the rest over all warps
+    for (int gi = w > 0 ? w - 1 : nw - 1; kGroup * gi < ncol; gi = (gi < nw - 1 ? nw - 1 + w : gi + nw)) {
+      const int c0 = kGroup * gi, c = c0 + l / 8;
+      if (gi >= nw - 1) d = g.load_dot(x, n, nt, c0, ncol, col);
+      const double yj = c < ncol ? col(c)[-1] : 0.0;
+      const double f = fma(v0, yj, d) * rn * rv;
+      g.update_store(x, f, n, nt, c0, ncol, col);
+      if (c < ncol && l % 8 == 0) col(c)[-1] = fma(-f, v0, yj);
+    }
+    group_sync(bar, 32 * nw);
   }
 }
 
-// y (p x r, ld ldy) <- Q y with Q = H_0 H_1 ... H_{q-1} from householder_qr.
-__device__ void apply_q(const double* v, int p, int q, int64_t ldv, const double* tau,
-                        double* y, int r, int64_t ldy) {
-  const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int j = q - 1; j >= 0; --j) {
-    const double t = tau[j];
-    if (t != 0.0) {
-      const double* vj = v + (int64_t)j * ldv;
-      for (int c = w; c < r; c += kWarps) {
-        double* yc = y + (int64_t)c * ldy;
-        double d = 0.0;
-        for (int i = j + 1 + l; i < p; i += 32) d += vj[i] * yc[i];
-        d = warp_sum(d) + yc[j];
-        const double f = t * d;
-        if (l == 0) yc[j] -= f;
-        for (int i = j + 1 + l; i < p; i += 32) yc[i] -= f * vj[i];
-      }
+// y (p x r, ld ldy) <- Q y with Q = H_0 H_1 ... H_{k-1}; the rows of reflector j are in column
+// perm[j] (j when perm is null) of v (ld p).  Each warp carries its four columns of y through all
+// reflectors in registers: no step waits for another warp.
+__device__ __noinline__ void apply_q(const double* v, int p, int k, const Reflectors& h,
+                                     const int* perm, double* y, int r, int64_t ldy, int w,
+                                     int nw) {
+  const int l = threadIdx.x % 32;
+  const int nt = (p + 31) / 32;
+  for (int g0 = kGroup * w; g0 < r; g0 += kGroup * nw) {
+    double yr[kGroup][kRowsPerLane];
+#pragma unroll
+    for (int c = 0; c < kGroup; ++c)
+#pragma unroll
+      for (int t = 0; t < kRowsPerLane; ++t)
+        yr[c][t] = g0 + c < r && l + 32 * t < p ? y[l + 32 * t + (int64_t)(g0 + c) * ldy] : 0.0;
+    for (int j = k - 1; j >= 0; --j) {
+      const double* vj = v + (int64_t)(perm ? perm[j] : j) * p;
+      const int t0 = j / 32;
+      const double v0 = h.v0[j];
+      double s[kGroup];
+      auto xv = [&](int i) { return i > j && i < p ? vj[i] : (i == j ? v0 : 0.0); };
+#pragma unroll
+      for (int c = 0; c < kGroup; ++c) s[c] = 0.0;
+#pragma unroll
+      for (int t = 0; t < kRowsPerLane; ++t)
+        if (t >= t0 && t < nt) {
+          const double x = xv(l + 32 * t);
+#pragma unroll
+          for (int c = 0; c < kGroup; ++c)
+            if (g0 + c < r) s[c] = fma(x, yr[c][t], s[c]);
+        }
+      const double f = warp_sum4(s) * h.rn[j] * h.rv[j];
+      double fc[kGroup];
+#pragma unroll
+      for (int c = 0; c < kGroup; ++c) fc[c] = __shfl_sync(0xffffffffu, f, 8 * c);
+#pragma unroll
+      for (int t = 0; t < kRowsPerLane; ++t)
+        if (t >= t0 && t < nt) {
+          const double x = xv(l + 32 * t);
+#pragma unroll
+          for (int c = 0; c < kGroup; ++c)
+            if (g0 + c < r) yr[c][t] = fma(-fc[c], x, yr[c][t]);
+        }
     }
-    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < kGroup; ++c)
+#pragma unroll
+      for (int t = 0; t < kRowsPerLane; ++t)
+        if (g0 + c < r && l + 32 * t < p) y[l + 32 * t + (int64_t)(g0 + c) * ldy] = yr[c][t];
   }
 }
 
@@ -346,6 +524,7 @@ struct SvdShared {
   double red[kWarps];
   double sigma[CLR_MAX_CLUSTER];    // by column
   double sorted[CLR_MAX_CLUSTER];   // descending
+  double sigma_inv[CLR_MAX_CLUSTER];   // tail_lower_bound_sq: 1 / R_ii
   int perm[CLR_MAX_CLUSTER];        // sorted position -> column
   int flag;
   int v_tracked;  // svd_mixed: 1 when v holds the right singular vectors (else recover_right)
@@ -353,10 +532,9 @@ struct SvdShared {
                   // reached): the right factor needs the least-squares form (ls_solve)
   int rank;
   double kept_sq;
-  // pivoted QR pre-reduction (compress_by_pivoted_qr): reflector coefficients and column order
-  double qr_tau[CLR_MAX_CLUSTER];
-  int qr_perm[CLR_MAX_CLUSTER];
-  int qr_pivot;
+  // reflectors of the pivoted QR, of rrqr_block, or of the QR route's X factor; and of its W
+  Reflectors refl, refl_w;
+  int qr_perm[CLR_MAX_CLUSTER];   // pivoted QR: column order (columns are not moved)
   double cert;    // tail_lower_bound_sq's result
   // compress_by_pivoted_qr: each column's trailing norm^2 when it was last summed exactly (the
   // downdated norms are recomputed once they fall below kDowndateFloor of it), and the FMAs
@@ -369,47 +547,67 @@ struct SvdShared {
 // so the relative error stays below ~1e-9 between recomputations.
 constexpr double kDowndateFloor = 1e-6;
 
-// Column norms of g, their descending order, and the truncation rank at eps.
+// Column norms of g, their descending order, and the truncation rank at eps.  (Norms >= 0 are
+// ordered by their bit patterns: integer comparisons instead of q^2 on the FP64 pipe, and the
+// rank from one warp's suffix sums instead of a serial chain with a square root per step.)
 __device__ void sort_and_truncate(const double* g, int p, int q, int64_t ldg, double eps,
                                   SvdShared& sh) {
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int c = w; c < q; c += kWarps) {
-    const double* gc = g + (int64_t)c * ldg;
-    double s = 0.0;
-    for (int i = l; i < p; i += 32) s = fma(gc[i], gc[i], s);
-    s = warp_sum(s);
-    if (l == 0) sh.sigma[c] = sqrt(s);
+  for (int c0 = kGroup * w; c0 < q; c0 += kGroup * kWarps) {
+    double s[kGroup];
+#pragma unroll
+    for (int c = 0; c < kGroup; ++c) {
+      s[c] = 0.0;
+      if (c0 + c < q) {
+        const double* gc = g + (int64_t)(c0 + c) * ldg;
+        for (int i = l; i < p; i += 32) s[c] = fma(gc[i], gc[i], s[c]);
+      }
+    }
+    const double d = warp_sum4(s);
+    if (l % 8 == 0 && c0 + l / 8 < q) sh.sigma[c0 + l / 8] = d;
   }
   __syncthreads();
+  for (int c = threadIdx.x; c < q; c += kThreads) sh.sigma[c] = sqrt(sh.sigma[c]);
+  __syncthreads();
   for (int j = threadIdx.x; j < q; j += kThreads) {
-    const double sj = sh.sigma[j];
+    const unsigned long long sj = (unsigned long long)__double_as_longlong(sh.sigma[j]);
     int pos = 0;
     for (int i = 0; i < q; ++i) {
-      const double si = sh.sigma[i];
+      const unsigned long long si = (unsigned long long)__double_as_longlong(sh.sigma[i]);
       pos += (si > sj) || (si == sj && i < j);
     }
     sh.perm[pos] = j;
-    sh.sorted[pos] = sj;
+    sh.sorted[pos] = sh.sigma[j];
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // smallest r with sqrt(sum_{i >= r} s_i^2) <= eps
-    double tail = 0.0;
-    int r = q;
-    for (int i = q - 1; i >= 0; --i) {
-      const double nt = tail + sh.sorted[i] * sh.sorted[i];
-      if (sqrt(nt) <= eps) {
-        tail = nt;
-        r = i;
-      } else {
-        break;
-      }
+  if (w == 0) {
+    // smallest r with sum_{i >= r} s_i^2 <= eps^2: lane l sums chunk l from the small end
+    const int ch = (q + 31) / 32;
+    const int hi = q - l * ch, lo = hi - ch > 0 ? hi - ch : 0;   // indices [lo, hi)
+    double own = 0.0;
+    for (int i = hi - 1; i >= lo; --i) own = fma(sh.sorted[i], sh.sorted[i], own);
+    double incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (l >= o) incl += v;
     }
-    if (q == 0) r = 0;
+    double tail = __shfl_up_sync(0xffffffffu, incl, 1);
+    if (l == 0) tail = 0.0;
+    const double eps2 = eps * eps;
+    int dropped = 0;
     double kept = 0.0;
-    for (int i = 0; i < r; ++i) kept += sh.sorted[i] * sh.sorted[i];
-    sh.rank = r;
-    sh.kept_sq = kept;
+    for (int i = hi - 1; i >= lo; --i) {
+      const double s2 = sh.sorted[i] * sh.sorted[i];
+      tail += s2;
+      if (tail <= eps2) ++dropped; else kept += s2;
+    }
+    dropped = __reduce_add_sync(0xffffffffu, dropped);
+    kept = warp_sum(kept);
+    if (l == 0) {
+      sh.rank = q - dropped;
+      sh.kept_sq = kept;
+    }
   }
   __syncthreads();
 }
@@ -723,7 +921,7 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
 // ---------------------------------------------------------------------------------------------
 // ROUTE_QR tiles: X_cat (m x R) and W_cat (n x R) in the workspace slot.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) compress_qr_kernel(MatView C, const int* list,
+__global__ void __launch_bounds__(kThreads, 1) compress_qr_kernel(MatView C, const int* list,
                                                                const int* count,
                                                                const int* rsum, double* ws,
                                                                double* svd_scratch,
@@ -743,13 +941,14 @@ __global__ void __launch_bounds__(kThreads) compress_qr_kernel(MatView C, const 
     const int64_t sC = slot_of(C, I, J, m);
     double* Xc = ws + 2 * sC;
     double* Wc = Xc + (int64_t)m * R;
-    double* tauX = Wc + (int64_t)n * R;
-    double* tauW = tauX + R;
-    double* M = tauW + R;
+    double* M = Wc + (int64_t)n * R;
     double* V = M + (int64_t)R * R;
     double* G = V + (int64_t)R * R;
-    householder_qr(Xc, m, R, m, tauX, sh.red);
-    householder_qr(Wc, n, R, n, tauW, sh.red);
+    // the two QRs at once, eight warps each
+    const int half = threadIdx.x / (kThreads / 2), hw = (threadIdx.x / 32) % (kWarps / 2);
+    householder_qr(half ? Wc : Xc, half ? n : m, R, half ? sh.refl_w : sh.refl, hw, kWarps / 2,
+                   1 + half);
+    __syncthreads();
     // M = R_X R_W^T (both upper triangular R x R)
     for (int e = threadIdx.x; e < R * R; e += kThreads) {
       const int a = e % R, b = e / R;
@@ -790,8 +989,11 @@ __global__ void __launch_bounds__(kThreads) compress_qr_kernel(MatView C, const 
                         : V[j + (int64_t)c * R] / (sh.sorted[c] * sh.sorted[c]);
     }
     __syncthreads();
-    apply_q(Xc, m, R, m, tauX, Xo, r, m);
-    apply_q(Wc, n, R, n, tauW, Wo, r, n);
+    // (W's column groups start three warps on, so that few columns spread over the four
+    // sub-partitions' FP64 pipes)
+    apply_q(half ? Wc : Xc, half ? n : m, R, half ? sh.refl_w : sh.refl, nullptr,
+            half ? Wo : Xo, r, half ? n : m, half ? (hw + 5) % (kWarps / 2) : hw, kWarps / 2);
+    __syncthreads();
     if (jstats && threadIdx.x == 0) {
       // Householder QRs 2(m+n)R^2, core R_X R_W^T (2/3)R^3, recovery 2R^2 r (when not
       // accumulated), re-expansion 4(m+n)R r
@@ -843,8 +1045,8 @@ void launch_compress_qr(const MatView& C, const int* list, const int* count, con
 // QR with greedy column pivoting (at step j the remaining column of largest norm over rows
 // j..m-1, first maximum; the norms are recomputed exactly every step), stopped at the first j
 // whose trailing block has ||R_22||_F <= eps.  g: m x n work copy (ld m); on return its upper
-// trapezoid holds R, the reflectors lie below the diagonal (v_0 = 1), tau in sh.sorted and the
-// column order in sh.perm.  Returns the rank r.
+// trapezoid holds R, the reflector rows lie below the diagonal (sh.refl), the column order is in
+// sh.perm.  Returns the rank r.
 // ---------------------------------------------------------------------------------------------
 __device__ int rrqr_block(const double* S, int64_t s_r, int64_t s_c, int m, int n, double eps,
                           double* g, SvdShared& sh) {
@@ -897,38 +1099,32 @@ __device__ int rrqr_block(const double* S, int64_t s_r, int64_t s_c, int m, int 
       }
     }
     __syncthreads();
-    // Householder reflector of column j below the diagonal (as householder_qr)
-    double* col = g + (int64_t)j * m;
-    double part = 0.0;
-    for (int i = j + 1 + threadIdx.x; i < m; i += kThreads) part += col[i] * col[i];
-    const double s = block_sum(part, sh.red);
-    const double x0 = col[j];
-    double t = 0.0, beta = x0, v0 = 1.0;
-    if (s > 0.0) {
-      beta = -copysign(sqrt(x0 * x0 + s), x0);
-      v0 = x0 - beta;
-      t = (beta - x0) / beta;
-    }
-    __syncthreads();
-    if (s > 0.0) {
-      const double inv = 1.0 / v0;
-      for (int i = j + 1 + threadIdx.x; i < m; i += kThreads) col[i] *= inv;
-    }
-    if (threadIdx.x == 0) {
-      col[j] = beta;
-      sh.sorted[j] = t;
-    }
-    __syncthreads();
-    if (t != 0.0) {
-      for (int c = j + 1 + w; c < n; c += kWarps) {
-        double* y = g + (int64_t)c * m;
-        double d = 0.0;
-        for (int i = j + 1 + l; i < m; i += 32) d += col[i] * y[i];
-        d = warp_sum(d) + y[j];
-        const double f = t * d;
-        if (l == 0) y[j] -= f;
-        for (int i = j + 1 + l; i < m; i += 32) y[i] -= f * col[i];
+    // Householder reflector of column j and its application (as householder_qr)
+    double* cj = g + (int64_t)j * m;
+    const int nr = m - j - 1, nt = (nr + 31) / 32, ncol = n - j - 1;
+    auto col = [&](int c) { return g + (int64_t)(j + 1 + c) * m + j + 1; };
+    const double* x = cj + j + 1;
+    if (w == 0) {
+      double v0, rn, rv;
+      const double beta = make_reflector(x, nr, cj[j], &v0, &rn, &rv);
+      __syncwarp();
+      if (l == 0) {
+        cj[j] = beta;
+        sh.refl.v0[j] = v0;
+        sh.refl.rn[j] = rn;
+        sh.refl.rv[j] = rv;
       }
+    }
+    __syncthreads();
+    const double v0 = sh.refl.v0[j], rn = sh.refl.rn[j], rv = sh.refl.rv[j];
+    for (int c0 = kGroup * w; c0 < ncol; c0 += kGroup * kWarps) {
+      ColGroup cg;
+      const double d = cg.load_dot(x, nr, nt, c0, ncol, col);
+      const int c = c0 + l / 8;
+      const double yj = c < ncol ? col(c)[-1] : 0.0;
+      const double f = fma(v0, yj, d) * rn * rv;
+      cg.update_store(x, f, nr, nt, c0, ncol, col);
+      if (c < ncol && l % 8 == 0) col(c)[-1] = fma(-f, v0, yj);
     }
     __syncthreads();
   }
@@ -980,39 +1176,69 @@ __device__ int rrqr_block(const double* S, int64_t s_r, int64_t s_c, int m, int 
 // values), and the Cauchy-Schwarz inequality over the K' - h smallest singular values of R_K'
 // gives  sum_{i > h} sigma_i(R_K')^2 >= (K' - h)^2 / sum_{i > h} sigma_i(R_K')^-2
 // >= (K' - h)^2 / ||R_K'^-1||_F^2.  The columns of R_K^-1 come by back substitution of the unit
-// vectors, one warp per column (x: K x K scratch); column c depends only on the leading
+// vectors, one warp per column; column c depends only on the leading
 // (c + 1) x (c + 1) triangle, so R_K'^-1 is the leading block of R_K^-1 and its squared
 // Frobenius norm a prefix sum of column norms.  Returns the largest of the K - h bounds
 // (h = K - 1: 1 / ||R_K^-1||_F^2 <= sigma_min(R_K)^2).
-__device__ double tail_lower_bound_sq(const double* g, int p, int h, int K, double* x,
-                                      SvdShared& sh) {
+__device__ __noinline__ double tail_lower_bound_sq(const double* g, int p, int h, int K,
+                                                   SvdShared& sh) {
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
+  for (int i = threadIdx.x; i < K; i += kThreads)
+    sh.sigma_inv[i] = 1.0 / g[i + (int64_t)sh.qr_perm[i] * p];
+  __syncthreads();
+  // column c by columns of R from the last: x_i is final when its turn comes and is subtracted
+  // from the rows above it, so no step needs a reduction (with an inner product and a division
+  // per entry this test took half of a certified tile's time)
   for (int c = w; c < K; c += kWarps) {
-    double* xc = x + (int64_t)c * K;
-    double s2 = 0.0;
-    for (int i = c; i >= 0; --i) {
-      double d = 0.0;
-      for (int t = i + 1 + l; t <= c; t += 32) d = fma(g[i + (int64_t)t * p], xc[t], d);
-      d = warp_sum(d);
-      const double rhs = (i == c ? 1.0 : 0.0) - d;
-      const double xi = rhs / g[i + (int64_t)i * p];
-      __syncwarp();
-      if (l == 0) xc[i] = xi;
-      __syncwarp();
-      s2 = fma(xi, xi, s2);
+    double x[kRowsPerLane];
+#pragma unroll
+    for (int t = 0; t < kRowsPerLane; ++t) x[t] = l + 32 * t == c ? 1.0 : 0.0;
+#pragma unroll
+    for (int b = kRowsPerLane - 1; b >= 0; --b) {
+      if (32 * b > c) continue;
+      for (int i = min(c, 32 * b + 31); i >= 32 * b; --i) {
+        const double* ri = g + (int64_t)sh.qr_perm[i] * p;
+        const double xi = __shfl_sync(0xffffffffu, x[b], i - 32 * b) * sh.sigma_inv[i];
+#pragma unroll
+        for (int t = 0; t < kRowsPerLane; ++t)
+          if (t <= b) {
+            const double u = l + 32 * t < i ? ri[l + 32 * t] : 0.0;
+            x[t] = fma(-u, xi, x[t]);
+          }
+        if (l == i - 32 * b) x[b] = xi;
+      }
     }
+    double s2 = 0.0;
+#pragma unroll
+    for (int t = 0; t < kRowsPerLane; ++t)
+      if (32 * t <= c) s2 = fma(x[t], x[t], s2);
+    s2 = warp_sum(s2);
     if (l == 0) sh.sorted[c] = s2;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double f = 0.0, best = 0.0;
-    for (int c = 0; c < K; ++c) {
+  if (w == 0) {
+    // the prefix sums f_c, until a zero pivot makes them useless, and the best bound
+    const int ch = (K + 31) / 32, lo = l * ch, hi = min(K, lo + ch);
+    double own = 0.0;
+    for (int c = lo; c < hi; ++c) own += sh.sorted[c];
+    double incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (l >= o) incl += v;
+    }
+    double f = __shfl_up_sync(0xffffffffu, incl, 1);
+    if (l == 0) f = 0.0;
+    double best = 0.0;
+    for (int c = lo; c < hi; ++c) {
       f += sh.sorted[c];
       if (!(f > 0.0) || !isfinite(f)) break;   // a zero pivot: no larger K' bounds anything
       const int kk = c + 1;
       if (kk > h) best = fmax(best, (double)(kk - h) * (double)(kk - h) / f);
     }
-    sh.cert = best;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
+    if (l == 0) sh.cert = best;
   }
   __syncthreads();
   return sh.cert;
@@ -1061,39 +1287,61 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
   bool exact = true;   // the trailing norms were all summed exactly at this step
   int k = -1;
   for (int j = 0; j <= q; ++j) {
-    // trailing norm and pivot (warp 0)
+    // pivot (warp 0): the largest trailing norm, first maximum (norms >= 0: compared as
+    // integers); their sum only when the largest could let it meet the threshold.  Columns are
+    // exchanged in the order qr_perm, not moved.
     if (w == 0) {
-      double tot = 0.0, best = -1.0;
+      unsigned long long best = 0;
       int arg = j;
       for (int c = j + l; c < q; c += 32) {
-        const double v = sh.sigma[c];
-        tot += v;
+        const unsigned long long v = (unsigned long long)__double_as_longlong(sh.sigma[c]);
         if (v > best) { best = v; arg = c; }
       }
-      tot = warp_sum(tot);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
         const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
         if (ob > best || (ob == best && oa < arg)) { best = ob; arg = oa; }
       }
+      double tot = __longlong_as_double((long long)best);
+      if (tot <= tau2) {
+        tot = 0.0;
+        for (int c = j + l; c < q; c += 32) tot += sh.sigma[c];
+        tot = warp_sum(tot);
+      }
       if (l == 0) {
         sh.kept_sq = tot;
-        sh.qr_pivot = arg;
+        if (!(tot <= tau2) && arg != j) {
+          const double t = sh.sigma[j];
+          sh.sigma[j] = sh.sigma[arg];
+          sh.sigma[arg] = t;
+          const double tr = sh.qr_nref[j];
+          sh.qr_nref[j] = sh.qr_nref[arg];
+          sh.qr_nref[arg] = tr;
+          const int ti = sh.qr_perm[j];
+          sh.qr_perm[j] = sh.qr_perm[arg];
+          sh.qr_perm[arg] = ti;
+        }
       }
     }
     __syncthreads();
     if (sh.kept_sq <= tau2 && !exact) {
       // the downdated norms meet the threshold: sum the trailing norms exactly and decide (and
       // pivot) on those
-      for (int c = j + w; c < q; c += kWarps) {
-        const double* y = g + (int64_t)c * p;
-        double s2 = 0.0;
-        for (int i = j + l; i < p; i += 32) s2 = fma(y[i], y[i], s2);
-        s2 = warp_sum(s2);
-        if (l == 0) {
-          sh.sigma[c] = s2;
-          sh.qr_nref[c] = s2;
+      for (int c0 = j + kGroup * w; c0 < q; c0 += kGroup * kWarps) {
+        double s2[kGroup];
+#pragma unroll
+        for (int c = 0; c < kGroup; ++c) {
+          s2[c] = 0.0;
+          if (c0 + c < q) {
+            const double* y = g + (int64_t)sh.qr_perm[c0 + c] * p;
+            for (int i = j + l; i < p; i += 32) s2[c] = fma(y[i], y[i], s2[c]);
+          }
+        }
+        const double d = warp_sum4(s2);
+        if (l % 8 == 0 && c0 + l / 8 < q) {
+          sh.sigma[c0 + l / 8] = d;
+          sh.qr_nref[c0 + l / 8] = d;
         }
       }
       fma_count += (unsigned long long)(p - j) * (unsigned long long)(q - j);
@@ -1108,7 +1356,7 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     }
     if (j == jcert) {
       // still above the threshold after floor(q/2) + 1 steps: dense if sigma_min(R_11) > eps
-      const double b2 = tail_lower_bound_sq(g, p, jcert - 1, jcert, wv, sh);
+      const double b2 = tail_lower_bound_sq(g, p, jcert - 1, jcert, sh);
       if (jstats && threadIdx.x == 0)
         atomicAdd(&jstats[4], 2ull * fma_count + (unsigned long long)jcert * jcert * jcert / 3);
       fma_count = 0;
@@ -1116,75 +1364,60 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     }
     // (the trailing block after q steps is empty: only a non-finite norm gets here)
     if (j == q) break;
-    const int piv = sh.qr_pivot;
-    if (piv != j) {
-      double* x = g + (int64_t)j * p;
-      double* y = g + (int64_t)piv * p;
-      for (int i = threadIdx.x; i < p; i += kThreads) {
-        const double t = x[i];
-        x[i] = y[i];
-        y[i] = t;
+    // Householder reflector of the pivot column and its application to the remaining columns
+    // (as householder_qr).  The reflector keeps the norm of each column's rows j..p-1 and moves
+    // its row j into R, so the trailing norm^2 over rows j+1..p-1 is the old one minus the new
+    // row-j entry squared (downdate), summed again exactly when it has fallen below
+    // kDowndateFloor of its last exact value (or is not positive).
+    double* cj = g + (int64_t)sh.qr_perm[j] * p;
+    const int n = p - j - 1, nt = (n + 31) / 32, ncol = q - j - 1;
+    auto col = [&](int c) { return g + (int64_t)sh.qr_perm[j + 1 + c] * p + j + 1; };
+    const double* x = cj + j + 1;
+    ColGroup cg;
+    double d = 0.0;
+    if (w == 0) {
+      double v0, rn, rv;
+      const double beta = make_reflector(x, n, cj[j], &v0, &rn, &rv);
+      __syncwarp();
+      if (l == 0) {
+        cj[j] = beta;
+        sh.refl.v0[j] = v0;
+        sh.refl.rn[j] = rn;
+        sh.refl.rv[j] = rv;
       }
+    } else if (kGroup * (w - 1) < ncol) {
+      d = cg.load_dot(x, n, nt, kGroup * (w - 1), ncol, col);
     }
     __syncthreads();
-    if (piv != j && threadIdx.x == 0) {
-      const double t = sh.sigma[j];
-      sh.sigma[j] = sh.sigma[piv];
-      sh.sigma[piv] = t;
-      const double tr = sh.qr_nref[j];
-      sh.qr_nref[j] = sh.qr_nref[piv];
-      sh.qr_nref[piv] = tr;
-      const int ti = sh.qr_perm[j];
-      sh.qr_perm[j] = sh.qr_perm[piv];
-      sh.qr_perm[piv] = ti;
-    }
-    // Householder reflector of column j below the diagonal (as householder_qr)
-    double* col = g + (int64_t)j * p;
-    double part = 0.0;
-    for (int i = j + 1 + threadIdx.x; i < p; i += kThreads) part = fma(col[i], col[i], part);
-    const double sv = block_sum(part, sh.red);
-    const double x0 = col[j];
-    double t = 0.0, beta = x0, v0 = 1.0;
-    if (sv > 0.0) {
-      beta = -copysign(sqrt(x0 * x0 + sv), x0);
-      v0 = x0 - beta;
-      t = (beta - x0) / beta;
-    }
-    if (sv > 0.0) {
-      const double inv = 1.0 / v0;
-      for (int i = j + 1 + threadIdx.x; i < p; i += kThreads) col[i] *= inv;
-    }
-    if (threadIdx.x == 0) {
-      col[j] = beta;
-      sh.qr_tau[j] = t;
-    }
-    __syncthreads();
-    // apply to the remaining columns.  The reflector keeps the norm of each column's rows
-    // j..p-1 and moves its row j into R, so the trailing norm^2 over rows j+1..p-1 is the old
-    // one minus the new row-j entry squared (downdate), summed again exactly when it has fallen
-    // below kDowndateFloor of its last exact value (or is not positive).
-    for (int c = j + 1 + w; c < q; c += kWarps) {
-      double* y = g + (int64_t)c * p;
-      double d = 0.0;
-      for (int i = j + 1 + l; i < p; i += 32) d = fma(col[i], y[i], d);
-      d = warp_sum(d) + y[j];
-      const double f = t * d;
-      for (int i = j + 1 + l; i < p; i += 32) y[i] = fma(-f, col[i], y[i]);
-      const double yj = y[j] - f;
-      double nu2 = sh.sigma[c] - yj * yj;
-      if (!(nu2 > kDowndateFloor * sh.qr_nref[c])) {
-        double s2 = 0.0;
-        for (int i = j + 1 + l; i < p; i += 32) s2 = fma(y[i], y[i], s2);
-        nu2 = warp_sum(s2);
-        if (l == 0) {
-          sh.qr_nref[c] = nu2;
-          atomicAdd(&sh.qr_recomputed, (unsigned long long)(p - j - 1));
+    const double v0 = sh.refl.v0[j], rn = sh.refl.rn[j], rv = sh.refl.rv[j];
+    for (int gi = w > 0 ? w - 1 : kWarps - 1; kGroup * gi < ncol;
+         gi = (gi < kWarps - 1 ? kWarps - 1 + w : gi + kWarps)) {
+      const int c0 = kGroup * gi, c = c0 + l / 8;
+      if (gi >= kWarps - 1) d = cg.load_dot(x, n, nt, c0, ncol, col);
+      const double yj = c < ncol ? col(c)[-1] : 0.0;
+      const double f = fma(v0, yj, d) * rn * rv;
+      cg.update_store(x, f, n, nt, c0, ncol, col);
+      const double yn = fma(-f, v0, yj);
+      double nu2 = 0.0;
+      bool again = false;
+      if (c < ncol) {
+        nu2 = fma(-yn, yn, sh.sigma[j + 1 + c]);
+        again = !(nu2 > kDowndateFloor * sh.qr_nref[j + 1 + c]);
+      }
+      if (__any_sync(0xffffffffu, again)) {
+        const double s2 = cg.sum_squares(nt, c0, ncol);
+        if (again) {
+          nu2 = s2;
+          if (l % 8 == 0) {
+            sh.qr_nref[j + 1 + c] = nu2;
+            atomicAdd(&sh.qr_recomputed, (unsigned long long)n);
+          }
         }
       }
       __syncwarp();
-      if (l == 0) {
-        y[j] = yj;
-        sh.sigma[c] = nu2;
+      if (c < ncol && l % 8 == 0) {
+        col(c)[-1] = yn;
+        sh.sigma[j + 1 + c] = nu2;
       }
     }
     fma_count += 2ull * (unsigned long long)(p - j) * (unsigned long long)(q - j - 1) + (p - j);
@@ -1197,7 +1430,7 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
   if (k > jtail) {
     // dense when sum_{i > q/2} sigma_i^2 > eps^2 is certified by some leading triangle of the
     // k completed steps, else the SVD of R decides
-    const double b2 = tail_lower_bound_sq(g, p, kmax, k, wv, sh);
+    const double b2 = tail_lower_bound_sq(g, p, kmax, k, sh);
     if (jstats && threadIdx.x == 0)
       atomicAdd(&jstats[4], (unsigned long long)k * k * k / 3);
     if (b2 > eps * eps) return 2;
@@ -1217,7 +1450,7 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
   double part = 0.0;
   for (int e = threadIdx.x; e < k * q; e += kThreads) {
     const int i = e % k, c = e / k;
-    const double x = i <= c ? g[i + (int64_t)c * p] : 0.0;
+    const double x = i <= c ? g[i + (int64_t)sh.qr_perm[c] * p] : 0.0;
     rb[e] = x;
     part = fma(x, x, part);
   }
@@ -1270,7 +1503,7 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     wa[sh.qr_perm[j] + (int64_t)c * q] = ls ? v : v / sh.sorted[c];
   }
   __syncthreads();
-  apply_q(g, p, k, p, sh.qr_tau, xa, r, p);
+  apply_q(g, p, k, sh.refl, sh.qr_perm, xa, r, p, w, kWarps);
   if (threadIdx.x == 0) {
     *kind_out = CLR_KIND_LR;
     *rank_out = r;
@@ -1356,7 +1589,8 @@ __global__ void __launch_bounds__(kThreads, 1) compress_dense_kernel(
         double* Wo = slot + (int64_t)m * r;
         for (int e = threadIdx.x; e < m * r; e += kThreads) Xo[e] = (e % m == e / m) ? 1.0 : 0.0;
         __syncthreads();
-        apply_q(G, m, r, m, sh.sorted, Xo, r, m);
+        apply_q(G, m, r, sh.refl, nullptr, Xo, r, m, threadIdx.x / 32, kWarps);
+        __syncthreads();
         double part = 0.0;
         for (int e = threadIdx.x; e < n * r; e += kThreads) {
           const int c = e % n, i = e / n;
