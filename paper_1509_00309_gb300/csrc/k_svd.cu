@@ -33,7 +33,6 @@ constexpr int kFullStageCounters = 24;
 // truncation, recovery and the factors' stores; then the count
 constexpr int kPreStageCounters = 32;
 constexpr int kWarps = kThreads / 32;
-constexpr int kFp64SweepCap = 0;  // FP64 sweeps of svd_mixed when the right factor is recovered
 
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
@@ -528,8 +527,8 @@ struct SvdShared {
   int perm[CLR_MAX_CLUSTER];        // sorted position -> column
   int flag;
   int v_tracked;  // svd_mixed: 1 when v holds the right singular vectors (else recover_right)
-  int ls_recover; // svd_mixed: 1 when G's kept columns may be non-orthogonal (FP64 sweep cap
-                  // reached): the right factor needs the least-squares form (ls_solve)
+  int ls_recover; // svd_mixed: 1 when G's kept columns are orthogonal to the FP32 stages' tolerance
+                  // only: the right factor needs the least-squares form (ls_solve)
   int rank;
   double kept_sq;
   // reflectors of the pivoted QR, of rrqr_block, or of the QR route's X factor; and of its W
@@ -784,10 +783,9 @@ __device__ void right_multiply_fp64(double* m, int rows, int64_t ldm, int q, con
 //  3. FP32 sweeps on a copy of G, whose columns are rounded relative to their own norms, so
 //     the small columns are resolved against each other and against the large ones; V2
 //     orthonormalised in FP64 and G <- G V2;
-//  4. FP64 sweeps continuing on G -- a quadratically convergent clean-up from there.  The
-//     rotations are not accumulated: for kept columns G_r = U_r S_r the right factor is
-//     V_r = A^T G_r S_r^-2 (recover_right), and G_r (A^T G_r S_r^-2)^T = P A with P the
-//     orthogonal projector onto span(G_r), so rounding in V_r is scaled back by S_r.
+//  The right factor: for kept columns G_r = U_r S_r it is V_r = A^T G_r S_r^-2 (recover_right),
+//     and G_r (A^T G_r S_r^-2)^T = P A with P the orthogonal projector onto span(G_r), so
+//     rounding in V_r is scaled back by S_r; near the noise floor V is accumulated instead.
 // Pairs whose inner product is below the noise floor are not rotated: p u ||A||_F in FP32 on A,
 // and max(p u ||A||_F, 1e-3 eps) on G (columns that small cannot move a truncation at eps).
 // On return g = U S in FP64, and v the right factor when sh.v_tracked (else workspace).  sc:
@@ -873,9 +871,8 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
   const int sw32b = jacobi_svd<float>(g32, p, q, p, v32, q, max_sweeps, &sh.flag, true, 4.0f,
                                       floor_g * floor_g);
   mark(3);
-  // The FP64 sweeps rotate G alone when eps is well above the noise floor: the right factor
-  // of the kept columns is then recovered from A and G afterwards (recover_right), a p q r
-  // product instead of 4 q flops per rotation.  Near the floor (eps < 1e3 p u ||A||_F) kept
+  // When eps is well above the noise floor the right factor of the kept columns is recovered
+  // from A and G afterwards (recover_right).  Near the floor (eps < 1e3 p u ||A||_F) kept
   // columns may lie below it, unorthogonalised, where that recovery is not a projection: V is
   // accumulated instead.
   const bool track_v = floor64 > 1e-3 * eps;
@@ -890,28 +887,23 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
   }
   if (threadIdx.x == 0) sh.v_tracked = track_v ? 1 : 0;
   mark(4);
-  // Without V accumulation no FP64 sweep runs (kFp64SweepCap): after stage 3 the columns of G
-  // are orthogonal to the FP32 stages' tolerance (cosines ~1e-5 relative to their own norms),
-  // so the sorted column norms, whose tail decides the rank, are within ~1e-10 of the
-  // singular values; and with the least-squares right factor (ls_solve) X W^T is the
-  // orthogonal projection of A onto span(G_r) for any G = A V_eff with V_eff orthogonal, so the
-  // error is ||(I - P) G_tail|| <= ||G_tail||_F <= eps whether or not the kept columns are
-  // mutually orthogonal.  (One FP64 sweep, the earlier choice, took the cosines to ~1e-10 at
-  // 4 p q^2 FP64 flops; a tight cluster of singular values made it converge only linearly.)
-  const int cap64 = track_v || max_sweeps < kFp64SweepCap ? max_sweeps : kFp64SweepCap;
-  const int sw64 = cap64 > 0 ? jacobi_svd<double>(g, p, q, p, track_v ? v : nullptr, q, cap64,
-                                                  &sh.flag, false, 1.0, floor64 * floor64)
-                             : 0;
-  if (threadIdx.x == 0) sh.ls_recover = (!track_v && sw64 >= cap64) ? 1 : 0;
-  mark(5);
+  // No FP64 sweep follows: after stage 3 the columns of G are orthogonal to the FP32 stages'
+  // tolerance (cosines ~1e-5 relative to their own norms), so the sorted column norms, whose
+  // tail decides the rank, are within ~1e-10 of the singular values, and the truncation error
+  // does not depend on their being orthogonal: with V accumulated A = G V^T and dropping columns
+  // leaves ||G_tail V_tail^T||_F = ||G_tail||_F (V is orthogonal to FP64 rounding); without it,
+  // the least-squares right factor (ls_solve) makes X W^T the orthogonal projection of A onto
+  // span(G_r), with error ||(I - P) G_tail|| <= ||G_tail||_F <= eps for any G = A V_eff.
+  // (FP64 sweeps to convergence where V is accumulated, the earlier choice, took 3.6 of 12.5 G
+  // cycles of the lattice product's recompression at N = 4096.)
+  if (threadIdx.x == 0) sh.ls_recover = track_v ? 0 : 1;
   if (jstats && threadIdx.x == 0) {
     // algorithmic flops: Jacobi 4 p q^2 per sweep, orthonormalisation 2 q^3, products 2 p q^2
     const unsigned long long pq2 = (unsigned long long)p * q * q, q3 = (unsigned long long)q * q * q;
-    unsigned long long f64 = 2 * q3 + 2 * pq2 + 4 * pq2 * sw64;
+    unsigned long long f64 = 2 * q3 + 2 * pq2;
     if (sw32b > 0) f64 += 2 * q3 + 2 * pq2 + (track_v ? 2 * q3 : 0);
     atomicAdd(&jstats[0], 1ull);
     atomicAdd(&jstats[1], (unsigned long long)(sw32 + sw32b));
-    atomicAdd(&jstats[2], (unsigned long long)sw64);
     atomicAdd(&jstats[4], f64);
     atomicAdd(&jstats[5], 4 * pq2 * (unsigned long long)(sw32 + sw32b));
   }
