@@ -173,7 +173,7 @@ void clr_opts_default(clr_opts* opts);
  * not free matrices.
  * Workspaces are allocated on first use, grow to the largest product seen and stay until
  * clr_destroy.  For C = A B they take about 16 bytes per element of C's dense footprint (tile
- * accumulation and SVD workspace), 2 MiB per CTA of the low-rank and recompression kernels
+ * accumulation and SVD workspace), 2.5 MiB per CTA of the low-rank and recompression kernels
  * (2 CTAs per SM unless the autotuner picks another count), and with a tensor-core precision
  * the operands' panels: 4 (bf16x3), 6 (bf16x6) or 16 (exact slices, plus FP64 images of the
  * low-rank operand blocks) bytes per element of A and of B.  Newton-Schulz keeps a second set

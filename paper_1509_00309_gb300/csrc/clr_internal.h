@@ -59,56 +59,82 @@ __device__ __forceinline__ int next_item(int* counter, int* sh_slot) {
   return *sh_slot;
 }
 
-// out(i,j) (= or +=) sum_l a(i,l) b(l,j) for a P x Q output with arbitrary element strides, by a
-// CTA of NT threads.  FP64 runs at ~2 FMAs per clock per SM on this part, and a single
-// accumulator per thread leaves the pipe waiting on each FMA's latency and its two loads: the
-// output is cut into 4 x 2 micro-tiles (4 consecutive rows, 2 consecutive columns; the ragged
-// last ones clamped), taken by the threads in turn, so a thread runs 8 independent chains whose 6
-// loads per step feed 8 FMAs, and skinny outputs (a few dozen columns: the rank of a low-rank
-// factor) waste no lanes.  No synchronisation inside: the caller orders dependent calls.
+// out(i,j) (= or +=) sum_l a(i,l) b(l,j) for a P x Q output (column-major, ld ldo) with
+// arbitrary element strides of a and b, by a CTA of NT threads.  FP64 runs at ~2 FMAs per clock
+// per SM on this part: a warp's FMA holds its sub-partition's pipe for 64 cycles, in which the
+// loads of the next ones arrive, so what counts is that the FMAs are spread evenly over the warps
+// and waste no lanes.  The output is cut into MR x MC micro-tiles (ragged last ones clamped)
+// taken by the threads in turn, rows first (a should have unit stride along i; b is mostly
+// broadcast).  TRI = 1: a(i, l) is zero for l > i; TRI = 2: b(l, j) is zero for l < j (those
+// terms are skipped).  No synchronisation inside: the caller orders dependent calls.
+template <int NT, int MR, int MC, int TRI, class T>
+__device__ __forceinline__ void cta_gemm_micro(int P, int Q, int L, const T* a, int64_t a_r,
+                                               int64_t a_c, const T* b, int64_t b_r, int64_t b_c,
+                                               T* out, int64_t ldo, bool accumulate) {
+  const int mp = (P + MR - 1) / MR, mq = (Q + MC - 1) / MC;
+  for (int t = threadIdx.x; t < mp * mq; t += NT) {
+    const int i0 = (t % mp) * MR, j0 = (t / mp) * MC;
+    const int l0 = TRI == 2 ? j0 : 0;
+    const int l1 = TRI == 1 && i0 + MR < L ? i0 + MR : L;
+    const T* ap[MR];
+    const T* bp[MC];
+#pragma unroll
+    for (int x = 0; x < MR; ++x) ap[x] = a + (int64_t)(i0 + x < P ? i0 + x : i0) * a_r + l0 * a_c;
+#pragma unroll
+    for (int y = 0; y < MC; ++y) bp[y] = b + (int64_t)(j0 + y < Q ? j0 + y : j0) * b_c + l0 * b_r;
+    T acc[MR][MC];
+#pragma unroll
+    for (int x = 0; x < MR; ++x)
+#pragma unroll
+      for (int y = 0; y < MC; ++y) acc[x][y] = T(0);
+    for (int l = l0; l < l1; ++l) {
+      T av[MR], bv[MC];
+#pragma unroll
+      for (int x = 0; x < MR; ++x) {
+        av[x] = *ap[x];
+        ap[x] += a_c;
+      }
+#pragma unroll
+      for (int y = 0; y < MC; ++y) {
+        bv[y] = *bp[y];
+        bp[y] += b_r;
+      }
+#pragma unroll
+      for (int x = 0; x < MR; ++x)
+#pragma unroll
+        for (int y = 0; y < MC; ++y) acc[x][y] = fma(av[x], bv[y], acc[x][y]);
+    }
+#pragma unroll
+    for (int x = 0; x < MR; ++x)
+#pragma unroll
+      for (int y = 0; y < MC; ++y)
+        if (i0 + x < P && j0 + y < Q) {
+          T* o = out + (i0 + x) + (int64_t)(j0 + y) * ldo;
+          *o = accumulate ? *o + acc[x][y] : acc[x][y];
+        }
+  }
+}
+
 template <int NT>
 __device__ __forceinline__ void cta_gemm_tiled(int P, int Q, int L, const double* a,
                                                int64_t a_r, int64_t a_c, const double* b,
                                                int64_t b_r, int64_t b_c, double* out,
                                                int64_t ldo, bool accumulate) {
-  const int mp = (P + 3) / 4, mq = (Q + 1) / 2;
-  for (int t = threadIdx.x; t < mp * mq; t += NT) {
-    const int i0 = (t % mp) * 4, j0 = (t / mp) * 2;
-    const double* ap[4];
-    const double* bp[2];
-#pragma unroll
-    for (int x = 0; x < 4; ++x) ap[x] = a + (int64_t)(i0 + x < P ? i0 + x : i0) * a_r;
-#pragma unroll
-    for (int y = 0; y < 2; ++y) bp[y] = b + (int64_t)(j0 + y < Q ? j0 + y : j0) * b_c;
-    double acc[4][2];
-#pragma unroll
-    for (int x = 0; x < 4; ++x) acc[x][0] = acc[x][1] = 0.0;
-    for (int l = 0; l < L; ++l) {
-      double av[4], bv[2];
-#pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        av[x] = *ap[x];
-        ap[x] += a_c;
-      }
-#pragma unroll
-      for (int y = 0; y < 2; ++y) {
-        bv[y] = *bp[y];
-        bp[y] += b_r;
-      }
-#pragma unroll
-      for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < 2; ++y) acc[x][y] = fma(av[x], bv[y], acc[x][y]);
-    }
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int y = 0; y < 2; ++y)
-        if (i0 + x < P && j0 + y < Q) {
-          double* o = out + (i0 + x) + (int64_t)(j0 + y) * ldo;
-          *o = accumulate ? *o + acc[x][y] : acc[x][y];
-        }
-  }
+  cta_gemm_micro<NT, 4, 2, 0>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
+}
+
+// The micro-tile by the size of the output: 4 x 2 from four rounds of the CTA's threads on
+// (less than a quarter of a round idle at the end), 2 x 2 from one, else an entry per thread.
+template <int NT, int TRI = 0, class T>
+__device__ __forceinline__ void cta_gemm_auto(int P, int Q, int L, const T* a, int64_t a_r,
+                                              int64_t a_c, const T* b, int64_t b_r, int64_t b_c,
+                                              T* out, int64_t ldo) {
+  if (P * Q >= 32 * NT)
+    cta_gemm_micro<NT, 4, 2, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, false);
+  else if (P * Q >= 4 * NT)
+    cta_gemm_micro<NT, 2, 2, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, false);
+  else
+    cta_gemm_micro<NT, 1, 1, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, false);
 }
 
 struct Triple {
@@ -196,8 +222,9 @@ void launch_lr_products(const MatView& A, const MatView& B, const MatView& C, co
 // k_svd.cu
 // jstats (may be null): device counters {svd blocks, FP32 sweeps, FP64 sweeps, early dense}
 // svd_scratch: grid x kSvdScratchPerCta doubles (FP32 working copies and an FP64 q x q factor
-// of the mixed-precision SVD, then the pivoted-QR path's R and the right factor of its SVD).
-constexpr int64_t kSvdScratchPerCta = (int64_t)4 * CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
+// of the mixed-precision SVD, the pivoted-QR path's right factor and R, then the
+// orthonormalisations' E).
+constexpr int64_t kSvdScratchPerCta = (int64_t)5 * CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
 // sched: a zeroed work counter (dynamic tile distribution).
 void launch_compress_qr(const MatView& C, const int* list, const int* count, const int* rsum,
                         double* ws, double* svd_scratch, double eps, int max_sweeps, int grid,

@@ -15,7 +15,8 @@
 //                          (mixed FP32/FP64 stages, svd_mixed);
 //   rank-revealing QR      the paper's construction for building from dense (option).
 // FP64 working arrays live in the tile's workspace slot (2 m n doubles per tile, enough for
-// either route); the FP32 copies of the mixed-precision SVD in a per-CTA scratch (L1-cached).
+// either route); the FP32 copies of the mixed-precision SVD in shared memory, or in a per-CTA
+// scratch where they do not fit.
 #include <cfloat>
 #include <mutex>
 
@@ -183,9 +184,10 @@ __device__ __forceinline__ double make_reflector(const double* x, int n, double 
   s = warp_sum(s);
   double beta = x0, a = 0.0, b = 0.0, c = 0.0;
   if (s > 0.0) {
-    const double nrm = sqrt(fma(x0, x0, s));
+    const double t2 = fma(x0, x0, s);
+    b = rsqrt(t2);
+    const double nrm = t2 * b;
     a = x0 + copysign(nrm, x0);
-    b = 1.0 / nrm;
     c = 1.0 / fabs(a);
     beta = -copysign(nrm, x0);
   }
@@ -340,7 +342,10 @@ __device__ __forceinline__ float rot_tangent(float d, float g) {
 __device__ __forceinline__ void rotation(float al, float be, float g, float& c, float& s,
                                          float& t) {
   t = rot_tangent(be - al, g);
-  c = rsqrtf(1.f + t * t);
+  // (one Newton step on the approximate root: c^2 + s^2 drifts less from 1 over many rotations)
+  const float u = 1.f + t * t;
+  c = rsqrtf(u);
+  c = c * (1.5f - 0.5f * u * c * c);
   s = c * t;
 }
 __device__ __forceinline__ void rotation(double al, double be, double g, double& c, double& s,
@@ -519,6 +524,224 @@ __device__ int jacobi_svd(T* g, int p, int q, int64_t ldg, T* v, int64_t ldv,
   return sweep;
 }
 
+// One-sided Jacobi in FP32 with the working copies in shared memory (or, where they do not fit,
+// in the per-CTA scratch): the same sweeps, tests and skips as jacobi_svd, for the FP32 stages of
+// svd_mixed.  What bounds it is the latency of a round (a column pair's inner product, its
+// rotation, and a barrier), so a round is kept short:
+//  - LP lanes per pair and kPer rows a lane, so that a round's pairs fill the CTA once where
+//    they can: a warp alone issues an instruction every ~5 cycles, so a round costs what one of
+//    its warps has to issue (about 80 instructions and 12 a row);
+//  - the columns in shared memory;
+//  - only the warps that have pairs take part, with their own barrier (none for a single warp).
+// Measured (core of 16 columns, both FP32 stages): 259k SM cycles with the copies in the global
+// scratch, a warp per pair and 8 masked rows a lane; 190k now.
+// ldg, ldv: odd multiples of LP where LP < 32, so that the pairs of a warp meet different banks.
+// v is reset to I.
+struct JacobiShared {
+  float nrm2[CLR_MAX_CLUSTER];     // column norms squared
+  int last_rot[CLR_MAX_CLUSTER];   // the step of the column's last rotation, -1 if none
+  int rotated, sweeps;
+};
+
+template <int LP, int kPer>
+__device__ __noinline__ int jacobi32(float* g, int p, int q, int ldg, float* v, int ldv,
+                                     int max_sweeps, float floor2, JacobiShared& sh) {
+  float* nrm2 = sh.nrm2;
+  int* last_rot = sh.last_rot;
+  constexpr unsigned kAll = 0xffffffffu;
+  const int w = threadIdx.x / 32, li = threadIdx.x % LP, grp = threadIdx.x / LP;
+  const int qq = q + (q & 1), half = qq / 2;   // slot q is a dummy when q is odd
+  const int n_act = min(kWarps, (half * LP + 31) / 32);   // warps with pairs
+  const int ngrp = n_act * (32 / LP);
+  for (int e = threadIdx.x; e < q * q; e += kThreads)
+    v[(e % q) + (e / q) * ldv] = (e % q == e / q) ? 1.f : 0.f;
+  for (int c = threadIdx.x; c < q; c += kThreads) last_rot[c] = -1;
+  __syncthreads();
+  if (w < n_act) {
+    auto act_sync = [&]() {
+      if (n_act == 1) __syncwarp(); else group_sync(3, 32 * n_act);
+    };
+    auto sum_lp = [&](float x) {
+#pragma unroll
+      for (int o = LP / 2; o > 0; o >>= 1) x += __shfl_xor_sync(kAll, x, o);
+      return x;
+    };
+    const float tol = FLT_EPSILON * sqrtf((float)p) * 4.0f;
+    int sweep = 0;
+    for (; sweep < max_sweeps; ++sweep) {
+      for (int c0 = 0; c0 < q; c0 += ngrp) {
+        const int c = c0 + grp;
+        float s2 = 0.f;
+        if (c < q) {
+          const float* gc = g + c * ldg;
+#pragma unroll
+          for (int j = 0; j < kPer; ++j) {
+            const float x = li + LP * j < p ? gc[li + LP * j] : 0.f;
+            s2 = fmaf(x, x, s2);
+          }
+        }
+        s2 = sum_lp(s2);
+        if (li == 0 && c < q) nrm2[c] = s2;
+      }
+      if (threadIdx.x == 0) sh.rotated = 0;
+      act_sync();
+      for (int round = 0; round < qq - 1; ++round) {
+        const int step = sweep * (qq - 1) + round;
+        for (int k0 = 0; k0 < half; k0 += ngrp) {
+          const int k = k0 + grp;
+          int a = round, b = qq - 1;
+          if (k > 0) {
+            a = round + k;
+            if (a >= qq - 1) a -= qq - 1;
+            b = round - k;
+            if (b < 0) b += qq - 1;
+          }
+          bool on = k < half && a < q && b < q;
+          float al = 0.f, be = 0.f;
+          if (on) {
+            // neither column rotated since this pair's check one sweep ago
+            on = !(sweep > 0 && last_rot[a] < step - (qq - 1) && last_rot[b] < step - (qq - 1));
+            al = nrm2[a];
+            be = nrm2[b];
+            on = on && !pair_below_floor(al, be, floor2);
+          }
+          if (!__any_sync(kAll, on)) continue;
+          float* ga = g + a * ldg;
+          float* gb = g + b * ldg;
+          float xa[kPer], xb[kPer], d = 0.f;
+#pragma unroll
+          for (int j = 0; j < kPer; ++j) {
+            const int i = li + LP * j;
+            const bool in = on && i < p;
+            xa[j] = in ? ga[i] : 0.f;
+            xb[j] = in ? gb[i] : 0.f;
+            d = fmaf(xa[j], xb[j], d);
+          }
+          d = sum_lp(d);
+          on = on && !pair_converged(al, be, d, tol, floor2);
+          if (!__any_sync(kAll, on)) continue;
+          float* va = v + a * ldv;
+          float* vb = v + b * ldv;
+          float na = al, nb = be;
+          bool again = false;
+          if (on) {
+            float ya[kPer], yb[kPer];
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+              const int i = li + LP * j;
+              ya[j] = i < q ? va[i] : 0.f;
+              yb[j] = i < q ? vb[i] : 0.f;
+            }
+            float c, sn, t;
+            rotation(al, be, d, c, sn, t);
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+              const int i = li + LP * j;
+              const float x = c * xa[j] - sn * xb[j];
+              xb[j] = sn * xa[j] + c * xb[j];
+              xa[j] = x;
+              if (i < p) {
+                ga[i] = xa[j];
+                gb[i] = xb[j];
+              }
+              if (i < q) {
+                va[i] = c * ya[j] - sn * yb[j];
+                vb[i] = sn * ya[j] + c * yb[j];
+              }
+            }
+            // a - t g and b + t g, recomputed from the rotated columns when that cancels
+            na = al - t * d;
+            nb = be + t * d;
+            again = !(na > al * 0.015625f) || !(nb > be * 0.015625f);
+          }
+          if (__any_sync(kAll, again)) {
+            float sa = 0.f, sb = 0.f;
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+              sa = fmaf(xa[j], xa[j], sa);
+              sb = fmaf(xb[j], xb[j], sb);
+            }
+            sa = sum_lp(sa);
+            sb = sum_lp(sb);
+            if (again) {
+              na = sa;
+              nb = sb;
+            }
+          }
+          if (on && li == 0) {
+            nrm2[a] = na;
+            nrm2[b] = nb;
+            last_rot[a] = step;
+            last_rot[b] = step;
+            sh.rotated = 1;
+          }
+        }
+        act_sync();
+      }
+      const int rotated = sh.rotated;
+      act_sync();
+      if (!rotated) break;
+    }
+    if (threadIdx.x == 0) sh.sweeps = sweep;
+  }
+  __syncthreads();
+  return sh.sweeps;
+}
+
+// The FP32 working copies of svd_mixed (G: p x q, V: q x q): lanes per pair and rows per lane,
+// leading dimensions and place.
+struct Work32 {
+  float *g, *v;
+  int ldg, ldv, lp, per;
+};
+// Dynamic shared memory of the recompression kernels: with their static part (27 KB) all that a
+// CTA can have, enough for a 256 x 136 pair of copies or a 158 x 158 one.
+constexpr int kSvdSmemBytes = 196 * 1024;
+
+__device__ __forceinline__ Work32 work32(int p, int q, double* sc) {
+  extern __shared__ float svd_smem[];
+  Work32 k;
+  // 16 lanes a pair put up to 32 pairs into one pass over the CTA's 16 warps, 32 lanes up to 16
+  const bool wide = q <= 32 || p > 128;
+  k.lp = p <= 16 || !wide ? 16 : 32;
+  k.per = p <= k.lp ? 1 : p <= 2 * k.lp ? 2 : p <= 4 * k.lp ? 4 : 8;
+  auto ld = [&](int n) { return k.lp == 32 ? n : (((n + k.lp - 1) / k.lp) | 1) * k.lp; };
+  k.ldg = ld(p);
+  k.ldv = ld(q);
+  const bool fits = (int64_t)(k.ldg + k.ldv) * q * (int)sizeof(float) <= kSvdSmemBytes;
+  // (outside shared memory p > 128: the leading dimensions are p and q, p q + q^2 floats)
+  k.g = fits ? svd_smem : reinterpret_cast<float*>(sc);
+  k.v = k.g + k.ldg * q;
+  return k;
+}
+
+__device__ __forceinline__ int run_jacobi32(const Work32& k, int p, int q, int max_sweeps,
+                                            float floor2,
+                                            JacobiShared& sh) {
+  if (k.lp == 16) {
+    switch (k.per) {
+      case 1: return jacobi32<16, 1>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, floor2, sh);
+      case 2:
+      case 4: return jacobi32<16, 4>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, floor2, sh);
+      default: return jacobi32<16, 8>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, floor2, sh);
+    }
+  }
+  switch (k.per) {
+    case 1: return jacobi32<32, 1>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, floor2, sh);
+    case 2: return jacobi32<32, 2>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, floor2, sh);
+    case 4: return jacobi32<32, 4>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, floor2, sh);
+    default: return jacobi32<32, 8>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, floor2, sh);
+  }
+}
+
+// Where small_series keeps its 2 q^2 floats: the place of the FP32 copies, which the
+// orthonormalisation has read by then.
+__device__ __forceinline__ float* series_f32(int q, double* sc) {
+  extern __shared__ float svd_smem[];
+  return (int64_t)2 * q * q * (int)sizeof(float) <= kSvdSmemBytes ? svd_smem
+                                                                 : reinterpret_cast<float*>(sc);
+}
+
 struct SvdShared {
   double red[kWarps];
   double sigma[CLR_MAX_CLUSTER];    // by column
@@ -534,6 +757,7 @@ struct SvdShared {
   // reflectors of the pivoted QR, of rrqr_block, or of the QR route's X factor; and of its W
   Reflectors refl, refl_w;
   int qr_perm[CLR_MAX_CLUSTER];   // pivoted QR: column order (columns are not moved)
+  JacobiShared jac;
   double cert;    // tail_lower_bound_sq's result
   // compress_by_pivoted_qr: each column's trailing norm^2 when it was last summed exactly (the
   // downdated norms are recomputed once they fall below kDowndateFloor of it), and the FMAs
@@ -622,76 +846,192 @@ struct SrcView {
   }
 };
 
-// v (q x q, ld q) <- the columns of the FP32 matrix v32 orthonormalised in FP64 (modified
-// Gram-Schmidt).
-__device__ void orthonormalise_fp64(const float* v32, double* v, int q, SvdShared& sh) {
-  const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int e = threadIdx.x; e < q * q; e += kThreads) v[e] = (double)v32[e];
+// The matrix function of a small symmetric E (q x q) that both uses below need, in place:
+//   e <- c1 E + c2 E^2 + c3 E^3.
+// The powers are taken in FP32 (f: 2 q^2 floats): E is at most a few 1e-4, so their error is
+// below 1e-16.  Returns ||E||_F^2.
+__device__ __noinline__ double small_series(double* e, int q, double c1, float c2, float c3,
+                                            float* f, SvdShared& sh) {
+  float* t = f + q * q;
+  float part = 0.f;
+  for (int x = threadIdx.x; x < q * q; x += kThreads) {
+    const float v = (float)e[x];
+    f[x] = v;
+    part = fmaf(v, v, part);
+  }
+  const double fro2 = block_sum((double)part, sh.red);
+  cta_gemm_auto<kThreads>(q, q, q, f, 1, q, f, 1, q, t, q);
   __syncthreads();
-  for (int j = 0; j < q; ++j) {
-    double* vj = v + (int64_t)j * q;
-    double part = 0.0;
-    for (int i = threadIdx.x; i < q; i += kThreads) part = fma(vj[i], vj[i], part);
-    const double nrm = sqrt(block_sum(part, sh.red));
-    const double inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
-    for (int i = threadIdx.x; i < q; i += kThreads) vj[i] *= inv;
-    __syncthreads();
-    for (int k = j + 1 + w; k < q; k += kWarps) {
-      double* vk = v + (int64_t)k * q;
-      double d = 0.0;
-      for (int i = l; i < q; i += 32) d = fma(vj[i], vk[i], d);
-      d = warp_sum(d);
-      for (int i = l; i < q; i += 32) vk[i] = fma(-d, vj[i], vk[i]);
+  // E^3 = F T an output at a time, added to the rest of the series
+  for (int x = threadIdx.x; x < q * q; x += kThreads) {
+    const int i = x % q, j = x / q;
+    float s = 0.f;
+    for (int l = 0; l < q; ++l) s = fmaf(f[i + l * q], t[l + j * q], s);
+    e[x] = fma(c1, e[x], (double)fmaf(c2, t[x], c3 * s));
+  }
+  __syncthreads();
+  return fro2;
+}
+
+// e (q x q) <- G^T G scaled by d on both sides (d null: unscaled) minus I, for G (n x q) given
+// row-major (element (l, i) at a[l q + i]): the lower triangle in 2 x 2 blocks, mirrored.
+__device__ void gram_minus_identity(const double* a, int n, int q, const double* d, double* e) {
+  const int nb = (q + 1) / 2;
+  for (int t = threadIdx.x; t < nb * (nb + 1) / 2; t += kThreads) {
+    int bi = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+    while (bi * (bi + 1) / 2 > t) --bi;
+    while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
+    const int i0 = 2 * bi, j0 = 2 * (t - bi * (bi + 1) / 2);
+    const int i1 = i0 + 1 < q ? i0 + 1 : i0, j1 = j0 + 1 < q ? j0 + 1 : j0;
+    double s00 = 0.0, s01 = 0.0, s10 = 0.0, s11 = 0.0;
+    const double* r = a;
+    for (int l = 0; l < n; ++l, r += q) {
+      const double x0 = r[i0], x1 = r[i1], y0 = r[j0], y1 = r[j1];
+      s00 = fma(x0, y0, s00);
+      s01 = fma(x0, y1, s01);
+      s10 = fma(x1, y0, s10);
+      s11 = fma(x1, y1, s11);
     }
-    __syncthreads();
+    auto put = [&](int i, int j, double s) {
+      if (d) s *= d[i] * d[j];
+      if (i == j) s -= 1.0;
+      e[i + (int64_t)j * q] = s;
+      e[j + (int64_t)i * q] = s;
+    };
+    put(i0, j0, s00);
+    if (j0 + 1 < q) put(i0, j1, s01);
+    if (i0 + 1 < q) put(i1, j0, s10);
+    if (i0 + 1 < q && j0 + 1 < q) put(i1, j1, s11);
+  }
+  __syncthreads();
+}
+
+// m (rows x q, row-major) <- m (I + w) (add_identity) or m w in FP64, w q x q row-major, row by
+// row in place: one warp per row, the row held in registers (8 entries per lane) and broadcast
+// by shuffles, 8 output columns per lane.  m's element (i, k) is at m[i m_r + k m_c].
+__device__ void right_multiply_fp64(double* m, int rows, int64_t m_r, int64_t m_c, int q,
+                                    const double* wt, bool add_identity) {
+  constexpr int kPer = CLR_MAX_CLUSTER / 32;
+  const int wp = threadIdx.x / 32, l = threadIdx.x % 32;
+  for (int i = wp; i < rows; i += kWarps) {
+    double r[kPer], acc[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      const int k = l + 32 * j;
+      r[j] = k < q ? m[i * m_r + k * m_c] : 0.0;
+      acc[j] = add_identity ? r[j] : 0.0;
+    }
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      if (32 * j >= q) break;
+      for (int kk = 0; kk < 32; ++kk) {
+        const int k = 32 * j + kk;
+        const double rk = __shfl_sync(0xffffffffu, r[j], kk);
+        if (k >= q) break;
+#pragma unroll
+        for (int o = 0; o < kPer; ++o) {
+          if (32 * o < q) {
+            const int c = l + 32 * o;
+            acc[o] = fma(rk, c < q ? wt[(int64_t)k * q + c] : 0.0, acc[o]);
+          }
+        }
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 0; o < kPer; ++o) {
+      const int c = l + 32 * o;
+      if (c < q) m[i * m_r + c * m_c] = acc[o];
+    }
+  }
+  __syncthreads();
+}
+
+// Above this ||E||_F the series in small_series, cut after E^3 and with FP32 powers, is not FP64
+// accurate (the first term left out is 35/128 E^4, the powers' error 4e-8 E^2).
+constexpr double kSeriesFro = 2e-4;
+
+// v (q x q, row-major) <- the orthogonal polar factor of the FP32 matrix v32 (ld ldv) in FP64:
+// V (V^T V)^-1/2 by its series in E = V^T V - I, which rotations accumulated in FP32 keep at
+// about 1e-5; repeated until ||E||_F has been below kSeriesFro.  Two products of q^3 FMAs (one of
+// them symmetric) that fill the CTA, against Gram-Schmidt's q^3 FMAs in q dependent steps of
+// reductions.  Measured (q = 16, with the product that follows): 218k -> 25k SM cycles; 3D lattice
+// product at N = 4096, both stages over all blocks: 3.1 -> 2.1 G cycles.  e: q^2 doubles, f: 2 q^2 floats, not overlapping v32's
+// matrix until it has been read.
+__device__ __noinline__ void orthonormalise_fp64(const float* v32, int ldv, double* v, int q,
+                                                 double* e, float* f, SvdShared& sh) {
+  for (int x = threadIdx.x; x < q * q; x += kThreads) {
+    const int i = x / q, j = x - i * q;
+    v[x] = (double)v32[i + j * ldv];
+  }
+  __syncthreads();
+  for (int pass = 0; pass < 4; ++pass) {
+    gram_minus_identity(v, q, q, nullptr, e);
+    const double fro2 = small_series(e, q, -0.5, 0.375f, -0.3125f, f, sh);
+    right_multiply_fp64(v, q, q, 1, q, e, true);
+    if (!(fro2 > kSeriesFro * kSeriesFro)) break;
   }
 }
 
-// g (p x q, ld p) = A v in FP64 (register-tiled, cta_gemm_tiled).
-__device__ void project_fp64(const SrcView& a, int p, int q, const double* v, double* g) {
+// g (p x q, ld p) = A v in FP64, v row-major.  lower: A(i, l) = 0 for l > i (the transposed
+// triangular factor), half of its first q rows.
+__device__ void project_fp64(const SrcView& a, int p, int q, const double* v, double* g,
+                             bool lower) {
   const int64_t a_i = a.tr ? a.s_c : a.s_r, a_k = a.tr ? a.s_r : a.s_c;
-  cta_gemm_tiled<kThreads>(p, q, q, a.src, a_i, a_k, v, 1, q, g, p, false);
+  if (lower)
+    cta_gemm_auto<kThreads, 1>(p, q, q, a.src, a_i, a_k, v, q, 1, g, p);
+  else
+    cta_gemm_auto<kThreads>(p, q, q, a.src, a_i, a_k, v, q, 1, g, p);
   __syncthreads();
 }
 
-// y (q x r, ld q) = A^T G_r in FP64, G_r the r kept columns of g (p x q, ld p) in the order
-// perm; with G_r = U_r S_r this is V_r S_r^2.  G_r is first gathered into `gather` (p r
-// doubles, not overlapping g or y) so that the product runs register-tiled.
+// y (q x r, row-major) = A^T G_r in FP64, G_r the r kept columns of g (p x q, ld p) in the order
+// perm; with G_r = U_r S_r this is V_r S_r^2.  G_r is first gathered row-major into `gather`
+// (p r doubles, not overlapping g or y).  lower: A(i, j) = 0 for i < j.
 __device__ void recover_right(const SrcView& a, int p, int q, const double* g, const int* perm,
-                              int r, double* y, double* gather) {
+                              int r, double* y, double* gather, bool lower) {
   for (int e = threadIdx.x; e < p * r; e += kThreads) {
-    const int k = e % p, c = e / p;
+    const int k = e / r, c = e - k * r;
     gather[e] = g[k + (int64_t)perm[c] * p];
   }
   __syncthreads();
-  // y(j, c) = sum_k A(k, j) G_r(k, c)
+  // y^T(c, j) = sum_k G_r(k, c) A(k, j)
   const int64_t a_j = a.tr ? a.s_r : a.s_c, a_k = a.tr ? a.s_c : a.s_r;
-  cta_gemm_tiled<kThreads>(q, r, p, a.src, a_j, a_k, gather, 1, p, y, q, false);
+  if (lower)
+    cta_gemm_auto<kThreads, 2>(r, q, p, gather, 1, r, a.src, a_k, a_j, y, r);
+  else
+    cta_gemm_auto<kThreads>(r, q, p, gather, 1, r, a.src, a_k, a_j, y, r);
   __syncthreads();
 }
 
-// y (q x r, ld q) <- y (G_r^T G_r)^-1 in FP64, G_r the r kept columns of g (p x q, ld p) in the
-// order perm, with norms d: the least-squares right factor when G_r is not orthogonal to FP64
-// precision.  The Gram matrix of the normalised columns (unit diagonal, off-diagonal at the
-// FP32 stages' tolerance, so well conditioned) is factored by Cholesky in mw (r x r).
-// Returns false, with y unchanged, when that factorisation meets a pivot that is not positive
-// (kept columns at the rounding level of a block whose norm is near eps); the caller then uses
-// the orthogonal-columns formula y S^-2.
-__device__ bool ls_solve(double* y, int q, int r, const double* g, int p, const int* perm,
-                         const double* d, double* mw, SvdShared& sh) {
-  const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int e = w; e < r * r; e += kWarps) {
-    const int i = e % r, j = e / r;
-    if (i < j) continue;
-    const double* gi = g + (int64_t)perm[i] * p;
-    const double* gj = g + (int64_t)perm[j] * p;
-    double s2 = 0.0;
-    for (int k = l; k < p; k += 32) s2 = fma(gi[k], gj[k], s2);
-    s2 = warp_sum(s2);
-    if (l == 0) mw[i + (int64_t)j * r] = s2 / (d[i] * d[j]);
-  }
+// y (q x r, row-major) <- y (G_r^T G_r)^-1 in FP64, G_r the kept columns gathered row-major in
+// `gr` (p x r), with norms d: the least-squares right factor when G_r is not orthogonal to FP64
+// precision.  The Gram matrix of the normalised columns is I + E, E at the FP32 stages' tolerance
+// (~1e-5), and its inverse I - E + E^2 - E^3; above kSeriesFro a Cholesky factorisation (in mw,
+// r^2 doubles, like e; f: 2 r^2 floats).  Returns false, with y unchanged, when that meets a
+// pivot that is not positive (kept columns at the rounding level of a block whose norm is near
+// eps); the caller then uses the orthogonal-columns formula y S^-2.
+__device__ __noinline__ bool ls_solve(double* y, int q, int r, const double* gr, int p,
+                                      const double* d, double* e, double* mw, float* f,
+                                      SvdShared& sh) {
+  double* rd = sh.sigma_inv;
+  for (int c = threadIdx.x; c < r; c += kThreads) rd[c] = 1.0 / d[c];
   __syncthreads();
+  gram_minus_identity(gr, p, r, rd, e);
+  for (int x = threadIdx.x; x < r * r; x += kThreads) mw[x] = e[x];
+  __syncthreads();
+  const double fro2 = small_series(e, r, -1.0, 1.0f, -1.0f, f, sh);
+  if (fro2 <= kSeriesFro * kSeriesFro) {
+    for (int x = threadIdx.x; x < q * r; x += kThreads) y[x] *= rd[x % r];
+    __syncthreads();
+    right_multiply_fp64(y, q, r, 1, r, e, true);
+    for (int x = threadIdx.x; x < q * r; x += kThreads) y[x] *= rd[x % r];
+    __syncthreads();
+    return true;
+  }
   if (threadIdx.x == 0) sh.flag = 1;
+  for (int x = threadIdx.x; x < r; x += kThreads) mw[x + (int64_t)x * r] += 1.0;
+  __syncthreads();
   for (int j = 0; j < r; ++j) {  // lower Cholesky, column by column
     if (threadIdx.x == 0) {
       double a = mw[j + (int64_t)j * r];
@@ -717,60 +1057,21 @@ __device__ bool ls_solve(double* y, int q, int r, const double* g, int p, const 
   }
   // each row t: x = (y_t D^-1) (L L^T)^-1 D^-1
   for (int t = threadIdx.x; t < q; t += kThreads) {
-    double* yt = y + t;  // stride q
+    double* yt = y + (int64_t)t * r;
     for (int i = 0; i < r; ++i) {  // forward: L u = (y_t D^-1)^T
-      double a = yt[(int64_t)i * q] / d[i];
-      for (int k = 0; k < i; ++k) a -= mw[i + (int64_t)k * r] * yt[(int64_t)k * q];
-      yt[(int64_t)i * q] = a / mw[i + (int64_t)i * r];
+      double a = yt[i] / d[i];
+      for (int k = 0; k < i; ++k) a -= mw[i + (int64_t)k * r] * yt[k];
+      yt[i] = a / mw[i + (int64_t)i * r];
     }
     for (int i = r - 1; i >= 0; --i) {  // back: L^T x = u
-      double a = yt[(int64_t)i * q];
-      for (int k = i + 1; k < r; ++k) a -= mw[k + (int64_t)i * r] * yt[(int64_t)k * q];
-      yt[(int64_t)i * q] = a / mw[i + (int64_t)i * r];
+      double a = yt[i];
+      for (int k = i + 1; k < r; ++k) a -= mw[k + (int64_t)i * r] * yt[k];
+      yt[i] = a / mw[i + (int64_t)i * r];
     }
-    for (int i = 0; i < r; ++i) yt[(int64_t)i * q] /= d[i];
+    for (int i = 0; i < r; ++i) yt[i] /= d[i];
   }
   __syncthreads();
   return true;
-}
-
-// m (rows x q, ld ldm) <- m w in FP64 with the q x q factor w given row-major (wt[k q + c] =
-// w(k, c)), row by row in place: one warp per row, the row held in registers (8 entries per
-// lane) and broadcast by shuffles, 8 output columns per lane (consecutive lanes read
-// consecutive entries of wt).
-__device__ void right_multiply_fp64(double* m, int rows, int64_t ldm, int q, const double* wt) {
-  constexpr int kPer = CLR_MAX_CLUSTER / 32;
-  const int wp = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int i = wp; i < rows; i += kWarps) {
-    double r[kPer], acc[kPer];
-#pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-      const int k = l + 32 * j;
-      r[j] = k < q ? m[i + (int64_t)k * ldm] : 0.0;
-      acc[j] = 0.0;
-    }
-#pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-      if (32 * j >= q) break;
-      for (int kk = 0; kk < 32; ++kk) {
-        const int k = 32 * j + kk;
-        const double rk = __shfl_sync(0xffffffffu, r[j], kk);
-        if (k >= q) break;
-#pragma unroll
-        for (int o = 0; o < kPer; ++o) {
-          const int c = l + 32 * o;
-          if (c < q) acc[o] = fma(rk, wt[(int64_t)k * q + c], acc[o]);
-        }
-      }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int o = 0; o < kPer; ++o) {
-      const int c = l + 32 * o;
-      if (c < q) m[i + (int64_t)c * ldm] = acc[o];
-    }
-  }
-  __syncthreads();
 }
 
 // Mixed-precision one-sided Jacobi SVD of the p x q (p >= q) matrix A given by `a`.  FP64 runs
@@ -801,7 +1102,8 @@ __device__ void right_multiply_fp64(double* m, int rows, int64_t ldm, int q, con
 // later stages could only confirm "dense": they are skipped and the function returns 1.
 __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g, double* v,
                                       double* sc, int max_sweeps, double eps, int dense_h,
-                                      double fro, SvdShared& sh, unsigned long long* jstats,
+                                      double fro, bool lower, SvdShared& sh,
+                                      unsigned long long* jstats,
                                       unsigned long long* stage_clk = nullptr) {
   // while profiling the full-SVD path: SM cycles per stage (1..5 of kFullStageCounters)
   long long ck = stage_clk ? clock64() : 0;
@@ -812,23 +1114,21 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
       ck = now;
     }
   };
-  // FP32 copies in the per-CTA scratch: the kernels run with the largest L1 carveout, which
-  // measured as fast as holding the copies in shared memory and gives the 256-column tiles
-  // (copies of 512 KB) the most cache
-  const int64_t pq = (int64_t)p * q;
-  float* g32 = reinterpret_cast<float*>(sc);
-  float* v32 = g32 + pq;
-  double* v2 = sc + (int64_t)CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;  // after p q + q^2 floats
+  const Work32 wk = work32(p, q, sc);
+  constexpr int64_t kSq = (int64_t)CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
+  double* v2 = sc + kSq;       // after p q + q^2 floats
+  double* e = sc + 4 * kSq;    // the orthonormalisations' E, and their FP32 powers
+  float* f = series_f32(q, sc);
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int e = threadIdx.x; e < p * q; e += kThreads) g32[e] = (float)a.at(e % p, e / p);
+  for (int e = threadIdx.x; e < p * q; e += kThreads)
+    wk.g[e % p + (e / p) * wk.ldg] = (float)a.at(e % p, e / p);
   __syncthreads();
   const float floor32 = (float)((double)p * FLT_EPSILON * fro);
-  const int sw32 = jacobi_svd<float>(g32, p, q, p, v32, q, max_sweeps, &sh.flag, true, 4.0f,
-                                     floor32 * floor32);
+  const int sw32 = run_jacobi32(wk, p, q, max_sweeps, floor32 * floor32, sh.jac);
   mark(1);
   if (dense_h >= 0 && dense_h < q) {
     for (int c = w; c < q; c += kWarps) {
-      const float* gc = g32 + (int64_t)c * p;
+      const float* gc = wk.g + c * wk.ldg;
       double s2 = 0.0;
       for (int i = l; i < p; i += 32) s2 = fma((double)gc[i], (double)gc[i], s2);
       s2 = warp_sum(s2);
@@ -858,18 +1158,18 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
       return 1;
     }
   }
-  orthonormalise_fp64(v32, v, q, sh);
-  project_fp64(a, p, q, v, g);
+  orthonormalise_fp64(wk.v, wk.ldv, v, q, e, f, sh);
+  project_fp64(a, p, q, v, g, lower);
   mark(2);
   // FP64 noise floor, raised to 1e-3 eps: columns below it hold less than 1e-6 eps^2 each, so
   // their mutual (non-)orthogonality cannot move a truncation decision at eps except within a
   // hair of the threshold, while orthogonalising them costs most of the sweeps
   const double floor64 = fmax((double)p * DBL_EPSILON * fro, 1e-3 * eps);
-  for (int e = threadIdx.x; e < p * q; e += kThreads) g32[e] = (float)g[e];
+  for (int e = threadIdx.x; e < p * q; e += kThreads)
+    wk.g[e % p + (e / p) * wk.ldg] = (float)g[e];
   __syncthreads();
   const float floor_g = (float)floor64;
-  const int sw32b = jacobi_svd<float>(g32, p, q, p, v32, q, max_sweeps, &sh.flag, true, 4.0f,
-                                      floor_g * floor_g);
+  const int sw32b = run_jacobi32(wk, p, q, max_sweeps, floor_g * floor_g, sh.jac);
   mark(3);
   // When eps is well above the noise floor the right factor of the kept columns is recovered
   // from A and G afterwards (recover_right).  Near the floor (eps < 1e3 p u ||A||_F) kept
@@ -877,13 +1177,9 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
   // accumulated instead.
   const bool track_v = floor64 > 1e-3 * eps;
   if (sw32b > 0) {
-    orthonormalise_fp64(v32, v2, q, sh);
-    // V2 row-major into the scratch's first half (the FP32 copies there are dead now)
-    double* v2t = sc;
-    for (int e = threadIdx.x; e < q * q; e += kThreads) v2t[e] = v2[e / q + (int64_t)(e % q) * q];
-    __syncthreads();
-    right_multiply_fp64(g, p, p, q, v2t);
-    if (track_v) right_multiply_fp64(v, q, q, q, v2t);
+    orthonormalise_fp64(wk.v, wk.ldv, v2, q, e, f, sh);
+    right_multiply_fp64(g, p, 1, p, q, v2, false);
+    if (track_v) right_multiply_fp64(v, q, q, 1, q, v2, false);
   }
   if (threadIdx.x == 0) sh.v_tracked = track_v ? 1 : 0;
   mark(4);
@@ -898,7 +1194,7 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
   // cycles of the lattice product's recompression at N = 4096.)
   if (threadIdx.x == 0) sh.ls_recover = track_v ? 0 : 1;
   if (jstats && threadIdx.x == 0) {
-    // algorithmic flops: Jacobi 4 p q^2 per sweep, orthonormalisation 2 q^3, products 2 p q^2
+    // algorithmic flops: Jacobi 4 p q^2 per sweep, orthonormalisation 3 q^3, products 2 p q^2
     const unsigned long long pq2 = (unsigned long long)p * q * q, q3 = (unsigned long long)q * q * q;
     unsigned long long f64 = 2 * q3 + 2 * pq2;
     if (sw32b > 0) f64 += 2 * q3 + 2 * pq2 + (track_v ? 2 * q3 : 0);
@@ -922,6 +1218,7 @@ __global__ void __launch_bounds__(kThreads, 1) compress_qr_kernel(MatView C, con
                                                                unsigned long long* jstats) {
   __shared__ SvdShared sh;
   __shared__ int sh_next;
+  constexpr int64_t kSq = (int64_t)CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
   double* sc = svd_scratch + (int64_t)blockIdx.x * kSvdScratchPerCta;
   const int n_items = *count;
   for (int it = next_item(sched, &sh_next); it < n_items; it = next_item(sched, &sh_next)) {
@@ -955,7 +1252,7 @@ __global__ void __launch_bounds__(kThreads, 1) compress_qr_kernel(MatView C, con
       for (int e = threadIdx.x; e < R * R; e += kThreads) part = fma(M[e], M[e], part);
       const double mfro = sqrt(block_sum(part, sh.red));
       SrcView mv{M, 1, R, false};
-      svd_mixed(mv, R, R, G, V, sc, max_sweeps, eps, -1, mfro, sh, jstats);
+      svd_mixed(mv, R, R, G, V, sc, max_sweeps, eps, -1, mfro, false, sh, jstats);
     }
     sort_and_truncate(G, R, R, R, eps, sh);
     const int r = sh.rank;
@@ -964,8 +1261,10 @@ __global__ void __launch_bounds__(kThreads, 1) compress_qr_kernel(MatView C, con
     if (!tracked) {
       // V_r S_r^2 = M^T G_r into V (M is still intact), or the least-squares V_r
       SrcView mv{M, 1, R, false};
-      recover_right(mv, R, R, G, sh.perm, r, V, sc);
-      if (ls) ls = ls_solve(V, R, r, G, R, sh.perm, sh.sorted, sc, sh);
+      recover_right(mv, R, R, G, sh.perm, r, V, sc, false);
+      if (ls)
+        ls = ls_solve(V, R, r, sc, R, sh.sorted, sc + 4 * kSq, sc + kSq, series_f32(r, sc + 2 * kSq),
+                      sh);
     }
     double* Xo = C.pool + sC;
     double* Wo = Xo + (int64_t)m * r;
@@ -976,9 +1275,9 @@ __global__ void __launch_bounds__(kThreads, 1) compress_qr_kernel(MatView C, con
     for (int e = threadIdx.x; e < n * r; e += kThreads) {
       const int j = e % n, c = e / n;
       Wo[e] = j >= R ? 0.0
-              : tracked ? V[j + (int64_t)sh.perm[c] * R]
-              : ls      ? V[j + (int64_t)c * R]
-                        : V[j + (int64_t)c * R] / (sh.sorted[c] * sh.sorted[c]);
+              : tracked ? V[(int64_t)j * R + sh.perm[c]]
+              : ls      ? V[(int64_t)j * r + c]
+                        : V[(int64_t)j * r + c] / (sh.sorted[c] * sh.sorted[c]);
     }
     __syncthreads();
     // (W's column groups start three warps on, so that few columns spread over the four
@@ -1003,8 +1302,8 @@ __global__ void __launch_bounds__(kThreads, 1) compress_qr_kernel(MatView C, con
 }
 
 // Launch shape of a recompression kernel: one CTA per SM (512 threads x 128 registers fill the
-// register file) within the caller's grid (the scratch is sized for it), with the shared memory
-// carveout at its minimum so that L1 caches the FP32 working copies.
+// register file) within the caller's grid (the scratch is sized for it), with all the shared
+// memory a CTA can have for the FP32 working copies.
 template <typename K>
 int svd_launch_grid(K kernel, int grid_max, bool* attr_done) {
   int dev = 0;
@@ -1013,7 +1312,7 @@ int svd_launch_grid(K kernel, int grid_max, bool* attr_done) {
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   // set once per device (outside any stream capture the first time a product runs)
   if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSvdSmemBytes);
     attr_done[dev] = true;
   }
   int grid = n_sm;
@@ -1028,7 +1327,7 @@ void launch_compress_qr(const MatView& C, const int* list, const int* count, con
   (void)err;
   static bool attr_done[64] = {false};
   const int g = svd_launch_grid(compress_qr_kernel, grid, attr_done);
-  compress_qr_kernel<<<g, kThreads, 0, st>>>(C, list, count, rsum, ws, svd_scratch, eps,
+  compress_qr_kernel<<<g, kThreads, kSvdSmemBytes, st>>>(C, list, count, rsum, ws, svd_scratch, eps,
                                              max_sweeps, sched, jstats);
 }
 
@@ -1434,25 +1733,26 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     __syncthreads();
     return 1;
   }
-  // R (k x q, ld k, zero below the diagonal) and the SVD of M = R^T (q x k)
+  // M = R^T (q x k, ld q, zero above the diagonal: consecutive threads of its products read
+  // consecutive rows) and its SVD
   constexpr int64_t kSq = (int64_t)CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
-  double* rb = sc + 3 * kSq;   // k x q
+  double* rb = sc + 3 * kSq;   // q x k
   double* gs = wv;             // q x k
   double* vs = sc + 2 * kSq;   // k x k
   double part = 0.0;
   for (int e = threadIdx.x; e < k * q; e += kThreads) {
     const int i = e % k, c = e / k;
     const double x = i <= c ? g[i + (int64_t)sh.qr_perm[c] * p] : 0.0;
-    rb[e] = x;
+    rb[c + (int64_t)i * q] = x;
     part = fma(x, x, part);
   }
   const double rfro = sqrt(block_sum(part, sh.red));
   const double budget = sqrt(fmax(eps * eps - trail2, 0.0));
-  const SrcView mv{rb, k, 1, false};   // M(i, j) = R(j, i)
+  const SrcView mv{rb, 1, q, false};
   unsigned long long* stage_clk = jstats ? jstats + kPreStageCounters : nullptr;
   if (stage_clk && threadIdx.x == 0)
     atomicAdd(&stage_clk[0], (unsigned long long)(clock64() - c_entry));
-  svd_mixed(mv, q, k, gs, vs, sc, max_sweeps, budget, -1, rfro, sh, jstats, stage_clk);
+  svd_mixed(mv, q, k, gs, vs, sc, max_sweeps, budget, -1, rfro, true, sh, jstats, stage_clk);
   const long long c_after = clock64();
   sort_and_truncate(gs, q, k, q, budget, sh);
   const int r = sh.rank;
@@ -1473,8 +1773,12 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
   }
   const bool tracked = sh.v_tracked;
   bool ls = !tracked && sh.ls_recover;
-  if (!tracked) recover_right(mv, q, k, gs, sh.perm, r, vs, sc);   // Y = R G_r (k x r)
-  if (ls) ls = ls_solve(vs, k, r, gs, q, sh.perm, sh.sorted, sc, sh);
+  if (!tracked) recover_right(mv, q, k, gs, sh.perm, r, vs, sc, true);   // Y = R G_r (k x r)
+  // (R is no longer needed: its place takes the Cholesky factor and FP32 powers too large for
+  // shared memory)
+  if (ls)
+    ls = ls_solve(vs, k, r, sc, q, sh.sorted, sc + 4 * kSq, sc + kSq, series_f32(r, sc + 3 * kSq),
+                  sh);
   // R = V_M S U_M^T:  X_R = (V_M S)_r (k x r), W_R = (U_M)_r (q x r); A ~ (Q_k X_R) (P W_R)^T
   // (the source in the slot is no longer read: the factors overwrite it)
   __syncthreads();
@@ -1484,9 +1788,9 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     const int i = e % p, c = e / p;
     double v = 0.0;
     if (i < k)
-      v = tracked ? vs[i + (int64_t)sh.perm[c] * k] * sh.sorted[c]
-          : ls    ? vs[i + (int64_t)c * k]
-                  : vs[i + (int64_t)c * k] / sh.sorted[c];
+      v = tracked ? vs[(int64_t)i * k + sh.perm[c]] * sh.sorted[c]
+          : ls    ? vs[(int64_t)i * r + c]
+                  : vs[(int64_t)i * r + c] / sh.sorted[c];
     xa[e] = v;
   }
   for (int e = threadIdx.x; e < q * r; e += kThreads) {
@@ -1613,7 +1917,7 @@ __global__ void __launch_bounds__(kThreads, 1) compress_dense_kernel(
         if (stage_clk && threadIdx.x == 0)
           atomicAdd(&stage_clk[0], (unsigned long long)(clock64() - c0));
         const int early_dense = svd_mixed(view, p, q, G, V, sc, max_sweeps, eps, q / 2, nrm,
-                                          sh, jstats, stage_clk);
+                                          false, sh, jstats, stage_clk);
         if (!early_dense) {
           c_full = clock64();
           sort_and_truncate(G, p, q, p, eps, sh);
@@ -1649,8 +1953,11 @@ __global__ void __launch_bounds__(kThreads, 1) compress_dense_kernel(
       const SrcView view{S, s_r, s_c, tr};
       const bool tracked = sh.v_tracked;
       bool ls = !tracked && sh.ls_recover;
-      if (!tracked) recover_right(view, p, q, G, sh.perm, r, V, sc);
-      if (ls) ls = ls_solve(V, q, r, G, p, sh.perm, sh.sorted, sc, sh);
+      constexpr int64_t kSq = (int64_t)CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
+      if (!tracked) recover_right(view, p, q, G, sh.perm, r, V, sc, false);
+      if (ls)
+        ls = ls_solve(V, q, r, sc, p, sh.sorted, sc + 4 * kSq, sc + kSq,
+                      series_f32(r, sc + 2 * kSq), sh);
       if (jstats && threadIdx.x == 0 && !tracked)
         atomicAdd(&jstats[4], 2ull * p * q * r);
       double* Xo = slot;
@@ -1663,18 +1970,18 @@ __global__ void __launch_bounds__(kThreads, 1) compress_dense_kernel(
         }
         for (int e = threadIdx.x; e < n * r; e += kThreads) {
           const int j = e % n, c = e / n;
-          Wo[e] = tracked ? V[j + (int64_t)sh.perm[c] * q]
-                  : ls    ? V[j + (int64_t)c * q]
-                          : V[j + (int64_t)c * q] / (sh.sorted[c] * sh.sorted[c]);
+          Wo[e] = tracked ? V[(int64_t)j * q + sh.perm[c]]
+                  : ls    ? V[(int64_t)j * r + c]
+                          : V[(int64_t)j * r + c] / (sh.sorted[c] * sh.sorted[c]);
         }
       } else {
         // G = U' S (n x m) of the transposed block, Y = V' S^2 (m x r): block = V' S U'^T ->
         // X = V'_r S_r = Y S^-1, W = U'_r = G_r S^-1
         for (int e = threadIdx.x; e < m * r; e += kThreads) {
           const int i = e % m, c = e / m;
-          Xo[e] = tracked ? V[i + (int64_t)sh.perm[c] * q] * sh.sorted[c]
-                  : ls    ? V[i + (int64_t)c * q]
-                          : V[i + (int64_t)c * q] / sh.sorted[c];
+          Xo[e] = tracked ? V[(int64_t)i * q + sh.perm[c]] * sh.sorted[c]
+                  : ls    ? V[(int64_t)i * r + c]
+                          : V[(int64_t)i * r + c] / sh.sorted[c];
         }
         for (int e = threadIdx.x; e < n * r; e += kThreads) {
           const int j = e % n, c = e / n;
@@ -1704,7 +2011,7 @@ void launch_compress_dense(const MatView& C, const int* list, const int* count,
                            int* err, int* sched, unsigned long long* jstats, cudaStream_t st) {
   static bool attr_done[64] = {false};
   const int g = svd_launch_grid(compress_dense_kernel, grid, attr_done);
-  compress_dense_kernel<<<g, kThreads, 0, st>>>(C, list, count, order, src, lds, ws, svd_scratch,
+  compress_dense_kernel<<<g, kThreads, kSvdSmemBytes, st>>>(C, list, count, order, src, lds, ws, svd_scratch,
                                                 eps, drop_norm, dense_only, rrqr, prereduce,
                                                 max_sweeps, err, sched, jstats);
 }
