@@ -1,6 +1,8 @@
 // K6/K7 -- CLR linear combination (the T_n polynomial of Section 4.2 is
 // (15 I - 10 X_n + 3 X_n^2) / 8), distance to the identity (NS convergence test), CLR
 // matrix-vector products (alpha estimate) and transposes (adjoint products).
+#include <cooperative_groups.h>
+
 #include "clr_internal.h"
 
 namespace clr {
@@ -202,51 +204,97 @@ void launch_identity_distance(const MatView& X, double* out_sq, cudaStream_t st)
   sum_kernel<<<1, 1024, 0, st>>>(out_sq + 1, nb, out_sq);
 }
 
-// y_I = sum_J M_IJ x_J, one CTA per block-row.
-__global__ void __launch_bounds__(kT) matvec_kernel(MatView M, const double* x, double* y) {
-  __shared__ double acc[CLR_MAX_CLUSTER];
-  __shared__ double tw[CLR_MAX_CLUSTER / 2];
-  const int I = blockIdx.x;
+// y_I = sum_J M_IJ x_J.  Bound by reading the blocks once (70 MB for the 3D lattice at N = 4096)
+// and by the FP64 pipe (an FMA per double read), 15 us each there, so the block-row is spread
+// over a cluster of 8 CTAs (blocks J in turn) whose partial sums are added, in a fixed order,
+// through distributed shared memory: no workspace, so calls on different streams do not meet.
+// (One CTA per block-row, walking its blocks one after the other, took 690 us;
+// this takes 60.)  Inside a CTA a warp
+// takes four columns of W at a time for W^T x and sums them together; for X t (and dense blocks)
+// it owns a group of 32 rows and a share of the columns, its row sums in registers until the end.
+constexpr int kMvCtas = 8;
+constexpr int kMvThreads = 512;
+constexpr int kMvWarps = kMvThreads / 32;
+
+__global__ void __cluster_dims__(kMvCtas, 1, 1) __launch_bounds__(kMvThreads)
+    matvec_kernel(MatView M, const double* x, double* y) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ double part[kMvWarps][CLR_MAX_CLUSTER];   // [0] ends as this CTA's sum
+  __shared__ double tw[2][CLR_MAX_CLUSTER / 2];
+  const int I = blockIdx.x / kMvCtas, rank = (int)cluster.block_rank();
   const int m = M.row_off[I + 1] - M.row_off[I];
-  for (int i = threadIdx.x; i < m; i += kT) acc[i] = 0.0;
-  __syncthreads();
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int J = 0; J < M.nc; ++J) {
+  const int groups = (m + 31) / 32, slices = kMvWarps / groups;
+  const int i = (w % groups) * 32 + l, slice = w / groups;
+  const bool mine = slice < slices && i < m;
+  double acc = 0.0;
+  int buf = 0;
+  for (int J = rank; J < M.nc; J += kMvCtas) {
     const int t = I * M.nc + J;
     const int kind = M.kind[t];
     if (kind == CLR_KIND_ZERO) continue;
     const int n = M.col_off[J + 1] - M.col_off[J];
     const double* s = M.pool + slot_of(M, I, J, m);
     const double* xj = x + M.col_off[J];
-    if (kind == CLR_KIND_DENSE) {
-      for (int i = threadIdx.x; i < m; i += kT) {
-        double v = 0.0;
-        for (int j = 0; j < n; ++j) v = fma(s[i + (int64_t)j * m], xj[j], v);
-        acc[i] += v;
-      }
-    } else {
+    const double* v = xj;
+    int cols = n;
+    if (kind == CLR_KIND_LR) {
       const int r = M.rank[t];
       const double* W = s + (int64_t)m * r;
-      for (int c = w; c < r; c += kT / 32) {
-        double v = 0.0;
-        for (int j = l; j < n; j += 32) v = fma(W[j + (int64_t)c * n], xj[j], v);
-        v = wsum(v);
-        if (l == 0) tw[c] = v;
+      for (int c0 = 4 * w; c0 < r; c0 += 4 * kMvWarps) {
+        double d[4] = {0.0, 0.0, 0.0, 0.0};
+        const double* wc[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) wc[c] = W + (int64_t)(c0 + c < r ? c0 + c : c0) * n;
+#pragma unroll 4
+        for (int j = l; j < n; j += 32) {
+          const double xv = xj[j];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) d[c] = fma(wc[c][j], xv, d[c]);
+        }
+        // lane l: the sum of column c0 + l / 8
+        const bool h16 = (l & 16) != 0, h8 = (l & 8) != 0;
+        double a0 = h16 ? d[2] : d[0], a1 = h16 ? d[3] : d[1];
+        a0 += __shfl_xor_sync(0xffffffffu, h16 ? d[0] : d[2], 16);
+        a1 += __shfl_xor_sync(0xffffffffu, h16 ? d[1] : d[3], 16);
+        double a = h8 ? a1 : a0;
+        a += __shfl_xor_sync(0xffffffffu, h8 ? a0 : a1, 8);
+        a += __shfl_xor_sync(0xffffffffu, a, 4);
+        a += __shfl_xor_sync(0xffffffffu, a, 2);
+        a += __shfl_xor_sync(0xffffffffu, a, 1);
+        if (l % 8 == 0 && c0 + l / 8 < r) tw[buf][c0 + l / 8] = a;
       }
+      // (the other buffer is written only past the next barrier: one barrier per block)
       __syncthreads();
-      for (int i = threadIdx.x; i < m; i += kT) {
-        double v = 0.0;
-        for (int c = 0; c < r; ++c) v = fma(s[i + (int64_t)c * m], tw[c], v);
-        acc[i] += v;
-      }
+      v = tw[buf];
+      cols = r;
+      buf ^= 1;
     }
-    __syncthreads();
+    if (mine) {
+      const double* si = s + i;
+#pragma unroll 8
+      for (int c = slice; c < cols; c += slices) acc = fma(si[(int64_t)c * m], v[c], acc);
+    }
   }
-  for (int i = threadIdx.x; i < m; i += kT) y[M.row_off[I] + i] = acc[i];
+  if (mine) part[slice][i] = acc;
+  __syncthreads();
+  for (int r = threadIdx.x; r < m; r += kMvThreads) {
+    double sum = part[0][r];
+    for (int q = 1; q < slices; ++q) sum += part[q][r];
+    part[0][r] = sum;
+  }
+  cluster.sync();
+  for (int r = rank + kMvCtas * threadIdx.x; r < m; r += kMvCtas * kMvThreads) {
+    double sum = 0.0;
+    for (int q = 0; q < kMvCtas; ++q) sum += cluster.map_shared_rank(&part[0][0], q)[r];
+    y[M.row_off[I] + r] = sum;
+  }
+  cluster.sync();   // no CTA's shared memory goes before the others have read it
 }
 
 void launch_matvec(const MatView& M, const double* x, double* y, cudaStream_t st) {
-  matvec_kernel<<<M.nr, kT, 0, st>>>(M, x, y);
+  matvec_kernel<<<M.nr * kMvCtas, kMvThreads, 0, st>>>(M, x, y);
 }
 
 // T = S^T: block (J,I) of T is block (I,J) of S transposed (dense) or with X and W swapped.
