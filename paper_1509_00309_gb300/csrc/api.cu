@@ -1158,7 +1158,7 @@ int multiply_into(clr_ctx_t ctx, clr_mat_t a, clr_mat_t b, clr_mat_t c, double a
   prof_launches(ctx, 4);
   prof_mark(ctx, s, PH_PLAN);
   if (prec == CLR_PREC_FP64) {
-    launch_dd_fp64(av, bv, cv, p, grid_of(ctx, 4), s);
+    launch_dd_fp64(av, bv, cv, p, ctx->n_sm, s);
     CLR_CHECK_LAUNCH("dense x dense (FP64)");
     prof_launches(ctx, 1);
     if (ctx->prof_on) ctx->prof.dense_launches++;

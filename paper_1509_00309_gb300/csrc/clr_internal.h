@@ -203,7 +203,7 @@ void launch_plan_scan(const Plan& p, int recompress_dense, cudaStream_t st);
 // k_dense64.cu
 // uses p.counters->sched[3]
 void launch_dd_fp64(const MatView& A, const MatView& B, const MatView& C, const Plan& p,
-                    int grid, cudaStream_t st);
+                    int n_sm, cudaStream_t st);
 void launch_set_route_kinds(const MatView& C, const Plan& p, cudaStream_t st);
 void launch_dense_tile_norms(const MatView& C, const Plan& p, cudaStream_t st);
 // norm = sqrt(norm) of the route-DENSE tiles (their sums of squares came from the GEMM epilogue)

@@ -3,94 +3,179 @@
 // bookkeeping.
 //
 // On GB300 FP64 runs on the CUDA cores at a small fraction of the tensor rate (~2 FMAs per clock
-// per SM), so these kernels are FP64-pipe-bound and the work is cut to waste no lanes: a C tile
-// (m x n, up to 256 x 256) is split into ceil(m/64) x ceil(n/64) sub-tiles of equal size (at
-// most 64 x 64, so a 170-row tile gives three 57-row sub-tiles rather than two full ones and a
-// 42-row one); one CTA computes a sub-tile in registers (4 x 4 per thread), walking that tile's
-// dense x dense products in k order (deterministic, no atomics).  Sub-tiles are taken from a
-// launch-wide counter over the tiles in decreasing cost order (longest-processing-time
-// scheduling: tiles differ in size and in their number of products).
+// per SM: a warp's FMA holds its sub-partition's pipe for 64 cycles), so these kernels are
+// FP64-pipe-bound and the work is cut to waste no FMAs and to reach every SM: a C tile (m x n, up
+// to 256 x 256) is cut into sub-tiles of 64, 32 or 16 rows and columns and a ragged last one; one
+// CTA computes a sub-tile in registers (16 x 16 threads, up to 4 x 4 entries each, rows and
+// columns beyond the next multiple of 16 skipped), walking that tile's dense x dense products in
+// k order (deterministic, no atomics).  Sub-tiles are taken from a launch-wide counter over the
+// tiles in decreasing cost order (longest-processing-time scheduling).
 #include "clr_internal.h"
 
 namespace clr {
 
-constexpr int kSub = 64;      // sub-tile edge
-constexpr int kKc = 16;       // k chunk staged in shared memory
+constexpr int kSub = 64;                     // largest sub-tile edge
+constexpr int kStage = 64 * 17;              // doubles of an operand's staged k chunk
 constexpr int kSubPerTile = (CLR_MAX_CLUSTER / kSub) * (CLR_MAX_CLUSTER / kSub);
+constexpr int kDdThreads = 256;
+constexpr int kPrefixTiles = 1024;           // tiles whose sub-tiles are numbered exactly
+constexpr int kItemsPerSm = 6;
 
-__global__ void __launch_bounds__(256) dd_fp64_kernel(MatView A, MatView B, MatView C, Plan p) {
-  __shared__ double As[kKc][kSub + 1];
-  __shared__ double Bs[kKc][kSub + 1];
+// The sub-tile of edge 16 NA at (i0, j0) of C tile t.  Chunks of 64 / NA k are staged.
+template <int NA>
+__device__ __forceinline__ void dd_sub_tile(const MatView& A, const MatView& B, const MatView& C,
+                                            const Plan& p, int t, int i0, int j0, double* As,
+                                            double* Bs) {
+  constexpr int E = 16 * NA, LD = E + 1, KC = 64 / NA;
+  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+  const int I = t / p.nJ, J = t % p.nJ;
+  const int m = C.row_off[I + 1] - C.row_off[I];
+  const int n = C.col_off[J + 1] - C.col_off[J];
+  const int h = min(E, m - i0), g = min(E, n - j0);
+  const int na = (h + 15) / 16, nb = (g + 15) / 16;
+  double acc[NA][NA];
+#pragma unroll
+  for (int a = 0; a < NA; ++a)
+#pragma unroll
+    for (int b = 0; b < NA; ++b) acc[a][b] = 0.0;
+  const int start = p.t_start[t], count = p.t_count[t];
+  for (int q = 0; q < count; ++q) {
+    const Triple tr = p.triples[start + q];
+    if (tr.kind != T_DD) continue;
+    const int K = tr.k;
+    const int k = A.col_off[K + 1] - A.col_off[K];
+    const double* Ab = A.pool + slot_of(A, I, K, m) + i0;                // m x k, column-major
+    const double* Bb = B.pool + slot_of(B, K, J, k) + (int64_t)j0 * k;   // k x n, column-major
+    for (int k0 = 0; k0 < k; k0 += KC) {
+      const int kc = min(KC, k - k0);
+      for (int e = tid; e < KC * E; e += kDdThreads) {
+        const int r = e % E, kk = e / E;
+        As[kk * LD + r] = (r < h && kk < kc) ? Ab[r + (int64_t)(k0 + kk) * m] : 0.0;
+        const int kk2 = e % KC, c = e / KC;
+        Bs[kk2 * LD + c] = (c < g && kk2 < kc) ? Bb[(k0 + kk2) + (int64_t)c * k] : 0.0;
+      }
+      __syncthreads();
+#pragma unroll 4
+      for (int kk = 0; kk < kc; ++kk) {
+        double av[NA], bv[NA];
+#pragma unroll
+        for (int a = 0; a < NA; ++a) av[a] = As[kk * LD + ty + 16 * a];
+#pragma unroll
+        for (int b = 0; b < NA; ++b) bv[b] = Bs[kk * LD + tx + 16 * b];
+#pragma unroll
+        for (int a = 0; a < NA; ++a)
+          if (a < na) {
+#pragma unroll
+            for (int b = 0; b < NA; ++b)
+              if (b < nb) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
+          }
+      }
+      __syncthreads();
+    }
+  }
+  double* D = C.pool + slot_of(C, I, J, m);
+#pragma unroll
+  for (int a = 0; a < NA; ++a)
+#pragma unroll
+    for (int b = 0; b < NA; ++b) {
+      const int r = ty + 16 * a, c = tx + 16 * b;
+      if (r < h && c < g) D[i0 + r + (int64_t)(j0 + c) * m] = acc[a][b];
+    }
+}
+
+// The sub-tile edge: the largest of 64, 32, 16 that still gives every SM kItemsPerSm sub-tiles
+// (16 x 128^2 tiles, the 1D chain at N = 2048: 64 sub-tiles of 64 on 152 SMs took 525 us, 1024 of 16 take 98), with
+// the tiles' sub-tiles numbered by a prefix sum; with more than kPrefixTiles tiles, 64 with 16
+// numbers per tile, of which those past the tile's end are empty.
+__global__ void __launch_bounds__(kDdThreads) dd_fp64_kernel(MatView A, MatView B, MatView C,
+                                                             Plan p, int n_sm) {
+  __shared__ double As[kStage], Bs[kStage];
+  __shared__ int prefix[kPrefixTiles];   // inclusive, of the chosen edge
+  __shared__ int warp_tot[3][kDdThreads / 32];
   __shared__ int sh_next;
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
-  const int n_items = p.counters->n_dense * kSubPerTile;
+  const int tid = threadIdx.x, w = tid / 32, l = tid % 32;
+  const int n_dense = p.counters->n_dense;
   int* sched = &p.counters->sched[3];
+  auto subs = [&](int it, int edge, int* nsi) {
+    const int t = p.l_dense_s[it];
+    const int I = t / p.nJ, J = t % p.nJ;
+    *nsi = (C.row_off[I + 1] - C.row_off[I] + edge - 1) / edge;
+    return *nsi * ((C.col_off[J + 1] - C.col_off[J] + edge - 1) / edge);
+  };
+  int edge = kSub, n_items = n_dense * kSubPerTile;
+  const bool exact = n_dense <= kPrefixTiles;
+  if (exact) {
+    constexpr int kPer = kPrefixTiles / kDdThreads;
+    int tot[3] = {0, 0, 0}, nsi;
+    for (int x = 0; x < kPer; ++x) {
+      const int it = tid * kPer + x;
+      if (it < n_dense)
+        for (int e = 0; e < 3; ++e) tot[e] += subs(it, kSub >> e, &nsi);
+    }
+    for (int e = 0; e < 3; ++e) {
+      const int s = __reduce_add_sync(0xffffffffu, tot[e]);
+      if (l == 0) warp_tot[e][w] = s;
+    }
+    __syncthreads();
+    int sel = 2;
+    for (int e = 1; e >= 0; --e) {
+      int s = 0;
+      for (int q = 0; q < kDdThreads / 32; ++q) s += warp_tot[e][q];
+      if (s >= kItemsPerSm * n_sm) sel = e;
+    }
+    edge = kSub >> sel;
+    int own = tot[0];
+    if (sel == 1) own = tot[1];
+    if (sel == 2) own = tot[2];
+    int incl = own;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (l >= o) incl += v;
+    }
+    int base = incl - own;
+    n_items = 0;
+    for (int q = 0; q < kDdThreads / 32; ++q) {
+      if (q < w) base += warp_tot[sel][q];
+      n_items += warp_tot[sel][q];
+    }
+    for (int x = 0; x < kPer; ++x) {
+      const int it = tid * kPer + x;
+      if (it < n_dense) prefix[it] = base += subs(it, edge, &nsi);
+    }
+    __syncthreads();
+  }
   for (int item = next_item(sched, &sh_next); item < n_items;
        item = next_item(sched, &sh_next)) {
-    const int t = p.l_dense_s[item / kSubPerTile];
-    const int s = item % kSubPerTile;
-    const int I = t / p.nJ, J = t % p.nJ;
-    const int mt = C.row_off[I + 1] - C.row_off[I];
-    const int nt = C.col_off[J + 1] - C.col_off[J];
-    // equal sub-tiles of at most kSub x kSub
-    const int nsi = (mt + kSub - 1) / kSub, nsj = (nt + kSub - 1) / kSub;
-    const int si = s / (CLR_MAX_CLUSTER / kSub), sj = s % (CLR_MAX_CLUSTER / kSub);
-    if (si >= nsi || sj >= nsj) continue;
-    const int hi = (mt + nsi - 1) / nsi, hj = (nt + nsj - 1) / nsj;
-    const int i0 = si * hi, j0 = sj * hj;
-    const int m = mt, n = nt;
-    const int ie = min(mt, i0 + hi), je = min(nt, j0 + hj);
-    double acc[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-    const int start = p.t_start[t], count = p.t_count[t];
-    for (int q = 0; q < count; ++q) {
-      const Triple tr = p.triples[start + q];
-      if (tr.kind != T_DD) continue;
-      const int K = tr.k;
-      const int k = A.col_off[K + 1] - A.col_off[K];
-      const double* Ab = A.pool + slot_of(A, I, K, m);   // m x k, column-major
-      const double* Bb = B.pool + slot_of(B, K, J, k);   // k x n, column-major
-      for (int k0 = 0; k0 < k; k0 += kKc) {
-        for (int e = tid; e < kKc * kSub; e += 256) {
-          const int r = e % kSub, kk = e / kSub;
-          As[kk][r] = (i0 + r < ie && k0 + kk < k) ? Ab[(i0 + r) + (int64_t)(k0 + kk) * m] : 0.0;
-          const int kk2 = e % kKc, c = e / kKc;
-          Bs[kk2][c] = (j0 + c < je && k0 + kk2 < k) ? Bb[(k0 + kk2) + (int64_t)(j0 + c) * k] : 0.0;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < kKc; ++kk) {
-          double av[4], bv[4];
-#pragma unroll
-          for (int a = 0; a < 4; ++a) av[a] = As[kk][ty + 16 * a];
-#pragma unroll
-          for (int b = 0; b < 4; ++b) bv[b] = Bs[kk][tx + 16 * b];
-#pragma unroll
-          for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
-        }
-        __syncthreads();
+    int it, si, sj, nsi;
+    if (exact) {
+      int lo = 0, hi = n_dense - 1;   // the first tile whose inclusive count exceeds item
+      while (lo < hi) {
+        const int mid = (lo + hi) / 2;
+        if (prefix[mid] > item) hi = mid; else lo = mid + 1;
       }
+      it = lo;
+      const int s = item - (it > 0 ? prefix[it - 1] : 0);
+      subs(it, edge, &nsi);
+      si = s % nsi;
+      sj = s / nsi;
+    } else {
+      it = item / kSubPerTile;
+      const int s = item % kSubPerTile;
+      si = s / (CLR_MAX_CLUSTER / kSub);
+      sj = s % (CLR_MAX_CLUSTER / kSub);
+      const int total = subs(it, edge, &nsi);
+      if (si >= nsi || sj >= total / nsi) continue;
     }
-    double* D = C.pool + slot_of(C, I, J, m);
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int r = i0 + ty + 16 * a, c = j0 + tx + 16 * b;
-        if (r < ie && c < je) D[r + (int64_t)c * m] = acc[a][b];
-      }
+    const int t = p.l_dense_s[it];
+    if (edge == 64) dd_sub_tile<4>(A, B, C, p, t, si * 64, sj * 64, As, Bs);
+    else if (edge == 32) dd_sub_tile<2>(A, B, C, p, t, si * 32, sj * 32, As, Bs);
+    else dd_sub_tile<1>(A, B, C, p, t, si * 16, sj * 16, As, Bs);
   }
 }
 
 void launch_dd_fp64(const MatView& A, const MatView& B, const MatView& C, const Plan& p,
-                    int grid, cudaStream_t st) {
-  dd_fp64_kernel<<<grid, 256, 0, st>>>(A, B, C, p);
+                    int n_sm, cudaStream_t st) {
+  dd_fp64_kernel<<<4 * n_sm, kDdThreads, 0, st>>>(A, B, C, p, n_sm);
 }
 
 // After planning: kinds of tiles that get no contribution (zero) or a dense accumulation.
