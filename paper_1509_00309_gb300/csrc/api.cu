@@ -494,14 +494,9 @@ void prof_launches(clr_ctx_t ctx, int n) {
   if (ctx->prof_on && !ctx->capturing) ctx->prof.launches += n;
 }
 
-constexpr int64_t kScratchPerCta =
-    (int64_t)(CLR_MAX_CLUSTER / 2) * (CLR_MAX_CLUSTER / 2) +
-    (int64_t)CLR_MAX_CLUSTER * (CLR_MAX_CLUSTER / 2);
 // Per-CTA scratch shared by the low-rank product kernel and (after it, on the same stream) the
 // recompression kernels' mixed-precision SVD.
-inline int64_t scratch_per_cta() {
-  return kScratchPerCta > kSvdScratchPerCta ? kScratchPerCta : kSvdScratchPerCta;
-}
+inline int64_t scratch_per_cta() { return kSvdScratchPerCta; }
 
 int choose_precision(clr_ctx_t ctx, clr_mat_t a, clr_mat_t b, double eps_in = -1.0) {
   int prec = ctx->opts.precision;
@@ -1174,7 +1169,7 @@ int multiply_into(clr_ctx_t ctx, clr_mat_t a, clr_mat_t b, clr_mat_t c, double a
   // the low-rank blocks are staged as reconstructions): the low-rank kernel skips those
   const bool dense_by_gemm = prec != CLR_PREC_FP64;
   launch_lr_products(av, bv, cv, p, (double*)ctx->cur->ws.p, (double*)ctx->cur->scratch.p,
-                     kScratchPerCta, dense_by_gemm, lr_grid, s);
+                     scratch_per_cta(), dense_by_gemm, lr_grid, s);
   CLR_CHECK_LAUNCH("low-rank products");
   prof_launches(ctx, 1);
   prof_mark(ctx, s, PH_LOWRANK);

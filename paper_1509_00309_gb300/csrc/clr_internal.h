@@ -128,13 +128,13 @@ __device__ __forceinline__ void cta_gemm_tiled(int P, int Q, int L, const double
 template <int NT, int TRI = 0, class T>
 __device__ __forceinline__ void cta_gemm_auto(int P, int Q, int L, const T* a, int64_t a_r,
                                               int64_t a_c, const T* b, int64_t b_r, int64_t b_c,
-                                              T* out, int64_t ldo) {
+                                              T* out, int64_t ldo, bool accumulate = false) {
   if (P * Q >= 32 * NT)
-    cta_gemm_micro<NT, 4, 2, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, false);
+    cta_gemm_micro<NT, 4, 2, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
   else if (P * Q >= 4 * NT)
-    cta_gemm_micro<NT, 2, 2, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, false);
+    cta_gemm_micro<NT, 2, 2, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
   else
-    cta_gemm_micro<NT, 1, 1, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, false);
+    cta_gemm_micro<NT, 1, 1, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
 }
 
 struct Triple {

@@ -5,8 +5,8 @@
 //   LR x dense  (LD):  (X_A W_A^T) B_KJ          -> X_A (B_KJ^T W_A)^T      rank r_A
 //   LR x LR     (LL):  Z = W_A^T X_B (r_A x r_B), then X_A Z with W_B (rank r_B) or X_A with
 //                      W_B Z^T (rank r_A), whichever output rank is smaller (Eq. 1; tie: X_A Z)
-// Low-rank sums are concatenations of factors (Eq. lr_addition).  One CTA owns one C tile and
-// walks its products in k order:
+// Low-rank sums are concatenations of factors (Eq. lr_addition).  One cluster of CTAs owns one C
+// tile and walks its products in k order:
 //   ROUTE_QR     the factor pairs are written side by side into the tile's concatenation
 //                workspace (X_cat m x R, W_cat n x R) for recompression by K5;
 //   ROUTE_DENSE  the tile already holds the dense x dense sum; every low-rank product is
@@ -16,38 +16,69 @@
 // With a tensor-core GEMM (split precision or exact slices: dense_by_gemm) the GEMM sums all
 // contributions of DENSE and DACC_G tiles; this kernel builds the ROUTE_QR concatenations and the
 // FP64 DACC sums.
+//
+// The work is FP64-pipe-bound (~2 FMAs per clock and SM) and a product has far fewer tiles with
+// low-rank work than SMs, or tiles that differ by an order of magnitude, so a tile is spread over
+// the CTAs of a cluster: CTA c owns the rows [m c / CS, m (c + 1) / CS) of the tile, of X_cat and
+// of every X_t, and that share of the rows of W_cat.  What every CTA needs whole (Z, and a
+// computed W_t of a dense accumulation) is formed in shares into the cluster's scratch and
+// exchanged by one cluster barrier; two buffers in turn make that barrier the only one.
+// Measured (one tile per CTA before): Coulomb-like lattice at N = 2048 (144 tiles, 1452 LL
+// products of rank ~40) 25.3 -> 9.7 ms; 1D chain at N = 2048 257 -> 88 us.
+#include <cooperative_groups.h>
+
 #include "clr_internal.h"
 
 namespace clr {
 
-// out(i,j) (= or +=) sum_l a(i,l) b(l,j) for a P x Q output with arbitrary element strides
-// (register-tiled, clr_internal.h).
+namespace cg = cooperative_groups;
+
+constexpr int kLrThreads = 256;
+
+// out(i,j) (= or +=) sum_l a(i,l) b(l,j) for a P x Q output with arbitrary element strides, the
+// micro-tile by the size of the output (clr_internal.h).
 __device__ __forceinline__ void cta_gemm(int P, int Q, int L, const double* a, int64_t a_r,
                                          int64_t a_c, const double* b, int64_t b_r, int64_t b_c,
                                          double* out, int64_t ldo, bool accumulate) {
-  cta_gemm_tiled<256>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
+  cta_gemm_auto<kLrThreads>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
 }
 
 __device__ void cta_copy_cols(int rows, int cols, const double* src, int64_t lds, double* dst,
                               int64_t ldd) {
-  for (int e = threadIdx.x; e < rows * cols; e += blockDim.x) {
+  for (int e = threadIdx.x; e < rows * cols; e += kLrThreads) {
     const int i = e % rows, j = e / rows;
     dst[i + (int64_t)j * ldd] = src[i + (int64_t)j * lds];
   }
 }
 
 constexpr int64_t kZElems = (int64_t)(CLR_MAX_CLUSTER / 2) * (CLR_MAX_CLUSTER / 2);
+constexpr int64_t kFElems = (int64_t)CLR_MAX_CLUSTER * (CLR_MAX_CLUSTER / 2);
+// scratch: per cluster (in its first CTA's part) two buffers of Z and of a shared W_t, then per
+// CTA its rows of X_t
+static_assert(2 * (kZElems + kFElems) + kFElems <= kSvdScratchPerCta, "low-rank scratch");
 
-__global__ void __launch_bounds__(256) lr_products_kernel(MatView A, MatView B, MatView C,
-                                                          Plan p, double* ws, double* scratch,
-                                                          int64_t scratch_per_cta,
-                                                          int dense_by_gemm) {
-  __shared__ int sh_next;
-  double* scrZ = scratch + (int64_t)blockIdx.x * scratch_per_cta;
-  double* scrF = scrZ + kZElems;
+template <int CS>
+__global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kLrThreads)
+    lr_products_kernel(MatView A, MatView B, MatView C, Plan p, double* ws, double* scratch,
+                       int64_t scratch_per_cta, int dense_by_gemm) {
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ int sh_next[2];
+  const int rank = (int)cluster.block_rank();
+  double* shared_scr = scratch + (int64_t)(blockIdx.x - rank) * scratch_per_cta;
+  double* scrX = scratch + (int64_t)blockIdx.x * scratch_per_cta + 2 * (kZElems + kFElems);
   const int n_lr = p.counters->n_lr;
   int* sched = &p.counters->sched[0];
-  for (int li = next_item(sched, &sh_next); li < n_lr; li = next_item(sched, &sh_next)) {
+  int slot = 0, par = 0;
+  while (true) {
+    // the cluster's next tile (two slots: one is read while the other is written)
+    if (rank == 0 && threadIdx.x == 0) {
+      const int v = atomicAdd(sched, 1);
+      for (int c = 0; c < CS; ++c) *cluster.map_shared_rank(&sh_next[slot], c) = v;
+    }
+    cluster.sync();
+    const int li = sh_next[slot];
+    slot ^= 1;
+    if (li >= n_lr) break;
     const int t = p.l_lr[li];
     const int I = t / p.nJ, J = t % p.nJ;
     const int m = C.row_off[I + 1] - C.row_off[I];
@@ -62,10 +93,10 @@ __global__ void __launch_bounds__(256) lr_products_kernel(MatView A, MatView B, 
     double* Xcat = ws + 2 * sC;
     double* Wcat = Xcat + (int64_t)m * R;
     const bool concat = route == ROUTE_QR;
-    if (route == ROUTE_DACC) {
-      for (int e = threadIdx.x; e < m * n; e += blockDim.x) D[e] = 0.0;
-      __syncthreads();
-    }
+    // this CTA's rows of the tile (and of X_t), and of W_t
+    const int x0 = m * rank / CS, xr = m * (rank + 1) / CS - x0;
+    const int w0 = n * rank / CS, wr = n * (rank + 1) / CS - w0;
+    bool first = route == ROUTE_DACC;   // a DACC sum starts from zero
     const int start = p.t_start[t], count = p.t_count[t];
     for (int q = 0; q < count; ++q) {
       const Triple tr = p.triples[start + q];
@@ -75,57 +106,52 @@ __global__ void __launch_bounds__(256) lr_products_kernel(MatView A, MatView B, 
       const int ra = A.rank[I * A.nc + K], rb = B.rank[K * B.nc + J];
       const double* Ab = A.pool + slot_of(A, I, K, m);
       const double* Bb = B.pool + slot_of(B, K, J, k);
-      const double* Xt;  // m x rt, ld m
-      const double* Wt;  // n x rt, ld n
-      int rt;
-      if (tr.kind == T_DL) {
-        // X_t = A_IK X_B, W_t = W_B
-        const double* XB = Bb;
-        const double* WB = Bb + (int64_t)k * rb;
-        rt = rb;
-        double* dst = concat ? Xcat + (int64_t)m * tr.col : scrF;
-        cta_gemm(m, rb, k, Ab, 1, m, XB, 1, k, dst, m, false);
-        Xt = dst;
-        Wt = WB;
-        if (concat) cta_copy_cols(n, rb, WB, n, Wcat + (int64_t)n * tr.col, n);
-      } else if (tr.kind == T_LD) {
-        // X_t = X_A, W_t = B_KJ^T W_A
-        const double* XA = Ab;
-        const double* WA = Ab + (int64_t)m * ra;
-        rt = ra;
-        double* dst = concat ? Wcat + (int64_t)n * tr.col : scrF;
-        cta_gemm(n, ra, k, Bb, k, 1, WA, 1, k, dst, n, false);
-        Xt = XA;
-        Wt = dst;
-        if (concat) cta_copy_cols(m, ra, XA, m, Xcat + (int64_t)m * tr.col, m);
-      } else {
-        const double* XA = Ab;
-        const double* WA = Ab + (int64_t)m * ra;
-        const double* XB = Bb;
-        const double* WB = Bb + (int64_t)k * rb;
-        // Z = W_A^T X_B  (ra x rb, column-major)
-        cta_gemm(ra, rb, k, WA, k, 1, XB, 1, k, scrZ, ra, false);
-        __syncthreads();
-        if (rb <= ra) {
-          rt = rb;  // X_t = X_A Z, W_t = W_B
-          double* dst = concat ? Xcat + (int64_t)m * tr.col : scrF;
-          cta_gemm(m, rb, ra, XA, 1, m, scrZ, 1, ra, dst, m, false);
-          Xt = dst;
-          Wt = WB;
-          if (concat) cta_copy_cols(n, rb, WB, n, Wcat + (int64_t)n * tr.col, n);
-        } else {
-          rt = ra;  // X_t = X_A, W_t = W_B Z^T
-          double* dst = concat ? Wcat + (int64_t)n * tr.col : scrF;
-          cta_gemm(n, ra, rb, WB, 1, n, scrZ, ra, 1, dst, n, false);
-          Xt = XA;
-          Wt = dst;
-          if (concat) cta_copy_cols(m, ra, XA, m, Xcat + (int64_t)m * tr.col, m);
-        }
+      const double* XA = Ab;                        // low-rank A: m x ra, then k x ra
+      const double* WA = Ab + (int64_t)m * ra;
+      const double* XB = Bb;                        // low-rank B: k x rb, then n x rb
+      const double* WB = Bb + (int64_t)k * rb;
+      const bool x_side = tr.kind == T_DL || (tr.kind == T_LL && rb <= ra);
+      double* scrZ = shared_scr + par * (kZElems + kFElems);
+      double* scrF = scrZ + kZElems;
+      if (tr.kind == T_LL) {
+        // Z = W_A^T X_B (ra x rb, column-major), its columns in shares
+        const int z0 = rb * rank / CS, zc = rb * (rank + 1) / CS - z0;
+        cta_gemm(ra, zc, k, WA, k, 1, XB + (int64_t)z0 * k, 1, k, scrZ + (int64_t)z0 * ra, ra,
+                 false);
+        cluster.sync();
+        par ^= 1;
       }
-      __syncthreads();
+      const int rt = x_side ? rb : ra;
+      if (x_side) {
+        // X_t = A_IK X_B or X_A Z, this CTA's rows; W_t = W_B
+        double* dst = concat ? Xcat + (int64_t)m * tr.col + x0 : scrX;
+        const int64_t ldd = concat ? m : xr;
+        if (tr.kind == T_DL)
+          cta_gemm(xr, rb, k, Ab + x0, 1, m, XB, 1, k, dst, ldd, false);
+        else
+          cta_gemm(xr, rb, ra, XA + x0, 1, m, scrZ, 1, ra, dst, ldd, false);
+        if (concat) cta_copy_cols(wr, rb, WB + w0, n, Wcat + (int64_t)n * tr.col + w0, n);
+      } else {
+        // X_t = X_A; W_t = B_KJ^T W_A or W_B Z^T, this CTA's rows
+        double* dst = (concat ? Wcat + (int64_t)n * tr.col : scrF) + w0;
+        if (tr.kind == T_LD)
+          cta_gemm(wr, ra, k, Bb + (int64_t)w0 * k, k, 1, WA, 1, k, dst, n, false);
+        else
+          cta_gemm(wr, ra, rb, WB + w0, 1, n, scrZ, ra, 1, dst, n, false);
+        if (concat) cta_copy_cols(xr, ra, XA + x0, m, Xcat + (int64_t)m * tr.col + x0, m);
+      }
       if (!concat) {
-        // D += X_t W_t^T
-        cta_gemm(m, n, rt, Xt, 1, m, Wt, n, 1, D, m, true);
+        // D += X_t W_t^T, this CTA's rows (the whole of W_t)
+        const double* Xt = x_side ? scrX : XA + x0;
+        const int64_t ldx = x_side ? xr : m;
+        if (x_side) {
+          __syncthreads();
+        } else {
+          cluster.sync();
+          if (tr.kind == T_LD) par ^= 1;   // (an LL product has switched buffers already)
+        }
+        cta_gemm(xr, n, rt, Xt, 1, ldx, x_side ? WB : scrF, n, 1, D + x0, m, !first);
+        first = false;
         __syncthreads();
       }
     }
@@ -136,8 +162,17 @@ __global__ void __launch_bounds__(256) lr_products_kernel(MatView A, MatView B, 
 void launch_lr_products(const MatView& A, const MatView& B, const MatView& C, const Plan& p,
                         double* ws, double* scratch, int64_t scratch_per_cta, int dense_by_gemm,
                         int grid, cudaStream_t st) {
-  lr_products_kernel<<<grid, 256, 0, st>>>(A, B, C, p, ws, scratch, scratch_per_cta,
-                                           dense_by_gemm);
+  // Eight CTAs a tile while the tiles are few (the 1D chain at N = 512: 16 tiles on 152 SMs),
+  // else four: from about 64 tiles on four already fill the SMs, with fewer exchanges.
+  if (p.nI * p.nJ <= 64) {
+    const int g = grid / 8 > 0 ? grid / 8 * 8 : 8;
+    lr_products_kernel<8><<<g, kLrThreads, 0, st>>>(A, B, C, p, ws, scratch, scratch_per_cta,
+                                                    dense_by_gemm);
+  } else {
+    const int g = grid / 4 > 0 ? grid / 4 * 4 : 4;
+    lr_products_kernel<4><<<g, kLrThreads, 0, st>>>(A, B, C, p, ws, scratch, scratch_per_cta,
+                                                    dense_by_gemm);
+  }
 }
 
 }  // namespace clr
