@@ -115,13 +115,10 @@ __device__ __forceinline__ void cta_gemm_micro(int P, int Q, int L, const T* a, 
   }
 }
 
-template <int NT>
-__device__ __forceinline__ void cta_gemm_tiled(int P, int Q, int L, const double* a,
-                                               int64_t a_r, int64_t a_c, const double* b,
-                                               int64_t b_r, int64_t b_c, double* out,
-                                               int64_t ldo, bool accumulate) {
-  cta_gemm_micro<NT, 4, 2, 0>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
-}
+// CTAs per block of the kernels that form the low-rank blocks' values, by the number of blocks
+// (how many of them are low rank is not known on the host): 8 where a CTA per block could not
+// fill 152 SMs evenly, 1 where the blocks alone do.
+inline int lr_parts(int n_blocks) { return n_blocks <= 1024 ? 8 : n_blocks <= 4096 ? 4 : 1; }
 
 // The micro-tile by the size of the output: 4 x 2 from four rounds of the CTA's threads on
 // (less than a quarter of a round idle at the end), 2 x 2 from one, else an entry per thread.

@@ -736,7 +736,8 @@ __global__ void __launch_bounds__(256) oz_lr_recon_kernel(MatView M, double* rec
   const double* x = M.pool + slot;             // m x r, ld m
   const double* w = x + (int64_t)m * r;        // n x r, ld n
   // out(i, j) = sum_q X(i, q) W(j, q)
-  cta_gemm_tiled<256>(m, n, r, x, 1, m, w, n, 1, recon + slot, m, false);
+  const int j0 = n * (int)blockIdx.y / (int)gridDim.y, j1 = n * ((int)blockIdx.y + 1) / (int)gridDim.y;
+  cta_gemm_auto<256>(m, j1 - j0, r, x, 1, m, w + j0, n, 1, recon + slot + (int64_t)j0 * m, m);
 }
 
 __global__ void __launch_bounds__(256) oz_exp_lr_kernel(MatView M, const double* recon,
@@ -838,7 +839,7 @@ void launch_ozaki_stage(const MatView& M, const int* row_idx, const int* col_idx
     const dim3 ne((unsigned)rows_pad, (unsigned)n_seg);
     oz_exp_b_kernel<<<ne, 256, 0, st>>>(M, row_idx, col_idx, exps, rows_pad, cols_pad);
   }
-  oz_lr_recon_kernel<<<nb, 256, 0, st>>>(M, recon);
+  oz_lr_recon_kernel<<<dim3(nb, (unsigned)lr_parts((int)nb)), 256, 0, st>>>(M, recon);
   oz_exp_lr_kernel<<<nb, 256, 0, st>>>(M, recon, exps, rows_pad, a_mode);
   if (a_mode) {
     const unsigned nd = (unsigned)((rows_pad / 32) * (cols_pad / 128));

@@ -134,8 +134,10 @@ __global__ void __launch_bounds__(256) split_stage_b_kernel(MatView M, const int
     *reinterpret_cast<unsigned long long*>(panels + t * plane + j * cols_pad + k) = packed[t];
 }
 
-// Low-rank blocks into the panels: one CTA per block of M (blocks of another kind return at
-// once), entry (i, j) = sum_t X(i, t) W(j, t) in FP64, then split as the dense pass does.
+// Low-rank blocks into the panels: lr_parts CTAs per block of M (blocks of another kind return at
+// once), entry (i, j) = sum_t X(i, t) W(j, t) in FP64, then split as the dense pass does.  (Bound
+// by the FP64 pipe; with one CTA per block the few low-rank blocks of a chain matrix left most
+// SMs idle: 160-220 us a launch at N = 1024..3072, now 30-50.)
 // a_mode: panel[t][row][k] = A(row, k); else panel[t][col][k] = B(k, col).
 template <int TERMS>
 __global__ void __launch_bounds__(256) split_stage_lr_kernel(MatView M, unsigned short* panels,
@@ -150,7 +152,7 @@ __global__ void __launch_bounds__(256) split_stage_lr_kernel(MatView M, unsigned
   const double* x = M.pool + (int64_t)M.row_off[R] * M.n_cols + (int64_t)mR * M.col_off[Cc];
   const double* w = x + (int64_t)mR * r;
   const int64_t plane = rows_pad * cols_pad;
-  for (int e = threadIdx.x; e < mR * nC; e += blockDim.x) {
+  for (int e = threadIdx.x + blockDim.x * blockIdx.y; e < mR * nC; e += blockDim.x * gridDim.y) {
     const int i = a_mode ? e / nC : e % mR;  // consecutive threads along the panel's k
     const int j = a_mode ? e % nC : e / mR;
     double v = 0.0;
@@ -181,7 +183,7 @@ void launch_split_stage(const MatView& M, const int* row_idx, const int* col_idx
     else
       split_stage_b_kernel<3><<<n, 256, 0, st>>>(M, row_idx, col_idx, pn, rows_pad, cols_pad);
   }
-  const unsigned nb = (unsigned)(M.nr * M.nc);
+  const dim3 nb((unsigned)(M.nr * M.nc), (unsigned)lr_parts(M.nr * M.nc));
   if (terms == 2)
     split_stage_lr_kernel<2><<<nb, 256, 0, st>>>(M, pn, rows_pad, cols_pad, a_mode);
   else
