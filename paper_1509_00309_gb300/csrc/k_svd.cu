@@ -68,11 +68,11 @@ __device__ double block_sum(double v, double* sh) {
 // SM, an addition in a reduction as dear as a fused multiply-add, and a scalar square root or
 // division (9 such instructions) repeated by 16 warps dearer than the column work of a small
 // step.  So:
-//  - a warp takes four columns at a time and sums their four inner products together
-//    (warp_sum4: 6 additions instead of 20); the scalars that follow (the multiplier, the new
-//    entry of R, the downdated norm) are then formed for the four columns by one instruction
-//    each, in the lanes that hold their sums; the columns stay in registers from the inner
-//    product to the update;
+//  - a warp takes eight columns at a time, eight lanes to a column and two columns to a lane: the
+//    inner products need 3 additions for the eight columns (with a warp per column 5 each), no
+//    more than 7 rows' lanes idle in a column's last instruction, and the scalars that follow
+//    (the multiplier, the new entry of R, the downdated norm) are formed for the eight columns
+//    by one instruction each, in the lanes that hold their sums;
 //  - the reflector is not scaled: v = (v_0, x_{j+1}, ...) with x the column as it is, and
 //    H y = y - v (v.y) rn rv with rn = 1 / ||x_j..||, rv = 1 / |v_0| (v.v / 2 = ||x|| |v_0|; two
 //    factors, so that neither over- nor underflows before ||x||^2 does).  One warp forms these
@@ -82,10 +82,11 @@ __device__ double block_sum(double v, double* sh) {
 // N = 4096 (pivoted QR of every block) 28.5 -> 24.5 ms.
 // ---------------------------------------------------------------------------------------------
 constexpr int kRowsPerLane = CLR_MAX_CLUSTER / 32;
-constexpr int kGroup = 4;   // columns a warp takes together
+constexpr int kGroup = 8;   // columns a warp takes together in a step
+constexpr int kQuad = 4;    // and where it holds whole columns (warp_sum4)
 
 // The warp's sums of s[0..3]: lane l receives the sum of s[l / 8].
-__device__ __forceinline__ double warp_sum4(const double (&s)[kGroup]) {
+__device__ __forceinline__ double warp_sum4(const double (&s)[kQuad]) {
   const int l = threadIdx.x % 32;
   const bool h16 = (l & 16) != 0, h8 = (l & 8) != 0;
   double a0 = h16 ? s[2] : s[0], a1 = h16 ? s[3] : s[1];
@@ -103,77 +104,76 @@ __device__ __forceinline__ void group_sync(int bar, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(threads) : "memory");
 }
 
-// Up to four columns held by a warp (rows l, l + 32, ... of n; nt = ceil(n / 32)).  The reflector
-// x is read again where it is used: the registers hold the four columns.
-struct ColGroup {
-  double y[kGroup][kRowsPerLane];
-  template <class Col>
-  __device__ __forceinline__ double load_dot(const double* x, int n, int nt, int c0, int ncol,
+// One group of a step: columns c0 .. c0 + 7 of ncol (col(c): the column's n rows), lane l works on
+// columns c0 + l / 8 and c0 + 4 + l / 8, rows l % 8, l % 8 + 8, ...; the sums arrive in the lanes
+// of group_column.
+__device__ __forceinline__ int group_column(int c0) {
+  const int l = threadIdx.x % 32;
+  return c0 + l / 8 + (l & 4);
+}
+__device__ __forceinline__ double group_sum(double s0, double s1) {
+  const bool hi = (threadIdx.x & 4) != 0;
+  double a = hi ? s1 : s0;
+  a += __shfl_xor_sync(0xffffffffu, hi ? s0 : s1, 4);
+  a += __shfl_xor_sync(0xffffffffu, a, 2);
+  a += __shfl_xor_sync(0xffffffffu, a, 1);
+  return a;
+}
+template <class Col>
+__device__ __forceinline__ double group_dot(const double* x, int n, int c0, int ncol, Col col) {
+  const int l = threadIdx.x % 32, a = c0 + l / 8, b = a + 4;
+  const double* ya = col(a < ncol ? a : c0);
+  const double* yb = col(b < ncol ? b : c0);
+  double s0 = 0.0, s1 = 0.0;
+  if (c0 + 4 < ncol) {
+#pragma unroll 4
+    for (int i = l % 8; i < n; i += 8) {
+      const double xv = x[i];
+      s0 = fma(xv, ya[i], s0);
+      s1 = fma(xv, yb[i], s1);
+    }
+  } else {
+#pragma unroll 4
+    for (int i = l % 8; i < n; i += 8) s0 = fma(x[i], ya[i], s0);
+  }
+  return group_sum(s0, s1);
+}
+// y_c -= f_c x, f_c in the lanes of group_column
+template <class Col>
+__device__ __forceinline__ void group_update(const double* x, double f, int n, int c0, int ncol,
                                              Col col) {
-    const int l = threadIdx.x % 32;
-    const double* yc[kGroup];
-    double s[kGroup];
-#pragma unroll
-    for (int c = 0; c < kGroup; ++c) {
-      s[c] = 0.0;
-      yc[c] = col(c0 + c < ncol ? c0 + c : c0);
+  const int l = threadIdx.x % 32, a = c0 + l / 8, b = a + 4;
+  const double fa = -__shfl_sync(0xffffffffu, f, l & 24);
+  const double fb = -__shfl_sync(0xffffffffu, f, (l & 24) + 4);
+  double* ya = col(a < ncol ? a : c0);
+  double* yb = col(b < ncol ? b : c0);
+  if (b < ncol) {
+#pragma unroll 4
+    for (int i = l % 8; i < n; i += 8) {
+      const double xv = x[i];
+      const double u = fma(fa, xv, ya[i]), v = fma(fb, xv, yb[i]);
+      ya[i] = u;
+      yb[i] = v;
     }
-#pragma unroll
-    for (int t = 0; t < kRowsPerLane; ++t)
-      if (t < nt) {
-        const bool in = l + 32 * t < n;
-#pragma unroll
-        for (int c = 0; c < kGroup; ++c) y[c][t] = in ? yc[c][l + 32 * t] : 0.0;
-      }
-#pragma unroll
-    for (int t = 0; t < kRowsPerLane; ++t)
-      if (t < nt) {
-        const double xv = l + 32 * t < n ? x[l + 32 * t] : 0.0;
-#pragma unroll
-        for (int c = 0; c < kGroup; ++c)
-          if (c0 + c < ncol) s[c] = fma(xv, y[c][t], s[c]);
-      }
-    return warp_sum4(s);
+  } else if (a < ncol) {
+#pragma unroll 4
+    for (int i = l % 8; i < n; i += 8) ya[i] = fma(fa, x[i], ya[i]);
   }
-  // y_c -= f_c x, f_c in the lanes 8 c .. 8 c + 7
-  template <class Col>
-  __device__ __forceinline__ void update_store(const double* x, double f, int n, int nt, int c0,
-                                               int ncol, Col col) {
-    const int l = threadIdx.x % 32;
-    double fc[kGroup];
-    double* yc[kGroup];
-#pragma unroll
-    for (int c = 0; c < kGroup; ++c) {
-      fc[c] = __shfl_sync(0xffffffffu, f, 8 * c);
-      yc[c] = col(c0 + c < ncol ? c0 + c : c0);
-    }
-#pragma unroll
-    for (int t = 0; t < kRowsPerLane; ++t)
-      if (t < nt) {
-        const bool in = l + 32 * t < n;
-        const double xv = in ? x[l + 32 * t] : 0.0;
-#pragma unroll
-        for (int c = 0; c < kGroup; ++c)
-          if (c0 + c < ncol) {
-            y[c][t] = fma(-fc[c], xv, y[c][t]);
-            if (in) yc[c][l + 32 * t] = y[c][t];
-          }
-      }
+  __syncwarp();
+}
+template <class Col>
+__device__ __forceinline__ double group_squares(int n, int c0, int ncol, Col col) {
+  const int l = threadIdx.x % 32, a = c0 + l / 8, b = a + 4;
+  const double* ya = col(a < ncol ? a : c0);
+  const double* yb = col(b < ncol ? b : c0);
+  double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
+  for (int i = l % 8; i < n; i += 8) {
+    s0 = fma(ya[i], ya[i], s0);
+    s1 = fma(yb[i], yb[i], s1);
   }
-  __device__ __forceinline__ double sum_squares(int nt, int c0, int ncol) const {
-    double s[kGroup];
-#pragma unroll
-    for (int c = 0; c < kGroup; ++c) {
-      s[c] = 0.0;
-      if (c0 + c < ncol) {
-#pragma unroll
-        for (int t = 0; t < kRowsPerLane; ++t)
-          if (t < nt) s[c] = fma(y[c][t], y[c][t], s[c]);
-      }
-    }
-    return warp_sum4(s);
-  }
-};
+  return group_sum(s0, s1);
+}
 
 // The reflector of a column (x0 above the n rows x), by one warp: *v0, *rn, *rv as above (rn =
 // 0 and H = I when the rows below are zero) and the new diagonal entry (returned).
@@ -211,10 +211,9 @@ __device__ __noinline__ void householder_qr(double* a, int p, int q, Reflectors&
   const int l = threadIdx.x % 32;
   for (int j = 0; j < q; ++j) {
     double* cj = a + (int64_t)j * p;
-    const int n = p - j - 1, nt = (n + 31) / 32, ncol = q - j - 1;
+    const int n = p - j - 1, ncol = q - j - 1;
     auto col = [&](int c) { return a + (int64_t)(j + 1 + c) * p + j + 1; };
     const double* x = cj + j + 1;
-    ColGroup g;
     double d = 0.0;
     if (w == 0) {
       double v0, rn, rv;
@@ -227,18 +226,18 @@ __device__ __noinline__ void householder_qr(double* a, int p, int q, Reflectors&
         h.rv[j] = rv;
       }
     } else if (kGroup * (w - 1) < ncol) {
-      d = g.load_dot(x, n, nt, kGroup * (w - 1), ncol, col);
+      d = group_dot(x, n, kGroup * (w - 1), ncol, col);
     }
     group_sync(bar, 32 * nw);
     const double v0 = h.v0[j], rn = h.rn[j], rv = h.rv[j];
     // the groups taken above, then the rest over all warps
     for (int gi = w > 0 ? w - 1 : nw - 1; kGroup * gi < ncol; gi = (gi < nw - 1 ? nw - 1 + w : gi + nw)) {
-      const int c0 = kGroup * gi, c = c0 + l / 8;
-      if (gi >= nw - 1) d = g.load_dot(x, n, nt, c0, ncol, col);
+      const int c0 = kGroup * gi, c = group_column(c0);
+      if (gi >= nw - 1) d = group_dot(x, n, c0, ncol, col);
       const double yj = c < ncol ? col(c)[-1] : 0.0;
       const double f = fma(v0, yj, d) * rn * rv;
-      g.update_store(x, f, n, nt, c0, ncol, col);
-      if (c < ncol && l % 8 == 0) col(c)[-1] = fma(-f, v0, yj);
+      group_update(x, f, n, c0, ncol, col);
+      if (c < ncol && l % 4 == 0) col(c)[-1] = fma(-f, v0, yj);
     }
     group_sync(bar, 32 * nw);
   }
@@ -252,10 +251,10 @@ __device__ __noinline__ void apply_q(const double* v, int p, int k, const Reflec
                                      int nw) {
   const int l = threadIdx.x % 32;
   const int nt = (p + 31) / 32;
-  for (int g0 = kGroup * w; g0 < r; g0 += kGroup * nw) {
-    double yr[kGroup][kRowsPerLane];
+  for (int g0 = kQuad * w; g0 < r; g0 += kQuad * nw) {
+    double yr[kQuad][kRowsPerLane];
 #pragma unroll
-    for (int c = 0; c < kGroup; ++c)
+    for (int c = 0; c < kQuad; ++c)
 #pragma unroll
       for (int t = 0; t < kRowsPerLane; ++t)
         yr[c][t] = g0 + c < r && l + 32 * t < p ? y[l + 32 * t + (int64_t)(g0 + c) * ldy] : 0.0;
@@ -263,103 +262,80 @@ __device__ __noinline__ void apply_q(const double* v, int p, int k, const Reflec
       const double* vj = v + (int64_t)(perm ? perm[j] : j) * p;
       const int t0 = j / 32;
       const double v0 = h.v0[j];
-      double s[kGroup];
+      double s[kQuad];
       auto xv = [&](int i) { return i > j && i < p ? vj[i] : (i == j ? v0 : 0.0); };
 #pragma unroll
-      for (int c = 0; c < kGroup; ++c) s[c] = 0.0;
+      for (int c = 0; c < kQuad; ++c) s[c] = 0.0;
 #pragma unroll
       for (int t = 0; t < kRowsPerLane; ++t)
         if (t >= t0 && t < nt) {
           const double x = xv(l + 32 * t);
 #pragma unroll
-          for (int c = 0; c < kGroup; ++c)
+          for (int c = 0; c < kQuad; ++c)
             if (g0 + c < r) s[c] = fma(x, yr[c][t], s[c]);
         }
       const double f = warp_sum4(s) * h.rn[j] * h.rv[j];
-      double fc[kGroup];
+      double fc[kQuad];
 #pragma unroll
-      for (int c = 0; c < kGroup; ++c) fc[c] = __shfl_sync(0xffffffffu, f, 8 * c);
+      for (int c = 0; c < kQuad; ++c) fc[c] = __shfl_sync(0xffffffffu, f, 8 * c);
 #pragma unroll
       for (int t = 0; t < kRowsPerLane; ++t)
         if (t >= t0 && t < nt) {
           const double x = xv(l + 32 * t);
 #pragma unroll
-          for (int c = 0; c < kGroup; ++c)
+          for (int c = 0; c < kQuad; ++c)
             if (g0 + c < r) yr[c][t] = fma(-fc[c], x, yr[c][t]);
         }
     }
 #pragma unroll
-    for (int c = 0; c < kGroup; ++c)
+    for (int c = 0; c < kQuad; ++c)
 #pragma unroll
       for (int t = 0; t < kRowsPerLane; ++t)
         if (g0 + c < r && l + 32 * t < p) y[l + 32 * t + (int64_t)(g0 + c) * ldy] = yr[c][t];
   }
 }
 
-// Per-pair arithmetic of the Jacobi sweeps.  FP64 runs at 1/64 of the FP32 rate on this part
-// and each FP64 instruction of a warp occupies its sub-partition's FP64 pipe for many cycles,
-// so the scalar steps avoid FP64 square roots and most divisions: the tests compare squares,
-// the rotation's tangent t is found in FP32 from zeta (its accuracy only sets how far one
-// rotation reduces the pair's inner product) and c = (1 + t^2)^-1/2 is refined in FP64 by two
-// Newton steps from the FP32 seed, so that c^2 + s^2 = 1 to FP64 rounding and the rotation is
-// orthogonal.
-// In FP32 the hardware approximations (a few ulp) serve throughout: the FP32 stages only find
-// rotations that the FP64 stages apply and refine.
-__device__ __forceinline__ float rt_sqrt(float x) {
-  return x > 0.f ? (x <= FLT_MAX ? x * rsqrtf(x) : x) : 0.f;
+// ---------------------------------------------------------------------------------------------
+// One-sided Jacobi.  The columns' pairs of a round are disjoint (cyclic round-robin order).  A
+// pair found converged (or below the floor) is checked again only once one of its columns has
+// been rotated: each pair meets at the same round of every sweep, so when neither column has been
+// rotated since the pair's check one sweep earlier, its inner product is the one that check
+// computed and the pair is skipped.  Late sweeps, and the refinement of columns that are already
+// orthogonal to each other, then touch only the pairs of recently rotated columns.
+//
+// The rotation (Rutishauser): zeta = (b - a) / 2g, t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)),
+// c = 1 / sqrt(1 + t^2), s = c t, with a, b the squared norms and g the inner product.
+// ---------------------------------------------------------------------------------------------
+// columns (a, b) of pair k in a round over qq slots
+__device__ __forceinline__ void round_pair(int round, int k, int qq, int* a, int* b) {
+  int x = round, y = qq - 1;
+  if (k > 0) {
+    x = round + k;
+    if (x >= qq - 1) x -= qq - 1;
+    y = round - k;
+    if (y < 0) y += qq - 1;
+  }
+  *a = x;
+  *b = y;
 }
 
-__device__ __forceinline__ bool pair_below_floor(float al, float be, float f2) {
-  const float s = rt_sqrt(al * be);
-  return s == 0.f || s <= f2;
-}
-__device__ __forceinline__ bool pair_below_floor(double al, double be, double f2) {
-  const double p2 = al * be;
-  return p2 == 0.0 || p2 <= f2 * f2;
-}
-
-// |g| <= tol |g_a| |g_b| or |g| <= floor2
-__device__ __forceinline__ bool pair_converged(float al, float be, float g, float tol, float f2) {
-  const float s = rt_sqrt(al * be);
-  return fabsf(g) <= tol * s || fabsf(g) <= f2;
-}
-__device__ __forceinline__ bool pair_converged(double al, double be, double g, double tol,
-                                               double f2) {
-  const double g2 = g * g;
-  return g2 <= tol * tol * (al * be) || g2 <= f2 * f2;
-}
-
-// Rutishauser's rotation: zeta = (b - a) / 2g, t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)),
-// c = 1 / sqrt(1 + t^2), s = c t.
-// (for |zeta| > 2^40, where zeta^2 may overflow, the asymptote 1 / (2 zeta))
-__device__ __forceinline__ float tangent_of(float zeta) {
-  if (fabsf(zeta) > 0x1p40f) return __fdividef(0.5f, zeta);
-  return copysignf(__fdividef(1.f, fabsf(zeta) + rt_sqrt(1.f + zeta * zeta)), zeta);
-}
-__device__ __forceinline__ float rot_tangent(float d, float g) {
-  return tangent_of(__fdividef(d, 2.f * g));
-}
-__device__ __forceinline__ void rotation(float al, float be, float g, float& c, float& s,
-                                         float& t) {
-  t = rot_tangent(be - al, g);
-  // (one Newton step on the approximate root: c^2 + s^2 drifts less from 1 over many rotations)
-  const float u = 1.f + t * t;
-  c = rsqrtf(u);
-  c = c * (1.5f - 0.5f * u * c * c);
-  s = c * t;
-}
+// FP64 (the allocation-free entry point): the tests compare squares, the rotation's tangent t is
+// found in FP32 from zeta where the angle is small (its accuracy only sets how far one rotation
+// reduces the pair's inner product) and c is refined in FP64 by two Newton steps from the FP32
+// seed, so that c^2 + s^2 = 1 to FP64 rounding and the rotation is orthogonal.
 __device__ __forceinline__ void rotation(double al, double be, double g, double& c, double& s,
                                          double& t) {
   // zeta in FP64 (the operands may lie far outside the FP32 range).  For a large angle
   // (|cos| > 1e-3: the first sweeps of a fresh start, nearly parallel columns) the tangent in
   // FP64, since a rotation that is off by u32 there leaves a leak that is large relative to the
-  // smaller column; for the small angles of a refinement in FP32 where |zeta| < 2^100, else its
+  // smaller column; for the small angles of a refinement in FP32 where |zeta| < 2^40, else its
   // asymptote 1 / (2 zeta).
   const double zeta = (be - al) / (2.0 * g);
   if (g * g > 1e-6 * (al * be)) {
     t = copysign(1.0 / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0))), zeta);
-  } else if (fabs(zeta) < 0x1p100) {
-    t = (double)tangent_of((float)zeta);
+  } else if (fabs(zeta) < 0x1p40) {
+    const float z = (float)zeta;
+    t = (double)copysignf(__fdividef(1.f, fabsf(z) + sqrtf(1.f + z * z)), z);
   } else {
     t = 0.5 / zeta;
   }
@@ -371,43 +347,29 @@ __device__ __forceinline__ void rotation(double al, double be, double g, double&
   s = r * t;
 }
 
-// One-sided Jacobi on the q columns of g (p x q, ld ldg); v (q x q, ld ldv) accumulates the
-// rotations (initialised to I here unless reset_v is false; not accumulated when v is null).
-// On return g = U S and the input
-// equals g v^T (times the initial v^T when v is not reset).  T is float or double; the
-// convergence threshold is the type's epsilon times sqrt(p) (times tol_scale); pairs whose inner
-// product is below floor2 are left alone.
-// A pair found converged (or below the floor) is checked again only once one of its columns has
-// been rotated: each pair meets at the same round of every sweep (cyclic round-robin order), so
-// when neither column has been rotated since the pair's check one sweep earlier, its inner
-// product is the one that check computed and the pair is skipped.  Late sweeps, and the
-// refinement of columns that are already orthogonal to each other, then touch only the pairs
-// of recently rotated columns.
-template <typename T>
-__device__ int jacobi_svd(T* g, int p, int q, int64_t ldg, T* v, int64_t ldv,
-                          int max_sweeps, int* sh_flag, bool reset_v = true,
-                          T tol_scale = T(1), T floor2 = T(0)) {
+// One-sided Jacobi in FP64 on the q columns of g (p x q, ld p); v (q x q, ld q), initialised to I
+// here, accumulates the rotations.  On return g = U S and the input equals g v^T.  Pairs whose
+// inner product is below floor2, or below the FP64 epsilon times sqrt(p) relative to the norms,
+// are left alone.  Returns the number of sweeps.
+__device__ int jacobi_svd(double* g, int p, int q, double* v, int max_sweeps, int* sh_flag,
+                          double floor2) {
   // Column norms squared, kept in shared memory: recomputed exactly at every sweep start and
   // refreshed (fused into the rotation pass) for the two columns of every rotated pair, so a
   // pair costs one inner product unless it is rotated.
-  __shared__ T nrm2[CLR_MAX_CLUSTER];
+  __shared__ double nrm2[CLR_MAX_CLUSTER];
   // per column: the step (sweep * (qq - 1) + round) of its last rotation, -1 if none
   __shared__ int last_rot[CLR_MAX_CLUSTER];
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  if (reset_v && v) {
-    for (int e = threadIdx.x; e < q * q; e += kThreads)
-      v[(e % q) + (int64_t)(e / q) * ldv] = (e % q == e / q) ? T(1) : T(0);
-    __syncthreads();
-  }
+  for (int e = threadIdx.x; e < q * q; e += kThreads) v[e] = (e % q == e / q) ? 1.0 : 0.0;
   const int qq = q + (q & 1);  // even number of slots; slot q is a dummy when q is odd
-  const T eps_t = sizeof(T) == 4 ? T(FLT_EPSILON) : T(DBL_EPSILON);
-  const T tol = eps_t * sqrt(T(p)) * tol_scale;
+  const double tol = DBL_EPSILON * sqrt((double)p);
   for (int c = threadIdx.x; c < q; c += kThreads) last_rot[c] = -1;
+  __syncthreads();
   int sweep = 0;
   for (; sweep < max_sweeps; ++sweep) {
     for (int c = w; c < q; c += kWarps) {
-      const T* gc = g + (int64_t)c * ldg;
-      T s2 = 0;
+      const double* gc = g + (int64_t)c * p;
+      double s2 = 0;
       for (int i = l; i < p; i += 32) s2 = fma(gc[i], gc[i], s2);
       s2 = warp_sum(s2);
       if (l == 0) nrm2[c] = s2;
@@ -417,59 +379,31 @@ __device__ int jacobi_svd(T* g, int p, int q, int64_t ldg, T* v, int64_t ldv,
     for (int round = 0; round < qq - 1; ++round) {
       for (int k = w; k < qq / 2; k += kWarps) {
         int a, b;
-        if (k == 0) {
-          a = round;
-          b = qq - 1;
-        } else {
-          a = round + k;
-          if (a >= qq - 1) a -= qq - 1;
-          b = round - k;
-          if (b < 0) b += qq - 1;
-        }
+        round_pair(round, k, qq, &a, &b);
         if (a >= q || b >= q) continue;
         const int step = sweep * (qq - 1) + round;
-        // neither column rotated since this pair's check one sweep ago (step - (qq - 1))
         if (sweep > 0 && last_rot[a] < step - (qq - 1) && last_rot[b] < step - (qq - 1))
           continue;
-        const T al = nrm2[a], be = nrm2[b];
+        const double al = nrm2[a], be = nrm2[b], ab = al * be;
         // both columns at the noise floor: |g_a . g_b| <= |g_a| |g_b| <= floor2, nothing to do
-        if (pair_below_floor(al, be, floor2)) continue;
-        T* ga = g + (int64_t)a * ldg;
-        T* gb = g + (int64_t)b * ldg;
-        // The working copies live in global scratch (L2 for the largest blocks): the two
-        // columns stay in registers between the inner product and the rotation, and in FP32
-        // the two columns of v are fetched before the rotation is formed, so that their latency
-        // overlaps it (in FP64 the registers that takes would spill)
-        constexpr int kPer = CLR_MAX_CLUSTER / 32;
-        constexpr bool kPrefetchV = sizeof(T) == 4;
-        T xa[kPer], xb[kPer];
-        T ga_gb = 0;
+        if (ab == 0.0 || ab <= floor2 * floor2) continue;
+        double* ga = g + (int64_t)a * p;
+        double* gb = g + (int64_t)b * p;
+        // the two columns stay in registers between the inner product and the rotation
+        double xa[kRowsPerLane], xb[kRowsPerLane], d = 0;
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
+        for (int j = 0; j < kRowsPerLane; ++j) {
           const int i = l + 32 * j;
-          xa[j] = i < p ? ga[i] : T(0);
-          xb[j] = i < p ? gb[i] : T(0);
-          ga_gb = fma(xa[j], xb[j], ga_gb);
+          xa[j] = i < p ? ga[i] : 0.0;
+          xb[j] = i < p ? gb[i] : 0.0;
+          d = fma(xa[j], xb[j], d);
         }
-        ga_gb = warp_sum(ga_gb);
-        if (pair_converged(al, be, ga_gb, tol, floor2)) continue;
-        T* va = v ? v + (int64_t)a * ldv : nullptr;
-        T* vb = v ? v + (int64_t)b * ldv : nullptr;
-        T ya[kPrefetchV ? kPer : 1], yb[kPrefetchV ? kPer : 1];
-        if constexpr (kPrefetchV) {
-          if (v) {
+        d = warp_sum(d);
+        if (d * d <= tol * tol * ab || d * d <= floor2 * floor2) continue;
+        double c, sn, t;
+        rotation(al, be, d, c, sn, t);
 #pragma unroll
-            for (int j = 0; j < kPer; ++j) {
-              const int i = l + 32 * j;
-              ya[j] = i < q ? va[i] : T(0);
-              yb[j] = i < q ? vb[i] : T(0);
-            }
-          }
-        }
-        T c, sn, t;
-        rotation(al, be, ga_gb, c, sn, t);
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
+        for (int j = 0; j < kRowsPerLane; ++j) {
           const int i = l + 32 * j;
           if (i < p) {
             ga[i] = c * xa[j] - sn * xb[j];
@@ -478,10 +412,10 @@ __device__ int jacobi_svd(T* g, int p, int q, int64_t ldg, T* v, int64_t ldv,
         }
         // new squared norms: a - t g and b + t g exactly; recomputed from the rotated columns
         // when the update cancels (a column losing more than 63/64 of its square)
-        T na = al - t * ga_gb, nb = be + t * ga_gb;
-        if (!(na > al * T(0.015625)) || !(nb > be * T(0.015625))) {
+        double na = al - t * d, nb = be + t * d;
+        if (!(na > al * 0.015625) || !(nb > be * 0.015625)) {
           __syncwarp();
-          T sa = 0, sb = 0;
+          double sa = 0, sb = 0;
           for (int i = l; i < p; i += 32) {
             sa = fma(ga[i], ga[i], sa);
             sb = fma(gb[i], gb[i], sb);
@@ -489,23 +423,12 @@ __device__ int jacobi_svd(T* g, int p, int q, int64_t ldg, T* v, int64_t ldv,
           na = warp_sum(sa);
           nb = warp_sum(sb);
         }
-        if (v) {
-          if constexpr (kPrefetchV) {
-#pragma unroll
-            for (int j = 0; j < kPer; ++j) {
-              const int i = l + 32 * j;
-              if (i < q) {
-                va[i] = c * ya[j] - sn * yb[j];
-                vb[i] = sn * ya[j] + c * yb[j];
-              }
-            }
-          } else {
-            for (int i = l; i < q; i += 32) {
-              const T x = va[i], y = vb[i];
-              va[i] = c * x - sn * y;
-              vb[i] = sn * x + c * y;
-            }
-          }
+        double* va = v + (int64_t)a * q;
+        double* vb = v + (int64_t)b * q;
+        for (int i = l; i < q; i += 32) {
+          const double x = va[i], y = vb[i];
+          va[i] = c * x - sn * y;
+          vb[i] = sn * x + c * y;
         }
         if (l == 0) {
           nrm2[a] = na;
@@ -524,38 +447,76 @@ __device__ int jacobi_svd(T* g, int p, int q, int64_t ldg, T* v, int64_t ldv,
   return sweep;
 }
 
-// One-sided Jacobi in FP32 with the working copies in shared memory (or, where they do not fit,
-// in the per-CTA scratch): the same sweeps, tests and skips as jacobi_svd, for the FP32 stages of
-// svd_mixed.  What bounds it is the latency of a round (a column pair's inner product, its
-// rotation, and a barrier), so a round is kept short:
-//  - LP lanes per pair and kPer rows a lane, so that a round's pairs fill the CTA once where
-//    they can: a warp alone issues an instruction every ~5 cycles, so a round costs what one of
-//    its warps has to issue (about 80 instructions and 12 a row);
-//  - the columns in shared memory;
-//  - only the warps that have pairs take part, with their own barrier (none for a single warp).
-// Measured (core of 16 columns, both FP32 stages): 259k SM cycles with the copies in the global
-// scratch, a warp per pair and 8 masked rows a lane; 190k now.
-// ldg, ldv: odd multiples of LP where LP < 32, so that the pairs of a warp meet different banks.
-// v is reset to I.
+// FP32 building blocks: the approximate units (a few ulp) serve throughout, as the FP32 stages
+// only find rotations that FP64 products apply; two rows at a time by the packed FP32 pipe.
+__device__ __forceinline__ float fast_rsqrt(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float fast_rcp(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float fast_sqrt(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float sum2(f32x2 a) {
+  float x, y;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a));
+  return x + y;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 struct JacobiShared {
-  float nrm2[CLR_MAX_CLUSTER];     // column norms squared
+  float nrm[CLR_MAX_CLUSTER];      // column norms
   int last_rot[CLR_MAX_CLUSTER];   // the step of the column's last rotation, -1 if none
   int rotated, sweeps;
 };
 
-template <int LP, int kPer>
+// One-sided Jacobi in FP32 with the working copies in shared memory (or, where they do not fit,
+// in the per-CTA scratch), for the FP32 stages of svd_mixed.  What bounds it is the latency of a
+// round (a column pair's inner product, its rotation, and a barrier), so a round is kept short:
+//  - LP lanes per pair and 2 kVec rows a lane (as packed pairs), so that a round's pairs fill the
+//    CTA once where they can: a warp alone issues an instruction every ~5 cycles, so a round
+//    costs what one of its warps has to issue;
+//  - norms, not their squares, are kept, so that the tests need no square root;
+//  - only the warps that have pairs take part, with their own barrier (none for a single warp).
+// g: p x q, ld ldg (even, the row p of an odd p zero); v: q x q, ld ldv (even), reset to I.
+// tol, floor2: a pair is converged when its inner product is at most tol times the norms, or
+// floor2.  Measured (core of 16 columns, both FP32 stages): 259k SM cycles with the copies in the
+// global scratch, a warp per pair and 8 masked rows a lane.
+template <int LP, int kVec>
 __device__ __noinline__ int jacobi32(float* g, int p, int q, int ldg, float* v, int ldv,
                                      int max_sweeps, float tol, float floor2,
                                      JacobiShared& sh) {
-  float* nrm2 = sh.nrm2;
+  float* nrm = sh.nrm;
   int* last_rot = sh.last_rot;
   constexpr unsigned kAll = 0xffffffffu;
   const int w = threadIdx.x / 32, li = threadIdx.x % LP, grp = threadIdx.x / LP;
   const int qq = q + (q & 1), half = qq / 2;   // slot q is a dummy when q is odd
   const int n_act = min(kWarps, (half * LP + 31) / 32);   // warps with pairs
   const int ngrp = n_act * (32 / LP);
-  for (int e = threadIdx.x; e < q * q; e += kThreads)
-    v[(e % q) + (e / q) * ldv] = (e % q == e / q) ? 1.f : 0.f;
+  const int p2 = ldg / 2, q2 = ldv / 2;        // packed rows
+  for (int e = threadIdx.x; e < ldv * q; e += kThreads) v[e] = e % ldv == e / ldv ? 1.f : 0.f;
   for (int c = threadIdx.x; c < q; c += kThreads) last_rot[c] = -1;
   __syncthreads();
   if (w < n_act) {
@@ -571,17 +532,17 @@ __device__ __noinline__ int jacobi32(float* g, int p, int q, int ldg, float* v, 
     for (; sweep < max_sweeps; ++sweep) {
       for (int c0 = 0; c0 < q; c0 += ngrp) {
         const int c = c0 + grp;
-        float s2 = 0.f;
+        f32x2 s2 = 0;
         if (c < q) {
-          const float* gc = g + c * ldg;
+          const f32x2* gc = reinterpret_cast<const f32x2*>(g + c * ldg);
 #pragma unroll
-          for (int j = 0; j < kPer; ++j) {
-            const float x = li + LP * j < p ? gc[li + LP * j] : 0.f;
-            s2 = fmaf(x, x, s2);
+          for (int j = 0; j < kVec; ++j) {
+            const f32x2 x = li + LP * j < p2 ? gc[li + LP * j] : 0;
+            s2 = fma2(x, x, s2);
           }
         }
-        s2 = sum_lp(s2);
-        if (li == 0 && c < q) nrm2[c] = s2;
+        const float s = sum_lp(sum2(s2));
+        if (li == 0 && c < q) nrm[c] = fast_sqrt(s);
       }
       if (threadIdx.x == 0) sh.rotated = 0;
       act_sync();
@@ -589,88 +550,94 @@ __device__ __noinline__ int jacobi32(float* g, int p, int q, int ldg, float* v, 
         const int step = sweep * (qq - 1) + round;
         for (int k0 = 0; k0 < half; k0 += ngrp) {
           const int k = k0 + grp;
-          int a = round, b = qq - 1;
-          if (k > 0) {
-            a = round + k;
-            if (a >= qq - 1) a -= qq - 1;
-            b = round - k;
-            if (b < 0) b += qq - 1;
-          }
+          int a, b;
+          round_pair(round, k, qq, &a, &b);
           bool on = k < half && a < q && b < q;
-          float al = 0.f, be = 0.f;
+          float na = 0.f, nb = 0.f;
           if (on) {
             // neither column rotated since this pair's check one sweep ago
             on = !(sweep > 0 && last_rot[a] < step - (qq - 1) && last_rot[b] < step - (qq - 1));
-            al = nrm2[a];
-            be = nrm2[b];
-            on = on && !pair_below_floor(al, be, floor2);
+            na = nrm[a];
+            nb = nrm[b];
           }
+          const float ab = na * nb;
+          on = on && ab > floor2;
           if (!__any_sync(kAll, on)) continue;
-          float* ga = g + a * ldg;
-          float* gb = g + b * ldg;
-          float xa[kPer], xb[kPer], d = 0.f;
+          f32x2* ga = reinterpret_cast<f32x2*>(g + a * ldg);
+          f32x2* gb = reinterpret_cast<f32x2*>(g + b * ldg);
+          f32x2 xa[kVec], xb[kVec], d2 = 0;
 #pragma unroll
-          for (int j = 0; j < kPer; ++j) {
+          for (int j = 0; j < kVec; ++j) {
             const int i = li + LP * j;
-            const bool in = on && i < p;
-            xa[j] = in ? ga[i] : 0.f;
-            xb[j] = in ? gb[i] : 0.f;
-            d = fmaf(xa[j], xb[j], d);
+            const bool in = on && i < p2;
+            xa[j] = in ? ga[i] : 0;
+            xb[j] = in ? gb[i] : 0;
+            d2 = fma2(xa[j], xb[j], d2);
           }
-          d = sum_lp(d);
-          on = on && !pair_converged(al, be, d, tol, floor2);
+          const float d = sum_lp(sum2(d2)), ad = fabsf(d);
+          // (inner products at the end of the FP32 range are left alone)
+          on = on && ad > tol * ab && ad > floor2 && ad > 1e-37f;
           if (!__any_sync(kAll, on)) continue;
-          float* va = v + a * ldv;
-          float* vb = v + b * ldv;
-          float na = al, nb = be;
+          float a2 = na * na, b2 = nb * nb;
           bool again = false;
           if (on) {
-            float ya[kPer], yb[kPer];
+            f32x2* va = reinterpret_cast<f32x2*>(v + a * ldv);
+            f32x2* vb = reinterpret_cast<f32x2*>(v + b * ldv);
+            f32x2 ya[kVec], yb[kVec];
 #pragma unroll
-            for (int j = 0; j < kPer; ++j) {
+            for (int j = 0; j < kVec; ++j) {
               const int i = li + LP * j;
-              ya[j] = i < q ? va[i] : 0.f;
-              yb[j] = i < q ? vb[i] : 0.f;
+              ya[j] = i < q2 ? va[i] : 0;
+              yb[j] = i < q2 ? vb[i] : 0;
             }
-            float c, sn, t;
-            rotation(al, be, d, c, sn, t);
+            const float z = (b2 - a2) * (0.5f * fast_rcp(d)), az = fabsf(z);
+            // (for |zeta| > 2^40, where its square may overflow, the asymptote 1 / (2 zeta))
+            const float t =
+                copysignf(fast_rcp(az + (az > 0x1p40f ? az : fast_sqrt(fmaf(az, az, 1.f)))), z);
+            // one Newton step on the approximate root: c^2 + s^2 drifts less from 1 over many
+            // rotations
+            const float u = fmaf(t, t, 1.f);
+            float c = fast_rsqrt(u);
+            c = c * fmaf(-0.5f * u, c * c, 1.5f);
+            const float sn = c * t;
+            const f32x2 cc = pack2(c, c), ss = pack2(sn, sn), ns = pack2(-sn, -sn);
 #pragma unroll
-            for (int j = 0; j < kPer; ++j) {
+            for (int j = 0; j < kVec; ++j) {
               const int i = li + LP * j;
-              const float x = c * xa[j] - sn * xb[j];
-              xb[j] = sn * xa[j] + c * xb[j];
+              const f32x2 x = fma2(ns, xb[j], mul2(cc, xa[j]));
+              xb[j] = fma2(cc, xb[j], mul2(ss, xa[j]));
               xa[j] = x;
-              if (i < p) {
+              if (i < p2) {
                 ga[i] = xa[j];
                 gb[i] = xb[j];
               }
-              if (i < q) {
-                va[i] = c * ya[j] - sn * yb[j];
-                vb[i] = sn * ya[j] + c * yb[j];
+              if (i < q2) {
+                va[i] = fma2(ns, yb[j], mul2(cc, ya[j]));
+                vb[i] = fma2(cc, yb[j], mul2(ss, ya[j]));
               }
             }
             // a - t g and b + t g, recomputed from the rotated columns when that cancels
-            na = al - t * d;
-            nb = be + t * d;
-            again = !(na > al * 0.015625f) || !(nb > be * 0.015625f);
+            const float ra = fmaf(-t, d, a2), rb = fmaf(t, d, b2);
+            again = !(ra > a2 * 0.015625f) || !(rb > b2 * 0.015625f);
+            a2 = ra;
+            b2 = rb;
           }
           if (__any_sync(kAll, again)) {
-            float sa = 0.f, sb = 0.f;
+            f32x2 sa = 0, sb = 0;
 #pragma unroll
-            for (int j = 0; j < kPer; ++j) {
-              sa = fmaf(xa[j], xa[j], sa);
-              sb = fmaf(xb[j], xb[j], sb);
+            for (int j = 0; j < kVec; ++j) {
+              sa = fma2(xa[j], xa[j], sa);
+              sb = fma2(xb[j], xb[j], sb);
             }
-            sa = sum_lp(sa);
-            sb = sum_lp(sb);
+            const float fa = sum_lp(sum2(sa)), fb = sum_lp(sum2(sb));
             if (again) {
-              na = sa;
-              nb = sb;
+              a2 = fa;
+              b2 = fb;
             }
           }
           if (on && li == 0) {
-            nrm2[a] = na;
-            nrm2[b] = nb;
+            nrm[a] = fast_sqrt(a2);
+            nrm[b] = fast_sqrt(b2);
             last_rot[a] = step;
             last_rot[b] = step;
             sh.rotated = 1;
@@ -688,56 +655,53 @@ __device__ __noinline__ int jacobi32(float* g, int p, int q, int ldg, float* v, 
   return sh.sweeps;
 }
 
-// The FP32 working copies of svd_mixed (G: p x q, V: q x q): lanes per pair and rows per lane,
-// leading dimensions and place.
+// The FP32 working copies of svd_mixed (G: p x q, V: q x q): lanes per pair and packed rows per
+// lane, leading dimensions and place.
 struct Work32 {
   float *g, *v;
-  int ldg, ldv, lp, per;
+  int ldg, ldv, lp, vec;
 };
 // Dynamic shared memory of the recompression kernels: with their static part (27 KB) all that a
 // CTA can have, enough for a 256 x 136 pair of copies or a 158 x 158 one.
 constexpr int kSvdSmemBytes = 196 * 1024;
 
 __device__ __forceinline__ Work32 work32(int p, int q, double* sc) {
-  extern __shared__ float svd_smem[];
+  extern __shared__ __align__(16) float svd_smem[];
   Work32 k;
-  // 16 lanes a pair put up to 32 pairs into one pass over the CTA's 16 warps, 32 lanes up to 16
-  const bool wide = q <= 32 || p > 128;
-  k.lp = p <= 16 || !wide ? 16 : 32;
-  k.per = p <= k.lp ? 1 : p <= 2 * k.lp ? 2 : p <= 4 * k.lp ? 4 : 8;
-  auto ld = [&](int n) { return k.lp == 32 ? n : (((n + k.lp - 1) / k.lp) | 1) * k.lp; };
-  k.ldg = ld(p);
-  k.ldv = ld(q);
+  // 16 lanes a pair put up to 32 pairs into one pass over the CTA's 16 warps, 32 lanes up to 16;
+  // one packed row a lane while the rows are few
+  k.ldg = (p + 1) & ~1;
+  k.ldv = (q + 1) & ~1;
+  k.lp = p <= 32 || (q > 32 && p <= 128) ? 16 : 32;
+  k.vec = (k.ldg / 2 + k.lp - 1) / k.lp;
   const bool fits = (int64_t)(k.ldg + k.ldv) * q * (int)sizeof(float) <= kSvdSmemBytes;
-  // (outside shared memory p > 128: the leading dimensions are p and q, p q + q^2 floats)
   k.g = fits ? svd_smem : reinterpret_cast<float*>(sc);
   k.v = k.g + k.ldg * q;
   return k;
 }
 
 __device__ __forceinline__ int run_jacobi32(const Work32& k, int p, int q, int max_sweeps,
-                                            float tol, float floor2,
-                                            JacobiShared& sh) {
+                                            float tol, float floor2, JacobiShared& sh) {
   if (k.lp == 16) {
-    switch (k.per) {
+    switch (k.vec) {
       case 1: return jacobi32<16, 1>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
-      case 2:
-      case 4: return jacobi32<16, 4>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
-      default: return jacobi32<16, 8>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
+      case 2: return jacobi32<16, 2>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
+      case 3: return jacobi32<16, 3>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
+      default: return jacobi32<16, 4>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
     }
   }
-  switch (k.per) {
-    case 1: return jacobi32<32, 1>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
+  switch (k.vec) {
+    case 1:
     case 2: return jacobi32<32, 2>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
-    case 4: return jacobi32<32, 4>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
-    default: return jacobi32<32, 8>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
+    case 3: return jacobi32<32, 3>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
+    default: return jacobi32<32, 4>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
   }
 }
 
 // Where small_series keeps its 2 q^2 floats: the place of the FP32 copies, which the
 // orthonormalisation has read by then.
 __device__ __forceinline__ float* series_f32(int q, double* sc) {
-  extern __shared__ float svd_smem[];
+  extern __shared__ __align__(16) float svd_smem[];
   return (int64_t)2 * q * q * (int)sizeof(float) <= kSvdSmemBytes ? svd_smem
                                                                  : reinterpret_cast<float*>(sc);
 }
@@ -776,10 +740,10 @@ constexpr double kDowndateFloor = 1e-6;
 __device__ void sort_and_truncate(const double* g, int p, int q, int64_t ldg, double eps,
                                   SvdShared& sh) {
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int c0 = kGroup * w; c0 < q; c0 += kGroup * kWarps) {
-    double s[kGroup];
+  for (int c0 = kQuad * w; c0 < q; c0 += kQuad * kWarps) {
+    double s[kQuad];
 #pragma unroll
-    for (int c = 0; c < kGroup; ++c) {
+    for (int c = 0; c < kQuad; ++c) {
       s[c] = 0.0;
       if (c0 + c < q) {
         const double* gc = g + (int64_t)(c0 + c) * ldg;
@@ -1146,8 +1110,10 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
   double* e = sc + 4 * kSq;    // the orthonormalisations' E, and their FP32 powers
   float* f = series_f32(q, sc);
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int e = threadIdx.x; e < p * q; e += kThreads)
-    wk.g[e % p + (e / p) * wk.ldg] = (float)a.at(e % p, e / p);
+  for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
+    const int i = e % wk.ldg;
+    wk.g[e] = i < p ? (float)a.at(i, e / wk.ldg) : 0.f;
+  }
   __syncthreads();
   // The FP64 noise floor, raised to 1e-3 eps: columns below it hold less than 1e-6 eps^2 each, so
   // their mutual (non-)orthogonality cannot move a truncation decision at eps except within a
@@ -1193,8 +1159,10 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
   orthonormalise_fp64(wk.v, wk.ldv, v, q, e, f, sh);
   project_fp64(a, p, q, v, g, lower);
   mark(2);
-  for (int e = threadIdx.x; e < p * q; e += kThreads)
-    wk.g[e % p + (e / p) * wk.ldg] = (float)g[e];
+  for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
+    const int i = e % wk.ldg;
+    wk.g[e] = i < p ? (float)g[i + (int64_t)(e / wk.ldg) * p] : 0.f;
+  }
   __syncthreads();
   const int sw32b = run_jacobi32(wk, p, q, max_sweeps, lower ? 16.f * tol32 : tol32,
                                  floor_g * floor_g, sh.jac);
@@ -1261,10 +1229,11 @@ __global__ void __launch_bounds__(kThreads, 1) compress_qr_kernel(MatView C, con
     double* M = Wc + (int64_t)n * R;
     double* V = M + (int64_t)R * R;
     double* G = V + (int64_t)R * R;
-    // the two QRs at once, eight warps each
+    // the two QRs at once, eight warps each (W's first warp on another sub-partition than X's:
+    // those two form the reflectors)
     const int half = threadIdx.x / (kThreads / 2), hw = (threadIdx.x / 32) % (kWarps / 2);
-    householder_qr(half ? Wc : Xc, half ? n : m, R, half ? sh.refl_w : sh.refl, hw, kWarps / 2,
-                   1 + half);
+    householder_qr(half ? Wc : Xc, half ? n : m, R, half ? sh.refl_w : sh.refl,
+                   half ? (hw + 6) % (kWarps / 2) : hw, kWarps / 2, 1 + half);
     __syncthreads();
     // M = R_X R_W^T (both upper triangular R x R)
     for (int e = threadIdx.x; e < R * R; e += kThreads) {
@@ -1420,7 +1389,7 @@ __device__ int rrqr_block(const double* S, int64_t s_r, int64_t s_c, int m, int 
     __syncthreads();
     // Householder reflector of column j and its application (as householder_qr)
     double* cj = g + (int64_t)j * m;
-    const int nr = m - j - 1, nt = (nr + 31) / 32, ncol = n - j - 1;
+    const int nr = m - j - 1, ncol = n - j - 1;
     auto col = [&](int c) { return g + (int64_t)(j + 1 + c) * m + j + 1; };
     const double* x = cj + j + 1;
     if (w == 0) {
@@ -1437,13 +1406,12 @@ __device__ int rrqr_block(const double* S, int64_t s_r, int64_t s_c, int m, int 
     __syncthreads();
     const double v0 = sh.refl.v0[j], rn = sh.refl.rn[j], rv = sh.refl.rv[j];
     for (int c0 = kGroup * w; c0 < ncol; c0 += kGroup * kWarps) {
-      ColGroup cg;
-      const double d = cg.load_dot(x, nr, nt, c0, ncol, col);
-      const int c = c0 + l / 8;
+      const double d = group_dot(x, nr, c0, ncol, col);
+      const int c = group_column(c0);
       const double yj = c < ncol ? col(c)[-1] : 0.0;
       const double f = fma(v0, yj, d) * rn * rv;
-      cg.update_store(x, f, nr, nt, c0, ncol, col);
-      if (c < ncol && l % 8 == 0) col(c)[-1] = fma(-f, v0, yj);
+      group_update(x, f, nr, c0, ncol, col);
+      if (c < ncol && l % 4 == 0) col(c)[-1] = fma(-f, v0, yj);
     }
     __syncthreads();
   }
@@ -1647,10 +1615,10 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     if (sh.kept_sq <= tau2 && !exact) {
       // the downdated norms meet the threshold: sum the trailing norms exactly and decide (and
       // pivot) on those
-      for (int c0 = j + kGroup * w; c0 < q; c0 += kGroup * kWarps) {
-        double s2[kGroup];
+      for (int c0 = j + kQuad * w; c0 < q; c0 += kQuad * kWarps) {
+        double s2[kQuad];
 #pragma unroll
-        for (int c = 0; c < kGroup; ++c) {
+        for (int c = 0; c < kQuad; ++c) {
           s2[c] = 0.0;
           if (c0 + c < q) {
             const double* y = g + (int64_t)sh.qr_perm[c0 + c] * p;
@@ -1689,10 +1657,9 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     // row-j entry squared (downdate), summed again exactly when it has fallen below
     // kDowndateFloor of its last exact value (or is not positive).
     double* cj = g + (int64_t)sh.qr_perm[j] * p;
-    const int n = p - j - 1, nt = (n + 31) / 32, ncol = q - j - 1;
+    const int n = p - j - 1, ncol = q - j - 1;
     auto col = [&](int c) { return g + (int64_t)sh.qr_perm[j + 1 + c] * p + j + 1; };
     const double* x = cj + j + 1;
-    ColGroup cg;
     double d = 0.0;
     if (w == 0) {
       double v0, rn, rv;
@@ -1705,17 +1672,17 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
         sh.refl.rv[j] = rv;
       }
     } else if (kGroup * (w - 1) < ncol) {
-      d = cg.load_dot(x, n, nt, kGroup * (w - 1), ncol, col);
+      d = group_dot(x, n, kGroup * (w - 1), ncol, col);
     }
     __syncthreads();
     const double v0 = sh.refl.v0[j], rn = sh.refl.rn[j], rv = sh.refl.rv[j];
     for (int gi = w > 0 ? w - 1 : kWarps - 1; kGroup * gi < ncol;
          gi = (gi < kWarps - 1 ? kWarps - 1 + w : gi + kWarps)) {
-      const int c0 = kGroup * gi, c = c0 + l / 8;
-      if (gi >= kWarps - 1) d = cg.load_dot(x, n, nt, c0, ncol, col);
+      const int c0 = kGroup * gi, c = group_column(c0);
+      if (gi >= kWarps - 1) d = group_dot(x, n, c0, ncol, col);
       const double yj = c < ncol ? col(c)[-1] : 0.0;
       const double f = fma(v0, yj, d) * rn * rv;
-      cg.update_store(x, f, n, nt, c0, ncol, col);
+      group_update(x, f, n, c0, ncol, col);
       const double yn = fma(-f, v0, yj);
       double nu2 = 0.0;
       bool again = false;
@@ -1724,17 +1691,17 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
         again = !(nu2 > kDowndateFloor * sh.qr_nref[j + 1 + c]);
       }
       if (__any_sync(0xffffffffu, again)) {
-        const double s2 = cg.sum_squares(nt, c0, ncol);
+        const double s2 = group_squares(n, c0, ncol, col);
         if (again) {
           nu2 = s2;
-          if (l % 8 == 0) {
+          if (l % 4 == 0) {
             sh.qr_nref[j + 1 + c] = nu2;
             atomicAdd(&sh.qr_recomputed, (unsigned long long)n);
           }
         }
       }
       __syncwarp();
-      if (c < ncol && l % 8 == 0) {
+      if (c < ncol && l % 4 == 0) {
         col(c)[-1] = yn;
         sh.sigma[j + 1 + c] = nu2;
       }
@@ -2164,8 +2131,7 @@ __global__ void __launch_bounds__(kThreads) compress_block_noalloc_kernel(
   // rotating them changes nothing that a truncation can see, and they would keep the sweeps
   // from ever converging
   const double floor64 = (double)p * DBL_EPSILON * sqrt(nsq);
-  const int sweeps = jacobi_svd(G, p, q, p, V, q, max_sweeps, &sh.flag, true, 1.0,
-                                floor64 * floor64);
+  const int sweeps = jacobi_svd(G, p, q, V, max_sweeps, &sh.flag, floor64 * floor64);
   // every sweep still rotated a pair: the column norms the truncation uses may be inexact
   if (sweeps >= max_sweeps && threadIdx.x == 0) status[2] = 4;
   sort_and_truncate(G, p, q, p, eps, sh);
