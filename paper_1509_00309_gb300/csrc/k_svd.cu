@@ -17,6 +17,8 @@
 // FP64 working arrays live in the tile's workspace slot (2 m n doubles per tile, enough for
 // either route); the FP32 copies of the mixed-precision SVD in shared memory, or in a per-CTA
 // scratch where they do not fit.
+#include <cooperative_groups.h>
+
 #include <cfloat>
 #include <mutex>
 
@@ -201,6 +203,7 @@ __device__ __forceinline__ double make_reflector(const double* x, int n, double 
 // below the diagonal of column j).
 struct Reflectors {
   double v0[CLR_MAX_CLUSTER], rn[CLR_MAX_CLUSTER], rv[CLR_MAX_CLUSTER];
+  double x0, beta;   // of the current step (householder_qr_regs)
 };
 
 // In-place Householder QR of the p x q column-major matrix a (ld p), p >= q, by the nw warps of
@@ -243,56 +246,148 @@ __device__ __noinline__ void householder_qr(double* a, int p, int q, Reflectors&
   }
 }
 
+// The same QR where a lane can keep its share of a column: each of the group's nw warps holds four
+// columns (q <= 4 nw) in registers from the first step to the last, eight lanes a column, rows
+// l % 8, l % 8 + 8, ... of them (kRows >= ceil(p / 8)); only the step's reflector goes through
+// shared memory (xs: 512 doubles of the group, two buffers in turn).  A step of a small factor is
+// bound by latency, its loads above all: with the columns in global memory a step took 16k SM
+// cycles at 16 columns.  The last warp forms the scalars.
+template <int kRows>
+__device__ __noinline__ void householder_qr_regs(double* a, int p, int q, Reflectors& h,
+                                                 double* xs, int w, int nw, int bar) {
+  const int l = threadIdx.x % 32, r8 = l % 8;
+  const int c = kQuad * w + l / 8;   // this lane's column
+  double y[kRows];
+#pragma unroll
+  for (int t = 0; t < kRows; ++t)
+    y[t] = c < q && r8 + 8 * t < p ? a[r8 + 8 * t + (int64_t)c * p] : 0.0;
+  const int nt = (p + 7) / 8;
+  for (int j = 0; j < q; ++j) {
+    double* x = xs + (j & 1) * CLR_MAX_CLUSTER;
+    const int t0 = j / 8;
+    const bool mine = kQuad * w < q && kQuad * w + kQuad - 1 >= j;   // a column from j on (warp)
+    double yj = 0.0;   // row j of this lane's column
+    if (mine) {
+#pragma unroll
+      for (int t = 0; t < kRows; ++t)
+        if (t == t0) yj = y[t];
+      yj = __shfl_sync(0xffffffffu, yj, (l & 24) + j % 8);
+      if (c == j) {
+#pragma unroll
+        for (int t = 0; t < kRows; ++t)
+          if (t <= nt) x[r8 + 8 * t] = r8 + 8 * t > j ? y[t] : 0.0;
+        if (r8 == 0) h.x0 = yj;
+      }
+    }
+    group_sync(bar, 32 * nw);
+    const double x0 = h.x0;
+    if (w == nw - 1) {
+      double v0, rn, rv;
+      const double beta = make_reflector(x + j + 1, p - j - 1, x0, &v0, &rn, &rv);
+      if (l == 0) {
+        h.beta = beta;
+        h.v0[j] = v0;
+        h.rn[j] = rn;
+        h.rv[j] = rv;
+      }
+    }
+    double d = 0.0;
+    if (mine) {
+#pragma unroll
+      for (int t = 0; t < kRows; t += 2)   // (two rows' loads together)
+        if (t + 1 >= t0 && t < nt) {
+          const double xa = x[r8 + 8 * t], xb = x[r8 + 8 * t + 8];
+          d = fma(xa, y[t], d);
+          d = fma(xb, y[t + 1], d);
+        }
+      d += __shfl_xor_sync(0xffffffffu, d, 4);
+      d += __shfl_xor_sync(0xffffffffu, d, 2);
+      d += __shfl_xor_sync(0xffffffffu, d, 1);
+    }
+    group_sync(bar, 32 * nw);
+    if (mine) {
+      const double v0 = h.v0[j];
+      const double f = c > j ? fma(v0, yj, d) * h.rn[j] * h.rv[j] : 0.0;
+#pragma unroll
+      for (int t = 0; t < kRows; t += 2)
+        if (t + 1 >= t0 && t < nt) {
+          const double xa = x[r8 + 8 * t], xb = x[r8 + 8 * t + 8];
+          y[t] = fma(-f, xa, y[t]);
+          y[t + 1] = fma(-f, xb, y[t + 1]);
+        }
+      const double yn = c == j ? h.beta : fma(-f, v0, yj);
+      const bool row_j = r8 == j % 8 && c >= j;
+#pragma unroll
+      for (int t = 0; t < kRows; ++t)
+        if (t == t0 && row_j) y[t] = yn;
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < kRows; ++t)
+    if (c < q && r8 + 8 * t < p) a[r8 + 8 * t + (int64_t)c * p] = y[t];
+}
+
+// The QR of a factor by a warp group, in registers where it fits.
+__device__ __forceinline__ void factor_qr(double* a, int p, int q, Reflectors& h, double* xs,
+                                          int w, int nw, int bar) {
+  if (q > kQuad * nw) householder_qr(a, p, q, h, w, nw, bar);
+  else if (p <= 128) householder_qr_regs<16>(a, p, q, h, xs, w, nw, bar);
+  else if (p <= 192) householder_qr_regs<24>(a, p, q, h, xs, w, nw, bar);
+  else householder_qr_regs<32>(a, p, q, h, xs, w, nw, bar);
+}
+
 // y (p x r, ld ldy) <- Q y with Q = H_0 H_1 ... H_{k-1}; the rows of reflector j are in column
-// perm[j] (j when perm is null) of v (ld p).  Each warp carries its four columns of y through all
-// reflectors in registers: no step waits for another warp.
-__device__ __noinline__ void apply_q(const double* v, int p, int k, const Reflectors& h,
-                                     const int* perm, double* y, int r, int64_t ldy, int w,
-                                     int nw) {
-  const int l = threadIdx.x % 32;
-  const int nt = (p + 31) / 32;
+// perm[j] (j when perm is null) of v (ld p).  Each warp carries four columns of y at a time through
+// all reflectors in registers (eight lanes a column): no step waits for another warp.
+template <int kRows>
+__device__ __noinline__ void apply_q_regs(const double* v, int p, int k, const Reflectors& h,
+                                          const int* perm, double* y, int r, int64_t ldy, int w,
+                                          int nw) {
+  const int l = threadIdx.x % 32, r8 = l % 8;
+  const int nt = (p + 7) / 8;
   for (int g0 = kQuad * w; g0 < r; g0 += kQuad * nw) {
-    double yr[kQuad][kRowsPerLane];
+    const int c = g0 + l / 8;
+    double* yc = y + (int64_t)c * ldy;
+    double yr[kRows];
 #pragma unroll
-    for (int c = 0; c < kQuad; ++c)
-#pragma unroll
-      for (int t = 0; t < kRowsPerLane; ++t)
-        yr[c][t] = g0 + c < r && l + 32 * t < p ? y[l + 32 * t + (int64_t)(g0 + c) * ldy] : 0.0;
+    for (int t = 0; t < kRows; ++t) yr[t] = c < r && r8 + 8 * t < p ? yc[r8 + 8 * t] : 0.0;
     for (int j = k - 1; j >= 0; --j) {
       const double* vj = v + (int64_t)(perm ? perm[j] : j) * p;
-      const int t0 = j / 32;
       const double v0 = h.v0[j];
-      double s[kQuad];
+      // rows two at a time, so that their loads go out together
       auto xv = [&](int i) { return i > j && i < p ? vj[i] : (i == j ? v0 : 0.0); };
+      double s = 0.0;
 #pragma unroll
-      for (int c = 0; c < kQuad; ++c) s[c] = 0.0;
-#pragma unroll
-      for (int t = 0; t < kRowsPerLane; ++t)
-        if (t >= t0 && t < nt) {
-          const double x = xv(l + 32 * t);
-#pragma unroll
-          for (int c = 0; c < kQuad; ++c)
-            if (g0 + c < r) s[c] = fma(x, yr[c][t], s[c]);
+      for (int t = 0; t < kRows; t += 2)
+        if (8 * (t + 2) > j && t < nt) {
+          const double xa = xv(r8 + 8 * t), xb = xv(r8 + 8 * t + 8);
+          s = fma(xa, yr[t], s);
+          s = fma(xb, yr[t + 1], s);
         }
-      const double f = warp_sum4(s) * h.rn[j] * h.rv[j];
-      double fc[kQuad];
+      s += __shfl_xor_sync(0xffffffffu, s, 4);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      const double f = -s * h.rn[j] * h.rv[j];
 #pragma unroll
-      for (int c = 0; c < kQuad; ++c) fc[c] = __shfl_sync(0xffffffffu, f, 8 * c);
-#pragma unroll
-      for (int t = 0; t < kRowsPerLane; ++t)
-        if (t >= t0 && t < nt) {
-          const double x = xv(l + 32 * t);
-#pragma unroll
-          for (int c = 0; c < kQuad; ++c)
-            if (g0 + c < r) yr[c][t] = fma(-fc[c], x, yr[c][t]);
+      for (int t = 0; t < kRows; t += 2)
+        if (8 * (t + 2) > j && t < nt) {
+          const double xa = xv(r8 + 8 * t), xb = xv(r8 + 8 * t + 8);
+          yr[t] = fma(f, xa, yr[t]);
+          yr[t + 1] = fma(f, xb, yr[t + 1]);
         }
     }
 #pragma unroll
-    for (int c = 0; c < kQuad; ++c)
-#pragma unroll
-      for (int t = 0; t < kRowsPerLane; ++t)
-        if (g0 + c < r && l + 32 * t < p) y[l + 32 * t + (int64_t)(g0 + c) * ldy] = yr[c][t];
+    for (int t = 0; t < kRows; ++t)
+      if (c < r && r8 + 8 * t < p) yc[r8 + 8 * t] = yr[t];
   }
+}
+
+__device__ __forceinline__ void apply_q(const double* v, int p, int k, const Reflectors& h,
+                                        const int* perm, double* y, int r, int64_t ldy, int w,
+                                        int nw) {
+  if (p <= 128) apply_q_regs<16>(v, p, k, h, perm, y, r, ldy, w, nw);
+  else if (p <= 192) apply_q_regs<24>(v, p, k, h, perm, y, r, ldy, w, nw);
+  else apply_q_regs<32>(v, p, k, h, perm, y, r, ldy, w, nw);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1204,20 +1299,31 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
 
 // ---------------------------------------------------------------------------------------------
 // ROUTE_QR tiles: X_cat (m x R) and W_cat (n x R) in the workspace slot.
+//
+// Small factors (the 1D chain's have 16 columns) make this a chain of latencies on a few SMs, so
+// the CTAs come in clusters of two: while the tiles are at most half the CTAs a pair takes one
+// tile, one CTA the QR of X_cat and the final Q_X product, the other W_cat's; the core and its SVD
+// both compute (the same bits: nothing needs to be exchanged but the triangular factors, which
+// are read after one cluster barrier).  With more tiles each CTA takes its own, eight warps a
+// factor.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads, 1) compress_qr_kernel(MatView C, const int* list,
-                                                               const int* count,
-                                                               const int* rsum, double* ws,
-                                                               double* svd_scratch,
-                                                               double eps, int max_sweeps,
-                                                               int* sched,
-                                                               unsigned long long* jstats) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+    compress_qr_kernel(MatView C, const int* list, const int* count, const int* rsum, double* ws,
+                       double* svd_scratch, double eps, int max_sweeps, int* sched,
+                       unsigned long long* jstats) {
+  extern __shared__ __align__(16) float svd_smem[];
   __shared__ SvdShared sh;
   __shared__ int sh_next;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
   constexpr int64_t kSq = (int64_t)CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
   double* sc = svd_scratch + (int64_t)blockIdx.x * kSvdScratchPerCta;
   const int n_items = *count;
-  for (int it = next_item(sched, &sh_next); it < n_items; it = next_item(sched, &sh_next)) {
+  const bool pair = 2 * n_items <= (int)gridDim.x;
+  const int rank = (int)cluster.block_rank();
+  const bool lead = !pair || rank == 0;   // writes what a tile has once
+  int it = pair ? (int)(blockIdx.x / 2) : next_item(sched, &sh_next);
+  while (it < n_items) {
     const int t = list[it];
     const int I = t / C.nc, J = t % C.nc;
     const int m = C.row_off[I + 1] - C.row_off[I];
@@ -1226,15 +1332,21 @@ __global__ void __launch_bounds__(kThreads, 1) compress_qr_kernel(MatView C, con
     const int64_t sC = slot_of(C, I, J, m);
     double* Xc = ws + 2 * sC;
     double* Wc = Xc + (int64_t)m * R;
-    double* M = Wc + (int64_t)n * R;
+    // R <= 128: the core and its SVD's factors in the third part of the CTA's scratch
+    double* M = sc + 2 * kSq;
     double* V = M + (int64_t)R * R;
     double* G = V + (int64_t)R * R;
-    // the two QRs at once, eight warps each (W's first warp on another sub-partition than X's:
-    // those two form the reflectors)
-    const int half = threadIdx.x / (kThreads / 2), hw = (threadIdx.x / 32) % (kWarps / 2);
-    householder_qr(half ? Wc : Xc, half ? n : m, R, half ? sh.refl_w : sh.refl,
-                   half ? (hw + 6) % (kWarps / 2) : hw, kWarps / 2, 1 + half);
-    __syncthreads();
+    // this warp's factor (X_cat or W_cat), its group of warps and the group's barrier
+    const int wg = threadIdx.x / 32, half = pair ? rank : wg / (kWarps / 2);
+    const int nw = pair ? kWarps : kWarps / 2;
+    // (alone, W's first warps sit on other sub-partitions than X's)
+    const int hw = pair ? wg : half ? (wg + 6) % (kWarps / 2) : wg;
+    double* F = half ? Wc : Xc;
+    const int f_rows = half ? n : m;
+    Reflectors& refl = half ? sh.refl_w : sh.refl;
+    factor_qr(F, f_rows, R, refl, reinterpret_cast<double*>(svd_smem) + half * 2 * CLR_MAX_CLUSTER,
+              hw, nw, 1 + half);
+    if (pair) cluster.sync(); else __syncthreads();
     // M = R_X R_W^T (both upper triangular R x R)
     for (int e = threadIdx.x; e < R * R; e += kThreads) {
       const int a = e % R, b = e / R;
@@ -1244,12 +1356,13 @@ __global__ void __launch_bounds__(kThreads, 1) compress_qr_kernel(MatView C, con
       M[e] = s;
     }
     __syncthreads();
+    unsigned long long* js = lead ? jstats : nullptr;
     {
       double part = 0.0;
       for (int e = threadIdx.x; e < R * R; e += kThreads) part = fma(M[e], M[e], part);
       const double mfro = sqrt(block_sum(part, sh.red));
       SrcView mv{M, 1, R, false};
-      svd_mixed(mv, R, R, G, V, sc, max_sweeps, eps, -1, mfro, false, sh, jstats);
+      svd_mixed(mv, R, R, G, V, sc, max_sweeps, eps, -1, mfro, false, sh, js);
     }
     sort_and_truncate(G, R, R, R, eps, sh);
     const int r = sh.rank;
@@ -1260,41 +1373,51 @@ __global__ void __launch_bounds__(kThreads, 1) compress_qr_kernel(MatView C, con
       SrcView mv{M, 1, R, false};
       recover_right(mv, R, R, G, sh.perm, r, V, sc, false);
       if (ls)
-        ls = ls_solve(V, R, r, sc, R, sh.sorted, sc + 4 * kSq, sc + kSq, series_f32(r, sc + 2 * kSq),
+        ls = ls_solve(V, R, r, sc, R, sh.sorted, sc + 4 * kSq, sc + kSq, series_f32(r, sc + 3 * kSq),
                       sh);
     }
     double* Xo = C.pool + sC;
     double* Wo = Xo + (int64_t)m * r;
-    for (int e = threadIdx.x; e < m * r; e += kThreads) {
-      const int i = e % m, c = e / m;
-      Xo[e] = i < R ? G[i + (int64_t)sh.perm[c] * R] : 0.0;
-    }
-    for (int e = threadIdx.x; e < n * r; e += kThreads) {
-      const int j = e % n, c = e / n;
-      Wo[e] = j >= R ? 0.0
-              : tracked ? V[(int64_t)j * R + sh.perm[c]]
-              : ls      ? V[(int64_t)j * r + c]
-                        : V[(int64_t)j * r + c] / (sh.sorted[c] * sh.sorted[c]);
+    if (!pair || rank == 0)
+      for (int e = threadIdx.x; e < m * r; e += kThreads) {
+        const int i = e % m, c = e / m;
+        Xo[e] = i < R ? G[i + (int64_t)sh.perm[c] * R] : 0.0;
+      }
+    if (!pair || rank == 1)
+      for (int e = threadIdx.x; e < n * r; e += kThreads) {
+        const int j = e % n, c = e / n;
+        Wo[e] = j >= R ? 0.0
+                : tracked ? V[(int64_t)j * R + sh.perm[c]]
+                : ls      ? V[(int64_t)j * r + c]
+                          : V[(int64_t)j * r + c] / (sh.sorted[c] * sh.sorted[c]);
+      }
+    // the reflectors in shared memory where they fit (the FP32 copies there are dead): a lone
+    // warp's step would wait for each reflector from L2
+    const double* Fs = F;
+    const int64_t room = (pair ? 1 : 2) * (int64_t)f_rows * R * (int64_t)sizeof(double);
+    if (room <= kSvdSmemBytes) {
+      double* st = reinterpret_cast<double*>(svd_smem) +
+                   (pair || !half ? 0 : kSvdSmemBytes / (int64_t)sizeof(double) / 2);
+      for (int e = hw * 32 + threadIdx.x % 32; e < f_rows * R; e += nw * 32) st[e] = F[e];
+      Fs = st;
     }
     __syncthreads();
-    // (W's column groups start three warps on, so that few columns spread over the four
-    // sub-partitions' FP64 pipes)
-    apply_q(half ? Wc : Xc, half ? n : m, R, half ? sh.refl_w : sh.refl, nullptr,
-            half ? Wo : Xo, r, half ? n : m, half ? (hw + 5) % (kWarps / 2) : hw, kWarps / 2);
-    __syncthreads();
-    if (jstats && threadIdx.x == 0) {
+    apply_q(Fs, f_rows, R, refl, nullptr, half ? Wo : Xo, r, f_rows, hw, nw);
+    if (js && threadIdx.x == 0) {
       // Householder QRs 2(m+n)R^2, core R_X R_W^T (2/3)R^3, recovery 2R^2 r (when not
       // accumulated), re-expansion 4(m+n)R r
       const unsigned long long mn = (unsigned long long)(m + n), RR = (unsigned long long)R * R;
-      atomicAdd(&jstats[4], 2 * mn * RR + 2 * RR * R / 3 + (tracked ? 0 : 2 * RR * r) +
-                                4 * mn * R * r);
+      atomicAdd(&js[4], 2 * mn * RR + 2 * RR * R / 3 + (tracked ? 0 : 2 * RR * r) +
+                            4 * mn * R * r);
     }
-    if (threadIdx.x == 0) {
+    if (lead && threadIdx.x == 0) {
       C.kind[t] = r > 0 ? CLR_KIND_LR : CLR_KIND_ZERO;
       C.rank[t] = r;
       C.norm[t] = sqrt(sh.kept_sq);
     }
     __syncthreads();
+    if (pair) break;   // at most one tile a pair
+    it = next_item(sched, &sh_next);
   }
 }
 
@@ -1323,7 +1446,8 @@ void launch_compress_qr(const MatView& C, const int* list, const int* count, con
                         unsigned long long* jstats, cudaStream_t st) {
   (void)err;
   static bool attr_done[64] = {false};
-  const int g = svd_launch_grid(compress_qr_kernel, grid, attr_done);
+  int g = svd_launch_grid(compress_qr_kernel, grid, attr_done);
+  g = g < 2 ? 2 : g & ~1;   // pairs of CTAs
   compress_qr_kernel<<<g, kThreads, kSvdSmemBytes, st>>>(C, list, count, rsum, ws, svd_scratch, eps,
                                              max_sweeps, sched, jstats);
 }
@@ -1794,7 +1918,17 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     wa[sh.qr_perm[j] + (int64_t)c * q] = ls ? v : v / sh.sorted[c];
   }
   __syncthreads();
-  apply_q(g, p, k, sh.refl, sh.qr_perm, xa, r, p, w, kWarps);
+  // the reflectors in shared memory where they fit
+  if ((int64_t)p * k * (int64_t)sizeof(double) <= kSvdSmemBytes) {
+    extern __shared__ __align__(16) float svd_smem[];
+    double* st = reinterpret_cast<double*>(svd_smem);
+    for (int c = w; c < k; c += kWarps)
+      for (int i = c + 1 + l; i < p; i += 32) st[i + c * p] = g[i + (int64_t)sh.qr_perm[c] * p];
+    __syncthreads();
+    apply_q(st, p, k, sh.refl, nullptr, xa, r, p, w, kWarps);
+  } else {
+    apply_q(g, p, k, sh.refl, sh.qr_perm, xa, r, p, w, kWarps);
+  }
   if (threadIdx.x == 0) {
     *kind_out = CLR_KIND_LR;
     *rank_out = r;
