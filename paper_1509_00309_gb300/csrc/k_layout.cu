@@ -65,51 +65,89 @@ void launch_dense_kinds(const MatView& M, double drop_norm, int* err, cudaStream
   dense_kinds_kernel<<<(n + 127) / 128, 128, 0, st>>>(M, drop_norm, err);
 }
 
-// row-major out <- reconstruction of every block.
+// row-major out <- reconstruction of every block.  Dense blocks are bound by HBM (16 bytes an
+// element), low-rank ones by the FP64 pipe (rank FMAs an element).  A CTA takes a 64 x 64 tile and a
+// lane 16 of its elements, all of whose kinds and then values are loaded before the first is used:
+// with 32 x 32 tiles and a chain of index, kind and value loads per element the dense N = 16384
+// result took 1.73 ms, now 0.80 (4.3 GB: 0.63 at the copy rate).
+constexpr int kOutTile = 64;
 __global__ void __launch_bounds__(256) pool_to_rowmajor_kernel(MatView M, const int* row_idx,
                                                                const int* col_idx, double* out,
                                                                int64_t ldo) {
-  __shared__ double tile[32][33];
-  const int64_t tiles_r = (M.n_rows + 31) / 32;
-  const int64_t r0 = (int64_t)(blockIdx.x % tiles_r) * 32;
-  const int64_t c0 = (int64_t)(blockIdx.x / tiles_r) * 32;
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  const int64_t r = r0 + tx;
-  if (r < M.n_rows) {
-    const int R = row_idx[r];
-    const int mR = M.row_off[R + 1] - M.row_off[R];
-    const int64_t rloc = r - M.row_off[R];
-    for (int cc = ty; cc < 32; cc += 8) {
-      const int64_t c = c0 + cc;
-      double v = 0.0;
-      if (c < M.n_cols) {
-        const int Cc = col_idx[c];
-        const int b = R * M.nc + Cc;
-        const int kind = M.kind[b];
-        if (kind == CLR_KIND_DENSE) {
-          v = M.pool[panel_index(M, R, r, c, mR)];
-        } else if (kind == CLR_KIND_LR) {
-          const int n = M.col_off[Cc + 1] - M.col_off[Cc];
-          const int rk = M.rank[b];
-          const double* X = M.pool + slot_of(M, R, Cc, mR);
-          const double* W = X + (int64_t)mR * rk;
-          const int64_t cloc = c - M.col_off[Cc];
-          for (int q = 0; q < rk; ++q) v = fma(X[rloc + (int64_t)q * mR], W[cloc + (int64_t)q * n], v);
-        }
-      }
-      tile[tx][cc] = v;
-    }
+  __shared__ double tile[kOutTile][kOutTile + 1];
+  const int64_t tiles_r = (M.n_rows + kOutTile - 1) / kOutTile;
+  const int64_t r0 = (int64_t)(blockIdx.x % tiles_r) * kOutTile;
+  const int64_t c0 = (int64_t)(blockIdx.x / tiles_r) * kOutTile;
+  const int l = threadIdx.x % 32, w = threadIdx.x / 32;
+  int R[2], mR[2], rloc[2];
+  int64_t base[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int64_t r = r0 + l + 32 * h;
+    R[h] = r < M.n_rows ? row_idx[r] : -1;
+    const int off = R[h] >= 0 ? M.row_off[R[h]] : 0;
+    mR[h] = R[h] >= 0 ? M.row_off[R[h] + 1] - off : 0;
+    rloc[h] = (int)(r - off);
+    base[h] = (int64_t)off * M.n_cols + rloc[h];
   }
+  constexpr int kCols = kOutTile / 8;
+  int Cc[kCols], kind[kCols][2];
+  double v[kCols][2];
+#pragma unroll
+  for (int q = 0; q < kCols; ++q) {
+    const int64_t c = c0 + w + 8 * q;
+    Cc[q] = c < M.n_cols ? col_idx[c] : -1;
+  }
+#pragma unroll
+  for (int q = 0; q < kCols; ++q)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      kind[q][h] = R[h] >= 0 && Cc[q] >= 0 ? M.kind[(int64_t)R[h] * M.nc + Cc[q]] : CLR_KIND_ZERO;
+  bool lr = false;
+#pragma unroll
+  for (int q = 0; q < kCols; ++q)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      v[q][h] = kind[q][h] == CLR_KIND_DENSE ? M.pool[base[h] + (c0 + w + 8 * q) * mR[h]] : 0.0;
+      lr = lr || kind[q][h] == CLR_KIND_LR;
+    }
+  if (lr) {
+#pragma unroll
+    for (int q = 0; q < kCols; ++q)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (kind[q][h] == CLR_KIND_LR) {
+          const int coff = M.col_off[Cc[q]];
+          const int n = M.col_off[Cc[q] + 1] - coff;
+          const int rk = M.rank[(int64_t)R[h] * M.nc + Cc[q]];
+          const double* X = M.pool + base[h] - rloc[h] + (int64_t)mR[h] * coff;
+          const double* W = X + (int64_t)mR[h] * rk + (c0 + w + 8 * q - coff);
+          X += rloc[h];
+          double s = 0.0;
+          for (int k = 0; k < rk; ++k) s = fma(X[(int64_t)k * mR[h]], W[(int64_t)k * n], s);
+          v[q][h] = s;
+        }
+  }
+#pragma unroll
+  for (int q = 0; q < kCols; ++q)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) tile[l + 32 * h][w + 8 * q] = v[q][h];
   __syncthreads();
-  for (int rr = ty; rr < 32; rr += 8) {
-    const int64_t rw = r0 + rr, c = c0 + tx;
-    if (rw < M.n_rows && c < M.n_cols) out[rw * ldo + c] = tile[rr][tx];
+  for (int rr = w; rr < kOutTile; rr += 8) {
+    const int64_t r = r0 + rr;
+    if (r >= M.n_rows) break;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int64_t c = c0 + l + 32 * h;
+      if (c < M.n_cols) out[r * ldo + c] = tile[rr][l + 32 * h];
+    }
   }
 }
 
 void launch_pool_to_rowmajor(const MatView& M, const int* row_idx, const int* col_idx,
                              double* out, int64_t ldo, cudaStream_t st) {
-  const int64_t n = ((M.n_rows + 31) / 32) * ((M.n_cols + 31) / 32);
+  const int64_t n =
+      ((M.n_rows + kOutTile - 1) / kOutTile) * ((M.n_cols + kOutTile - 1) / kOutTile);
   pool_to_rowmajor_kernel<<<(unsigned)n, 256, 0, st>>>(M, row_idx, col_idx, out, ldo);
 }
 
