@@ -58,11 +58,21 @@ __global__ void lincomb_route_kernel(double a, MatView X, double b, MatView Y, d
   // the copy case is re-derived by the apply kernel from the operand kinds
 }
 
-__global__ void __launch_bounds__(kT) lincomb_apply_kernel(double a, MatView X, double b,
-                                                           MatView Y, double diag, MatView O,
-                                                           Plan p, double* ws) {
+// A cluster of CTAs per block, its elements in turn (a dense sum of low-rank blocks takes m n r
+// FMAs on the FP64 pipe, and with one CTA per block the largest block was the kernel's time: 4.9 ms
+// for the 3D lattice's iterates at N = 2048, now 1.2); the norm's parts are added in a fixed order.
+constexpr int kLcCtas = 8;
+
+__global__ void __cluster_dims__(kLcCtas, 1, 1) __launch_bounds__(kT)
+    lincomb_apply_kernel(double a, MatView X, double b, MatView Y, double diag, MatView O, Plan p,
+                         double* ws) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
   __shared__ double red[kT / 32];
-  const int t = blockIdx.x;
+  __shared__ double part_sq;
+  const int t = blockIdx.x / kLcCtas, rank = (int)cluster.block_rank();
+  const int tid = threadIdx.x + kT * rank;
+  constexpr int kAll = kT * kLcCtas;
   const int I = t / p.nJ, J = t % p.nJ;
   const int m = X.row_off[I + 1] - X.row_off[I];
   const int n = X.col_off[J + 1] - X.col_off[J];
@@ -77,7 +87,7 @@ __global__ void __launch_bounds__(kT) lincomb_apply_kernel(double a, MatView X, 
   const int route = p.t_route[t];
   const int rx = X.rank[t], ry = Y.rank[t];
   if (kx == CLR_KIND_ZERO && ky == CLR_KIND_ZERO && !shift) {
-    if (threadIdx.x == 0) { O.kind[t] = CLR_KIND_ZERO; O.rank[t] = 0; O.norm[t] = 0.0; }
+    if (tid == 0) { O.kind[t] = CLR_KIND_ZERO; O.rank[t] = 0; O.norm[t] = 0.0; }
     return;
   }
   if (!shift && (kx == CLR_KIND_ZERO || ky == CLR_KIND_ZERO)) {
@@ -87,27 +97,27 @@ __global__ void __launch_bounds__(kT) lincomb_apply_kernel(double a, MatView X, 
     const double* ss = fromx ? xs : ys;
     const int kind = S.kind[t], r = S.rank[t];
     if (kind == CLR_KIND_DENSE) {
-      for (int e = threadIdx.x; e < m * n; e += kT) os[e] = c * ss[e];
+      for (int e = tid; e < m * n; e += kAll) os[e] = c * ss[e];
     } else {
-      for (int e = threadIdx.x; e < m * r; e += kT) os[e] = c * ss[e];
-      for (int e = threadIdx.x; e < n * r; e += kT) os[m * r + e] = ss[m * r + e];
+      for (int e = tid; e < m * r; e += kAll) os[e] = c * ss[e];
+      for (int e = tid; e < n * r; e += kAll) os[m * r + e] = ss[m * r + e];
     }
-    if (threadIdx.x == 0) { O.kind[t] = kind; O.rank[t] = r; O.norm[t] = fabs(c) * S.norm[t]; }
+    if (tid == 0) { O.kind[t] = kind; O.rank[t] = r; O.norm[t] = fabs(c) * S.norm[t]; }
     return;
   }
   if (route == ROUTE_QR) {
     const int R = rx + ry;
     double* Xc = ws + 2 * sl;
     double* Wc = Xc + (int64_t)m * R;
-    for (int e = threadIdx.x; e < m * rx; e += kT) Xc[e] = a * xs[e];
-    for (int e = threadIdx.x; e < m * ry; e += kT) Xc[m * rx + e] = b * ys[e];
-    for (int e = threadIdx.x; e < n * rx; e += kT) Wc[e] = xs[m * rx + e];
-    for (int e = threadIdx.x; e < n * ry; e += kT) Wc[n * rx + e] = ys[m * ry + e];
+    for (int e = tid; e < m * rx; e += kAll) Xc[e] = a * xs[e];
+    for (int e = tid; e < m * ry; e += kAll) Xc[m * rx + e] = b * ys[e];
+    for (int e = tid; e < n * rx; e += kAll) Wc[e] = xs[m * rx + e];
+    for (int e = tid; e < n * ry; e += kAll) Wc[n * rx + e] = ys[m * ry + e];
     return;
   }
   // dense sum (ROUTE_DENSE or ROUTE_DACC)
   double part = 0.0;
-  for (int e = threadIdx.x; e < m * n; e += kT) {
+  for (int e = tid; e < m * n; e += kAll) {
     const int i = e % m, j = e / m;
     double v = 0.0;
     if (kx == CLR_KIND_DENSE) {
@@ -128,12 +138,17 @@ __global__ void __launch_bounds__(kT) lincomb_apply_kernel(double a, MatView X, 
     os[e] = v;
     part = fma(v, v, part);
   }
-  const double nsq = bsum(part, red);
-  if (threadIdx.x == 0) {
+  const double own = bsum(part, red);
+  if (threadIdx.x == 0) part_sq = own;
+  cluster.sync();
+  if (tid == 0) {
+    double nsq = 0.0;
+    for (int c = 0; c < kLcCtas; ++c) nsq += *cluster.map_shared_rank(&part_sq, c);
     O.kind[t] = CLR_KIND_DENSE;
     O.rank[t] = m < n ? m : n;
     O.norm[t] = sqrt(nsq);
   }
+  cluster.sync();   // no CTA's part goes before it has been read
 }
 
 void launch_plan_scan(const Plan& p, int recompress_dense, cudaStream_t st);
@@ -145,7 +160,7 @@ void launch_lincomb_plan(double a, const MatView& X, double b, const MatView& Y,
   cudaMemsetAsync(p.counters, 0, kPlanCountersClear, st);
   lincomb_route_kernel<<<(n + 127) / 128, 128, 0, st>>>(a, X, b, Y, diag, p);
   launch_plan_scan(p, recompress_dense, st);
-  lincomb_apply_kernel<<<n, kT, 0, st>>>(a, X, b, Y, diag, O, p, ws);
+  lincomb_apply_kernel<<<n * kLcCtas, kT, 0, st>>>(a, X, b, Y, diag, O, p, ws);
 }
 
 // Per block: ||M_IJ - delta_IJ I||_F^2, then a deterministic single-CTA sum.
@@ -297,8 +312,11 @@ void launch_matvec(const MatView& M, const double* x, double* y, cudaStream_t st
   matvec_kernel<<<M.nr * kMvCtas, kMvThreads, 0, st>>>(M, x, y);
 }
 
-// T = S^T: block (J,I) of T is block (I,J) of S transposed (dense) or with X and W swapped.
-__global__ void transpose_kernel(MatView S, MatView T) {
+// T = S^T: block (J,I) of T is block (I,J) of S transposed (dense, 32 x 32 tiles through shared
+// memory so that both sides are accessed along their columns) or with X and W swapped.  Several
+// CTAs per block (lr_parts).
+__global__ void __launch_bounds__(256) transpose_kernel(MatView S, MatView T) {
+  __shared__ double tile[32][33];
   const int t = blockIdx.x;
   const int I = t / S.nc, J = t % S.nc;
   const int m = S.row_off[I + 1] - S.row_off[I];
@@ -308,15 +326,22 @@ __global__ void transpose_kernel(MatView S, MatView T) {
   const int tt = J * T.nc + I;
   double* d = T.pool + slot_of(T, J, I, n);
   if (kind == CLR_KIND_DENSE) {
-    for (int e = threadIdx.x; e < m * n; e += blockDim.x) {
-      const int i = e % m, j = e / m;
-      d[j + (int64_t)i * n] = s[e];
+    const int ti = (m + 31) / 32, tj = (n + 31) / 32, x = threadIdx.x % 32, y = threadIdx.x / 32;
+    for (int q = blockIdx.y; q < ti * tj; q += gridDim.y) {
+      const int i0 = (q % ti) * 32, j0 = (q / ti) * 32;
+      for (int c = y; c < 32; c += 8)
+        if (i0 + x < m && j0 + c < n) tile[c][x] = s[i0 + x + (int64_t)(j0 + c) * m];
+      __syncthreads();
+      for (int c = y; c < 32; c += 8)
+        if (j0 + x < n && i0 + c < m) d[j0 + x + (int64_t)(i0 + c) * n] = tile[x][c];
+      __syncthreads();
     }
   } else if (kind == CLR_KIND_LR) {
-    for (int e = threadIdx.x; e < n * r; e += blockDim.x) d[e] = s[(int64_t)m * r + e];
-    for (int e = threadIdx.x; e < m * r; e += blockDim.x) d[(int64_t)n * r + e] = s[e];
+    const int e0 = threadIdx.x + blockDim.x * blockIdx.y, step = blockDim.x * gridDim.y;
+    for (int e = e0; e < n * r; e += step) d[e] = s[(int64_t)m * r + e];
+    for (int e = e0; e < m * r; e += step) d[(int64_t)n * r + e] = s[e];
   }
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && blockIdx.y == 0) {
     T.kind[tt] = kind;
     T.rank[tt] = r;
     T.norm[tt] = S.norm[t];
@@ -324,7 +349,8 @@ __global__ void transpose_kernel(MatView S, MatView T) {
 }
 
 void launch_transpose(const MatView& S, const MatView& T, cudaStream_t st) {
-  transpose_kernel<<<S.nr * S.nc, 256, 0, st>>>(S, T);
+  transpose_kernel<<<dim3((unsigned)(S.nr * S.nc), (unsigned)lr_parts(S.nr * S.nc)), 256, 0,
+                     st>>>(S, T);
 }
 
 }  // namespace clr
