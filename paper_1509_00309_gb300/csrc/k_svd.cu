@@ -79,9 +79,8 @@ __device__ double block_sum(double v, double* sh) {
 //    H y = y - v (v.y) rn rv with rn = 1 / ||x_j..||, rv = 1 / |v_0| (v.v / 2 = ||x|| |v_0|; two
 //    factors, so that neither over- nor underflows before ||x||^2 does).  One warp forms these
 //    while the others already take their columns' inner products with x, which need no scalar.
-// Measured: the two 16-column QRs of a 164 x 132 tile took 580k SM cycles before, 18k a step;
-// recompression of the 1D-chain product (N = 512) 757 -> 485 us, the build of the 3D lattice at
-// N = 4096 (pivoted QR of every block) 28.5 -> 24.5 ms.
+// Measured: the two 16-column QRs of a 164 x 132 tile took 580k SM cycles with a warp per column
+// and the scalars by every warp; 96k now (in registers, a CTA each, below).
 // ---------------------------------------------------------------------------------------------
 constexpr int kRowsPerLane = CLR_MAX_CLUSTER / 32;
 constexpr int kGroup = 8;   // columns a warp takes together in a step
@@ -582,7 +581,7 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
 }
 
 struct JacobiShared {
-  float nrm[CLR_MAX_CLUSTER];      // column norms
+  float2 nrm[CLR_MAX_CLUSTER];     // column norms: squared, and the root
   int last_rot[CLR_MAX_CLUSTER];   // the step of the column's last rotation, -1 if none
   int rotated, sweeps;
 };
@@ -593,7 +592,9 @@ struct JacobiShared {
 //  - LP lanes per pair and 2 kVec rows a lane (as packed pairs), so that a round's pairs fill the
 //    CTA once where they can: a warp alone issues an instruction every ~5 cycles, so a round
 //    costs what one of its warps has to issue;
-//  - norms, not their squares, are kept, so that the tests need no square root;
+//  - the norms' roots are kept beside their squares, so that the tests need no square root (and
+//    the squares so that the rotation angles see no more than the rounding of their updates:
+//    squared approximate roots drift, and clustered columns then stop converging);
 //  - only the warps that have pairs take part, with their own barrier (none for a single warp).
 // g: p x q, ld ldg (even, the row p of an odd p zero); v: q x q, ld ldv (even), reset to I.
 // tol, floor2: a pair is converged when its inner product is at most tol times the norms, or
@@ -603,7 +604,7 @@ template <int LP, int kVec>
 __device__ __noinline__ int jacobi32(float* g, int p, int q, int ldg, float* v, int ldv,
                                      int max_sweeps, float tol, float floor2,
                                      JacobiShared& sh) {
-  float* nrm = sh.nrm;
+  float2* nrm = sh.nrm;
   int* last_rot = sh.last_rot;
   constexpr unsigned kAll = 0xffffffffu;
   const int w = threadIdx.x / 32, li = threadIdx.x % LP, grp = threadIdx.x / LP;
@@ -637,7 +638,7 @@ __device__ __noinline__ int jacobi32(float* g, int p, int q, int ldg, float* v, 
           }
         }
         const float s = sum_lp(sum2(s2));
-        if (li == 0 && c < q) nrm[c] = fast_sqrt(s);
+        if (li == 0 && c < q) nrm[c] = make_float2(s, fast_sqrt(s));
       }
       if (threadIdx.x == 0) sh.rotated = 0;
       act_sync();
@@ -648,14 +649,14 @@ __device__ __noinline__ int jacobi32(float* g, int p, int q, int ldg, float* v, 
           int a, b;
           round_pair(round, k, qq, &a, &b);
           bool on = k < half && a < q && b < q;
-          float na = 0.f, nb = 0.f;
+          float2 na = make_float2(0.f, 0.f), nb = na;
           if (on) {
             // neither column rotated since this pair's check one sweep ago
             on = !(sweep > 0 && last_rot[a] < step - (qq - 1) && last_rot[b] < step - (qq - 1));
             na = nrm[a];
             nb = nrm[b];
           }
-          const float ab = na * nb;
+          const float ab = na.y * nb.y;
           on = on && ab > floor2;
           if (!__any_sync(kAll, on)) continue;
           f32x2* ga = reinterpret_cast<f32x2*>(g + a * ldg);
@@ -673,7 +674,7 @@ __device__ __noinline__ int jacobi32(float* g, int p, int q, int ldg, float* v, 
           // (inner products at the end of the FP32 range are left alone)
           on = on && ad > tol * ab && ad > floor2 && ad > 1e-37f;
           if (!__any_sync(kAll, on)) continue;
-          float a2 = na * na, b2 = nb * nb;
+          float a2 = na.x, b2 = nb.x;
           bool again = false;
           if (on) {
             f32x2* va = reinterpret_cast<f32x2*>(v + a * ldv);
@@ -731,8 +732,8 @@ __device__ __noinline__ int jacobi32(float* g, int p, int q, int ldg, float* v, 
             }
           }
           if (on && li == 0) {
-            nrm[a] = fast_sqrt(a2);
-            nrm[b] = fast_sqrt(b2);
+            nrm[a] = make_float2(a2, fast_sqrt(a2));
+            nrm[b] = make_float2(b2, fast_sqrt(b2));
             last_rot[a] = step;
             last_rot[b] = step;
             sh.rotated = 1;
@@ -1009,7 +1010,7 @@ __device__ void right_multiply_fp64(double* m, int rows, int64_t m_r, int64_t m_
 // Above this ||E||_F the series in small_series, cut after E^3 and with FP32 powers, is not FP64
 // accurate (the first term left out is 35/128 E^4, the powers' error 4e-8 E^2).
 constexpr double kSeriesFro = 2e-4;
-constexpr double kRefineFro = 1e-3;   // up to this, accurate after one refinement (ls_solve)
+constexpr double kRefineFro = 0.05;   // up to this, by refinement (ls_solve)
 
 // v (q x q, row-major) <- the orthogonal polar factor of the FP32 matrix v32 (ld ldv) in FP64:
 // V (V^T V)^-1/2 by its series in E = V^T V - I, which rotations accumulated in FP32 keep at
@@ -1067,15 +1068,17 @@ __device__ void recover_right(const SrcView& a, int p, int q, const double* g, c
 // y (q x r, row-major) <- y (G_r^T G_r)^-1 in FP64, G_r the kept columns gathered row-major in
 // `gr` (p x r), with norms d: the least-squares right factor when G_r is not orthogonal to FP64
 // precision.  The Gram matrix of the normalised columns is I + E, E at the FP32 stages' tolerance
-// (~1e-5), and its inverse I - E + E^2 - E^3; above kSeriesFro a Cholesky factorisation (in mw,
-// r^2 doubles, like e; f: 2 r^2 floats; gr and e are used again as work space, q r doubles each).
-// Between kSeriesFro and kRefineFro the series' result is refined once.  Returns false, with y
-// unchanged, when the Cholesky factorisation meets a pivot that is not positive (kept columns at
+// (~1e-5), and its inverse N = I - E + E^2 - E^3; above kSeriesFro the result is refined,
+// x += (y - x (I + E)) N, until the series' relative error to the power of the steps is below
+// 1e-16; above kRefineFro a Cholesky factorisation in mw (a chain of one row's steps per thread:
+// 10-40 M SM cycles at r ~ 110, which the relaxed test of a graded A made common before the
+// refinement).  mw, e: r^2 doubles, f: 2 r^2 floats, z: q r doubles; gr is used again (q r).
+// Returns false, with y unchanged, when the Cholesky factorisation meets a pivot that is not positive (kept columns at
 // the rounding level of a block whose norm is near eps); the caller then uses the
 // orthogonal-columns formula y S^-2.
 __device__ __noinline__ bool ls_solve(double* y, int q, int r, double* gr, int p,
-                                      const double* d, double* e, double* mw, float* f,
-                                      SvdShared& sh) {
+                                      const double* d, double* e, double* mw, double* z,
+                                      float* f, SvdShared& sh) {
   double* rd = sh.sigma_inv;
   for (int c = threadIdx.x; c < r; c += kThreads) rd[c] = 1.0 / d[c];
   __syncthreads();
@@ -1084,20 +1087,26 @@ __device__ __noinline__ bool ls_solve(double* y, int q, int r, double* gr, int p
   __syncthreads();
   const double fro2 = small_series(e, r, -1.0, 1.0f, -1.0f, f, sh);
   if (fro2 <= kRefineFro * kRefineFro) {
-    const bool refine = fro2 > kSeriesFro * kSeriesFro;
+    // the series' relative error: its first omitted term and the FP32 powers'
+    const double err = fro2 * fro2 + 1e-7 * fro2;
+    int steps = 0;
+    if (fro2 > kSeriesFro * kSeriesFro)
+      for (double x = err; x > 1e-16; x *= err) ++steps;
     for (int x = threadIdx.x; x < q * r; x += kThreads) {
       const double v = y[x] * rd[x % r];
       y[x] = v;
-      if (refine) gr[x] = v;
+      gr[x] = v;
     }
     __syncthreads();
     right_multiply_fp64(y, q, r, 1, r, e, true);
-    if (refine) {
-      // x + (y - x (I + E)): the error of x, ~E^4, times E remains
-      for (int x = threadIdx.x; x < q * r; x += kThreads) e[x] = y[x];
+    for (; steps > 0; --steps) {
+      for (int x = threadIdx.x; x < q * r; x += kThreads) z[x] = y[x];
       __syncthreads();
-      right_multiply_fp64(e, q, r, 1, r, mw, true);
-      for (int x = threadIdx.x; x < q * r; x += kThreads) y[x] += gr[x] - e[x];
+      right_multiply_fp64(z, q, r, 1, r, mw, true);
+      for (int x = threadIdx.x; x < q * r; x += kThreads) z[x] = gr[x] - z[x];
+      __syncthreads();
+      right_multiply_fp64(z, q, r, 1, r, e, true);
+      for (int x = threadIdx.x; x < q * r; x += kThreads) y[x] += z[x];
       __syncthreads();
     }
     for (int x = threadIdx.x; x < q * r; x += kThreads) y[x] *= rd[x % r];
@@ -1305,7 +1314,8 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
 // tile, one CTA the QR of X_cat and the final Q_X product, the other W_cat's; the core and its SVD
 // both compute (the same bits: nothing needs to be exchanged but the triangular factors, which
 // are read after one cluster barrier).  With more tiles each CTA takes its own, eight warps a
-// factor.
+// factor.  Measured, a 164 x 132 tile with R = 16 (SM cycles): QRs 262k -> 96k, application of Q
+// 149k -> 70k; compress_qr_kernel of the 1D chain at N = 512 374 -> 260 us.
 // ---------------------------------------------------------------------------------------------
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     compress_qr_kernel(MatView C, const int* list, const int* count, const int* rsum, double* ws,
@@ -1373,8 +1383,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       SrcView mv{M, 1, R, false};
       recover_right(mv, R, R, G, sh.perm, r, V, sc, false);
       if (ls)
-        ls = ls_solve(V, R, r, sc, R, sh.sorted, sc + 4 * kSq, sc + kSq, series_f32(r, sc + 3 * kSq),
-                      sh);
+        ls = ls_solve(V, R, r, sc, R, sh.sorted, sc + 4 * kSq, sc + kSq, sc + 3 * kSq,
+                      series_f32(r, sc), sh);
     }
     double* Xo = C.pool + sC;
     double* Wo = Xo + (int64_t)m * r;
@@ -1893,11 +1903,9 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
   const bool tracked = sh.v_tracked;
   bool ls = !tracked && sh.ls_recover;
   if (!tracked) recover_right(mv, q, k, gs, sh.perm, r, vs, sc, true);   // Y = R G_r (k x r)
-  // (R is no longer needed: its place takes the Cholesky factor and FP32 powers too large for
-  // shared memory)
+  // (R is no longer needed: its place is work space)
   if (ls)
-    ls = ls_solve(vs, k, r, sc, q, sh.sorted, sc + 4 * kSq, sc + kSq, series_f32(r, sc + 3 * kSq),
-                  sh);
+    ls = ls_solve(vs, k, r, sc, q, sh.sorted, sc + 4 * kSq, sc + kSq, rb, series_f32(r, sc), sh);
   // R = V_M S U_M^T:  X_R = (V_M S)_r (k x r), W_R = (U_M)_r (q x r); A ~ (Q_k X_R) (P W_R)^T
   // (the source in the slot is no longer read: the factors overwrite it)
   __syncthreads();
@@ -2085,8 +2093,8 @@ __global__ void __launch_bounds__(kThreads, 1) compress_dense_kernel(
       constexpr int64_t kSq = (int64_t)CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
       if (!tracked) recover_right(view, p, q, G, sh.perm, r, V, sc, false);
       if (ls)
-        ls = ls_solve(V, q, r, sc, p, sh.sorted, sc + 4 * kSq, sc + kSq,
-                      series_f32(r, sc + 2 * kSq), sh);
+        ls = ls_solve(V, q, r, sc, p, sh.sorted, sc + 4 * kSq, sc + kSq, sc + 3 * kSq,
+                      series_f32(r, sc), sh);
       if (jstats && threadIdx.x == 0 && !tracked)
         atomicAdd(&jstats[4], 2ull * p * q * r);
       double* Xo = slot;
@@ -2197,7 +2205,8 @@ void launch_block_norms(const MatView& M, cudaStream_t st) {
   block_norms_kernel<<<M.nr * M.nc, kThreads, 0, st>>>(M);
 }
 
-// alpha * M in place: dense values or the X factor, and the norms.
+// alpha * M in place: dense values or the X factor, and the norms; several CTAs per block
+// (lr_parts).
 __global__ void scale_blocks_kernel(MatView M, double alpha) {
   const int t = blockIdx.x;
   const int I = t / M.nc, J = t % M.nc;
@@ -2207,12 +2216,15 @@ __global__ void scale_blocks_kernel(MatView M, double alpha) {
   double* s = M.pool + slot_of(M, I, J, m);
   int64_t len = kind == CLR_KIND_DENSE ? (int64_t)m * n
               : kind == CLR_KIND_LR ? (int64_t)m * M.rank[t] : 0;
-  for (int64_t e = threadIdx.x; e < len; e += blockDim.x) s[e] *= alpha;
-  if (threadIdx.x == 0) M.norm[t] *= fabs(alpha);
+  const int64_t step = (int64_t)blockDim.x * gridDim.y;
+  for (int64_t e = threadIdx.x + (int64_t)blockDim.x * blockIdx.y; e < len; e += step)
+    s[e] *= alpha;
+  if (threadIdx.x == 0 && blockIdx.y == 0) M.norm[t] *= fabs(alpha);
 }
 
 void launch_scale_blocks(const MatView& M, double alpha, cudaStream_t st) {
-  scale_blocks_kernel<<<M.nr * M.nc, 256, 0, st>>>(M, alpha);
+  scale_blocks_kernel<<<dim3((unsigned)(M.nr * M.nc), (unsigned)lr_parts(M.nr * M.nc)), 256, 0,
+                        st>>>(M, alpha);
 }
 
 }  // namespace clr
