@@ -60,19 +60,19 @@ __device__ __forceinline__ int next_item(int* counter, int* sh_slot) {
 }
 
 // out(i,j) (= or +=) sum_l a(i,l) b(l,j) for a P x Q output (column-major, ld ldo) with
-// arbitrary element strides of a and b, by a CTA of NT threads.  FP64 runs at ~2 FMAs per clock
+// arbitrary element strides of a and b, by nt threads (tid this one).  FP64 runs at ~2 FMAs per clock
 // per SM on this part: a warp's FMA holds its sub-partition's pipe for 64 cycles, in which the
 // loads of the next ones arrive, so what counts is that the FMAs are spread evenly over the warps
 // and waste no lanes.  The output is cut into MR x MC micro-tiles (ragged last ones clamped)
 // taken by the threads in turn, rows first (a should have unit stride along i; b is mostly
 // broadcast).  TRI = 1: a(i, l) is zero for l > i; TRI = 2: b(l, j) is zero for l < j (those
 // terms are skipped).  No synchronisation inside: the caller orders dependent calls.
-template <int NT, int MR, int MC, int TRI, class T>
-__device__ __forceinline__ void cta_gemm_micro(int P, int Q, int L, const T* a, int64_t a_r,
+template <int MR, int MC, int TRI, class T>
+__device__ __forceinline__ void cta_gemm_micro(int tid, int nt, int P, int Q, int L, const T* a, int64_t a_r,
                                                int64_t a_c, const T* b, int64_t b_r, int64_t b_c,
                                                T* out, int64_t ldo, bool accumulate) {
   const int mp = (P + MR - 1) / MR, mq = (Q + MC - 1) / MC;
-  for (int t = threadIdx.x; t < mp * mq; t += NT) {
+  for (int t = tid; t < mp * mq; t += nt) {
     const int i0 = (t % mp) * MR, j0 = (t / mp) * MC;
     const int l0 = TRI == 2 ? j0 : 0;
     const int l1 = TRI == 1 && i0 + MR < L ? i0 + MR : L;
@@ -120,18 +120,18 @@ __device__ __forceinline__ void cta_gemm_micro(int P, int Q, int L, const T* a, 
 // fill 152 SMs evenly, 1 where the blocks alone do.
 inline int lr_parts(int n_blocks) { return n_blocks <= 1024 ? 8 : n_blocks <= 4096 ? 4 : 1; }
 
-// The micro-tile by the size of the output: 4 x 2 from four rounds of the CTA's threads on
+// The micro-tile by the size of the output: 4 x 2 from four rounds of the threads on
 // (less than a quarter of a round idle at the end), 2 x 2 from one, else an entry per thread.
-template <int NT, int TRI = 0, class T>
-__device__ __forceinline__ void cta_gemm_auto(int P, int Q, int L, const T* a, int64_t a_r,
+template <int TRI = 0, class T>
+__device__ __forceinline__ void cta_gemm_auto(int tid, int nt, int P, int Q, int L, const T* a, int64_t a_r,
                                               int64_t a_c, const T* b, int64_t b_r, int64_t b_c,
                                               T* out, int64_t ldo, bool accumulate = false) {
-  if (P * Q >= 32 * NT)
-    cta_gemm_micro<NT, 4, 2, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
-  else if (P * Q >= 4 * NT)
-    cta_gemm_micro<NT, 2, 2, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
+  if (P * Q >= 32 * nt)
+    cta_gemm_micro<4, 2, TRI>(tid, nt, P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
+  else if (P * Q >= 4 * nt)
+    cta_gemm_micro<2, 2, TRI>(tid, nt, P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
   else
-    cta_gemm_micro<NT, 1, 1, TRI>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
+    cta_gemm_micro<1, 1, TRI>(tid, nt, P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
 }
 
 struct Triple {

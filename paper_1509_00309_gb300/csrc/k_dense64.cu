@@ -10,6 +10,8 @@
 // columns beyond the next multiple of 16 skipped), walking that tile's dense x dense products in
 // k order (deterministic, no atomics).  Sub-tiles are taken from a launch-wide counter over the
 // tiles in decreasing cost order (longest-processing-time scheduling).
+#include <cooperative_groups.h>
+
 #include "clr_internal.h"
 
 namespace clr {
@@ -202,18 +204,26 @@ void launch_set_route_kinds(const MatView& C, const Plan& p, cudaStream_t st) {
   set_route_kinds_kernel<<<(n + 127) / 128, 128, 0, st>>>(C, p);
 }
 
-// Frobenius norms of the dense-accumulated tiles (those not recompressed afterwards).
-__global__ void __launch_bounds__(256) dense_tile_norms_kernel(MatView C, Plan p) {
+// Frobenius norms of the dense-accumulated tiles (those not recompressed afterwards): a cluster of
+// CTAs per tile, its parts added in a fixed order (with one CTA a tile's loads took 20 us).
+constexpr int kNormCtas = 8;
+__global__ void __cluster_dims__(kNormCtas, 1, 1) __launch_bounds__(256)
+    dense_tile_norms_kernel(MatView C, Plan p) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
   __shared__ double red[8];
+  __shared__ double part;
+  const int rank = (int)cluster.block_rank();
   const int n_items = p.counters->n_dense;
-  for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
+  for (int it = blockIdx.x / kNormCtas; it < n_items; it += gridDim.x / kNormCtas) {
     const int t = p.l_dense[it];
     const int I = t / p.nJ, J = t % p.nJ;
     const int m = C.row_off[I + 1] - C.row_off[I];
     const int n = C.col_off[J + 1] - C.col_off[J];
     const double* D = C.pool + slot_of(C, I, J, m);
     double s = 0.0;
-    for (int e = threadIdx.x; e < m * n; e += 256) s = fma(D[e], D[e], s);
+#pragma unroll 4
+    for (int e = threadIdx.x + 256 * rank; e < m * n; e += 256 * kNormCtas) s = fma(D[e], D[e], s);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = s;
@@ -221,9 +231,15 @@ __global__ void __launch_bounds__(256) dense_tile_norms_kernel(MatView C, Plan p
     if (threadIdx.x == 0) {
       double tot = 0.0;
       for (int i = 0; i < 8; ++i) tot += red[i];
+      part = tot;
+    }
+    cluster.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+      double tot = 0.0;
+      for (int c = 0; c < kNormCtas; ++c) tot += *cluster.map_shared_rank(&part, c);
       C.norm[t] = sqrt(tot);
     }
-    __syncthreads();
+    cluster.sync();   // the parts have been read
   }
 }
 

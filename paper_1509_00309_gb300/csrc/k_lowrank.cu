@@ -40,7 +40,7 @@ constexpr int kLrThreads = 256;
 __device__ __forceinline__ void cta_gemm(int P, int Q, int L, const double* a, int64_t a_r,
                                          int64_t a_c, const double* b, int64_t b_r, int64_t b_c,
                                          double* out, int64_t ldo, bool accumulate) {
-  cta_gemm_auto<kLrThreads>(P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
+  cta_gemm_auto((int)threadIdx.x, kLrThreads, P, Q, L, a, a_r, a_c, b, b_r, b_c, out, ldo, accumulate);
 }
 
 __device__ void cta_copy_cols(int rows, int cols, const double* src, int64_t lds, double* dst,

@@ -737,7 +737,7 @@ __global__ void __launch_bounds__(256) oz_lr_recon_kernel(MatView M, double* rec
   const double* w = x + (int64_t)m * r;        // n x r, ld n
   // out(i, j) = sum_q X(i, q) W(j, q)
   const int j0 = n * (int)blockIdx.y / (int)gridDim.y, j1 = n * ((int)blockIdx.y + 1) / (int)gridDim.y;
-  cta_gemm_auto<256>(m, j1 - j0, r, x, 1, m, w + j0, n, 1, recon + slot + (int64_t)j0 * m, m);
+  cta_gemm_auto((int)threadIdx.x, 256, m, j1 - j0, r, x, 1, m, w + j0, n, 1, recon + slot + (int64_t)j0 * m, m);
 }
 
 __global__ void __launch_bounds__(256) oz_exp_lr_kernel(MatView M, const double* recon,

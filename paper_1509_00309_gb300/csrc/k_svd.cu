@@ -65,6 +65,42 @@ __device__ double block_sum(double v, double* sh) {
   return s;
 }
 
+// The CTAs that work on one tile: one, or a whole cluster (compress_dense_kernel while tiles are
+// few).  Data in global memory is shared out by tid / nt and w / nw; what every CTA needs in
+// shared memory each keeps a copy of, computed alike from the same data or written to every copy
+// by put().
+// (One is the team of a single CTA, known when the kernel is compiled.)
+struct Team {
+  int rank, size;   // this CTA and the number of CTAs
+  int tid, nt;      // this thread and the threads of the team
+  int w, nw;        // this warp (warps are dealt over the CTAs) and the warps of the team
+  __device__ __forceinline__ Team(int r, int n)
+      : rank(r), size(n), tid(r * kThreads + threadIdx.x), nt(n * kThreads),
+        w(r + n * (int)(threadIdx.x / 32)), nw(n * kWarps) {}
+  __device__ __forceinline__ void sync() const {
+    if (size == 1) __syncthreads(); else cooperative_groups::this_cluster().sync();
+  }
+  template <class T>
+  __device__ __forceinline__ void put(T* local, T v) const {
+    if (size == 1) {
+      *local = v;
+    } else {
+      cooperative_groups::cluster_group c = cooperative_groups::this_cluster();
+      for (int r = 0; r < size; ++r) *c.map_shared_rank(local, r) = v;
+    }
+  }
+};
+struct One {
+  static constexpr int rank = 0, size = 1, nt = kThreads, nw = kWarps;
+  int tid, w;
+  __device__ __forceinline__ One() : tid(threadIdx.x), w(threadIdx.x / 32) {}
+  __device__ __forceinline__ void sync() const { __syncthreads(); }
+  template <class T>
+  __device__ __forceinline__ void put(T* local, T v) const {
+    *local = v;
+  }
+};
+
 // ---------------------------------------------------------------------------------------------
 // Householder steps.  What bounds them is the FP64 pipe: one warp-instruction per 19 cycles and
 // SM, an addition in a reduction as dear as a fused multiply-add, and a scalar square root or
@@ -600,10 +636,15 @@ struct JacobiShared {
 // tol, floor2: a pair is converged when its inner product is at most tol times the norms, or
 // floor2.  Measured (core of 16 columns, both FP32 stages): 259k SM cycles with the copies in the
 // global scratch, a warp per pair and 8 masked rows a lane.
-template <int LP, int kVec>
-__device__ __noinline__ int jacobi32(float* g, int p, int q, int ldg, float* v, int ldv,
+// kShared: both copies in shared memory, g and v given as offsets into it (addressed as such: a
+// generic pointer's loads are slower).
+template <int LP, int kVec, bool kShared>
+__device__ __noinline__ int jacobi32(float* g_ptr, int q, int ldg, float* v_ptr, int ldv,
                                      int max_sweeps, float tol, float floor2,
                                      JacobiShared& sh) {
+  extern __shared__ __align__(16) float svd_smem[];
+  float* const g = kShared ? svd_smem + (int)(g_ptr - svd_smem) : g_ptr;
+  float* const v = kShared ? svd_smem + (int)(v_ptr - svd_smem) : v_ptr;
   float2* nrm = sh.nrm;
   int* last_rot = sh.last_rot;
   constexpr unsigned kAll = 0xffffffffu;
@@ -757,41 +798,128 @@ struct Work32 {
   float *g, *v;
   int ldg, ldv, lp, vec;
 };
-// Dynamic shared memory of the recompression kernels: with their static part (27 KB) all that a
-// CTA can have, enough for a 256 x 136 pair of copies or a 158 x 158 one.
-constexpr int kSvdSmemBytes = 196 * 1024;
+// Dynamic shared memory of the recompression kernels: with their static part (34 KB) nearly all
+// that a CTA can have, enough for a 256 x 133 pair of copies or a 156 x 156 one.
+constexpr int kSvdSmemBytes = 192 * 1024;
 
-__device__ __forceinline__ Work32 work32(int p, int q, double* sc) {
-  extern __shared__ __align__(16) float svd_smem[];
-  Work32 k;
-  // 16 lanes a pair put up to 32 pairs into one pass over the CTA's 16 warps, 32 lanes up to 16;
-  // one packed row a lane while the rows are few
+// Lanes and packed rows per lane for columns of p rows: 16 lanes a pair put up to 32 pairs into one
+// pass over the CTA's 16 warps, 32 lanes up to 16; one packed row a lane while the rows are few.
+__device__ __forceinline__ void split32(Work32& k, int p, int q) {
   k.ldg = (p + 1) & ~1;
   k.ldv = (q + 1) & ~1;
   k.lp = p <= 32 || (q > 32 && p <= 128) ? 16 : 32;
   k.vec = (k.ldg / 2 + k.lp - 1) / k.lp;
+}
+
+__device__ __forceinline__ Work32 work32(int p, int q, double* sc) {
+  extern __shared__ __align__(16) float svd_smem[];
+  Work32 k;
+  split32(k, p, q);
   const bool fits = (int64_t)(k.ldg + k.ldv) * q * (int)sizeof(float) <= kSvdSmemBytes;
   k.g = fits ? svd_smem : reinterpret_cast<float*>(sc);
   k.v = k.g + k.ldg * q;
   return k;
 }
 
-__device__ __forceinline__ int run_jacobi32(const Work32& k, int p, int q, int max_sweeps,
-                                            float tol, float floor2, JacobiShared& sh) {
+// Whether the sweeps on a graded p x q matrix run on its FP32 triangular factor instead: rotations
+// of A = Q R from the right are those of R, whose columns are q long, and Householder QR keeps
+// each column's error relative to its own norm, as the grading needs.  The QR works in shared
+// memory (p q floats).
+__device__ __forceinline__ bool use_qr32(int p, int q) {
+  return 8 * p >= 9 * q && (int64_t)((p + 1) & ~1) * q * (int)sizeof(float) <= kSvdSmemBytes;
+}
+
+// k.g (p x q, ld k.ldg, in shared memory) <- its triangular factor (q x q, zero below the diagonal),
+// k set up for it: V beside it in shared memory, or in the scratch.  One barrier a step: every
+// warp forms the reflector itself and takes its columns.  Measured (256 x 100): 4.0 M SM cycles of
+// sweeps on A, 2.4 M with this.
+__device__ __noinline__ void qr32(Work32& k, int p, int q, double* sc) {
+  extern __shared__ __align__(16) float svd_smem[];
+  const int w = threadIdx.x / 32, l = threadIdx.x % 32;
+  constexpr int kPer = CLR_MAX_CLUSTER / 32;
+  float beta = 0.f;
+  for (int j = 0; j < q; ++j) {
+    const float* x = k.g + j * k.ldg;
+    float xr[kPer], s = 0.f;
+#pragma unroll
+    for (int t = 0; t < kPer; ++t) {
+      const int i = l + 32 * t;
+      xr[t] = i > j && i < p ? x[i] : 0.f;
+      s = fmaf(xr[t], xr[t], s);
+    }
+    const float x0 = x[j];
+    s = warp_sum(s);
+    // v = (v0, x below the diagonal), H = I - v v^T / (||x|| |v0|)
+    const float nrm = sqrtf(fmaf(x0, x0, s)), v0 = x0 + copysignf(nrm, x0);
+    const float tau = s > 0.f ? __fdividef(1.f, nrm) * __fdividef(1.f, fabsf(v0)) : 0.f;
+    beta = s > 0.f ? -copysignf(nrm, x0) : x0;
+    if (l == j % 32) {
+#pragma unroll
+      for (int t = 0; t < kPer; ++t)
+        if (t == j / 32) xr[t] = v0;
+    }
+    for (int c = j + 1 + w; c < q; c += kWarps) {
+      float* y = k.g + c * k.ldg;
+      float yr[kPer], d = 0.f;
+#pragma unroll
+      for (int t = 0; t < kPer; ++t) {
+        const int i = l + 32 * t;
+        yr[t] = i >= j && i < p ? y[i] : 0.f;
+        d = fmaf(xr[t], yr[t], d);
+      }
+      const float f = tau * warp_sum(d);
+#pragma unroll
+      for (int t = 0; t < kPer; ++t) {
+        const int i = l + 32 * t;
+        if (i >= j && i < p) y[i] = fmaf(-f, xr[t], yr[t]);
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) k.g[j * k.ldg + j] = beta;   // (read no more by the steps to come)
+  }
+  __syncthreads();
+  // columns moved together, to the even leading dimension of q rows: a column's new place ends
+  // before the next one's old place starts
+  const int ldp = k.ldg;
+  Work32 n = k;
+  split32(n, q, q);
+  for (int c = 0; c < q; ++c) {
+    const int i = threadIdx.x;
+    const float v = i <= c ? k.g[c * ldp + i] : 0.f;
+    __syncthreads();
+    if (i < n.ldg) n.g[c * n.ldg + i] = v;
+  }
+  const bool fits = (int64_t)2 * n.ldg * q * (int)sizeof(float) <= kSvdSmemBytes;
+  n.v = fits ? n.g + n.ldg * q : reinterpret_cast<float*>(sc);
+  k = n;
+  __syncthreads();
+}
+
+__device__ __forceinline__ int run_jacobi32(const Work32& k, int q, int max_sweeps, float tol,
+                                            float floor2, JacobiShared& sh) {
+  extern __shared__ __align__(16) float svd_smem[];
+#define CLR_JACOBI32(LP, VEC, SH) \
+  return jacobi32<LP, VEC, SH>(k.g, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh)
+  const float* end = svd_smem + kSvdSmemBytes / sizeof(float);
+  if (!(k.g >= svd_smem && k.g < end && k.v >= svd_smem && k.v < end)) {
+    if (k.vec <= 3) CLR_JACOBI32(32, 3, false);   // (columns of more than 128 rows only)
+    CLR_JACOBI32(32, 4, false);
+  }
   if (k.lp == 16) {
     switch (k.vec) {
-      case 1: return jacobi32<16, 1>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
-      case 2: return jacobi32<16, 2>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
-      case 3: return jacobi32<16, 3>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
-      default: return jacobi32<16, 4>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
+      case 1: CLR_JACOBI32(16, 1, true);
+      case 2: CLR_JACOBI32(16, 2, true);
+      case 3: CLR_JACOBI32(16, 3, true);
+      default: CLR_JACOBI32(16, 4, true);
     }
   }
   switch (k.vec) {
     case 1:
-    case 2: return jacobi32<32, 2>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
-    case 3: return jacobi32<32, 3>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
-    default: return jacobi32<32, 4>(k.g, p, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh);
+    case 2: CLR_JACOBI32(32, 2, true);
+    case 3: CLR_JACOBI32(32, 3, true);
+    default: CLR_JACOBI32(32, 4, true);
   }
+#undef CLR_JACOBI32
 }
 
 // Where small_series keeps its 2 q^2 floats: the place of the FP32 copies, which the
@@ -817,12 +945,15 @@ struct SvdShared {
   // reflectors of the pivoted QR, of rrqr_block, or of the QR route's X factor; and of its W
   Reflectors refl, refl_w;
   int qr_perm[CLR_MAX_CLUSTER];   // pivoted QR: column order (columns are not moved)
+  double qr_diag[CLR_MAX_CLUSTER];   // and R's diagonal (the columns keep their x_j there)
+  int sweeps;      // of the second FP32 stage (every CTA's copy)
   JacobiShared jac;
   double cert;    // tail_lower_bound_sq's result
-  // compress_by_pivoted_qr: each column's trailing norm^2 when it was last summed exactly (the
-  // downdated norms are recomputed once they fall below kDowndateFloor of it), and the FMAs
-  // of those recomputations
-  double qr_nref[CLR_MAX_CLUSTER];
+  // compress_by_pivoted_qr, by parity of the step: each column's trailing norm^2, downdated, and
+  // its value when it was last summed exactly (the downdated norms are recomputed once they fall
+  // below kDowndateFloor of it); and the FMAs of those recomputations
+  double qr_nu[2][CLR_MAX_CLUSTER];
+  double qr_nref[2][CLR_MAX_CLUSTER];
   unsigned long long qr_recomputed;
 };
 // Downdated column norms^2 are summed again exactly once they fall below this fraction of the
@@ -910,8 +1041,10 @@ struct SrcView {
 //   e <- c1 E + c2 E^2 + c3 E^3.
 // The powers are taken in FP32 (f: 2 q^2 floats): E is at most a few 1e-4, so their error is
 // below 1e-16.  Returns ||E||_F^2.
-__device__ __noinline__ double small_series(double* e, int q, double c1, float c2, float c3,
-                                            float* f, SvdShared& sh) {
+template <class TM>
+__device__ __noinline__ double small_series(const TM& tm, double* e, int q, double c1, float c2,
+                                            float c3, float* f, SvdShared& sh) {
+  // (every CTA of the team takes the FP32 powers itself)
   float* t = f + q * q;
   float part = 0.f;
   for (int x = threadIdx.x; x < q * q; x += kThreads) {
@@ -920,24 +1053,26 @@ __device__ __noinline__ double small_series(double* e, int q, double c1, float c
     part = fmaf(v, v, part);
   }
   const double fro2 = block_sum((double)part, sh.red);
-  cta_gemm_auto<kThreads>(q, q, q, f, 1, q, f, 1, q, t, q);
-  __syncthreads();
+  cta_gemm_auto(threadIdx.x, kThreads, q, q, q, f, 1, q, f, 1, q, t, q);
+  tm.sync();
   // E^3 = F T an output at a time, added to the rest of the series
-  for (int x = threadIdx.x; x < q * q; x += kThreads) {
+  for (int x = tm.tid; x < q * q; x += tm.nt) {
     const int i = x % q, j = x / q;
     float s = 0.f;
     for (int l = 0; l < q; ++l) s = fmaf(f[i + l * q], t[l + j * q], s);
     e[x] = fma(c1, e[x], (double)fmaf(c2, t[x], c3 * s));
   }
-  __syncthreads();
+  tm.sync();
   return fro2;
 }
 
 // e (q x q) <- G^T G scaled by d on both sides (d null: unscaled) minus I, for G (n x q) given
 // row-major (element (l, i) at a[l q + i]): the lower triangle in 2 x 2 blocks, mirrored.
-__device__ void gram_minus_identity(const double* a, int n, int q, const double* d, double* e) {
+template <class TM>
+__device__ void gram_minus_identity(const TM& tm, const double* a, int n, int q,
+                                    const double* d, double* e) {
   const int nb = (q + 1) / 2;
-  for (int t = threadIdx.x; t < nb * (nb + 1) / 2; t += kThreads) {
+  for (int t = tm.tid; t < nb * (nb + 1) / 2; t += tm.nt) {
     int bi = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
     while (bi * (bi + 1) / 2 > t) --bi;
     while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
@@ -963,17 +1098,18 @@ __device__ void gram_minus_identity(const double* a, int n, int q, const double*
     if (i0 + 1 < q) put(i1, j0, s10);
     if (i0 + 1 < q && j0 + 1 < q) put(i1, j1, s11);
   }
-  __syncthreads();
+  tm.sync();
 }
 
 // m (rows x q, row-major) <- m (I + w) (add_identity) or m w in FP64, w q x q row-major, row by
 // row in place: one warp per row, the row held in registers (8 entries per lane) and broadcast
 // by shuffles, 8 output columns per lane.  m's element (i, k) is at m[i m_r + k m_c].
-__device__ void right_multiply_fp64(double* m, int rows, int64_t m_r, int64_t m_c, int q,
-                                    const double* wt, bool add_identity) {
+template <class TM>
+__device__ void right_multiply_fp64(const TM& tm, double* m, int rows, int64_t m_r, int64_t m_c,
+                                    int q, const double* wt, bool add_identity) {
   constexpr int kPer = CLR_MAX_CLUSTER / 32;
-  const int wp = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int i = wp; i < rows; i += kWarps) {
+  const int l = threadIdx.x % 32;
+  for (int i = tm.w; i < rows; i += tm.nw) {
     double r[kPer], acc[kPer];
 #pragma unroll
     for (int j = 0; j < kPer; ++j) {
@@ -1004,7 +1140,7 @@ __device__ void right_multiply_fp64(double* m, int rows, int64_t m_r, int64_t m_
       if (c < q) m[i * m_r + c * m_c] = acc[o];
     }
   }
-  __syncthreads();
+  tm.sync();
 }
 
 // Above this ||E||_F the series in small_series, cut after E^3 and with FP32 powers, is not FP64
@@ -1017,52 +1153,58 @@ constexpr double kRefineFro = 0.05;   // up to this, by refinement (ls_solve)
 // about 1e-5; repeated until ||E||_F has been below kSeriesFro.  Two products of q^3 FMAs (one of
 // them symmetric) that fill the CTA, against Gram-Schmidt's q^3 FMAs in q dependent steps of
 // reductions.  Measured (q = 16, with the product that follows): 218k -> 25k SM cycles; 3D lattice
-// product at N = 4096, both stages over all blocks: 3.1 -> 2.1 G cycles.  e: q^2 doubles, f: 2 q^2 floats, not overlapping v32's
-// matrix until it has been read.
-__device__ __noinline__ void orthonormalise_fp64(const float* v32, int ldv, double* v, int q,
-                                                 double* e, float* f, SvdShared& sh) {
-  for (int x = threadIdx.x; x < q * q; x += kThreads) {
-    const int i = x / q, j = x - i * q;
-    v[x] = (double)v32[i + j * ldv];
-  }
-  __syncthreads();
+// product at N = 4096, both stages over all blocks: 3.1 -> 2.1 G cycles.  v32 is
+// the team's first CTA's; e: q^2 doubles, f: 2 q^2 floats, not overlapping v32's matrix until it
+// has been read.
+template <class TM>
+__device__ __noinline__ void orthonormalise_fp64(const TM& tm, const float* v32, int ldv,
+                                                 double* v, int q, double* e, float* f,
+                                                 SvdShared& sh) {
+  if (tm.rank == 0)
+    for (int x = threadIdx.x; x < q * q; x += kThreads) {
+      const int i = x / q, j = x - i * q;
+      v[x] = (double)v32[i + j * ldv];
+    }
+  tm.sync();
   for (int pass = 0; pass < 4; ++pass) {
-    gram_minus_identity(v, q, q, nullptr, e);
-    const double fro2 = small_series(e, q, -0.5, 0.375f, -0.3125f, f, sh);
-    right_multiply_fp64(v, q, q, 1, q, e, true);
+    gram_minus_identity(tm, v, q, q, nullptr, e);
+    const double fro2 = small_series(tm, e, q, -0.5, 0.375f, -0.3125f, f, sh);
+    right_multiply_fp64(tm, v, q, q, 1, q, e, true);
     if (!(fro2 > kSeriesFro * kSeriesFro)) break;
   }
 }
 
 // g (p x q, ld p) = A v in FP64, v row-major.  lower: A(i, l) = 0 for l > i (the transposed
 // triangular factor), half of its first q rows.
-__device__ void project_fp64(const SrcView& a, int p, int q, const double* v, double* g,
-                             bool lower) {
+template <class TM>
+__device__ void project_fp64(const TM& tm, const SrcView& a, int p, int q, const double* v,
+                             double* g, bool lower) {
   const int64_t a_i = a.tr ? a.s_c : a.s_r, a_k = a.tr ? a.s_r : a.s_c;
   if (lower)
-    cta_gemm_auto<kThreads, 1>(p, q, q, a.src, a_i, a_k, v, q, 1, g, p);
+    cta_gemm_auto<1>(tm.tid, tm.nt, p, q, q, a.src, a_i, a_k, v, q, 1, g, p);
   else
-    cta_gemm_auto<kThreads>(p, q, q, a.src, a_i, a_k, v, q, 1, g, p);
-  __syncthreads();
+    cta_gemm_auto(tm.tid, tm.nt, p, q, q, a.src, a_i, a_k, v, q, 1, g, p);
+  tm.sync();
 }
 
 // y (q x r, row-major) = A^T G_r in FP64, G_r the r kept columns of g (p x q, ld p) in the order
 // perm; with G_r = U_r S_r this is V_r S_r^2.  G_r is first gathered row-major into `gather`
 // (p r doubles, not overlapping g or y).  lower: A(i, j) = 0 for i < j.
-__device__ void recover_right(const SrcView& a, int p, int q, const double* g, const int* perm,
-                              int r, double* y, double* gather, bool lower) {
-  for (int e = threadIdx.x; e < p * r; e += kThreads) {
+template <class TM>
+__device__ void recover_right(const TM& tm, const SrcView& a, int p, int q, const double* g,
+                              const int* perm, int r, double* y, double* gather, bool lower) {
+  for (int e = tm.tid; e < p * r; e += tm.nt) {
     const int k = e / r, c = e - k * r;
     gather[e] = g[k + (int64_t)perm[c] * p];
   }
-  __syncthreads();
+  tm.sync();
   // y^T(c, j) = sum_k G_r(k, c) A(k, j)
   const int64_t a_j = a.tr ? a.s_r : a.s_c, a_k = a.tr ? a.s_c : a.s_r;
   if (lower)
-    cta_gemm_auto<kThreads, 2>(r, q, p, gather, 1, r, a.src, a_k, a_j, y, r);
+    cta_gemm_auto<2>(tm.tid, tm.nt, r, q, p, gather, 1, r, a.src, a_k, a_j, y, r);
   else
-    cta_gemm_auto<kThreads>(r, q, p, gather, 1, r, a.src, a_k, a_j, y, r);
-  __syncthreads();
+    cta_gemm_auto(tm.tid, tm.nt, r, q, p, gather, 1, r, a.src, a_k, a_j, y, r);
+  tm.sync();
 }
 
 // y (q x r, row-major) <- y (G_r^T G_r)^-1 in FP64, G_r the kept columns gathered row-major in
@@ -1076,43 +1218,45 @@ __device__ void recover_right(const SrcView& a, int p, int q, const double* g, c
 // Returns false, with y unchanged, when the Cholesky factorisation meets a pivot that is not positive (kept columns at
 // the rounding level of a block whose norm is near eps); the caller then uses the
 // orthogonal-columns formula y S^-2.
-__device__ __noinline__ bool ls_solve(double* y, int q, int r, double* gr, int p,
+template <class TM>
+__device__ __noinline__ bool ls_solve(const TM& tm, double* y, int q, int r, double* gr, int p,
                                       const double* d, double* e, double* mw, double* z,
                                       float* f, SvdShared& sh) {
   double* rd = sh.sigma_inv;
   for (int c = threadIdx.x; c < r; c += kThreads) rd[c] = 1.0 / d[c];
   __syncthreads();
-  gram_minus_identity(gr, p, r, rd, e);
-  for (int x = threadIdx.x; x < r * r; x += kThreads) mw[x] = e[x];
-  __syncthreads();
-  const double fro2 = small_series(e, r, -1.0, 1.0f, -1.0f, f, sh);
+  gram_minus_identity(tm, gr, p, r, rd, e);
+  for (int x = tm.tid; x < r * r; x += tm.nt) mw[x] = e[x];
+  tm.sync();
+  const double fro2 = small_series(tm, e, r, -1.0, 1.0f, -1.0f, f, sh);
   if (fro2 <= kRefineFro * kRefineFro) {
     // the series' relative error: its first omitted term and the FP32 powers'
     const double err = fro2 * fro2 + 1e-7 * fro2;
     int steps = 0;
     if (fro2 > kSeriesFro * kSeriesFro)
       for (double x = err; x > 1e-16; x *= err) ++steps;
-    for (int x = threadIdx.x; x < q * r; x += kThreads) {
+    for (int x = tm.tid; x < q * r; x += tm.nt) {
       const double v = y[x] * rd[x % r];
       y[x] = v;
       gr[x] = v;
     }
-    __syncthreads();
-    right_multiply_fp64(y, q, r, 1, r, e, true);
+    tm.sync();
+    right_multiply_fp64(tm, y, q, r, 1, r, e, true);
     for (; steps > 0; --steps) {
-      for (int x = threadIdx.x; x < q * r; x += kThreads) z[x] = y[x];
-      __syncthreads();
-      right_multiply_fp64(z, q, r, 1, r, mw, true);
-      for (int x = threadIdx.x; x < q * r; x += kThreads) z[x] = gr[x] - z[x];
-      __syncthreads();
-      right_multiply_fp64(z, q, r, 1, r, e, true);
-      for (int x = threadIdx.x; x < q * r; x += kThreads) y[x] += z[x];
-      __syncthreads();
+      for (int x = tm.tid; x < q * r; x += tm.nt) z[x] = y[x];
+      tm.sync();
+      right_multiply_fp64(tm, z, q, r, 1, r, mw, true);
+      for (int x = tm.tid; x < q * r; x += tm.nt) z[x] = gr[x] - z[x];
+      tm.sync();
+      right_multiply_fp64(tm, z, q, r, 1, r, e, true);
+      for (int x = tm.tid; x < q * r; x += tm.nt) y[x] += z[x];
+      tm.sync();
     }
-    for (int x = threadIdx.x; x < q * r; x += kThreads) y[x] *= rd[x % r];
-    __syncthreads();
+    for (int x = tm.tid; x < q * r; x += tm.nt) y[x] *= rd[x % r];
+    tm.sync();
     return true;
   }
+  if (tm.rank == 0) {   // (by the first CTA alone)
   if (threadIdx.x == 0) sh.flag = 1;
   for (int x = threadIdx.x; x < r; x += kThreads) mw[x + (int64_t)x * r] += 1.0;
   __syncthreads();
@@ -1135,10 +1279,8 @@ __device__ __noinline__ bool ls_solve(double* y, int q, int r, double* gr, int p
     }
     __syncthreads();
   }
-  if (!sh.flag) {
-    __syncthreads();
-    return false;
-  }
+  __syncthreads();
+  if (sh.flag)
   // each row t: x = (y_t D^-1) (L L^T)^-1 D^-1
   for (int t = threadIdx.x; t < q; t += kThreads) {
     double* yt = y + (int64_t)t * r;
@@ -1154,8 +1296,10 @@ __device__ __noinline__ bool ls_solve(double* y, int q, int r, double* gr, int p
     }
     for (int i = 0; i < r; ++i) yt[i] /= d[i];
   }
-  __syncthreads();
-  return true;
+  if (threadIdx.x == 0) tm.put(&sh.flag, sh.flag);
+  }
+  tm.sync();
+  return sh.flag != 0;
 }
 
 // Mixed-precision one-sided Jacobi SVD of the p x q (p >= q) matrix A given by `a`.  FP64 runs
@@ -1194,31 +1338,30 @@ __device__ __noinline__ bool ls_solve(double* y, int q, int r, double* gr, int p
 // non-orthogonality of G32's columns: pairs within 4 u32 sqrt(p) of orthogonal or below the FP32
 // noise floor).  So tail(A) >= tail(c) - sqrt(q - dense_h) delta, and when that exceeds eps the
 // later stages could only confirm "dense": they are skipped and the function returns 1.
-__device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g, double* v,
+template <class TM>
+__device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int q, double* g, double* v,
                                       double* sc, int max_sweeps, double eps, int dense_h,
                                       double fro, bool lower, SvdShared& sh,
                                       unsigned long long* jstats,
                                       unsigned long long* stage_clk = nullptr) {
+  extern __shared__ __align__(16) float svd_smem[];
   // while profiling the full-SVD path: SM cycles per stage (1..5 of kFullStageCounters)
   long long ck = stage_clk ? clock64() : 0;
   auto mark = [&](int stage) {
-    if (stage_clk && threadIdx.x == 0) {
+    if (stage_clk && tm.tid == 0) {
       const long long now = clock64();
       atomicAdd(&stage_clk[stage], (unsigned long long)(now - ck));
       ck = now;
     }
   };
-  const Work32 wk = work32(p, q, sc);
+  Work32 wk = work32(p, q, sc);
+  const bool tri32 = lower && use_qr32(p, q);
+  if (tri32) wk.g = svd_smem;
   constexpr int64_t kSq = (int64_t)CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
   double* v2 = sc + kSq;       // after p q + q^2 floats
   double* e = sc + 4 * kSq;    // the orthonormalisations' E, and their FP32 powers
   float* f = series_f32(q, sc);
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
-    const int i = e % wk.ldg;
-    wk.g[e] = i < p ? (float)a.at(i, e / wk.ldg) : 0.f;
-  }
-  __syncthreads();
   // The FP64 noise floor, raised to 1e-3 eps: columns below it hold less than 1e-6 eps^2 each, so
   // their mutual (non-)orthogonality cannot move a truncation decision at eps except within a
   // hair of the threshold, while orthogonalising them costs most of the sweeps
@@ -1226,9 +1369,19 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
   const float floor_g = (float)floor64;
   const float tol32 = 4.f * FLT_EPSILON * sqrtf((float)p);
   const float floor32 = lower ? floor_g : (float)((double)p * FLT_EPSILON * fro);
-  const int sw32 = run_jacobi32(wk, p, q, max_sweeps, tol32, floor32 * floor32, sh.jac);
+  // (the FP32 stages are the first CTA's)
+  int sw32 = 0;
+  if (tm.rank == 0) {
+    for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
+      const int i = e % wk.ldg;
+      wk.g[e] = i < p ? (float)a.at(i, e / wk.ldg) : 0.f;
+    }
+    __syncthreads();
+    if (tri32) qr32(wk, p, q, sc);
+    sw32 = run_jacobi32(wk, q, max_sweeps, tol32, floor32 * floor32, sh.jac);
+  }
   mark(1);
-  if (dense_h >= 0 && dense_h < q) {
+  if (dense_h >= 0 && dense_h < q) {   // (full SVDs: a team of one)
     for (int c = w; c < q; c += kWarps) {
       const float* gc = wk.g + c * wk.ldg;
       double s2 = 0.0;
@@ -1251,7 +1404,7 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
     const double delta = 2.0 * FLT_EPSILON * fro *
                          (4.0 * q * sqrt((double)p) + p * sqrt((double)q) + 2.0 * sw32 * q + 1.0);
     if (tail - sqrt((double)(q - dense_h)) * delta > eps) {
-      if (jstats && threadIdx.x == 0) {
+      if (jstats && tm.tid == 0) {
         atomicAdd(&jstats[0], 1ull);
         atomicAdd(&jstats[1], (unsigned long long)sw32);
         atomicAdd(&jstats[3], 1ull);
@@ -1260,16 +1413,22 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
       return 1;
     }
   }
-  orthonormalise_fp64(wk.v, wk.ldv, v, q, e, f, sh);
-  project_fp64(a, p, q, v, g, lower);
+  orthonormalise_fp64(tm, wk.v, wk.ldv, v, q, e, f, sh);
+  project_fp64(tm, a, p, q, v, g, lower);
   mark(2);
-  for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
-    const int i = e % wk.ldg;
-    wk.g[e] = i < p ? (float)g[i + (int64_t)(e / wk.ldg) * p] : 0.f;
+  wk = work32(p, q, sc);
+  if (tm.rank == 0) {
+    for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
+      const int i = e % wk.ldg;
+      wk.g[e] = i < p ? (float)g[i + (int64_t)(e / wk.ldg) * p] : 0.f;
+    }
+    __syncthreads();
+    const int sw = run_jacobi32(wk, q, max_sweeps, lower ? 16.f * tol32 : tol32,
+                                floor_g * floor_g, sh.jac);
+    if (threadIdx.x == 0) tm.put(&sh.sweeps, sw);
   }
-  __syncthreads();
-  const int sw32b = run_jacobi32(wk, p, q, max_sweeps, lower ? 16.f * tol32 : tol32,
-                                 floor_g * floor_g, sh.jac);
+  tm.sync();
+  const int sw32b = sh.sweeps;
   mark(3);
   // When eps is well above the noise floor the right factor of the kept columns is recovered
   // from A and G afterwards (recover_right).  Near the floor (eps < 1e3 p u ||A||_F) kept
@@ -1277,9 +1436,9 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
   // accumulated instead.
   const bool track_v = floor64 > 1e-3 * eps;
   if (sw32b > 0) {
-    orthonormalise_fp64(wk.v, wk.ldv, v2, q, e, f, sh);
-    right_multiply_fp64(g, p, 1, p, q, v2, false);
-    if (track_v) right_multiply_fp64(v, q, q, 1, q, v2, false);
+    orthonormalise_fp64(tm, wk.v, wk.ldv, v2, q, e, f, sh);
+    right_multiply_fp64(tm, g, p, 1, p, q, v2, false);
+    if (track_v) right_multiply_fp64(tm, v, q, q, 1, q, v2, false);
   }
   if (threadIdx.x == 0) sh.v_tracked = track_v ? 1 : 0;
   mark(4);
@@ -1293,7 +1452,7 @@ __device__ __noinline__ int svd_mixed(const SrcView& a, int p, int q, double* g,
   // (FP64 sweeps to convergence where V is accumulated, the earlier choice, took 3.6 of 12.5 G
   // cycles of the lattice product's recompression at N = 4096.)
   if (threadIdx.x == 0) sh.ls_recover = track_v ? 0 : 1;
-  if (jstats && threadIdx.x == 0) {
+  if (jstats && tm.tid == 0) {
     // algorithmic flops: Jacobi 4 p q^2 per sweep, orthonormalisation 3 q^3, products 2 p q^2
     const unsigned long long pq2 = (unsigned long long)p * q * q, q3 = (unsigned long long)q * q * q;
     unsigned long long f64 = 2 * q3 + 2 * pq2;
@@ -1331,6 +1490,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int n_items = *count;
   const bool pair = 2 * n_items <= (int)gridDim.x;
   const int rank = (int)cluster.block_rank();
+  const One solo;   // the core is each CTA's own
   const bool lead = !pair || rank == 0;   // writes what a tile has once
   int it = pair ? (int)(blockIdx.x / 2) : next_item(sched, &sh_next);
   while (it < n_items) {
@@ -1372,7 +1532,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       for (int e = threadIdx.x; e < R * R; e += kThreads) part = fma(M[e], M[e], part);
       const double mfro = sqrt(block_sum(part, sh.red));
       SrcView mv{M, 1, R, false};
-      svd_mixed(mv, R, R, G, V, sc, max_sweeps, eps, -1, mfro, false, sh, js);
+      svd_mixed(solo, mv, R, R, G, V, sc, max_sweeps, eps, -1, mfro, false, sh, js);
     }
     sort_and_truncate(G, R, R, R, eps, sh);
     const int r = sh.rank;
@@ -1381,9 +1541,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     if (!tracked) {
       // V_r S_r^2 = M^T G_r into V (M is still intact), or the least-squares V_r
       SrcView mv{M, 1, R, false};
-      recover_right(mv, R, R, G, sh.perm, r, V, sc, false);
+      recover_right(solo, mv, R, R, G, sh.perm, r, V, sc, false);
       if (ls)
-        ls = ls_solve(V, R, r, sc, R, sh.sorted, sc + 4 * kSq, sc + kSq, sc + 3 * kSq,
+        ls = ls_solve(solo, V, R, r, sc, R, sh.sorted, sc + 4 * kSq, sc + kSq, sc + 3 * kSq,
                       series_f32(r, sc), sh);
     }
     double* Xo = C.pool + sC;
@@ -1601,16 +1761,16 @@ __device__ int rrqr_block(const double* S, int64_t s_r, int64_t s_c, int m, int 
 // (c + 1) x (c + 1) triangle, so R_K'^-1 is the leading block of R_K^-1 and its squared
 // Frobenius norm a prefix sum of column norms.  Returns the largest of the K - h bounds
 // (h = K - 1: 1 / ||R_K^-1||_F^2 <= sigma_min(R_K)^2).
-__device__ __noinline__ double tail_lower_bound_sq(const double* g, int p, int h, int K,
-                                                   SvdShared& sh) {
+template <class TM>
+__device__ __noinline__ double tail_lower_bound_sq(const TM& tm, const double* g, int p, int h,
+                                                   int K, SvdShared& sh) {
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int i = threadIdx.x; i < K; i += kThreads)
-    sh.sigma_inv[i] = 1.0 / g[i + (int64_t)sh.qr_perm[i] * p];
+  for (int i = threadIdx.x; i < K; i += kThreads) sh.sigma_inv[i] = 1.0 / sh.qr_diag[i];
   __syncthreads();
   // column c by columns of R from the last: x_i is final when its turn comes and is subtracted
   // from the rows above it, so no step needs a reduction (with an inner product and a division
   // per entry this test took half of a certified tile's time)
-  for (int c = w; c < K; c += kWarps) {
+  for (int c = tm.w; c < K; c += tm.nw) {
     double x[kRowsPerLane];
 #pragma unroll
     for (int t = 0; t < kRowsPerLane; ++t) x[t] = l + 32 * t == c ? 1.0 : 0.0;
@@ -1634,9 +1794,9 @@ __device__ __noinline__ double tail_lower_bound_sq(const double* g, int p, int h
     for (int t = 0; t < kRowsPerLane; ++t)
       if (32 * t <= c) s2 = fma(x[t], x[t], s2);
     s2 = warp_sum(s2);
-    if (l == 0) sh.sorted[c] = s2;
+    if (l == 0) tm.put(&sh.sorted[c], s2);
   }
-  __syncthreads();
+  tm.sync();
   if (w == 0) {
     // the prefix sums f_c, until a zero pivot makes them useless, and the best bound
     const int ch = (K + 31) / 32, lo = l * ch, hi = min(K, lo + ch);
@@ -1666,8 +1826,9 @@ __device__ __noinline__ double tail_lower_bound_sq(const double* g, int p, int h
 }
 
 // (not inlined: the kernel's register allocation stays with its own paths)
-__device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int q, bool tr,
-                                                   int m, int n, double eps, int max_sweeps,
+template <class TM>
+__device__ __noinline__ int compress_by_pivoted_qr(const TM& tm, const SrcView& a, int p, int q,
+                                                   bool tr, int m, int n, double eps, int max_sweeps,
                                                    double* g, double* wv, double* sc,
                                                    double* slot, int* kind_out, int* rank_out,
                                                    double* norm_out, SvdShared& sh,
@@ -1687,7 +1848,7 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
   const int jtail = (3 * q) / 5 > jcert ? (3 * q) / 5 : jcert;
   const double tau2 = (eps / 16.0) * (eps / 16.0);
   // copy with the column norms
-  for (int c = w; c < q; c += kWarps) {
+  for (int c = tm.w; c < q; c += tm.nw) {
     double* gc = g + (int64_t)c * p;
     double s2 = 0.0;
     for (int i = l; i < p; i += 32) {
@@ -1697,13 +1858,13 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     }
     s2 = warp_sum(s2);
     if (l == 0) {
-      sh.sigma[c] = s2;
-      sh.qr_nref[c] = s2;
-      sh.qr_perm[c] = c;
+      tm.put(&sh.qr_nu[0][c], s2);
+      tm.put(&sh.qr_nref[0][c], s2);
     }
   }
+  for (int c = threadIdx.x; c < q; c += kThreads) sh.qr_perm[c] = c;
   if (threadIdx.x == 0) sh.qr_recomputed = 0;
-  __syncthreads();
+  tm.sync();
   unsigned long long fma_count = 0;
   bool exact = true;   // the trailing norms were all summed exactly at this step
   int k = -1;
@@ -1711,11 +1872,15 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     // pivot (warp 0): the largest trailing norm, first maximum (norms >= 0: compared as
     // integers); their sum only when the largest could let it meet the threshold.  Columns are
     // exchanged in the order qr_perm, not moved.
+    // (two buffers of the norms, by step: a CTA of the team that is ahead writes the next step's
+    // into every copy while another still chooses its pivot)
+    double* nu = sh.qr_nu[j & 1];
+    double* nref = sh.qr_nref[j & 1];
     if (w == 0) {
       unsigned long long best = 0;
       int arg = j;
       for (int c = j + l; c < q; c += 32) {
-        const unsigned long long v = (unsigned long long)__double_as_longlong(sh.sigma[c]);
+        const unsigned long long v = (unsigned long long)__double_as_longlong(nu[c]);
         if (v > best) { best = v; arg = c; }
       }
 #pragma unroll
@@ -1727,18 +1892,18 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
       double tot = __longlong_as_double((long long)best);
       if (tot <= tau2) {
         tot = 0.0;
-        for (int c = j + l; c < q; c += 32) tot += sh.sigma[c];
+        for (int c = j + l; c < q; c += 32) tot += nu[c];
         tot = warp_sum(tot);
       }
       if (l == 0) {
         sh.kept_sq = tot;
         if (!(tot <= tau2) && arg != j) {
-          const double t = sh.sigma[j];
-          sh.sigma[j] = sh.sigma[arg];
-          sh.sigma[arg] = t;
-          const double tr = sh.qr_nref[j];
-          sh.qr_nref[j] = sh.qr_nref[arg];
-          sh.qr_nref[arg] = tr;
+          const double t = nu[j];
+          nu[j] = nu[arg];
+          nu[arg] = t;
+          const double tr = nref[j];
+          nref[j] = nref[arg];
+          nref[arg] = tr;
           const int ti = sh.qr_perm[j];
           sh.qr_perm[j] = sh.qr_perm[arg];
           sh.qr_perm[arg] = ti;
@@ -1747,9 +1912,10 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     }
     __syncthreads();
     if (sh.kept_sq <= tau2 && !exact) {
+      tm.sync();   // (every CTA has chosen)
       // the downdated norms meet the threshold: sum the trailing norms exactly and decide (and
       // pivot) on those
-      for (int c0 = j + kQuad * w; c0 < q; c0 += kQuad * kWarps) {
+      for (int c0 = j + kQuad * tm.w; c0 < q; c0 += kQuad * tm.nw) {
         double s2[kQuad];
 #pragma unroll
         for (int c = 0; c < kQuad; ++c) {
@@ -1761,13 +1927,13 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
         }
         const double d = warp_sum4(s2);
         if (l % 8 == 0 && c0 + l / 8 < q) {
-          sh.sigma[c0 + l / 8] = d;
-          sh.qr_nref[c0 + l / 8] = d;
+          tm.put(&nu[c0 + l / 8], d);
+          tm.put(&nref[c0 + l / 8], d);
         }
       }
       fma_count += (unsigned long long)(p - j) * (unsigned long long)(q - j);
       exact = true;
-      __syncthreads();
+      tm.sync();
       --j;   // the same step again
       continue;
     }
@@ -1777,8 +1943,8 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     }
     if (j == jcert) {
       // still above the threshold after floor(q/2) + 1 steps: dense if sigma_min(R_11) > eps
-      const double b2 = tail_lower_bound_sq(g, p, jcert - 1, jcert, sh);
-      if (jstats && threadIdx.x == 0)
+      const double b2 = tail_lower_bound_sq(tm, g, p, jcert - 1, jcert, sh);
+      if (jstats && tm.tid == 0)
         atomicAdd(&jstats[4], 2ull * fma_count + (unsigned long long)jcert * jcert * jcert / 3);
       fma_count = 0;
       if (b2 > eps * eps) return 2;
@@ -1794,71 +1960,77 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     const int n = p - j - 1, ncol = q - j - 1;
     auto col = [&](int c) { return g + (int64_t)sh.qr_perm[j + 1 + c] * p + j + 1; };
     const double* x = cj + j + 1;
+    // Groups of eight columns, or in a team of four where that still leaves no warp more than one
+    // (shorter, though more of the pipe in all); each CTA's first warp forms the reflector (all alike), so the first groups go to the others.
+    const int gc = tm.size > 1 && ncol <= 4 * (kWarps - 1) * tm.size ? 4 : kGroup;
+    const int first = (kWarps - 1) * tm.size;   // groups taken before the scalars are known
+    auto end = [&](int c0) { return c0 + gc < ncol ? c0 + gc : ncol; };
     double d = 0.0;
     if (w == 0) {
       double v0, rn, rv;
       const double beta = make_reflector(x, n, cj[j], &v0, &rn, &rv);
       __syncwarp();
       if (l == 0) {
-        cj[j] = beta;
+        sh.qr_diag[j] = beta;
         sh.refl.v0[j] = v0;
         sh.refl.rn[j] = rn;
         sh.refl.rv[j] = rv;
       }
-    } else if (kGroup * (w - 1) < ncol) {
-      d = group_dot(x, n, kGroup * (w - 1), ncol, col);
+    } else if (gc * (tm.w - tm.size) < ncol) {
+      const int c0 = gc * (tm.w - tm.size);
+      d = group_dot(x, n, c0, end(c0), col);
     }
     __syncthreads();
     const double v0 = sh.refl.v0[j], rn = sh.refl.rn[j], rv = sh.refl.rv[j];
-    for (int gi = w > 0 ? w - 1 : kWarps - 1; kGroup * gi < ncol;
-         gi = (gi < kWarps - 1 ? kWarps - 1 + w : gi + kWarps)) {
-      const int c0 = kGroup * gi, c = group_column(c0);
-      if (gi >= kWarps - 1) d = group_dot(x, n, c0, ncol, col);
+    for (int gi = w > 0 ? tm.w - tm.size : first + tm.w; gc * gi < ncol;
+         gi = gi < first ? first + tm.w : gi + tm.nw) {
+      const int c0 = gc * gi, c1 = end(c0);
+      const int cg = group_column(c0), c = cg < c1 ? cg : ncol;   // (ncol: no column)
+      if (gi >= first) d = group_dot(x, n, c0, c1, col);
       const double yj = c < ncol ? col(c)[-1] : 0.0;
       const double f = fma(v0, yj, d) * rn * rv;
-      group_update(x, f, n, c0, ncol, col);
+      group_update(x, f, n, c0, c1, col);
       const double yn = fma(-f, v0, yj);
-      double nu2 = 0.0;
+      double nu2 = 0.0, ref = 0.0;
       bool again = false;
       if (c < ncol) {
-        nu2 = fma(-yn, yn, sh.sigma[j + 1 + c]);
-        again = !(nu2 > kDowndateFloor * sh.qr_nref[j + 1 + c]);
+        ref = nref[j + 1 + c];
+        nu2 = fma(-yn, yn, nu[j + 1 + c]);
+        again = !(nu2 > kDowndateFloor * ref);
       }
       if (__any_sync(0xffffffffu, again)) {
-        const double s2 = group_squares(n, c0, ncol, col);
+        const double s2 = group_squares(n, c0, c1, col);
         if (again) {
-          nu2 = s2;
-          if (l % 4 == 0) {
-            sh.qr_nref[j + 1 + c] = nu2;
-            atomicAdd(&sh.qr_recomputed, (unsigned long long)n);
-          }
+          ref = nu2 = s2;
+          if (l % 4 == 0) atomicAdd(&sh.qr_recomputed, (unsigned long long)n);
         }
       }
       __syncwarp();
       if (c < ncol && l % 4 == 0) {
         col(c)[-1] = yn;
-        sh.sigma[j + 1 + c] = nu2;
+        tm.put(&sh.qr_nu[(j + 1) & 1][j + 1 + c], nu2);
+        tm.put(&sh.qr_nref[(j + 1) & 1][j + 1 + c], ref);
       }
     }
     fma_count += 2ull * (unsigned long long)(p - j) * (unsigned long long)(q - j - 1) + (p - j);
     exact = false;
-    __syncthreads();
+    tm.sync();
   }
-  if (jstats && threadIdx.x == 0)   // (the QR's flops after the certificate test)
+  if (jstats && tm.tid == 0)   // (the QR's flops after the certificate test)
     atomicAdd(&jstats[4], 2ull * (fma_count + sh.qr_recomputed));
   if (k < 0) return 0;
   if (k > jtail) {
     // dense when sum_{i > q/2} sigma_i^2 > eps^2 is certified by some leading triangle of the
     // k completed steps, else the SVD of R decides
-    const double b2 = tail_lower_bound_sq(g, p, kmax, k, sh);
-    if (jstats && threadIdx.x == 0)
+    const double b2 = tail_lower_bound_sq(tm, g, p, kmax, k, sh);
+    if (jstats && tm.tid == 0)
       atomicAdd(&jstats[4], (unsigned long long)k * k * k / 3);
     if (b2 > eps * eps) return 2;
   }
   const double trail2 = sh.kept_sq;
   __syncthreads();
   if (k == 0) {
-    if (threadIdx.x == 0) { *kind_out = CLR_KIND_ZERO; *rank_out = 0; *norm_out = 0.0; }
+    if (tm.tid == 0) { *kind_out = CLR_KIND_ZERO; *rank_out = 0; *norm_out = 0.0; }
     __syncthreads();
     return 1;
   }
@@ -1869,31 +2041,33 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
   double* gs = wv;             // q x k
   double* vs = sc + 2 * kSq;   // k x k
   double part = 0.0;
-  for (int e = threadIdx.x; e < k * q; e += kThreads) {
+  for (int e = tm.tid; e < k * q; e += tm.nt) {
     const int i = e % k, c = e / k;
-    const double x = i <= c ? g[i + (int64_t)sh.qr_perm[c] * p] : 0.0;
-    rb[c + (int64_t)i * q] = x;
-    part = fma(x, x, part);
+    rb[c + (int64_t)i * q] = i < c    ? g[i + (int64_t)sh.qr_perm[c] * p]
+                             : i == c ? sh.qr_diag[i]
+                                      : 0.0;
   }
+  tm.sync();
+  for (int e = threadIdx.x; e < k * q; e += kThreads) part = fma(rb[e], rb[e], part);
   const double rfro = sqrt(block_sum(part, sh.red));
   const double budget = sqrt(fmax(eps * eps - trail2, 0.0));
   const SrcView mv{rb, 1, q, false};
   unsigned long long* stage_clk = jstats ? jstats + kPreStageCounters : nullptr;
-  if (stage_clk && threadIdx.x == 0)
+  if (stage_clk && tm.tid == 0)
     atomicAdd(&stage_clk[0], (unsigned long long)(clock64() - c_entry));
-  svd_mixed(mv, q, k, gs, vs, sc, max_sweeps, budget, -1, rfro, true, sh, jstats, stage_clk);
+  svd_mixed(tm, mv, q, k, gs, vs, sc, max_sweeps, budget, -1, rfro, true, sh, jstats, stage_clk);
   const long long c_after = clock64();
   sort_and_truncate(gs, q, k, q, budget, sh);
   const int r = sh.rank;
   if (r == 0) {
-    if (threadIdx.x == 0) { *kind_out = CLR_KIND_ZERO; *rank_out = 0; *norm_out = 0.0; }
+    if (tm.tid == 0) { *kind_out = CLR_KIND_ZERO; *rank_out = 0; *norm_out = 0.0; }
     __syncthreads();
     return 1;
   }
   if (r > kmax) {
     // stored dense: the source is untouched (R lives in the scratch), so the block is kept
     // exactly (the caller copies an external source into the slot)
-    if (jstats && threadIdx.x == 0) {
+    if (jstats && tm.tid == 0) {
       atomicAdd(&stage_clk[6], (unsigned long long)(clock64() - c_after));
       atomicAdd(&stage_clk[7], 1ull);
     }
@@ -1902,16 +2076,16 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
   }
   const bool tracked = sh.v_tracked;
   bool ls = !tracked && sh.ls_recover;
-  if (!tracked) recover_right(mv, q, k, gs, sh.perm, r, vs, sc, true);   // Y = R G_r (k x r)
+  if (!tracked) recover_right(tm, mv, q, k, gs, sh.perm, r, vs, sc, true);   // Y = R G_r (k x r)
   // (R is no longer needed: its place is work space)
   if (ls)
-    ls = ls_solve(vs, k, r, sc, q, sh.sorted, sc + 4 * kSq, sc + kSq, rb, series_f32(r, sc), sh);
+    ls = ls_solve(tm, vs, k, r, sc, q, sh.sorted, sc + 4 * kSq, sc + kSq, rb, series_f32(r, sc), sh);
   // R = V_M S U_M^T:  X_R = (V_M S)_r (k x r), W_R = (U_M)_r (q x r); A ~ (Q_k X_R) (P W_R)^T
   // (the source in the slot is no longer read: the factors overwrite it)
-  __syncthreads();
+  tm.sync();
   double* xa = tr ? slot + (int64_t)m * r : slot;   // Q_k X_R: p x r, ld p
   double* wa = tr ? slot : slot + (int64_t)m * r;   // P W_R: q x r, ld q
-  for (int e = threadIdx.x; e < p * r; e += kThreads) {
+  for (int e = tm.tid; e < p * r; e += tm.nt) {
     const int i = e % p, c = e / p;
     double v = 0.0;
     if (i < k)
@@ -1920,7 +2094,7 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
                   : vs[(int64_t)i * r + c] / sh.sorted[c];
     xa[e] = v;
   }
-  for (int e = threadIdx.x; e < q * r; e += kThreads) {
+  for (int e = tm.tid; e < q * r; e += tm.nt) {
     const int j = e % q, c = e / q;
     const double v = gs[j + (int64_t)sh.perm[c] * q];
     wa[sh.qr_perm[j] + (int64_t)c * q] = ls ? v : v / sh.sorted[c];
@@ -1932,12 +2106,13 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
     double* st = reinterpret_cast<double*>(svd_smem);
     for (int c = w; c < k; c += kWarps)
       for (int i = c + 1 + l; i < p; i += 32) st[i + c * p] = g[i + (int64_t)sh.qr_perm[c] * p];
-    __syncthreads();
-    apply_q(st, p, k, sh.refl, nullptr, xa, r, p, w, kWarps);
+    tm.sync();   // (and the factors' entries)
+    apply_q(st, p, k, sh.refl, nullptr, xa, r, p, tm.w, tm.nw);
   } else {
-    apply_q(g, p, k, sh.refl, sh.qr_perm, xa, r, p, w, kWarps);
+    tm.sync();
+    apply_q(g, p, k, sh.refl, sh.qr_perm, xa, r, p, tm.w, tm.nw);
   }
-  if (threadIdx.x == 0) {
+  if (tm.tid == 0) {
     *kind_out = CLR_KIND_LR;
     *rank_out = r;
     *norm_out = sqrt(sh.kept_sq);
@@ -1955,27 +2130,54 @@ __device__ __noinline__ int compress_by_pivoted_qr(const SrcView& a, int p, int 
 // ---------------------------------------------------------------------------------------------
 // Dense truncated SVD of whole blocks (ROUTE_DACC tiles, recompressed dense tiles, building a
 // CLR matrix from a dense one).
+//
+// A tile is FP64-pipe-bound for 5 to 20 ms of one SM at 256 x 256, so with few tiles the launch
+// takes what its largest tile takes while most SMs idle.  With few tiles the CTAs come in clusters of
+// four, and while the tiles are at most half the CTAs a cluster works on one tile as a team (the
+// columns of the QR, the rows and blocks of the products; the FP32 sweeps stay with one CTA), else
+// each CTA takes its own.  A team takes a 256 x 240 tile in 9.8 M SM cycles, one CTA in 21, so that
+// half of its SMs' time is lost: with 144 tiles on 152 SMs (Coulomb-like lattice at N = 2048) teams
+// took 6.2 ms against 5.8, with 64 (gradient of the 1D chain at N = 1024) 3.6 against 5.1.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads, 1) compress_dense_kernel(
+constexpr int kTeamCtas = 4;
+
+template <bool kTeams>
+__device__ __forceinline__ void compress_dense_body(
     MatView C, const int* list, const int* count, const int* order, const double* src,
     int64_t lds, double* ws, double* svd_scratch, double eps, double drop_norm,
     int dense_only, int rrqr, int prereduce, int max_sweeps, int* err, int* sched,
     unsigned long long* jstats) {
   __shared__ SvdShared sh;
-  __shared__ int sh_next;
-  double* sc = svd_scratch + (int64_t)blockIdx.x * kSvdScratchPerCta;
+  __shared__ int sh_next[2];
   const int n_items = list ? *count : C.nr * C.nc;
+  const int cta = kTeams ? (int)cooperative_groups::this_cluster().block_rank() : 0;
+  const bool team = kTeams && 2 * n_items <= (int)gridDim.x;
+  auto make = [&]() {
+    if constexpr (kTeams) return Team(team ? cta : 0, team ? kTeamCtas : 1);
+    else return One();
+  };
+  const auto tm = make();
+  double* sc = svd_scratch + (int64_t)(blockIdx.x - tm.rank) * kSvdScratchPerCta;
+  int next_slot = 0;
+  auto next = [&]() {
+    if (!team) return next_item(sched, &sh_next[0]);
+    // (two slots: one is read while the other is written)
+    if (tm.tid == 0) tm.put(&sh_next[next_slot], atomicAdd(sched, 1));
+    tm.sync();
+    next_slot ^= 1;
+    return sh_next[next_slot ^ 1];
+  };
   // each tile's SM kilocycles go to C.cost (the next plan's scheduling cost), written when the
   // CTA takes its next tile (every path of the loop body ends there) and after the last one
   int prev_t = -1;
   long long prev_c = 0;
   auto record_cost = [&](long long now) {
-    if (C.cost && prev_t >= 0 && threadIdx.x == 0) {
+    if (C.cost && prev_t >= 0 && tm.tid == 0) {
       const long long kc = (now - prev_c) >> 10;
       C.cost[prev_t] = (unsigned int)(kc < 1 ? 1 : kc > 0xFFFFFFFFll ? 0xFFFFFFFFll : kc);
     }
   };
-  for (int it = next_item(sched, &sh_next); it < n_items; it = next_item(sched, &sh_next)) {
+  for (int it = next(); it < n_items; it = next()) {
     const int t = list ? list[it] : (order ? order[it] : it);
     const long long now = clock64();
     record_cost(now);
@@ -2002,17 +2204,19 @@ __global__ void __launch_bounds__(kThreads, 1) compress_dense_kernel(
     }
     const double nsq = block_sum(part, sh.red);
     if (!isfinite(nsq)) {
-      if (threadIdx.x == 0) atomicCAS(err, 0, 3);  // a timeout (1) keeps precedence
+      if (tm.tid == 0) atomicCAS(err, 0, 3);  // a timeout (1) keeps precedence
     }
     const double nrm = sqrt(nsq);
     int kind;
     if (!(nrm >= drop_norm) || nsq == 0.0 || !isfinite(nsq)) {
       kind = CLR_KIND_ZERO;
-      if (threadIdx.x == 0) { C.kind[t] = kind; C.rank[t] = 0; C.norm[t] = 0.0; }
+      if (tm.tid == 0) { C.kind[t] = kind; C.rank[t] = 0; C.norm[t] = 0.0; }
       __syncthreads();
       continue;
     }
+    const One solo;
     int r = q;
+    bool alone = false;      // a full SVD in a team: the rest is the first CTA's
     long long c_full = -1;   // while profiling: start of a full-SVD block's truncation
     if (rrqr && !dense_only) {
       r = rrqr_block(S, s_r, s_c, m, n, eps, G, sh);
@@ -2045,28 +2249,31 @@ __global__ void __launch_bounds__(kThreads, 1) compress_dense_kernel(
       const long long c0 = clock64();
       // pivoted QR first: blocks of low numerical rank are truncated through the SVD of
       // the k x q factor, blocks of rank above q/2 certified dense
-      const int pre = prereduce ? compress_by_pivoted_qr(view, p, q, tr, m, n, eps, max_sweeps,
+      const int pre = prereduce ? compress_by_pivoted_qr(tm, view, p, q, tr, m, n, eps, max_sweeps,
                                                          G, V, sc, slot, &C.kind[t], &C.rank[t],
                                                          &C.norm[t], sh, jstats)
                                 : 0;
+      // (the full SVD is one CTA's)
+      if (pre == 0 && tm.rank != 0) continue;
+      alone = pre == 0;
       if (pre == 0) {
         unsigned long long* stage_clk = jstats ? jstats + kFullStageCounters : nullptr;
         if (stage_clk && threadIdx.x == 0)
           atomicAdd(&stage_clk[0], (unsigned long long)(clock64() - c0));
-        const int early_dense = svd_mixed(view, p, q, G, V, sc, max_sweeps, eps, q / 2, nrm,
+        const int early_dense = svd_mixed(solo, view, p, q, G, V, sc, max_sweeps, eps, q / 2, nrm,
                                           false, sh, jstats, stage_clk);
         if (!early_dense) {
           c_full = clock64();
           sort_and_truncate(G, p, q, p, eps, sh);
           r = sh.rank;
         }
-      } else if (pre >= 2 && jstats && threadIdx.x == 0) {
+      } else if (pre >= 2 && jstats && tm.tid == 0) {
         atomicAdd(&jstats[3], 1ull);   // stored dense without a full SVD
       }
       // SM cycles per path while profiling (block 2 of the counters): QR and the SVD of R
       // stored low rank, certified dense by the QR's triangles, full SVD (prereduce off, or a
       // non-finite QR norm), QR and the SVD of R stored dense
-      if (jstats && threadIdx.x == 0) {
+      if (jstats && tm.tid == 0) {
         const int path = pre == 1 ? 0 : pre == 2 ? 1 : pre == 3 ? 3 : 2;
         atomicAdd(&jstats[kPathCounters + 2 * path], (unsigned long long)(clock64() - c0));
         atomicAdd(&jstats[kPathCounters + 2 * path + 1], 1ull);
@@ -2075,15 +2282,15 @@ __global__ void __launch_bounds__(kThreads, 1) compress_dense_kernel(
     }
     const int lim = q / 2;
     if (r == 0) {
-      if (threadIdx.x == 0) { C.kind[t] = CLR_KIND_ZERO; C.rank[t] = 0; C.norm[t] = 0.0; }
+      if (tm.tid == 0) { C.kind[t] = CLR_KIND_ZERO; C.rank[t] = 0; C.norm[t] = 0.0; }
     } else if (dense_only || r > lim) {
       if (src) {
-        for (int e = threadIdx.x; e < m * n; e += kThreads) {
+        for (int e = alone ? threadIdx.x : tm.tid; e < m * n; e += alone ? kThreads : tm.nt) {
           const int i = e % m, j = e / m;
           slot[e] = S[i * s_r + j * s_c];
         }
       }
-      if (threadIdx.x == 0) { C.kind[t] = CLR_KIND_DENSE; C.rank[t] = q; C.norm[t] = nrm; }
+      if (tm.tid == 0) { C.kind[t] = CLR_KIND_DENSE; C.rank[t] = q; C.norm[t] = nrm; }
     } else {
       // Y = A^T G_r (q x r) into V before the slot (possibly the source) is overwritten, or
       // Y = V_r S_r^2 from the accumulated V
@@ -2091,9 +2298,9 @@ __global__ void __launch_bounds__(kThreads, 1) compress_dense_kernel(
       const bool tracked = sh.v_tracked;
       bool ls = !tracked && sh.ls_recover;
       constexpr int64_t kSq = (int64_t)CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
-      if (!tracked) recover_right(view, p, q, G, sh.perm, r, V, sc, false);
+      if (!tracked) recover_right(solo, view, p, q, G, sh.perm, r, V, sc, false);
       if (ls)
-        ls = ls_solve(V, q, r, sc, p, sh.sorted, sc + 4 * kSq, sc + kSq, sc + 3 * kSq,
+        ls = ls_solve(solo, V, q, r, sc, p, sh.sorted, sc + 4 * kSq, sc + kSq, sc + 3 * kSq,
                       series_f32(r, sc), sh);
       if (jstats && threadIdx.x == 0 && !tracked)
         atomicAdd(&jstats[4], 2ull * p * q * r);
@@ -2141,16 +2348,46 @@ __global__ void __launch_bounds__(kThreads, 1) compress_dense_kernel(
   record_cost(clock64());
 }
 
+// The kernel with CTAs in clusters, which leave a few SMs of a GPC unused, and the one without for
+// launches that could not use a team.
+__global__ void __cluster_dims__(kTeamCtas, 1, 1) __launch_bounds__(kThreads, 1)
+    compress_dense_team_kernel(MatView C, const int* list, const int* count, const int* order,
+                               const double* src, int64_t lds, double* ws, double* svd_scratch,
+                               double eps, double drop_norm, int dense_only, int rrqr,
+                               int prereduce, int max_sweeps, int* err, int* sched,
+                               unsigned long long* jstats) {
+  compress_dense_body<true>(C, list, count, order, src, lds, ws, svd_scratch, eps, drop_norm, dense_only,
+                      rrqr, prereduce, max_sweeps, err, sched, jstats);
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+    compress_dense_kernel(MatView C, const int* list, const int* count, const int* order,
+                          const double* src, int64_t lds, double* ws, double* svd_scratch,
+                          double eps, double drop_norm, int dense_only, int rrqr, int prereduce,
+                          int max_sweeps, int* err, int* sched, unsigned long long* jstats) {
+  compress_dense_body<false>(C, list, count, order, src, lds, ws, svd_scratch, eps, drop_norm, dense_only,
+                      rrqr, prereduce, max_sweeps, err, sched, jstats);
+}
+
 void launch_compress_dense(const MatView& C, const int* list, const int* count,
                            const int* order, const double* src, int64_t lds, double* ws,
                            double* svd_scratch, double eps, double drop_norm,
                            int dense_only, int rrqr, int prereduce, int max_sweeps, int grid,
                            int* err, int* sched, unsigned long long* jstats, cudaStream_t st) {
-  static bool attr_done[64] = {false};
+  static bool attr_done[64] = {false}, attr_done_team[64] = {false};
   const int g = svd_launch_grid(compress_dense_kernel, grid, attr_done);
-  compress_dense_kernel<<<g, kThreads, kSvdSmemBytes, st>>>(C, list, count, order, src, lds, ws, svd_scratch,
-                                                eps, drop_norm, dense_only, rrqr, prereduce,
-                                                max_sweeps, err, sched, jstats);
+  const int gt =
+      svd_launch_grid(compress_dense_team_kernel, grid, attr_done_team) / kTeamCtas * kTeamCtas;
+  // (how many tiles a product has is the device's to know; launches with more blocks than this are
+  // rarely left with few enough for teams)
+  if (gt > 0 && prereduce && !rrqr && !dense_only && C.nr * C.nc <= 2 * gt)
+    compress_dense_team_kernel<<<gt, kThreads, kSvdSmemBytes, st>>>(
+        C, list, count, order, src, lds, ws, svd_scratch, eps, drop_norm, dense_only, rrqr,
+        prereduce, max_sweeps, err, sched, jstats);
+  else
+    compress_dense_kernel<<<g, kThreads, kSvdSmemBytes, st>>>(
+        C, list, count, order, src, lds, ws, svd_scratch, eps, drop_norm, dense_only, rrqr,
+        prereduce, max_sweeps, err, sched, jstats);
 }
 
 // ---------------------------------------------------------------------------------------------
