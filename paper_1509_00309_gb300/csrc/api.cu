@@ -404,6 +404,7 @@ int make_plan(clr_ctx_t ctx, int nI, int nJ, int nK, Plan* p) {
   p->nI = nI;
   p->nJ = nJ;
   p->nK = nK;
+  p->n_sm = ctx->n_sm;
   p->t_count = base;
   p->t_start = base + nt;
   p->t_route = base + 2 * nt;
@@ -747,7 +748,7 @@ extern "C" int clr_mat_from_dense(clr_ctx_t ctx, const double* a, int64_t lda, i
                           eps_lr, drop_norm, 0, ctx->opts.build_rrqr ? 1 : 0,
                           ctx->opts.svd_no_prereduce ? 0 : 1,
                           ctx->opts.jacobi_max_sweeps, grid_of(ctx, 2), &pc->err, &pc->sched[2],
-                          jst(ctx), s);
+                          nullptr, jst(ctx), s);
   }
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1181,7 +1182,7 @@ int multiply_into(clr_ctx_t ctx, clr_mat_t a, clr_mat_t b, clr_mat_t c, double a
                         (double*)ctx->cur->ws.p, (double*)ctx->cur->scratch.p,
                         eps_lr, 0.0, 0, 0, o.svd_no_prereduce ? 0 : 1, o.jacobi_max_sweeps,
                         lr_grid, &p.counters->err,
-                        &p.counters->sched[2], jst(ctx), s);
+                        &p.counters->sched[2], &p.counters->n_team, jst(ctx), s);
   CLR_CHECK_LAUNCH("recompression");
   prof_launches(ctx, 2);
   prof_mark(ctx, s, PH_COMPRESS);
@@ -1402,7 +1403,7 @@ extern "C" int clr_lincomb(clr_ctx_t ctx, double a, clr_mat_t x, double b, clr_m
                         (double*)ctx->cur->ws.p, (double*)ctx->cur->scratch.p,
                         o.eps_lr, 0.0, 0, 0, o.svd_no_prereduce ? 0 : 1, o.jacobi_max_sweeps,
                         grid, &p.counters->err,
-                        &p.counters->sched[2], jst(ctx), s);
+                        &p.counters->sched[2], &p.counters->n_team, jst(ctx), s);
   CLR_CHECK_LAUNCH("lincomb");
   return CLR_OK;
 }

@@ -150,6 +150,7 @@ struct PlanCounters {
   unsigned long long max_rsum;
   unsigned long long n_gemm_dacc;  // tiles routed ROUTE_DACC_G
   int n_dense, n_lr, n_qr, n_dacc, n_dcomp;
+  int n_team;     // leading tiles of l_dcomp_s that take a team of CTAs each (plan_scan)
   int sched[4];   // work counters of the tile-list kernels (next_item), zeroed with the plan
   // error flag raised by kernels (1: a bounded wait gave up, 2: triple list overflow, 3:
   // non-finite data).  Sticky: a plan clears only the fields before it, and the host reads and
@@ -161,6 +162,7 @@ constexpr size_t kPlanCountersClear = offsetof(PlanCounters, err);
 
 struct Plan {
   int nI, nJ, nK;
+  int n_sm;
   int* t_count;   // nI*nJ
   int* t_start;   // nI*nJ
   int* t_route;   // nI*nJ
@@ -236,13 +238,16 @@ void launch_compress_qr(const MatView& C, const int* list, const int* count, con
 // prereduce: reduce every block by a column-pivoted QR (stopped at eps/16) before the SVD of
 // its k x q factor R, unless the QR's triangles certify it dense; without it every block takes
 // the full SVD.
+// n_team (may be null): how many leading tiles of the list take a team of kTeamCtas CTAs each.
+constexpr int kTeamCtas = 4;
 // jstats (7 counters): SVD blocks, FP32 sweeps, FP64 sweeps, early dense exits, FP64 flops,
 // FP32 flops, pre-reduced blocks.
 void launch_compress_dense(const MatView& C, const int* list, const int* count,
                            const int* order, const double* src, int64_t lds, double* ws,
                            double* svd_scratch, double eps, double drop_norm,
                            int dense_only, int rrqr, int prereduce, int max_sweeps, int grid,
-                           int* err, int* sched, unsigned long long* jstats, cudaStream_t st);
+                           int* err, int* sched, const int* n_team, unsigned long long* jstats,
+                           cudaStream_t st);
 void launch_block_norms(const MatView& M, cudaStream_t st);
 void launch_block_norms_dense(const MatView& M, cudaStream_t st);
 void launch_scale_blocks(const MatView& M, double alpha, cudaStream_t st);

@@ -115,9 +115,9 @@ __global__ void plan_count_kernel(MatView A, MatView B, Plan p, double eps_sp,
 // contiguous chunks is enough.
 constexpr int kScanThreads = 1024;
 constexpr int kScanQ = 5;
-constexpr int kCostBuckets = 32;
+constexpr int kCostBuckets = 128;   // four an octave
 
-// log2 bucket of a tile's cost (which = 0: QR route recompression, 1: dense SVD, 2: dense x
+// Bucket (4 log2, rounded down) of a tile's cost (which = 0: QR route recompression, 1: dense SVD, 2: dense x
 // dense products, m n times the tile's number of products).  A dense recompression's cost
 // depends on the path the tile takes (dense certificate ~0.4, pivoted QR and the SVD of R
 // ~1.1 when stored low rank and ~2 when stored dense, SM cycles per m n min(m, n) on the
@@ -139,8 +139,81 @@ __device__ __forceinline__ int cost_bucket(const Plan& p, int t, int which) {
   } else {
     c = m * n * (long long)p.t_count[t];
   }
-  const int b = c > 0 ? 63 - __clzll(c) : 0;
-  return b < kCostBuckets ? b : kCostBuckets - 1;
+  if (c < 4) return 0;
+  const int b = 63 - __clzll(c);
+  const int q = 4 * b + (int)(c >> (b - 2) & 3);
+  return q < kCostBuckets ? q : kCostBuckets - 1;
+}
+
+// How many of the most expensive recompressions take a team of kTeamCtas CTAs each instead of one
+// CTA (compress_dense_team_kernel): with few tiles the launch takes what its largest tile takes
+// while most SMs idle.  A team halves a tile's time and so doubles what it costs, hence the
+// estimate max((E + E_K) / CTAs, e_0 / 2, e_K) of the launch's time for the K leading tiles, e_K
+// the cost of the next one; the cut lies at the end of a bucket, within one tile a team, and is
+// taken only for a tenth of the time or more.  By one warp; lane l holds the counts of the
+// buckets kCostBuckets - 1 - 4 l and the three below.
+__device__ __forceinline__ int team_tiles(const int (&cnt)[4], int n_ctas) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int l = threadIdx.x % 32;
+  float e[4], own = 0.f, first = 0.f;
+  int own_n = 0;
+#pragma unroll
+  for (int x = 3; x >= 0; --x) {
+    const int b = kCostBuckets - 1 - 4 * l - x;
+    e[x] = ldexpf(4.5f + (float)(b & 3), (b >> 2) - 2);   // the middle of the bucket
+    own += (float)cnt[x] * e[x];
+    own_n += cnt[x];
+    if (cnt[x]) first = e[x];
+  }
+  float sum = own;
+  int num = own_n;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const float v = __shfl_up_sync(kAll, sum, o);
+    const int u = __shfl_up_sync(kAll, num, o);
+    if (l >= o) {
+      sum += v;
+      num += u;
+    }
+  }
+  const float all = __shfl_sync(kAll, sum, 31);
+  const unsigned busy = __ballot_sync(kAll, own_n > 0);
+  if (!busy) return 0;
+  const float top = __shfl_sync(kAll, first, __ffs(busy) - 1);
+  const unsigned later = l < 31 ? busy >> (l + 1) : 0u;
+  float below = __shfl_sync(kAll, first, later ? l + __ffs(later) : l);
+  if (!later) below = 0.f;   // nothing below this lane's buckets
+  const float none = fmaxf(all / (float)n_ctas, top);
+  float best = none;
+  int cut = 0;
+  float next[4];
+#pragma unroll
+  for (int x = 3; x >= 0; --x) {
+    next[x] = below;
+    if (cnt[x]) below = e[x];
+  }
+  sum -= own;
+  num -= own_n;
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    sum += (float)cnt[x] * e[x];
+    num += cnt[x];
+    const float t = fmaxf(fmaxf((all + sum) / (float)n_ctas, 0.5f * top), next[x]);
+    if (cnt[x] && num <= n_ctas / kTeamCtas && t < best) {
+      best = t;
+      cut = num;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float t = __shfl_xor_sync(kAll, best, o);
+    const int c = __shfl_xor_sync(kAll, cut, o);
+    if (t < best || (t == best && c < cut)) {
+      best = t;
+      cut = c;
+    }
+  }
+  return best < 0.9f * none ? cut : 0;
 }
 
 __global__ void __launch_bounds__(kScanThreads) plan_scan_kernel(Plan p, int recompress_dense) {
@@ -191,13 +264,14 @@ __global__ void __launch_bounds__(kScanThreads) plan_scan_kernel(Plan p, int rec
   }
   // The recompression lists and the dense-product list again, largest cost first
   // (longest-processing-time order for the dynamically distributed kernels): a counting sort on
-  // log2 of the cost, m n min(m, n) for a dense SVD, (m + n) R^2 for a QR route, m n times the
+  // a quarter of an octave of the cost, m n min(m, n) for a dense SVD, (m + n) R^2 for a QR route, m n times the
   // number of products for dense x dense products.  The order within a bucket is immaterial:
   // every tile is processed independently.
   __syncthreads();
   const int n_qr = sh[3][kScanThreads - 1], n_dc = sh[4][kScanThreads - 1];
   const int n_de = sh[1][kScanThreads - 1];
   __shared__ int bcount[3][kCostBuckets], boff[3][kCostBuckets];
+  static_assert(3 * kCostBuckets <= kScanThreads && kCostBuckets == 4 * 32, "buckets");
   if (tid < 3 * kCostBuckets) (&bcount[0][0])[tid] = 0;
   __syncthreads();
   auto item = [&](int i, int* which) {
@@ -211,11 +285,26 @@ __global__ void __launch_bounds__(kScanThreads) plan_scan_kernel(Plan p, int rec
     atomicAdd(&bcount[which][cost_bucket(p, t, which)], 1);
   }
   __syncthreads();
-  if (tid < 3) {
-    int acc = 0;
-    for (int b = kCostBuckets - 1; b >= 0; --b) {
-      boff[tid][b] = acc;
-      acc += bcount[tid][b];
+  if (tid < 3 * 32) {
+    const int which = tid / 32, l = tid % 32;
+    int cnt[4], own = 0;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) own += cnt[x] = bcount[which][kCostBuckets - 1 - 4 * l - x];
+    int incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (l >= o) incl += v;
+    }
+    int acc = incl - own;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      boff[which][kCostBuckets - 1 - 4 * l - x] = acc;
+      acc += cnt[x];
+    }
+    if (which == 1) {
+      const int k = n_dc > 0 ? team_tiles(cnt, p.n_sm / kTeamCtas * kTeamCtas) : 0;
+      if (l == 0) p.counters->n_team = k;
     }
   }
   __syncthreads();

@@ -21,6 +21,7 @@
 
 #include <cfloat>
 #include <mutex>
+#include <type_traits>
 
 #include "clr_internal.h"
 
@@ -638,9 +639,13 @@ struct JacobiShared {
 // global scratch, a warp per pair and 8 masked rows a lane.
 // kShared: both copies in shared memory, g and v given as offsets into it (addressed as such: a
 // generic pointer's loads are slower).
-template <int LP, int kVec, bool kShared>
-__device__ __noinline__ int jacobi32(float* g_ptr, int q, int ldg, float* v_ptr, int ldv,
-                                     int max_sweeps, float tol, float floor2,
+// Copies that do not fit there (more than ~156 columns) make a sweep bound by what one SM can move
+// to and from L2 (8 KB a pair: 23k SM cycles a round of 119 pairs), so a team takes such a sweep
+// together: the pairs dealt over its warps, the norms and marks in every CTA's copy, a cluster
+// barrier a round.  The rotations are the same ones in the same order.
+template <int LP, int kVec, bool kShared, class TM>
+__device__ __noinline__ int jacobi32(const TM& tm, float* g_ptr, int q, int ldg, float* v_ptr,
+                                     int ldv, int max_sweeps, float tol, float floor2,
                                      JacobiShared& sh) {
   extern __shared__ __align__(16) float svd_smem[];
   float* const g = kShared ? svd_smem + (int)(g_ptr - svd_smem) : g_ptr;
@@ -648,17 +653,20 @@ __device__ __noinline__ int jacobi32(float* g_ptr, int q, int ldg, float* v_ptr,
   float2* nrm = sh.nrm;
   int* last_rot = sh.last_rot;
   constexpr unsigned kAll = 0xffffffffu;
-  const int w = threadIdx.x / 32, li = threadIdx.x % LP, grp = threadIdx.x / LP;
+  const int w = threadIdx.x / 32, li = threadIdx.x % LP;
   const int qq = q + (q & 1), half = qq / 2;   // slot q is a dummy when q is odd
   const int n_act = min(kWarps, (half * LP + 31) / 32);   // warps with pairs
-  const int ngrp = n_act * (32 / LP);
+  const int grp = tm.w * (32 / LP) + (threadIdx.x % 32) / LP;
+  const int ngrp = n_act * (32 / LP) * tm.size;
   const int p2 = ldg / 2, q2 = ldv / 2;        // packed rows
-  for (int e = threadIdx.x; e < ldv * q; e += kThreads) v[e] = e % ldv == e / ldv ? 1.f : 0.f;
+  for (int e = tm.tid; e < ldv * q; e += tm.nt) v[e] = e % ldv == e / ldv ? 1.f : 0.f;
   for (int c = threadIdx.x; c < q; c += kThreads) last_rot[c] = -1;
-  __syncthreads();
+  tm.sync();
   if (w < n_act) {
     auto act_sync = [&]() {
-      if (n_act == 1) __syncwarp(); else group_sync(3, 32 * n_act);
+      if (tm.size > 1) tm.sync();   // (all warps have pairs then)
+      else if (n_act == 1) __syncwarp();
+      else group_sync(3, 32 * n_act);
     };
     auto sum_lp = [&](float x) {
 #pragma unroll
@@ -679,7 +687,7 @@ __device__ __noinline__ int jacobi32(float* g_ptr, int q, int ldg, float* v_ptr,
           }
         }
         const float s = sum_lp(sum2(s2));
-        if (li == 0 && c < q) nrm[c] = make_float2(s, fast_sqrt(s));
+        if (li == 0 && c < q) tm.put(&nrm[c], make_float2(s, fast_sqrt(s)));
       }
       if (threadIdx.x == 0) sh.rotated = 0;
       act_sync();
@@ -773,11 +781,11 @@ __device__ __noinline__ int jacobi32(float* g_ptr, int q, int ldg, float* v_ptr,
             }
           }
           if (on && li == 0) {
-            nrm[a] = make_float2(a2, fast_sqrt(a2));
-            nrm[b] = make_float2(b2, fast_sqrt(b2));
-            last_rot[a] = step;
-            last_rot[b] = step;
-            sh.rotated = 1;
+            tm.put(&nrm[a], make_float2(a2, fast_sqrt(a2)));
+            tm.put(&nrm[b], make_float2(b2, fast_sqrt(b2)));
+            tm.put(&last_rot[a], step);
+            tm.put(&last_rot[b], step);
+            tm.put(&sh.rotated, 1);
           }
         }
         act_sync();
@@ -895,30 +903,35 @@ __device__ __noinline__ void qr32(Work32& k, int p, int q, double* sc) {
   __syncthreads();
 }
 
-__device__ __forceinline__ int run_jacobi32(const Work32& k, int q, int max_sweeps, float tol,
-                                            float floor2, JacobiShared& sh) {
+// (tm: one CTA, or the team with both copies in global memory)
+template <class TM>
+__device__ __forceinline__ int run_jacobi32(const TM& tm, const Work32& k, int q, int max_sweeps,
+                                            float tol, float floor2, JacobiShared& sh) {
   extern __shared__ __align__(16) float svd_smem[];
 #define CLR_JACOBI32(LP, VEC, SH) \
-  return jacobi32<LP, VEC, SH>(k.g, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh)
+  return jacobi32<LP, VEC, SH>(tm, k.g, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh)
   const float* end = svd_smem + kSvdSmemBytes / sizeof(float);
   if (!(k.g >= svd_smem && k.g < end && k.v >= svd_smem && k.v < end)) {
     if (k.vec <= 3) CLR_JACOBI32(32, 3, false);   // (columns of more than 128 rows only)
     CLR_JACOBI32(32, 4, false);
   }
-  if (k.lp == 16) {
+  if constexpr (std::is_same<TM, One>::value) {
+    if (k.lp == 16) {
+      switch (k.vec) {
+        case 1: CLR_JACOBI32(16, 1, true);
+        case 2: CLR_JACOBI32(16, 2, true);
+        case 3: CLR_JACOBI32(16, 3, true);
+        default: CLR_JACOBI32(16, 4, true);
+      }
+    }
     switch (k.vec) {
-      case 1: CLR_JACOBI32(16, 1, true);
-      case 2: CLR_JACOBI32(16, 2, true);
-      case 3: CLR_JACOBI32(16, 3, true);
-      default: CLR_JACOBI32(16, 4, true);
+      case 1:
+      case 2: CLR_JACOBI32(32, 2, true);
+      case 3: CLR_JACOBI32(32, 3, true);
+      default: CLR_JACOBI32(32, 4, true);
     }
   }
-  switch (k.vec) {
-    case 1:
-    case 2: CLR_JACOBI32(32, 2, true);
-    case 3: CLR_JACOBI32(32, 3, true);
-    default: CLR_JACOBI32(32, 4, true);
-  }
+  return 0;   // (not reached: a team's copies are in global memory)
 #undef CLR_JACOBI32
 }
 
@@ -1357,6 +1370,12 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
   Work32 wk = work32(p, q, sc);
   const bool tri32 = lower && use_qr32(p, q);
   if (tri32) wk.g = svd_smem;
+  // the team's sweeps where the copies (of A, or of its triangular factor) do not fit one CTA's
+  // shared memory
+  const int q_even = (q + 1) & ~1;
+  const bool spread1 =
+      tm.size > 1 && (tri32 ? 2 * q_even * q : (wk.ldg + wk.ldv) * q) * (int)sizeof(float) >
+                         kSvdSmemBytes;
   constexpr int64_t kSq = (int64_t)CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
   double* v2 = sc + kSq;       // after p q + q^2 floats
   double* e = sc + 4 * kSq;    // the orthonormalisations' E, and their FP32 powers
@@ -1369,16 +1388,35 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
   const float floor_g = (float)floor64;
   const float tol32 = 4.f * FLT_EPSILON * sqrtf((float)p);
   const float floor32 = lower ? floor_g : (float)((double)p * FLT_EPSILON * fro);
-  // (the FP32 stages are the first CTA's)
+  // (else the FP32 stages are the first CTA's)
   int sw32 = 0;
-  if (tm.rank == 0) {
+  const One solo;
+  if (spread1 && !tri32) {
+    for (int e = tm.tid; e < wk.ldg * q; e += tm.nt) {
+      const int i = e % wk.ldg;
+      wk.g[e] = i < p ? (float)a.at(i, e / wk.ldg) : 0.f;
+    }
+    tm.sync();
+    sw32 = run_jacobi32(tm, wk, q, max_sweeps, tol32, floor32 * floor32, sh.jac);
+  } else if (tm.rank == 0) {
     for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
       const int i = e % wk.ldg;
       wk.g[e] = i < p ? (float)a.at(i, e / wk.ldg) : 0.f;
     }
     __syncthreads();
     if (tri32) qr32(wk, p, q, sc);
-    sw32 = run_jacobi32(wk, q, max_sweeps, tol32, floor32 * floor32, sh.jac);
+    if (!spread1) sw32 = run_jacobi32(solo, wk, q, max_sweeps, tol32, floor32 * floor32, sh.jac);
+  }
+  if (spread1 && tri32) {
+    // the triangular factor from the first CTA's shared memory to where the team reads it
+    float* g32 = reinterpret_cast<float*>(sc);
+    split32(wk, q, q);
+    if (tm.rank == 0)
+      for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) g32[e] = wk.g[e];
+    wk.g = g32;
+    wk.v = g32 + wk.ldg * q;
+    tm.sync();
+    sw32 = run_jacobi32(tm, wk, q, max_sweeps, tol32, floor32 * floor32, sh.jac);
   }
   mark(1);
   if (dense_h >= 0 && dense_h < q) {   // (full SVDs: a team of one)
@@ -1417,18 +1455,28 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
   project_fp64(tm, a, p, q, v, g, lower);
   mark(2);
   wk = work32(p, q, sc);
-  if (tm.rank == 0) {
-    for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
+  const float tol_g = lower ? 16.f * tol32 : tol32;
+  int sw32b = 0;
+  if (tm.size > 1 && (wk.ldg + wk.ldv) * q * (int)sizeof(float) > kSvdSmemBytes) {
+    for (int e = tm.tid; e < wk.ldg * q; e += tm.nt) {
       const int i = e % wk.ldg;
       wk.g[e] = i < p ? (float)g[i + (int64_t)(e / wk.ldg) * p] : 0.f;
     }
-    __syncthreads();
-    const int sw = run_jacobi32(wk, q, max_sweeps, lower ? 16.f * tol32 : tol32,
-                                floor_g * floor_g, sh.jac);
-    if (threadIdx.x == 0) tm.put(&sh.sweeps, sw);
+    tm.sync();
+    sw32b = run_jacobi32(tm, wk, q, max_sweeps, tol_g, floor_g * floor_g, sh.jac);
+  } else {
+    if (tm.rank == 0) {
+      for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
+        const int i = e % wk.ldg;
+        wk.g[e] = i < p ? (float)g[i + (int64_t)(e / wk.ldg) * p] : 0.f;
+      }
+      __syncthreads();
+      const int sw = run_jacobi32(solo, wk, q, max_sweeps, tol_g, floor_g * floor_g, sh.jac);
+      if (threadIdx.x == 0) tm.put(&sh.sweeps, sw);
+    }
+    tm.sync();
+    sw32b = sh.sweeps;
   }
-  tm.sync();
-  const int sw32b = sh.sweeps;
   mark(3);
   // When eps is well above the noise floor the right factor of the kept columns is recovered
   // from A and G afterwards (recover_right).  Near the floor (eps < 1e3 p u ||A||_F) kept
@@ -2016,8 +2064,8 @@ __device__ __noinline__ int compress_by_pivoted_qr(const TM& tm, const SrcView& 
     exact = false;
     tm.sync();
   }
-  if (jstats && tm.tid == 0)   // (the QR's flops after the certificate test)
-    atomicAdd(&jstats[4], 2ull * (fma_count + sh.qr_recomputed));
+  if (jstats && threadIdx.x == 0)   // (the QR's flops after the certificate test)
+    atomicAdd(&jstats[4], 2ull * ((tm.rank == 0 ? fma_count : 0) + sh.qr_recomputed));
   if (k < 0) return 0;
   if (k > jtail) {
     // dense when sum_{i > q/2} sigma_i^2 > eps^2 is certified by some leading triangle of the
@@ -2131,49 +2179,64 @@ __device__ __noinline__ int compress_by_pivoted_qr(const TM& tm, const SrcView& 
 // Dense truncated SVD of whole blocks (ROUTE_DACC tiles, recompressed dense tiles, building a
 // CLR matrix from a dense one).
 //
-// A tile is FP64-pipe-bound for 5 to 20 ms of one SM at 256 x 256, so with few tiles the launch
-// takes what its largest tile takes while most SMs idle.  With few tiles the CTAs come in clusters of
-// four, and while the tiles are at most half the CTAs a cluster works on one tile as a team (the
-// columns of the QR, the rows and blocks of the products; the FP32 sweeps stay with one CTA), else
-// each CTA takes its own.  A team takes a 256 x 240 tile in 9.8 M SM cycles, one CTA in 21, so that
-// half of its SMs' time is lost: with 144 tiles on 152 SMs (Coulomb-like lattice at N = 2048) teams
-// took 6.2 ms against 5.8, with 64 (gradient of the 1D chain at N = 1024) 3.6 against 5.1.
+// A tile is FP64-pipe-bound for 5 to 20 ms of one SM at 256 x 256 (and bound by its FP32 sweeps for
+// up to 45 where its QR rank is ~240), so with few tiles the launch takes what its largest tile takes
+// while most SMs idle.  With few tiles the CTAs come in clusters of four, and a cluster can work on
+// one tile as a team (the columns of the QR, the rows and blocks of the products, the pairs of
+// FP32 sweeps that leave shared memory).  A team takes a 256 x 240 tile in 9.8 M SM cycles, one CTA
+// in 21, so that half of its SMs' time is lost.  Teams take all tiles while these are at most half
+// the CTAs (64 tiles, gradient of the 1D chain at N = 1024: 3.6 ms against 5.1), else the leading
+// n_team ones of the list (team_tiles, by their costs), after which each CTA takes its own: with
+// 144 tiles on 152 SMs all by teams were no faster than none (Coulomb-like lattice at N = 2048,
+// 6.2 ms against 5.8), the largest few are (3D lattice iterates at N = 2048, 29 launches: 247 ->
+// 197 ms, the longest 43 -> 20).  Either way a tile's arithmetic is the same to the bit.
 // ---------------------------------------------------------------------------------------------
-constexpr int kTeamCtas = 4;
-
 template <bool kTeams>
 __device__ __forceinline__ void compress_dense_body(
     MatView C, const int* list, const int* count, const int* order, const double* src,
     int64_t lds, double* ws, double* svd_scratch, double eps, double drop_norm,
     int dense_only, int rrqr, int prereduce, int max_sweeps, int* err, int* sched,
-    unsigned long long* jstats) {
+    const int* n_team, unsigned long long* jstats) {
   __shared__ SvdShared sh;
   __shared__ int sh_next[2];
   const int n_items = list ? *count : C.nr * C.nc;
   const int cta = kTeams ? (int)cooperative_groups::this_cluster().block_rank() : 0;
-  const bool team = kTeams && 2 * n_items <= (int)gridDim.x;
+  // the leading tiles of the list that teams take
+  const int lead = !kTeams ? 0 : 2 * n_items <= (int)gridDim.x ? n_items : n_team ? *n_team : 0;
+  bool team = lead > 0;
   auto make = [&]() {
     if constexpr (kTeams) return Team(team ? cta : 0, team ? kTeamCtas : 1);
     else return One();
   };
-  const auto tm = make();
+  auto tm = make();
   double* sc = svd_scratch + (int64_t)(blockIdx.x - tm.rank) * kSvdScratchPerCta;
   int next_slot = 0;
   auto next = [&]() {
-    if (!team) return next_item(sched, &sh_next[0]);
-    // (two slots: one is read while the other is written)
-    if (tm.tid == 0) tm.put(&sh_next[next_slot], atomicAdd(sched, 1));
-    tm.sync();
-    next_slot ^= 1;
-    return sh_next[next_slot ^ 1];
+    if constexpr (kTeams)
+      if (team) {
+        // (two slots: one is read while the other is written)
+        if (tm.tid == 0) tm.put(&sh_next[next_slot], atomicAdd(sched, 1));
+        tm.sync();
+        next_slot ^= 1;
+        const int it = sh_next[next_slot ^ 1];
+        if (it < lead) return it;
+        // from here on each CTA takes its own tiles, the first one this one
+        __syncthreads();
+        team = false;
+        tm = make();
+        sc = svd_scratch + (int64_t)blockIdx.x * kSvdScratchPerCta;
+        if (cta == 0) return it;
+      }
+    return next_item(sched, &sh_next[0]);
   };
   // each tile's SM kilocycles go to C.cost (the next plan's scheduling cost), written when the
   // CTA takes its next tile (every path of the loop body ends there) and after the last one
-  int prev_t = -1;
+  // (a team's time twice over: about what one CTA takes)
+  int prev_t = -1, prev_x = 1;
   long long prev_c = 0;
   auto record_cost = [&](long long now) {
-    if (C.cost && prev_t >= 0 && tm.tid == 0) {
-      const long long kc = (now - prev_c) >> 10;
+    if (C.cost && prev_t >= 0 && threadIdx.x == 0) {
+      const long long kc = (now - prev_c) * prev_x >> 10;
       C.cost[prev_t] = (unsigned int)(kc < 1 ? 1 : kc > 0xFFFFFFFFll ? 0xFFFFFFFFll : kc);
     }
   };
@@ -2181,8 +2244,9 @@ __device__ __forceinline__ void compress_dense_body(
     const int t = list ? list[it] : (order ? order[it] : it);
     const long long now = clock64();
     record_cost(now);
-    prev_t = t;
+    prev_t = tm.rank == 0 ? t : -1;
     prev_c = now;
+    prev_x = tm.size > 1 ? 2 : 1;
     const int I = t / C.nc, J = t % C.nc;
     const int m = C.row_off[I + 1] - C.row_off[I];
     const int n = C.col_off[J + 1] - C.col_off[J];
@@ -2355,9 +2419,9 @@ __global__ void __cluster_dims__(kTeamCtas, 1, 1) __launch_bounds__(kThreads, 1)
                                const double* src, int64_t lds, double* ws, double* svd_scratch,
                                double eps, double drop_norm, int dense_only, int rrqr,
                                int prereduce, int max_sweeps, int* err, int* sched,
-                               unsigned long long* jstats) {
+                               const int* n_team, unsigned long long* jstats) {
   compress_dense_body<true>(C, list, count, order, src, lds, ws, svd_scratch, eps, drop_norm, dense_only,
-                      rrqr, prereduce, max_sweeps, err, sched, jstats);
+                      rrqr, prereduce, max_sweeps, err, sched, n_team, jstats);
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -2366,14 +2430,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                           double eps, double drop_norm, int dense_only, int rrqr, int prereduce,
                           int max_sweeps, int* err, int* sched, unsigned long long* jstats) {
   compress_dense_body<false>(C, list, count, order, src, lds, ws, svd_scratch, eps, drop_norm, dense_only,
-                      rrqr, prereduce, max_sweeps, err, sched, jstats);
+                      rrqr, prereduce, max_sweeps, err, sched, nullptr, jstats);
 }
 
 void launch_compress_dense(const MatView& C, const int* list, const int* count,
                            const int* order, const double* src, int64_t lds, double* ws,
                            double* svd_scratch, double eps, double drop_norm,
                            int dense_only, int rrqr, int prereduce, int max_sweeps, int grid,
-                           int* err, int* sched, unsigned long long* jstats, cudaStream_t st) {
+                           int* err, int* sched, const int* n_team, unsigned long long* jstats,
+                           cudaStream_t st) {
   static bool attr_done[64] = {false}, attr_done_team[64] = {false};
   const int g = svd_launch_grid(compress_dense_kernel, grid, attr_done);
   const int gt =
@@ -2383,7 +2448,7 @@ void launch_compress_dense(const MatView& C, const int* list, const int* count,
   if (gt > 0 && prereduce && !rrqr && !dense_only && C.nr * C.nc <= 2 * gt)
     compress_dense_team_kernel<<<gt, kThreads, kSvdSmemBytes, st>>>(
         C, list, count, order, src, lds, ws, svd_scratch, eps, drop_norm, dense_only, rrqr,
-        prereduce, max_sweeps, err, sched, jstats);
+        prereduce, max_sweeps, err, sched, n_team, jstats);
   else
     compress_dense_kernel<<<g, kThreads, kSvdSmemBytes, st>>>(
         C, list, count, order, src, lds, ws, svd_scratch, eps, drop_norm, dense_only, rrqr,

@@ -174,3 +174,63 @@ def test_build_by_teams_and_single_ctas(ctx, sizes):
             d = np.linalg.norm(g.block_dense(i, j) - blk)
             assert d <= (0.0 if gk[i, j] == co.KIND_DENSE
                          else eps * (1 + 1e-6) + 1e-14 * np.linalg.norm(blk)), (i, j, d)
+
+
+def _slow_tail(rng, m, n, lead, decay, top):
+    """U diag(s) V^T: `lead` singular values from 1 to 1e-4, then a tail from `top` falling by
+    `decay` each."""
+    k = min(m, n)
+    u, v = (np.linalg.qr(rng.standard_normal((d, k)))[0] for d in (m, n))
+    s = np.concatenate([np.logspace(0, -4, lead), top * decay ** np.arange(k - lead)])
+    return (u * s) @ v.T
+
+
+# a team of four CTAs and a CTA alone do the same arithmetic: QR ranks of ~235 (sweeps on a copy in
+# global memory), ~190 (on the FP32 triangular factor, in global memory) and ~60 (in shared memory)
+@pytest.mark.parametrize("decay", [0.999, 0.985, 0.93])
+def test_teams_and_single_ctas_give_the_same_bits(ctx, decay):
+    rng = np.random.default_rng(int(1000 * decay))
+    big = [256, 240]
+    eps = 1e-8
+    a = np.zeros((496, 496))
+    for i, m in enumerate(big):
+        for j, n in enumerate(big):
+            # the tail's norm is 0.9 eps: the rank is the leading part's
+            tail = 0.9 * eps * np.sqrt(1.0 - decay ** 2)
+            a[256 * i:256 * i + m, 256 * j:256 * j + n] = _slow_tail(rng, m, n, 20, decay, tail)
+    team = ctx.from_dense(a, big, eps_lr=eps)
+    pad = np.zeros((514, 514))
+    pad[:496, :496] = a
+    alone = ctx.from_dense(pad, big + [1] * 18, eps_lr=eps)   # 400 blocks: no clusters of CTAs
+    kt, rt = team.get_blocks()[:2]
+    ka, ra = alone.get_blocks()[:2]
+    assert np.array_equal(kt, ka[:2, :2]) and np.array_equal(rt, ra[:2, :2])
+    assert (np.abs(rt - 20) <= 1).all()
+    assert np.array_equal(team.to_dense(), alone.to_dense()[:496, :496])
+    for i, m in enumerate(big):
+        for j, n in enumerate(big):
+            box = (slice(256 * i, 256 * i + m), slice(256 * j, 256 * j + n))
+            assert np.linalg.norm(team.to_dense()[box] - a[box]) <= eps * (1 + 1e-6) + 1e-13
+
+
+def test_leading_tiles_by_teams(ctx):
+    # 169 tiles whose costs differ by 1000: the largest take teams, by their size at first and by
+    # their measured cost when the product is repeated into the same matrix, with the same bits
+    sizes = [256, 230] + [40, 25, 33, 48, 7, 60, 22, 37, 51, 1, 44]
+    n = sum(sizes)
+    rng = np.random.default_rng(3)
+    r = 0.02 * np.arange(n) + rng.uniform(-0.004, 0.004, n)
+    a = np.exp(-(r[:, None] - r[None, :]) ** 2 / 2.0) + 1e-3 * np.eye(n)
+    s = ctx.from_dense(a, sizes, eps_lr=1e-10)
+    ctx.set_opts(recompress_dense=1)
+    try:
+        c = ctx.multiply(s, s)
+        first = c.to_dense()
+        for _ in range(2):
+            ctx.multiply_into(s, s, c)
+            assert np.array_equal(c.to_dense(), first)
+    finally:
+        ctx.set_opts(recompress_dense=0)
+    # 169 tiles truncated at 1e-8, their operands at 1e-10
+    tol = 13 * 1e-8 + 2 * 13 * 1e-10 * np.linalg.norm(a, 2) + 2 * n * U * np.linalg.norm(a) ** 2
+    assert np.linalg.norm(first - a @ a) <= tol
