@@ -395,7 +395,7 @@ int take_device_error(clr_ctx_t ctx, const std::vector<std::unique_ptr<WorkSet>>
 // Grow the context workspaces needed by a plan over nI x nJ tiles and nK inner clusters.
 int make_plan(clr_ctx_t ctx, int nI, int nJ, int nK, Plan* p) {
   const size_t nt = (size_t)nI * nJ;
-  CLR_CUDA(ctx->cur->plan_ints.ensure(11 * nt * sizeof(int)));
+  CLR_CUDA(ctx->cur->plan_ints.ensure(12 * nt * sizeof(int)));
   const int64_t max_tr = (int64_t)nt * nK;
   CLR_CUDA(ctx->cur->triples.ensure((size_t)max_tr * sizeof(Triple)));
   int st = ensure_counters(ctx, ctx->cur);
@@ -416,6 +416,7 @@ int make_plan(clr_ctx_t ctx, int nI, int nJ, int nK, Plan* p) {
   p->l_qr_s = base + 8 * nt;
   p->l_dcomp_s = base + 9 * nt;
   p->l_dense_s = base + 10 * nt;
+  p->l_lr_s = base + 11 * nt;
   p->row_off = nullptr;
   p->col_off = nullptr;
   p->c_cost = nullptr;

@@ -175,6 +175,7 @@ struct Plan {
   int* l_qr_s;    // l_qr and l_dcomp reordered by decreasing recompression cost (plan_scan)
   int* l_dcomp_s;
   int* l_dense_s;  // l_dense reordered by decreasing cost m n (number of products)
+  int* l_lr_s;     // l_lr reordered by decreasing cost
   const int* row_off;  // C's cluster offsets (device), for those costs
   const int* col_off;
   const unsigned int* c_cost;  // C's measured recompression costs (MatView::cost), or null

@@ -79,7 +79,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kLrThreads)
     const int li = sh_next[slot];
     slot ^= 1;
     if (li >= n_lr) break;
-    const int t = p.l_lr[li];
+    const int t = p.l_lr_s[li];
     const int I = t / p.nJ, J = t % p.nJ;
     const int m = C.row_off[I + 1] - C.row_off[I];
     const int n = C.col_off[J + 1] - C.col_off[J];

@@ -118,7 +118,8 @@ constexpr int kScanQ = 5;
 constexpr int kCostBuckets = 128;   // four an octave
 
 // Bucket (4 log2, rounded down) of a tile's cost (which = 0: QR route recompression, 1: dense SVD, 2: dense x
-// dense products, m n times the tile's number of products).  A dense recompression's cost
+// dense products, m n times the tile's number of products, 3: low-rank products: an X_t or W_t of
+// ~32 (m + n) FMAs a column of the concatenation and, unless it is concatenated, m n for the sum).  A dense recompression's cost
 // depends on the path the tile takes (dense certificate ~0.4, pivoted QR and the SVD of R
 // ~1.1 when stored low rank and ~2 when stored dense, SM cycles per m n min(m, n) on the
 // lattice iterates), known only once it ran: the cycles
@@ -136,8 +137,10 @@ __device__ __forceinline__ int cost_bucket(const Plan& p, int t, int which) {
   } else if (which == 1) {
     const unsigned kc = p.c_cost ? p.c_cost[t] : 0u;
     c = kc ? (long long)kc << 10 : 2 * m * n * (m < n ? m : n);
-  } else {
+  } else if (which == 2) {
     c = m * n * (long long)p.t_count[t];
+  } else {
+    c = (p.t_route[t] == ROUTE_QR ? 32 * (m + n) : m * n + 32 * (m + n)) * (long long)p.t_rsum[t];
   }
   if (c < 4) return 0;
   const int b = 63 - __clzll(c);
@@ -262,30 +265,33 @@ __global__ void __launch_bounds__(kScanThreads) plan_scan_kernel(Plan p, int rec
     p.counters->n_dcomp = sh[4][tid];
     p.counters->n_dacc = 0;
   }
-  // The recompression lists and the dense-product list again, largest cost first
+  // The recompression lists and those of dense and low-rank products again, largest cost first
   // (longest-processing-time order for the dynamically distributed kernels): a counting sort on
   // a quarter of an octave of the cost, m n min(m, n) for a dense SVD, (m + n) R^2 for a QR route, m n times the
   // number of products for dense x dense products.  The order within a bucket is immaterial:
   // every tile is processed independently.
   __syncthreads();
   const int n_qr = sh[3][kScanThreads - 1], n_dc = sh[4][kScanThreads - 1];
-  const int n_de = sh[1][kScanThreads - 1];
-  __shared__ int bcount[3][kCostBuckets], boff[3][kCostBuckets];
-  static_assert(3 * kCostBuckets <= kScanThreads && kCostBuckets == 4 * 32, "buckets");
-  if (tid < 3 * kCostBuckets) (&bcount[0][0])[tid] = 0;
+  const int n_de = sh[1][kScanThreads - 1], n_lr = sh[2][kScanThreads - 1];
+  __shared__ int bcount[4][kCostBuckets], boff[4][kCostBuckets];
+  static_assert(4 * kCostBuckets <= kScanThreads && kCostBuckets == 4 * 32, "buckets");
+  if (tid < 4 * kCostBuckets) (&bcount[0][0])[tid] = 0;
   __syncthreads();
   auto item = [&](int i, int* which) {
-    *which = i < n_qr ? 0 : (i < n_qr + n_dc ? 1 : 2);
-    return *which == 0 ? p.l_qr[i] : *which == 1 ? p.l_dcomp[i - n_qr]
-                                                  : p.l_dense[i - n_qr - n_dc];
+    *which = i < n_qr ? 0 : i < n_qr + n_dc ? 1 : i < n_qr + n_dc + n_de ? 2 : 3;
+    return *which == 0   ? p.l_qr[i]
+           : *which == 1 ? p.l_dcomp[i - n_qr]
+           : *which == 2 ? p.l_dense[i - n_qr - n_dc]
+                         : p.l_lr[i - n_qr - n_dc - n_de];
   };
-  for (int i = tid; i < n_qr + n_dc + n_de; i += kScanThreads) {
+  const int n_all = n_qr + n_dc + n_de + n_lr;
+  for (int i = tid; i < n_all; i += kScanThreads) {
     int which;
     const int t = item(i, &which);
     atomicAdd(&bcount[which][cost_bucket(p, t, which)], 1);
   }
   __syncthreads();
-  if (tid < 3 * 32) {
+  if (tid < 4 * 32) {
     const int which = tid / 32, l = tid % 32;
     int cnt[4], own = 0;
 #pragma unroll
@@ -308,11 +314,11 @@ __global__ void __launch_bounds__(kScanThreads) plan_scan_kernel(Plan p, int rec
     }
   }
   __syncthreads();
-  for (int i = tid; i < n_qr + n_dc + n_de; i += kScanThreads) {
+  for (int i = tid; i < n_all; i += kScanThreads) {
     int which;
     const int t = item(i, &which);
     const int pos = atomicAdd(&boff[which][cost_bucket(p, t, which)], 1);
-    (which == 0 ? p.l_qr_s : which == 1 ? p.l_dcomp_s : p.l_dense_s)[pos] = t;
+    (which == 0 ? p.l_qr_s : which == 1 ? p.l_dcomp_s : which == 2 ? p.l_dense_s : p.l_lr_s)[pos] = t;
   }
 }
 
