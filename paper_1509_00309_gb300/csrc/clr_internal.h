@@ -309,8 +309,8 @@ int ozaki_gemm_dd(const OzakiGemmArgs& a, cudaStream_t st, std::string* why);
 // per segment); panels: kOzakiSlices planes
 // recon: scratch of M.n_rows x M.n_cols doubles (the low-rank blocks' reconstructions)
 void launch_ozaki_stage(const MatView& M, const int* row_idx, const int* col_idx, void* panels,
-                        int* exps, double* recon, int64_t rows_pad, int64_t cols_pad,
-                        int a_mode, cudaStream_t st);
+                        int* exps, double* recon, bool recon_formed, int64_t rows_pad,
+                        int64_t cols_pad, int a_mode, cudaStream_t st);
 // out[c * n_seg + s] = sum over rows i in [off[c], off[c + 1]) of 4^exps[s * rows_pad + i]
 void launch_ozaki_scale_sums(const int* exps, int64_t rows_pad, const int* off, int n_cl,
                              int n_seg, double* out, cudaStream_t st);

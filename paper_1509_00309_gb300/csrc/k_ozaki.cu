@@ -740,6 +740,10 @@ __global__ void __launch_bounds__(256) oz_lr_recon_kernel(MatView M, double* rec
   cta_gemm_auto((int)threadIdx.x, 256, m, j1 - j0, r, x, 1, m, w + j0, n, 1, recon + slot + (int64_t)j0 * m, m);
 }
 
+// Exponents and digits of the low-rank blocks from the image, lr_parts CTAs per block: bound by
+// the latency of their loads (the image is read along its rows for A's panels) and integer work, so
+// what counts is warps in flight.  With a CTA per block the 144 blocks of the 3D lattice at N = 2048
+// took 76 and 218 us a launch.
 __global__ void __launch_bounds__(256) oz_exp_lr_kernel(MatView M, const double* recon,
                                                         int* exps, int64_t rows_pad,
                                                         int a_mode) {
@@ -751,7 +755,8 @@ __global__ void __launch_bounds__(256) oz_exp_lr_kernel(MatView M, const double*
   const int s0 = (int)(k0 / SEG_K);
   for (int i = threadIdx.x; i < np; i += blockDim.x) red[i][0] = red[i][1] = INT_MIN;
   __syncthreads();
-  for (int e = threadIdx.x; e < L.m * L.n; e += blockDim.x) {
+  for (int e = threadIdx.x + blockDim.x * blockIdx.y; e < L.m * L.n;
+       e += blockDim.x * gridDim.y) {
     const int i = a_mode ? e / L.n : e % L.m;
     const int j = a_mode ? e % L.n : e / L.m;
     const int x = exp_bound(L.v[i + (int64_t)j * L.m]);
@@ -773,7 +778,8 @@ __global__ void __launch_bounds__(256) oz_digits_lr_kernel(MatView M, const doub
   LrBlock L;
   if (!lr_block(M, recon, blockIdx.x, &L)) return;
   const int64_t plane = rows_pad * cols_pad;
-  for (int e = threadIdx.x; e < L.m * L.n; e += blockDim.x) {
+  for (int e = threadIdx.x + blockDim.x * blockIdx.y; e < L.m * L.n;
+       e += blockDim.x * gridDim.y) {
     const int i = a_mode ? e / L.n : e % L.m;
     const int j = a_mode ? e % L.n : e / L.m;
     const int64_t prow = a_mode ? L.row0 + i : L.col0 + j;
@@ -824,8 +830,8 @@ bool encode_panel(EncodeFn fn, CUtensorMap* tm, void* base, int64_t k_pad, int64
 }  // namespace oz
 
 void launch_ozaki_stage(const MatView& M, const int* row_idx, const int* col_idx, void* panels,
-                        int* exps, double* recon, int64_t rows_pad, int64_t cols_pad,
-                        int a_mode, cudaStream_t st) {
+                        int* exps, double* recon, bool recon_formed, int64_t rows_pad,
+                        int64_t cols_pad, int a_mode, cudaStream_t st) {
   using namespace oz;
   unsigned short* pn = (unsigned short*)panels;
   // sentinel exponent (bytes 0x80: a large negative int) for rows without entries in a segment
@@ -839,8 +845,9 @@ void launch_ozaki_stage(const MatView& M, const int* row_idx, const int* col_idx
     const dim3 ne((unsigned)rows_pad, (unsigned)n_seg);
     oz_exp_b_kernel<<<ne, 256, 0, st>>>(M, row_idx, col_idx, exps, rows_pad, cols_pad);
   }
-  oz_lr_recon_kernel<<<dim3(nb, (unsigned)lr_parts((int)nb)), 256, 0, st>>>(M, recon);
-  oz_exp_lr_kernel<<<nb, 256, 0, st>>>(M, recon, exps, rows_pad, a_mode);
+  const dim3 nl(nb, (unsigned)lr_parts((int)nb));
+  if (!recon_formed) oz_lr_recon_kernel<<<nl, 256, 0, st>>>(M, recon);
+  oz_exp_lr_kernel<<<nl, 256, 0, st>>>(M, recon, exps, rows_pad, a_mode);
   if (a_mode) {
     const unsigned nd = (unsigned)((rows_pad / 32) * (cols_pad / 128));
     oz_digits_a_kernel<<<nd, 256, 0, st>>>(M, row_idx, col_idx, exps, pn, rows_pad, cols_pad);
@@ -849,7 +856,7 @@ void launch_ozaki_stage(const MatView& M, const int* row_idx, const int* col_idx
     oz_digits_b_kernel<<<nd, 256, 0, st>>>(M, row_idx, col_idx, exps, pn, rows_pad, cols_pad);
   }
   // (after the dense pass, which writes zeros at the low-rank blocks' entries)
-  oz_digits_lr_kernel<<<nb, 256, 0, st>>>(M, recon, exps, pn, rows_pad, cols_pad, a_mode);
+  oz_digits_lr_kernel<<<nl, 256, 0, st>>>(M, recon, exps, pn, rows_pad, cols_pad, a_mode);
 }
 
 void launch_ozaki_scale_sums(const int* exps, int64_t rows_pad, const int* off, int n_cl,
