@@ -66,14 +66,19 @@ __device__ __forceinline__ int next_item(int* counter, int* sh_slot) {
 // and waste no lanes.  The output is cut into MR x MC micro-tiles (ragged last ones clamped)
 // taken by the threads in turn, rows first (a should have unit stride along i; b is mostly
 // broadcast).  TRI = 1: a(i, l) is zero for l > i; TRI = 2: b(l, j) is zero for l < j (those
-// terms are skipped).  No synchronisation inside: the caller orders dependent calls.
+// terms are skipped).  With TRI = 1 columns go first and the longest rows (b should have unit
+// stride along j): a warp's lanes then have the same number of terms, where rows first made a warp
+// wait for its longest row and gave two of the four sub-partitions all the long ones (the
+// projections of the 3D lattice product's recompression at N = 4096: 0.76 -> 0.70 G SM cycles).
+// No synchronisation inside: the caller orders dependent calls.
 template <int MR, int MC, int TRI, class T>
 __device__ __forceinline__ void cta_gemm_micro(int tid, int nt, int P, int Q, int L, const T* a, int64_t a_r,
                                                int64_t a_c, const T* b, int64_t b_r, int64_t b_c,
                                                T* out, int64_t ldo, bool accumulate) {
   const int mp = (P + MR - 1) / MR, mq = (Q + MC - 1) / MC;
   for (int t = tid; t < mp * mq; t += nt) {
-    const int i0 = (t % mp) * MR, j0 = (t / mp) * MC;
+    const int i0 = (TRI == 1 ? mp - 1 - t / mq : t % mp) * MR;
+    const int j0 = (TRI == 1 ? t % mq : t / mp) * MC;
     const int l0 = TRI == 2 ? j0 : 0;
     const int l1 = TRI == 1 && i0 + MR < L ? i0 + MR : L;
     const T* ap[MR];

@@ -743,7 +743,7 @@ __global__ void __launch_bounds__(256) oz_lr_recon_kernel(MatView M, double* rec
 // Exponents and digits of the low-rank blocks from the image, lr_parts CTAs per block: bound by
 // the latency of their loads (the image is read along its rows for A's panels) and integer work, so
 // what counts is warps in flight.  With a CTA per block the 144 blocks of the 3D lattice at N = 2048
-// took 76 and 218 us a launch.
+// took 76 and 218 us a launch, now 38 and 85.
 __global__ void __launch_bounds__(256) oz_exp_lr_kernel(MatView M, const double* recon,
                                                         int* exps, int64_t rows_pad,
                                                         int a_mode) {
