@@ -70,6 +70,8 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kLrThreads)
   const int n_lr = p.counters->n_lr;
   int* sched = &p.counters->sched[0];
   int slot = 0, par = 0;
+  // a CTA's shared memory may be written by another only once it is known to have started
+  cluster.sync();
   while (true) {
     // the cluster's next tile (two slots: one is read while the other is written)
     if (rank == 0 && threadIdx.x == 0) {
