@@ -2210,6 +2210,9 @@ __device__ __forceinline__ void compress_dense_body(
   };
   auto tm = make();
   double* sc = svd_scratch + (int64_t)(blockIdx.x - tm.rank) * kSvdScratchPerCta;
+  // a CTA's shared memory may be written by another (put) only once it is known to have started
+  // (lead is the same in all of a cluster's CTAs)
+  if (team) tm.sync();
   int next_slot = 0;
   auto next = [&]() {
     if constexpr (kTeams)

@@ -29,6 +29,7 @@ def _function(file, name):
     ("k_ns.cu", "lincomb_apply_kernel", "cluster.sync()", "map_shared_rank("),
     ("k_ns.cu", "matvec_kernel", "cluster.sync()", "map_shared_rank("),
     ("k_dense64.cu", "dense_tile_norms_kernel", "cluster.sync()", "map_shared_rank("),
+    ("k_svd.cu", "compress_dense_body", "if (team) tm.sync()", "tm.put("),
 ])
 def test_a_cluster_barrier_precedes_the_first_access_to_a_peer(file, kernel, barrier, access):
     body = _function(file, kernel)
