@@ -1057,16 +1057,21 @@ struct SrcView {
 template <class TM>
 __device__ __noinline__ double small_series(const TM& tm, double* e, int q, double c1, float c2,
                                             float c3, float* f, SvdShared& sh) {
-  // (every CTA of the team takes the FP32 powers itself)
+  // Where the powers lie in the CTA's shared memory every CTA of the team takes them itself; in the
+  // team's one global scratch (more than ~156 columns) they are dealt over the team.
+  extern __shared__ __align__(16) float svd_smem[];
+  const bool own = tm.size == 1 || f == svd_smem;
+  const int t0 = own ? (int)threadIdx.x : tm.tid, step = own ? kThreads : tm.nt;
   float* t = f + q * q;
   float part = 0.f;
   for (int x = threadIdx.x; x < q * q; x += kThreads) {
     const float v = (float)e[x];
-    f[x] = v;
     part = fmaf(v, v, part);
   }
+  for (int x = t0; x < q * q; x += step) f[x] = (float)e[x];
   const double fro2 = block_sum((double)part, sh.red);
-  cta_gemm_auto(threadIdx.x, kThreads, q, q, q, f, 1, q, f, 1, q, t, q);
+  if (!own) tm.sync();
+  cta_gemm_auto(t0, step, q, q, q, f, 1, q, f, 1, q, t, q);
   tm.sync();
   // E^3 = F T an output at a time, added to the rest of the series
   for (int x = tm.tid; x < q * q; x += tm.nt) {
