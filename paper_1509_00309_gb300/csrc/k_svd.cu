@@ -1390,23 +1390,29 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
   // their mutual (non-)orthogonality cannot move a truncation decision at eps except within a
   // hair of the threshold, while orthogonalising them costs most of the sweeps
   const double floor64 = fmax((double)p * DBL_EPSILON * fro, 1e-3 * eps);
-  const float floor_g = (float)floor64;
+  // The FP32 copies (and the floors beside them) are scaled by the power of two that brings
+  // ||A||_F to 1..2: their squares and inner products then stay inside the FP32 range whatever
+  // the block's norm is, and V does not depend on the scale.  (Unscaled, no pair of columns was
+  // rotated in blocks of norm below ~1e-18 or above 1.8e19, and their ranks were those of the
+  // columns as they came.)
+  const double sc32 = fro > 0.0 && isfinite(fro) ? scalbn(1.0, -ilogb(fro)) : 1.0;
+  const float floor_g = (float)(floor64 * sc32);
   const float tol32 = 4.f * FLT_EPSILON * sqrtf((float)p);
-  const float floor32 = lower ? floor_g : (float)((double)p * FLT_EPSILON * fro);
+  const float floor32 = lower ? floor_g : (float)((double)p * FLT_EPSILON * fro * sc32);
   // (else the FP32 stages are the first CTA's)
   int sw32 = 0;
   const One solo;
   if (spread1 && !tri32) {
     for (int e = tm.tid; e < wk.ldg * q; e += tm.nt) {
       const int i = e % wk.ldg;
-      wk.g[e] = i < p ? (float)a.at(i, e / wk.ldg) : 0.f;
+      wk.g[e] = i < p ? (float)(a.at(i, e / wk.ldg) * sc32) : 0.f;
     }
     tm.sync();
     sw32 = run_jacobi32(tm, wk, q, max_sweeps, tol32, floor32 * floor32, sh.jac);
   } else if (tm.rank == 0) {
     for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
       const int i = e % wk.ldg;
-      wk.g[e] = i < p ? (float)a.at(i, e / wk.ldg) : 0.f;
+      wk.g[e] = i < p ? (float)(a.at(i, e / wk.ldg) * sc32) : 0.f;
     }
     __syncthreads();
     if (tri32) qr32(wk, p, q, sc);
@@ -1430,7 +1436,7 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
       double s2 = 0.0;
       for (int i = l; i < p; i += 32) s2 = fma((double)gc[i], (double)gc[i], s2);
       s2 = warp_sum(s2);
-      if (l == 0) sh.sigma[c] = sqrt(s2);
+      if (l == 0) sh.sigma[c] = sqrt(s2) / sc32;
     }
     __syncthreads();
     double part = 0.0;
@@ -1465,7 +1471,7 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
   if (tm.size > 1 && (wk.ldg + wk.ldv) * q * (int)sizeof(float) > kSvdSmemBytes) {
     for (int e = tm.tid; e < wk.ldg * q; e += tm.nt) {
       const int i = e % wk.ldg;
-      wk.g[e] = i < p ? (float)g[i + (int64_t)(e / wk.ldg) * p] : 0.f;
+      wk.g[e] = i < p ? (float)(g[i + (int64_t)(e / wk.ldg) * p] * sc32) : 0.f;
     }
     tm.sync();
     sw32b = run_jacobi32(tm, wk, q, max_sweeps, tol_g, floor_g * floor_g, sh.jac);
@@ -1473,7 +1479,7 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
     if (tm.rank == 0) {
       for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
         const int i = e % wk.ldg;
-        wk.g[e] = i < p ? (float)g[i + (int64_t)(e / wk.ldg) * p] : 0.f;
+        wk.g[e] = i < p ? (float)(g[i + (int64_t)(e / wk.ldg) * p] * sc32) : 0.f;
       }
       __syncthreads();
       const int sw = run_jacobi32(solo, wk, q, max_sweeps, tol_g, floor_g * floor_g, sh.jac);
