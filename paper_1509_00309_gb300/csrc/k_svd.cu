@@ -450,10 +450,11 @@ __device__ __forceinline__ void round_pair(int round, int k, int qq, int* a, int
   *b = y;
 }
 
-// FP64 (the allocation-free entry point): the tests compare squares, the rotation's tangent t is
-// found in FP32 from zeta where the angle is small (its accuracy only sets how far one rotation
-// reduces the pair's inner product) and c is refined in FP64 by two Newton steps from the FP32
-// seed, so that c^2 + s^2 = 1 to FP64 rounding and the rotation is orthogonal.
+// FP64 (the allocation-free entry point, and svd_mixed near the noise floor): the tests compare
+// squares, the rotation's tangent t is found in FP32 from zeta where the angle is small (its
+// accuracy only sets how far one rotation reduces the pair's inner product) and c is refined in
+// FP64 by two Newton steps from the FP32 seed, so that c^2 + s^2 = 1 to FP64 rounding and the
+// rotation is orthogonal.
 __device__ __forceinline__ void rotation(double al, double be, double g, double& c, double& s,
                                          double& t) {
   // zeta in FP64 (the operands may lie far outside the FP32 range).  For a large angle
@@ -478,20 +479,28 @@ __device__ __forceinline__ void rotation(double al, double be, double g, double&
   s = r * t;
 }
 
-// One-sided Jacobi in FP64 on the q columns of g (p x q, ld p); v (q x q, ld q), initialised to I
-// here, accumulates the rotations.  On return g = U S and the input equals g v^T.  Pairs whose
+struct JacobiShared {
+  float2 nrm[CLR_MAX_CLUSTER];     // column norms: squared, and the root
+  int last_rot[CLR_MAX_CLUSTER];   // the step of the column's last rotation, -1 if none
+  int rotated, sweeps;
+};
+
+// One-sided Jacobi in FP64 on the q columns of g (p x q, ld p); v (q x q, element (i, c) at
+// v[i v_r + c v_c]) accumulates the rotations, from I when reset is set.  On return g = U S and the
+// input equals g v^T (times the initial v^T when v is not reset).  Pairs whose
 // inner product is below floor2, or below the FP64 epsilon times sqrt(p) relative to the norms,
-// are left alone.  Returns the number of sweeps.
-__device__ int jacobi_svd(double* g, int p, int q, double* v, int max_sweeps, int* sh_flag,
-                          double floor2) {
-  // Column norms squared, kept in shared memory: recomputed exactly at every sweep start and
-  // refreshed (fused into the rotation pass) for the two columns of every rotated pair, so a
-  // pair costs one inner product unless it is rotated.
-  __shared__ double nrm2[CLR_MAX_CLUSTER];
-  // per column: the step (sweep * (qq - 1) + round) of its last rotation, -1 if none
-  __shared__ int last_rot[CLR_MAX_CLUSTER];
+// are left alone.  Returns the number of sweeps.  jac: its norms' place holds the column norms
+// squared, recomputed exactly at every sweep start and refreshed (fused into the rotation pass) for
+// the two columns of every rotated pair, so a pair costs one inner product unless it is rotated.
+__device__ __noinline__ int jacobi_svd(double* g, int p, int q, double* v, int64_t v_r, int64_t v_c,
+                                       bool reset, int max_sweeps, int* sh_flag, double floor2,
+                                       JacobiShared& jac) {
+  double* nrm2 = reinterpret_cast<double*>(jac.nrm);
+  int* last_rot = jac.last_rot;   // the step (sweep * (qq - 1) + round) of its last rotation, -1
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  for (int e = threadIdx.x; e < q * q; e += kThreads) v[e] = (e % q == e / q) ? 1.0 : 0.0;
+  if (reset)
+    for (int e = threadIdx.x; e < q * q; e += kThreads)
+      v[e % q * v_r + e / q * v_c] = (e % q == e / q) ? 1.0 : 0.0;
   const int qq = q + (q & 1);  // even number of slots; slot q is a dummy when q is odd
   const double tol = DBL_EPSILON * sqrt((double)p);
   for (int c = threadIdx.x; c < q; c += kThreads) last_rot[c] = -1;
@@ -554,12 +563,12 @@ __device__ int jacobi_svd(double* g, int p, int q, double* v, int max_sweeps, in
           na = warp_sum(sa);
           nb = warp_sum(sb);
         }
-        double* va = v + (int64_t)a * q;
-        double* vb = v + (int64_t)b * q;
+        double* va = v + a * v_c;
+        double* vb = v + b * v_c;
         for (int i = l; i < q; i += 32) {
-          const double x = va[i], y = vb[i];
-          va[i] = c * x - sn * y;
-          vb[i] = sn * x + c * y;
+          const double x = va[i * v_r], y = vb[i * v_r];
+          va[i * v_r] = c * x - sn * y;
+          vb[i * v_r] = sn * x + c * y;
         }
         if (l == 0) {
           nrm2[a] = na;
@@ -616,12 +625,6 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
-
-struct JacobiShared {
-  float2 nrm[CLR_MAX_CLUSTER];     // column norms: squared, and the root
-  int last_rot[CLR_MAX_CLUSTER];   // the step of the column's last rotation, -1 if none
-  int rotated, sweeps;
-};
 
 // One-sided Jacobi in FP32 with the working copies in shared memory (or, where they do not fit,
 // in the per-CTA scratch), for the FP32 stages of svd_mixed.  What bounds it is the latency of a
@@ -1335,8 +1338,11 @@ __device__ __noinline__ bool ls_solve(const TM& tm, double* y, int q, int r, dou
 //     relative to their own norms already and one-sided Jacobi is relatively accurate on them
 //     (Drmac and Veselic).  Stage 1 then sweeps down to stage 3's floor, and stage 3 only runs
 //     where a pair of G's columns is further than 16 times the stages' tolerance (cosine ~1e-4)
-//     from orthogonal; at that angle the sorted norms are within 1e-8 relative of the singular
-//     values, and what a kept column can carry of a dropped one is 1e-4 eps.  Measured on the
+//     from orthogonal.  At that angle well separated columns' norms are within 1e-8 relative of the
+//     singular values; of a cluster only the sum of squares is (two equal columns at a cosine c have
+//     singular values c / 2 to either side), so a truncation inside a cluster may keep or drop a
+//     column whose singular value is within 1e-4 of its norm; the error is the dropped columns' norm
+//     either way, and what a kept column can carry of a dropped one is 1e-4 eps.  Measured on the
 //     3D lattice product at N = 4096 (376 blocks): stages 1, 3 and 4 took 0.26 + 1.34 + 1.38 G
 //     SM cycles, now 1.49 + 0.13 + 0.02.
 //  The right factor: for kept columns G_r = U_r S_r it is V_r = A^T G_r S_r^-2 (recover_right),
@@ -1501,23 +1507,31 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
   }
   if (threadIdx.x == 0) sh.v_tracked = track_v ? 1 : 0;
   mark(4);
-  // No FP64 sweep follows: after stage 3 the columns of G are orthogonal to the FP32 stages'
-  // tolerance (cosines ~1e-5 relative to their own norms), so the sorted column norms, whose
-  // tail decides the rank, are within ~1e-10 of the singular values, and the truncation error
-  // does not depend on their being orthogonal: with V accumulated A = G V^T and dropping columns
-  // leaves ||G_tail V_tail^T||_F = ||G_tail||_F (V is orthogonal to FP64 rounding); without it,
-  // the least-squares right factor (ls_solve) makes X W^T the orthogonal projection of A onto
+  // Near the noise floor a matrix that is not graded needs FP64 sweeps too: V2 is FP32, so the small
+  // columns of G V2 keep ~u32^2 ||A||_F sqrt(p q) of the large ones, which can exceed eps (a sum of
+  // two low-rank blocks of a common column space, eps = 1e-13: rank 48 where it is 24).
+  // Elsewhere no FP64 sweep follows: the columns of G are orthogonal to the FP32 stages' tolerance
+  // (cosines ~1e-5, for a graded A up to ~1e-4, relative to their own norms), and the truncation
+  // error does not depend on their being orthogonal: with V accumulated A = G V^T and dropping
+  // columns leaves ||G_tail V_tail^T||_F = ||G_tail||_F (V is orthogonal to FP64 rounding); without
+  // it, the least-squares right factor (ls_solve) makes X W^T the orthogonal projection of A onto
   // span(G_r), with error ||(I - P) G_tail|| <= ||G_tail||_F <= eps for any G = A V_eff.
-  // (FP64 sweeps to convergence where V is accumulated, the earlier choice, took 3.6 of 12.5 G
-  // cycles of the lattice product's recompression at N = 4096.)
+  // (FP64 sweeps to convergence wherever V is accumulated, the earlier choice, took 3.6 of 12.5 G
+  // cycles of the lattice product's recompression at N = 4096, of graded factors.)
+  int sw64 = 0;
+  if (track_v && !lower)   // (one CTA: teams have graded factors)
+    sw64 = jacobi_svd(g, p, q, v, q, 1, false, max_sweeps, &sh.flag, floor64 * floor64, sh.jac);
+  mark(5);
   if (threadIdx.x == 0) sh.ls_recover = track_v ? 0 : 1;
   if (jstats && tm.tid == 0) {
     // algorithmic flops: Jacobi 4 p q^2 per sweep, orthonormalisation 3 q^3, products 2 p q^2
     const unsigned long long pq2 = (unsigned long long)p * q * q, q3 = (unsigned long long)q * q * q;
     unsigned long long f64 = 2 * q3 + 2 * pq2;
     if (sw32b > 0) f64 += 2 * q3 + 2 * pq2 + (track_v ? 2 * q3 : 0);
+    f64 += 4 * pq2 * (unsigned long long)sw64;
     atomicAdd(&jstats[0], 1ull);
     atomicAdd(&jstats[1], (unsigned long long)(sw32 + sw32b));
+    atomicAdd(&jstats[2], (unsigned long long)sw64);
     atomicAdd(&jstats[4], f64);
     atomicAdd(&jstats[5], 4 * pq2 * (unsigned long long)(sw32 + sw32b));
   }
@@ -2593,7 +2607,8 @@ __global__ void __launch_bounds__(kThreads) compress_block_noalloc_kernel(
   // rotating them changes nothing that a truncation can see, and they would keep the sweeps
   // from ever converging
   const double floor64 = (double)p * DBL_EPSILON * sqrt(nsq);
-  const int sweeps = jacobi_svd(G, p, q, V, max_sweeps, &sh.flag, floor64 * floor64);
+  const int sweeps =
+      jacobi_svd(G, p, q, V, 1, q, true, max_sweeps, &sh.flag, floor64 * floor64, sh.jac);
   // every sweep still rotated a pair: the column norms the truncation uses may be inexact
   if (sweeps >= max_sweeps && threadIdx.x == 0) status[2] = 4;
   sort_and_truncate(G, p, q, p, eps, sh);
