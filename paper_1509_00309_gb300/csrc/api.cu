@@ -405,6 +405,7 @@ int make_plan(clr_ctx_t ctx, int nI, int nJ, int nK, Plan* p) {
   p->nJ = nJ;
   p->nK = nK;
   p->n_sm = ctx->n_sm;
+  p->dense_by_gemm = 0;
   p->t_count = base;
   p->t_start = base + nt;
   p->t_route = base + 2 * nt;
@@ -1132,6 +1133,7 @@ int multiply_into(clr_ctx_t ctx, clr_mat_t a, clr_mat_t b, clr_mat_t c, double a
   p.row_off = c->d_row_off;
   p.col_off = c->d_col_off;
   p.c_cost = c->d_cost;
+  p.dense_by_gemm = prec != CLR_PREC_FP64;
   CLR_CUDA(ctx->cur->ws.ensure(2 * (size_t)c->n_rows * c->n_cols * sizeof(double)));
   const int lr_grid = grid_of(ctx, tune.lr_mult);
   CLR_CUDA(ctx->cur->scratch.ensure((size_t)lr_grid * scratch_per_cta() * sizeof(double)));
@@ -1169,13 +1171,11 @@ int multiply_into(clr_ctx_t ctx, clr_mat_t a, clr_mat_t b, clr_mat_t c, double a
     st = run_split_dd(ctx, a, b, c, p, prec, recompress_dense, s, &fused_norms);
     if (st) return st;
   }
-  // the tensor-core GEMMs form the whole sum of the tiles they serve (route DENSE and DACC_G:
-  // the low-rank blocks are staged as reconstructions): the low-rank kernel skips those
-  const bool dense_by_gemm = prec != CLR_PREC_FP64;
-  launch_lr_products(av, bv, cv, p, (double*)ctx->cur->ws.p, (double*)ctx->cur->scratch.p,
-                     scratch_per_cta(), dense_by_gemm, lr_grid, s);
+  const int lr_launches =
+      launch_lr_products(av, bv, cv, p, (double*)ctx->cur->ws.p, (double*)ctx->cur->scratch.p,
+                         scratch_per_cta(), lr_grid, s);
   CLR_CHECK_LAUNCH("low-rank products");
-  prof_launches(ctx, 1);
+  prof_launches(ctx, lr_launches);
   prof_mark(ctx, s, PH_LOWRANK);
   launch_compress_qr(cv, p.l_qr_s, &p.counters->n_qr, p.t_rsum, (double*)ctx->cur->ws.p,
                      (double*)ctx->cur->scratch.p, eps_lr, o.jacobi_max_sweeps,

@@ -168,12 +168,13 @@ constexpr size_t kPlanCountersClear = offsetof(PlanCounters, err);
 struct Plan {
   int nI, nJ, nK;
   int n_sm;
+  int dense_by_gemm;  // the dense tiles' low-rank products are the tensor-core GEMM's too
   int* t_count;   // nI*nJ
   int* t_start;   // nI*nJ
   int* t_route;   // nI*nJ
   int* t_rsum;    // nI*nJ
   int* l_dense;   // tiles with ROUTE_DENSE
-  int* l_lr;      // tiles with at least one low-rank product (any route)
+  int* l_lr;      // tiles with low-rank products for launch_lr_products
   int* l_qr;      // ROUTE_QR
   int* l_dcomp;   // tiles needing a dense truncated SVD (ROUTE_DACC, or ROUTE_DENSE when
                   // dense tiles are recompressed)
@@ -220,10 +221,10 @@ void launch_dense_kinds(const MatView& M, double drop_norm, int* err, cudaStream
 void launch_pool_to_rowmajor(const MatView& M, const int* row_idx, const int* col_idx,
                              double* out, int64_t ldo, cudaStream_t st);
 // k_lowrank.cu
-// dense_by_gemm: DENSE and DACC tiles were fully summed by the split GEMM (skip them).
-void launch_lr_products(const MatView& A, const MatView& B, const MatView& C, const Plan& p,
-                        double* ws, double* scratch, int64_t scratch_per_cta, int dense_by_gemm,
-                        int grid, cudaStream_t st);  // uses p.counters->sched[0]
+// uses p.counters->sched[0]; returns the number of kernels launched
+int launch_lr_products(const MatView& A, const MatView& B, const MatView& C, const Plan& p,
+                       double* ws, double* scratch, int64_t scratch_per_cta, int grid,
+                       cudaStream_t st);
 // k_svd.cu
 // jstats (may be null): device counters {svd blocks, FP32 sweeps, FP64 sweeps, early dense}
 // svd_scratch: grid x kSvdScratchPerCta doubles (FP32 working copies and an FP64 q x q factor

@@ -13,19 +13,21 @@
 //                added as X_t W_t^T;
 //   ROUTE_DACC   the concatenated rank exceeds floor(min(m,n)/2), so the sum is accumulated
 //                densely (from zero) and K5 takes a dense truncated SVD.
-// With a tensor-core GEMM (split precision or exact slices: dense_by_gemm) the GEMM sums all
-// contributions of DENSE and DACC_G tiles; this kernel builds the ROUTE_QR concatenations and the
-// FP64 DACC sums.
+// With a tensor-core GEMM (split precision or exact slices: Plan::dense_by_gemm) the GEMM sums all
+// contributions of DENSE and DACC_G tiles, which are not in the list then; this kernel builds the
+// ROUTE_QR concatenations and the FP64 DACC sums.
 //
-// The work is FP64-pipe-bound (~2 FMAs per clock and SM) and a product has far fewer tiles with
-// low-rank work than SMs, or tiles that differ by an order of magnitude, so a tile is spread over
-// the CTAs of a cluster: CTA c owns the rows [m c / CS, m (c + 1) / CS) of the tile, of X_cat and
-// of every X_t, and that share of the rows of W_cat.  What every CTA needs whole (Z, and a
-// computed W_t of a dense accumulation) is formed in shares into the cluster's scratch and
-// exchanged by one cluster barrier; two buffers in turn make that barrier the only one.
-// Measured (one tile per CTA before): Coulomb-like lattice at N = 2048 (144 tiles, 1452 LL
-// products of rank ~40) 25.3 -> 7.7 ms (1 of it by taking the most expensive tiles first); 1D
-// chain at N = 2048 257 -> 70 us.
+// The work is FP64-pipe-bound (~2 FMAs per clock and SM).  While the tiles with low-rank work are
+// few, or differ by an order of magnitude, a tile is spread over the CTAs of a cluster: CTA c owns
+// the rows [m c / CS, m (c + 1) / CS) of the tile, of X_cat and of every X_t, and that share of the
+// rows of W_cat.  What every CTA needs whole (Z, and a computed W_t of a dense accumulation) is
+// formed in shares into the cluster's scratch and exchanged by one cluster barrier; two buffers in
+// turn make that barrier the only one.  Measured (one tile per CTA before): Coulomb-like lattice at
+// N = 2048 (144 tiles, 1452 LL products of rank ~40) 25.3 -> 7.7 ms (1 of it by taking the most
+// expensive tiles first); 1D chain at N = 2048 257 -> 70 us.  With more than kTilesPerCta tiles a
+// CTA they fill the SMs one to a CTA, and shares only cost barriers and ragged micro-tiles (CS = 1;
+// ms with CS = 4 / 1: 3D lattice, 529 tiles 48 / 49, 1156 tiles (Coulomb-like) 133 / 117, 2116
+// 306 / 263; clusters of at most 48 points, 48400 tiles, 1106 / 581).
 #include <cooperative_groups.h>
 
 #include "clr_internal.h"
@@ -35,6 +37,9 @@ namespace clr {
 namespace cg = cooperative_groups;
 
 constexpr int kLrThreads = 256;
+// Tiles with work, a CTA of the grid, from which each CTA takes its own (608 at two CTAs an SM:
+// between the 529 and the 784 tiles measured).
+constexpr int kTilesPerCta = 2;
 
 // out(i,j) (= or +=) sum_l a(i,l) b(l,j) for a P x Q output with arbitrary element strides, the
 // micro-tile by the size of the output (clr_internal.h).
@@ -61,24 +66,30 @@ static_assert(2 * (kZElems + kFElems) + kFElems <= kSvdScratchPerCta, "low-rank 
 template <int CS>
 __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kLrThreads)
     lr_products_kernel(MatView A, MatView B, MatView C, Plan p, double* ws, double* scratch,
-                       int64_t scratch_per_cta, int dense_by_gemm) {
+                       int64_t scratch_per_cta, int few) {
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ int sh_next[2];
-  const int rank = (int)cluster.block_rank();
+  const int n_lr = p.counters->n_lr;
+  if (few != 0 && (n_lr > few) != (CS == 1)) return;   // the other launch's work
+  const int rank = CS > 1 ? (int)cluster.block_rank() : 0;
+  auto tile_sync = [&]() {
+    if constexpr (CS == 1) __syncthreads(); else cluster.sync();
+  };
   double* shared_scr = scratch + (int64_t)(blockIdx.x - rank) * scratch_per_cta;
   double* scrX = scratch + (int64_t)blockIdx.x * scratch_per_cta + 2 * (kZElems + kFElems);
-  const int n_lr = p.counters->n_lr;
   int* sched = &p.counters->sched[0];
   int slot = 0, par = 0;
   // a CTA's shared memory may be written by another only once it is known to have started
-  cluster.sync();
+  if (CS > 1) cluster.sync();
   while (true) {
     // the cluster's next tile (two slots: one is read while the other is written)
     if (rank == 0 && threadIdx.x == 0) {
       const int v = atomicAdd(sched, 1);
-      for (int c = 0; c < CS; ++c) *cluster.map_shared_rank(&sh_next[slot], c) = v;
+      if (CS == 1) sh_next[slot] = v;
+      else
+        for (int c = 0; c < CS; ++c) *cluster.map_shared_rank(&sh_next[slot], c) = v;
     }
-    cluster.sync();
+    tile_sync();
     const int li = sh_next[slot];
     slot ^= 1;
     if (li >= n_lr) break;
@@ -87,9 +98,6 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kLrThreads)
     const int m = C.row_off[I + 1] - C.row_off[I];
     const int n = C.col_off[J + 1] - C.col_off[J];
     const int route = p.t_route[t];
-    // with a tensor-core GEMM the dense tiles and the DACC_G tiles already hold every
-    // contribution (low-rank operand blocks staged as X W^T)
-    if ((dense_by_gemm && route == ROUTE_DENSE) || route == ROUTE_DACC_G) continue;
     const int R = p.t_rsum[t];
     const int64_t sC = slot_of(C, I, J, m);
     double* D = C.pool + sC;
@@ -121,7 +129,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kLrThreads)
         const int z0 = rb * rank / CS, zc = rb * (rank + 1) / CS - z0;
         cta_gemm(ra, zc, k, WA, k, 1, XB + (int64_t)z0 * k, 1, k, scrZ + (int64_t)z0 * ra, ra,
                  false);
-        cluster.sync();
+        tile_sync();
         par ^= 1;
       }
       const int rt = x_side ? rb : ra;
@@ -150,7 +158,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kLrThreads)
         if (x_side) {
           __syncthreads();
         } else {
-          cluster.sync();
+          tile_sync();
           if (tr.kind == T_LD) par ^= 1;   // (an LL product has switched buffers already)
         }
         cta_gemm(xr, n, rt, Xt, 1, ldx, x_side ? WB : scrF, n, 1, D + x0, m, !first);
@@ -162,20 +170,22 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kLrThreads)
   }
 }
 
-void launch_lr_products(const MatView& A, const MatView& B, const MatView& C, const Plan& p,
-                        double* ws, double* scratch, int64_t scratch_per_cta, int dense_by_gemm,
-                        int grid, cudaStream_t st) {
-  // Eight CTAs a tile while the tiles are few (the 1D chain at N = 512: 16 tiles on 152 SMs),
-  // else four: from about 64 tiles on four already fill the SMs, with fewer exchanges.
-  if (p.nI * p.nJ <= 64) {
-    const int g = grid / 8 > 0 ? grid / 8 * 8 : 8;
-    lr_products_kernel<8><<<g, kLrThreads, 0, st>>>(A, B, C, p, ws, scratch, scratch_per_cta,
-                                                    dense_by_gemm);
-  } else {
-    const int g = grid / 4 > 0 ? grid / 4 * 4 : 4;
-    lr_products_kernel<4><<<g, kLrThreads, 0, st>>>(A, B, C, p, ws, scratch, scratch_per_cta,
-                                                    dense_by_gemm);
-  }
+int launch_lr_products(const MatView& A, const MatView& B, const MatView& C, const Plan& p,
+                       double* ws, double* scratch, int64_t scratch_per_cta, int grid,
+                       cudaStream_t st) {
+  // Eight CTAs a tile while the tiles are few (the 1D chain at N = 512: 16 tiles on 152 SMs), else
+  // four (from about 64 tiles on four already fill the SMs, with fewer exchanges) or one.  How many
+  // tiles have work is the device's to know: of two launches the one whose case it is not returns.
+  const int tiles = p.nI * p.nJ, few = kTilesPerCta * grid;
+  auto launch = [&](auto kernel, int cs) {
+    const int g = grid / cs > 0 ? grid / cs * cs : cs;
+    kernel<<<g, kLrThreads, 0, st>>>(A, B, C, p, ws, scratch, scratch_per_cta,
+                                     tiles > few ? few : 0);
+  };
+  if (tiles <= 64) launch(lr_products_kernel<8>, 8); else launch(lr_products_kernel<4>, 4);
+  if (tiles <= few) return 1;
+  launch(lr_products_kernel<1>, 1);
+  return 2;
 }
 
 }  // namespace clr

@@ -226,11 +226,16 @@ __global__ void __launch_bounds__(kScanThreads) plan_scan_kernel(Plan p, int rec
   const int chunk = (n + kScanThreads - 1) / kScanThreads;
   const int lo = min(n, tid * chunk), hi = min(n, lo + chunk);
   int s[kScanQ] = {0, 0, 0, 0, 0};
+  // with a tensor-core GEMM the dense tiles and the DACC_G tiles take every contribution there
+  // (low-rank operand blocks staged as X W^T)
+  auto takes_lr = [&](int i, int route) {
+    return p.t_rsum[i] > 0 && route != ROUTE_DACC_G && !(p.dense_by_gemm && route == ROUTE_DENSE);
+  };
   for (int i = lo; i < hi; ++i) {
     int route = p.t_route[i];
     s[0] += p.t_count[i];
     s[1] += route == ROUTE_DENSE;
-    s[2] += p.t_rsum[i] > 0;
+    s[2] += takes_lr(i, route);
     s[3] += route == ROUTE_QR;
     s[4] += route == ROUTE_DACC || route == ROUTE_DACC_G ||
             (route == ROUTE_DENSE && recompress_dense);
@@ -252,7 +257,7 @@ __global__ void __launch_bounds__(kScanThreads) plan_scan_kernel(Plan p, int rec
     p.t_start[i] = base[0];
     base[0] += p.t_count[i];
     if (route == ROUTE_DENSE) p.l_dense[base[1]++] = i;
-    if (p.t_rsum[i] > 0) p.l_lr[base[2]++] = i;
+    if (takes_lr(i, route)) p.l_lr[base[2]++] = i;
     if (route == ROUTE_QR) p.l_qr[base[3]++] = i;
     if (route == ROUTE_DACC || route == ROUTE_DACC_G ||
         (route == ROUTE_DENSE && recompress_dense))

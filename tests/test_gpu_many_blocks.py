@@ -1,0 +1,32 @@
+"""The forms of the kernels for many blocks, and for mostly zero ones, at the numbers of blocks where
+each begins, against plain FP64 (NumPy) or the oracle."""
+import numpy as np
+import pytest
+
+from oracle import clr_oracle as co
+from paper_1509_00309_gb300 import workloads as wl
+from tests import clr_pack
+from tests.test_gpu_product import _check_product
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1509_00309_gb300 import build, clr
+    build.build()
+    return clr.Context(0, precision="fp64", eps_lr=1e-8)
+
+
+# 676 tiles: each CTA takes its own (all with low-rank work, sums concatenated and accumulated
+# densely), or clusters do (few with work)
+@pytest.mark.parametrize("p_zero,p_dense,max_rank", [(0.1, 0.2, None), (0.7, 0.02, 2), (0.94, 0.02, 2)])
+def test_low_rank_products_of_many_tiles(ctx, p_zero, p_dense, max_rank):
+    sizes = [16, 1, 7, 33, 2, 20, 9, 3, 40, 12, 5, 8, 25] * 2
+    rng = np.random.default_rng(int(100 * p_zero))
+    a, b = (co.from_blocks(sizes, sizes, wl.random_blocks_spec(
+        rng, sizes, sizes, p_zero=p_zero, p_dense=p_dense, max_rank=max_rank)) for _ in range(2))
+    gc = ctx.multiply(clr_pack.to_library(ctx, a), clr_pack.to_library(ctx, b))
+    _check_product(ctx, a, b, 1e-8, gc)
