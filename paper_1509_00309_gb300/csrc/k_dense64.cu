@@ -205,17 +205,23 @@ void launch_set_route_kinds(const MatView& C, const Plan& p, cudaStream_t st) {
 }
 
 // Frobenius norms of the dense-accumulated tiles (those not recompressed afterwards): a cluster of
-// CTAs per tile, its parts added in a fixed order (with one CTA a tile's loads took 20 us).
+// CTAs per tile, its parts added in a fixed order (with one CTA a tile's loads took 20 us), while
+// the tiles are few (kNormFew a cluster: 512); beyond, CTAs fill the SMs with a tile each and a
+// cluster would only wait at its barriers (48400 tiles of at most 48^2: 2350 us by clusters, 330 by
+// CTAs).
 constexpr int kNormCtas = 8;
+constexpr int kNormGrid = 1024;
+constexpr int kNormFew = 4;
 __global__ void __cluster_dims__(kNormCtas, 1, 1) __launch_bounds__(256)
     dense_tile_norms_kernel(MatView C, Plan p) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ double red[8];
   __shared__ double part;
-  const int rank = (int)cluster.block_rank();
   const int n_items = p.counters->n_dense;
-  for (int it = blockIdx.x / kNormCtas; it < n_items; it += gridDim.x / kNormCtas) {
+  const bool alone = n_items > kNormFew * (int)(gridDim.x / kNormCtas);
+  const int rank = alone ? 0 : (int)cluster.block_rank(), ctas = alone ? 1 : kNormCtas;
+  for (int it = blockIdx.x / ctas; it < n_items; it += gridDim.x / ctas) {
     const int t = p.l_dense[it];
     const int I = t / p.nJ, J = t % p.nJ;
     const int m = C.row_off[I + 1] - C.row_off[I];
@@ -223,7 +229,7 @@ __global__ void __cluster_dims__(kNormCtas, 1, 1) __launch_bounds__(256)
     const double* D = C.pool + slot_of(C, I, J, m);
     double s = 0.0;
 #pragma unroll 4
-    for (int e = threadIdx.x + 256 * rank; e < m * n; e += 256 * kNormCtas) s = fma(D[e], D[e], s);
+    for (int e = threadIdx.x + 256 * rank; e < m * n; e += 256 * ctas) s = fma(D[e], D[e], s);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = s;
@@ -232,6 +238,11 @@ __global__ void __cluster_dims__(kNormCtas, 1, 1) __launch_bounds__(256)
       double tot = 0.0;
       for (int i = 0; i < 8; ++i) tot += red[i];
       part = tot;
+    }
+    if (alone) {
+      if (threadIdx.x == 0) C.norm[t] = sqrt(part);
+      __syncthreads();
+      continue;
     }
     cluster.sync();
     if (rank == 0 && threadIdx.x == 0) {
@@ -244,7 +255,7 @@ __global__ void __cluster_dims__(kNormCtas, 1, 1) __launch_bounds__(256)
 }
 
 void launch_dense_tile_norms(const MatView& C, const Plan& p, cudaStream_t st) {
-  dense_tile_norms_kernel<<<1024, 256, 0, st>>>(C, p);
+  dense_tile_norms_kernel<<<kNormGrid, 256, 0, st>>>(C, p);
 }
 
 __global__ void sqrt_dense_norms_kernel(MatView C, Plan p) {

@@ -30,3 +30,21 @@ def test_low_rank_products_of_many_tiles(ctx, p_zero, p_dense, max_rank):
         rng, sizes, sizes, p_zero=p_zero, p_dense=p_dense, max_rank=max_rank)) for _ in range(2))
     gc = ctx.multiply(clr_pack.to_library(ctx, a), clr_pack.to_library(ctx, b))
     _check_product(ctx, a, b, 1e-8, gc)
+
+
+# 529 and 484 dense tiles: a CTA a tile, or clusters; 1 x 1 tiles among them
+@pytest.mark.parametrize("nb", [22, 23])
+def test_norms_of_many_dense_tiles(ctx, nb):
+    sizes = ([40, 1, 17, 9, 64] * 5)[:nb]
+    n = sum(sizes)
+    rng = np.random.default_rng(nb)
+    a, b = rng.standard_normal((n, n)), rng.standard_normal((n, n))
+    norms = ctx.multiply(ctx.from_dense(a, sizes), ctx.from_dense(b, sizes)).get_blocks(pool=False)[2]
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    ab, mag = a @ b, np.abs(a) @ np.abs(b)
+    for i in range(nb):
+        for j in range(nb):
+            box = (slice(off[i], off[i + 1]), slice(off[j], off[j + 1]))
+            # n products and additions an entry on either side, m n <= 4096 squares
+            bound = 2.0 * (n + 4096) * U * np.linalg.norm(mag[box])
+            assert abs(norms[i, j] - np.linalg.norm(ab[box])) <= bound, (i, j)
