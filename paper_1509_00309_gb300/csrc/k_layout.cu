@@ -66,23 +66,27 @@ void launch_dense_kinds(const MatView& M, double drop_norm, int* err, cudaStream
 }
 
 // row-major out <- reconstruction of every block.  Dense blocks are bound by HBM (16 bytes an
-// element), low-rank ones by the FP64 pipe (rank FMAs an element).  A CTA takes a 64 x 64 tile and a
-// lane 16 of its elements, all of whose kinds and then values are loaded before the first is used:
-// with 32 x 32 tiles and a chain of index, kind and value loads per element the dense N = 16384
-// result took 1.73 ms, now 0.80 (4.3 GB: 0.63 at the copy rate).
-constexpr int kOutTile = 64;
+// element), low-rank ones by the FP64 pipe (rank FMAs an element).  A CTA takes a T x T tile and a
+// lane T / 32 of its rows in T / 8 adjacent columns, all of whose kinds and then dense values are
+// loaded before the first is used: with 32 x 32 tiles and a chain of index, kind and value loads per
+// element the dense N = 16384 result took 1.74 ms, with T = 64 0.77 (4.3 GB: 0.63 at the copy
+// rate).  Where the lane's columns lie in one block their low-rank sums run side by side: one load
+// of X a step for all of them, and no FMA waits for the one before (3D lattice, N = 8192: 4.22 ms, an
+// element at a time 4.74; its FMAs alone take 4.0).
+template <int T>
 __global__ void __launch_bounds__(256) pool_to_rowmajor_kernel(MatView M, const int* row_idx,
                                                                const int* col_idx, double* out,
                                                                int64_t ldo) {
-  __shared__ double tile[kOutTile][kOutTile + 1];
-  const int64_t tiles_r = (M.n_rows + kOutTile - 1) / kOutTile;
-  const int64_t r0 = (int64_t)(blockIdx.x % tiles_r) * kOutTile;
-  const int64_t c0 = (int64_t)(blockIdx.x / tiles_r) * kOutTile;
+  __shared__ double tile[T][T + 1];
+  constexpr int kRows = T / 32, kCols = T / 8;
+  const int64_t tiles_r = (M.n_rows + T - 1) / T;
+  const int64_t r0 = (int64_t)(blockIdx.x % tiles_r) * T;
+  const int64_t c0 = (int64_t)(blockIdx.x / tiles_r) * T;
   const int l = threadIdx.x % 32, w = threadIdx.x / 32;
-  int R[2], mR[2], rloc[2];
-  int64_t base[2];
+  int R[kRows], mR[kRows], rloc[kRows];
+  int64_t base[kRows];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < kRows; ++h) {
     const int64_t r = r0 + l + 32 * h;
     R[h] = r < M.n_rows ? row_idx[r] : -1;
     const int off = R[h] >= 0 ? M.row_off[R[h]] : 0;
@@ -90,54 +94,85 @@ __global__ void __launch_bounds__(256) pool_to_rowmajor_kernel(MatView M, const 
     rloc[h] = (int)(r - off);
     base[h] = (int64_t)off * M.n_cols + rloc[h];
   }
-  constexpr int kCols = kOutTile / 8;
-  int Cc[kCols], kind[kCols][2];
-  double v[kCols][2];
+  const int64_t cw = c0 + kCols * w;   // the warp's first column
+  unsigned dense = 0, lr = 0;          // by element: bit kRows q + h
+  bool one;                            // the warp's columns lie in one cluster
+  {
+    int Cc[kCols], kind[kCols][kRows];
 #pragma unroll
-  for (int q = 0; q < kCols; ++q) {
-    const int64_t c = c0 + w + 8 * q;
-    Cc[q] = c < M.n_cols ? col_idx[c] : -1;
-  }
-#pragma unroll
-  for (int q = 0; q < kCols; ++q)
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-      kind[q][h] = R[h] >= 0 && Cc[q] >= 0 ? M.kind[(int64_t)R[h] * M.nc + Cc[q]] : CLR_KIND_ZERO;
-  bool lr = false;
-#pragma unroll
-  for (int q = 0; q < kCols; ++q)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      v[q][h] = kind[q][h] == CLR_KIND_DENSE ? M.pool[base[h] + (c0 + w + 8 * q) * mR[h]] : 0.0;
-      lr = lr || kind[q][h] == CLR_KIND_LR;
-    }
-  if (lr) {
+    for (int q = 0; q < kCols; ++q) Cc[q] = cw + q < M.n_cols ? col_idx[cw + q] : -1;
 #pragma unroll
     for (int q = 0; q < kCols; ++q)
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        if (kind[q][h] == CLR_KIND_LR) {
-          const int coff = M.col_off[Cc[q]];
-          const int n = M.col_off[Cc[q] + 1] - coff;
-          const int rk = M.rank[(int64_t)R[h] * M.nc + Cc[q]];
-          const double* X = M.pool + base[h] - rloc[h] + (int64_t)mR[h] * coff;
-          const double* W = X + (int64_t)mR[h] * rk + (c0 + w + 8 * q - coff);
-          X += rloc[h];
-          double s = 0.0;
-          for (int k = 0; k < rk; ++k) s = fma(X[(int64_t)k * mR[h]], W[(int64_t)k * n], s);
-          v[q][h] = s;
-        }
+      for (int h = 0; h < kRows; ++h)
+        kind[q][h] = R[h] >= 0 && Cc[q] >= 0 ? M.kind[(int64_t)R[h] * M.nc + Cc[q]] : CLR_KIND_ZERO;
+#pragma unroll
+    for (int q = 0; q < kCols; ++q)
+#pragma unroll
+      for (int h = 0; h < kRows; ++h) {
+        dense |= (unsigned)(kind[q][h] == CLR_KIND_DENSE) << (kRows * q + h);
+        lr |= (unsigned)(kind[q][h] == CLR_KIND_LR) << (kRows * q + h);
+      }
+    one = Cc[0] >= 0 && Cc[0] == Cc[kCols - 1];
   }
+  {
+    double v[kCols][kRows];
 #pragma unroll
-  for (int q = 0; q < kCols; ++q)
+    for (int q = 0; q < kCols; ++q)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) tile[l + 32 * h][w + 8 * q] = v[q][h];
+      for (int h = 0; h < kRows; ++h)
+        v[q][h] = dense >> (kRows * q + h) & 1u ? M.pool[base[h] + (cw + q) * mR[h]] : 0.0;
+#pragma unroll
+    for (int q = 0; q < kCols; ++q)
+#pragma unroll
+      for (int h = 0; h < kRows; ++h) tile[l + 32 * h][kCols * w + q] = v[q][h];
+  }
+  // (the factors of the block of row h's cluster and column c)
+  auto factors = [&](int h, int64_t c, const double** X, const double** W, int* n) {
+    const int C = col_idx[c], coff = M.col_off[C];
+    const int rk = M.rank[(int64_t)R[h] * M.nc + C];
+    *n = M.col_off[C + 1] - coff;
+    *X = M.pool + base[h] + (int64_t)mR[h] * coff;
+    *W = *X - rloc[h] + (int64_t)mR[h] * rk + (c - coff);
+    return rk;
+  };
+#pragma unroll
+  for (int h = 0; h < kRows; ++h) {
+    const double *X, *W;
+    int n;
+    double* to = &tile[l + 32 * h][kCols * w];
+    if (one) {
+      if (!(lr >> h & 1u)) continue;
+      const int rk = factors(h, cw, &X, &W, &n);
+      double s[kCols];
+#pragma unroll
+      for (int q = 0; q < kCols; ++q) s[q] = 0.0;
+#pragma unroll 2
+      for (int k = 0; k < rk; ++k) {
+        const double x = *X;
+        X += mR[h];
+#pragma unroll
+        for (int q = 0; q < kCols; ++q) s[q] = fma(x, W[q], s[q]);
+        W += n;
+      }
+#pragma unroll
+      for (int q = 0; q < kCols; ++q) to[q] = s[q];
+    } else {
+      for (int q = 0; q < kCols; ++q) {
+        if (!(lr >> (kRows * q + h) & 1u)) continue;
+        const int rk = factors(h, cw + q, &X, &W, &n);
+        double s = 0.0;
+        for (int k = 0; k < rk; ++k) s = fma(X[(int64_t)k * mR[h]], W[(int64_t)k * n], s);
+        to[q] = s;
+      }
+    }
+  }
   __syncthreads();
-  for (int rr = w; rr < kOutTile; rr += 8) {
+  for (int rr = w; rr < T; rr += 8) {
     const int64_t r = r0 + rr;
     if (r >= M.n_rows) break;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < kRows; ++h) {
       const int64_t c = c0 + l + 32 * h;
       if (c < M.n_cols) out[r * ldo + c] = tile[rr][l + 32 * h];
     }
@@ -146,9 +181,13 @@ __global__ void __launch_bounds__(256) pool_to_rowmajor_kernel(MatView M, const 
 
 void launch_pool_to_rowmajor(const MatView& M, const int* row_idx, const int* col_idx,
                              double* out, int64_t ldo, cudaStream_t st) {
-  const int64_t n =
-      ((M.n_rows + kOutTile - 1) / kOutTile) * ((M.n_cols + kOutTile - 1) / kOutTile);
-  pool_to_rowmajor_kernel<<<(unsigned)n, 256, 0, st>>>(M, row_idx, col_idx, out, ldo);
+  // T = 64 once such tiles are enough (N = 512 to 4096 with low rank blocks: 77 to 1190 us with 64,
+  // 44 to 1127 with 32; dense N = 4096 66 and 80, N = 16384 0.77 and 1.0 ms)
+  auto tiles = [&](int64_t t) { return ((M.n_rows + t - 1) / t) * ((M.n_cols + t - 1) / t); };
+  if (tiles(64) > 4096)
+    pool_to_rowmajor_kernel<64><<<(unsigned)tiles(64), 256, 0, st>>>(M, row_idx, col_idx, out, ldo);
+  else
+    pool_to_rowmajor_kernel<32><<<(unsigned)tiles(32), 256, 0, st>>>(M, row_idx, col_idx, out, ldo);
 }
 
 }  // namespace clr

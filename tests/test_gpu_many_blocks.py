@@ -48,3 +48,30 @@ def test_norms_of_many_dense_tiles(ctx, nb):
             # n products and additions an entry on either side, m n <= 4096 squares
             bound = 2.0 * (n + 4096) * U * np.linalg.norm(mag[box])
             assert abs(norms[i, j] - np.linalg.norm(ab[box])) <= bound, (i, j)
+
+
+# 64 x 64 tiles from 4097 tiles on, 32 x 32 below; warps whose columns lie in one block and in
+# several, all zero, and ragged edges
+@pytest.mark.parametrize("big,sizes", [
+    (False, [256, 1, 100, 7, 33]), (True, [256, 200, 31, 1, 180, 64, 3] * 6 + [97]),
+    (True, [5, 1, 3, 17, 8, 2, 33, 9] * 53 + [63]),
+])
+def test_reconstruction_by_either_tile(ctx, big, sizes):
+    n = sum(sizes)
+    assert (((n + 63) // 64) ** 2 > 4096) == big
+    rng = np.random.default_rng(n)
+    many = len(sizes) > 100
+    a = co.from_blocks(sizes, sizes, wl.random_blocks_spec(
+        rng, sizes, sizes, p_zero=0.6 if many else 0.2, p_dense=0.2))
+    got = clr_pack.to_library(ctx, a).to_dense()
+    zero = np.ones((n, n), bool)
+    for (i, j), b in a.blocks.items():
+        box = (slice(a.row_off[i], a.row_off[i + 1]), slice(a.col_off[j], a.col_off[j + 1]))
+        zero[box] = False
+        if b.kind == co.KIND_DENSE:
+            assert np.array_equal(got[box], b.d)
+        else:
+            # ranks of at most 128
+            assert (np.abs(got[box] - b.x @ b.w.T)
+                    <= 2.0 * 130 * U * (np.abs(b.x) @ np.abs(b.w).T)).all()
+    assert (got[zero] == 0.0).all()
