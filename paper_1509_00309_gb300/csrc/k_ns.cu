@@ -58,21 +58,20 @@ __global__ void lincomb_route_kernel(double a, MatView X, double b, MatView Y, d
   // the copy case is re-derived by the apply kernel from the operand kinds
 }
 
-// A cluster of CTAs per block, its elements in turn (a dense sum of low-rank blocks takes m n r
+// A cluster of CS CTAs per block, its elements in turn (a dense sum of low-rank blocks takes m n r
 // FMAs on the FP64 pipe, and with one CTA per block the largest block was the kernel's time: 4.9 ms
 // for the 3D lattice's iterates at N = 2048, now 1.2); the norm's parts are added in a fixed order.
-constexpr int kLcCtas = 8;
-
-__global__ void __cluster_dims__(kLcCtas, 1, 1) __launch_bounds__(kT)
+template <int CS>
+__global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kT)
     lincomb_apply_kernel(double a, MatView X, double b, MatView Y, double diag, MatView O, Plan p,
                          double* ws) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ double red[kT / 32];
   __shared__ double part_sq;
-  const int t = blockIdx.x / kLcCtas, rank = (int)cluster.block_rank();
+  const int t = blockIdx.x / CS, rank = (int)cluster.block_rank();
   const int tid = threadIdx.x + kT * rank;
-  constexpr int kAll = kT * kLcCtas;
+  constexpr int kAll = kT * CS;
   const int I = t / p.nJ, J = t % p.nJ;
   const int m = X.row_off[I + 1] - X.row_off[I];
   const int n = X.col_off[J + 1] - X.col_off[J];
@@ -143,7 +142,7 @@ __global__ void __cluster_dims__(kLcCtas, 1, 1) __launch_bounds__(kT)
   cluster.sync();
   if (tid == 0) {
     double nsq = 0.0;
-    for (int c = 0; c < kLcCtas; ++c) nsq += *cluster.map_shared_rank(&part_sq, c);
+    for (int c = 0; c < CS; ++c) nsq += *cluster.map_shared_rank(&part_sq, c);
     O.kind[t] = CLR_KIND_DENSE;
     O.rank[t] = m < n ? m : n;
     O.norm[t] = sqrt(nsq);
@@ -160,7 +159,16 @@ void launch_lincomb_plan(double a, const MatView& X, double b, const MatView& Y,
   cudaMemsetAsync(p.counters, 0, kPlanCountersClear, st);
   lincomb_route_kernel<<<(n + 127) / 128, 128, 0, st>>>(a, X, b, Y, diag, p);
   launch_plan_scan(p, recompress_dense, st);
-  lincomb_apply_kernel<<<n * kLcCtas, kT, 0, st>>>(a, X, b, Y, diag, O, p, ws);
+  // CTAs per block, fewer the more blocks there are: starting CTAs for blocks without work is then
+  // what the launch takes (a sum of 141376 blocks, 1126 of them not zero: 2840 us with recompression
+  // by eights, 1360 by ones; 8281 blocks, 3D lattice: 95.3 and 97.9 ms, by twos 95.9; 2116: equal
+  // with 8 and 4).  A scaled copy has no FMAs to share: by ones from 3072 on (8100 blocks, chain:
+  // 214, 134 and 123 us by eights, twos and ones).
+  const int many = a == 0.0 || b == 0.0 ? 3072 : 16384;
+  if (n <= 1024) lincomb_apply_kernel<8><<<n * 8, kT, 0, st>>>(a, X, b, Y, diag, O, p, ws);
+  else if (n <= 3072) lincomb_apply_kernel<4><<<n * 4, kT, 0, st>>>(a, X, b, Y, diag, O, p, ws);
+  else if (n <= many) lincomb_apply_kernel<2><<<n * 2, kT, 0, st>>>(a, X, b, Y, diag, O, p, ws);
+  else lincomb_apply_kernel<1><<<n, kT, 0, st>>>(a, X, b, Y, diag, O, p, ws);
 }
 
 // Per block: ||M_IJ - delta_IJ I||_F^2, then a deterministic single-CTA sum.

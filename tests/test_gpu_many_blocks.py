@@ -50,6 +50,33 @@ def test_norms_of_many_dense_tiles(ctx, nb):
             assert abs(norms[i, j] - np.linalg.norm(ab[box])) <= bound, (i, j)
 
 
+# clusters of eight up to 1024 blocks, four up to 3072, two, one beyond 16384 (a scaled copy: beyond
+# 3072)
+@pytest.mark.parametrize("nb,p_zero", [(32, 0.3), (33, 0.3), (56, 0.5), (129, 0.97)])
+def test_linear_combination_of_many_blocks(ctx, nb, p_zero):
+    sizes = ([3, 1, 20, 9, 12, 2, 33] * 19)[:nb]
+    rng = np.random.default_rng(nb)
+    x, y = (co.from_blocks(sizes, sizes, wl.random_blocks_spec(rng, sizes, sizes, p_zero=p_zero,
+                                                               p_dense=0.5 * (1 - p_zero)))
+            for _ in range(2))
+    gx, gy = clr_pack.to_library(ctx, x), clr_pack.to_library(ctx, y)
+    n, dx, dy = sum(sizes), x.to_dense(), y.to_dense()
+    off = x.row_off
+    for a, b, diag in ((-1.25, 0.375, 1.875), (0.75, 0.0, 0.0), (0.0, 0.5, 0.0)):
+        out = ctx.lincomb(a, gx, b, gy, diag)
+        got, want = out.to_dense(), a * dx + b * dy + diag * np.eye(n)
+        norms = out.get_blocks(pool=False)[2]
+        # truncation at 1e-8 a block (none in a copy); 33 squares and products of entries of order 10
+        eps = 1e-8 if a != 0.0 and b != 0.0 else 0.0
+        for i in range(nb):
+            for j in range(nb):
+                box = (slice(off[i], off[i + 1]), slice(off[j], off[j + 1]))
+                w = np.linalg.norm(want[box])
+                tol = eps * (1 + 1e-6) + 1e-11
+                assert np.linalg.norm(got[box] - want[box]) <= tol, (a, i, j)
+                assert abs(norms[i, j] - w) <= tol, (a, i, j)
+
+
 # 64 x 64 tiles from 4097 tiles on, 32 x 32 below; warps whose columns lie in one block and in
 # several, all zero, and ragged edges
 @pytest.mark.parametrize("big,sizes", [
