@@ -229,23 +229,24 @@ void launch_identity_distance(const MatView& X, double* out_sq, cudaStream_t st)
 
 // y_I = sum_J M_IJ x_J.  Bound by reading the blocks once (70 MB for the 3D lattice at N = 4096)
 // and by the FP64 pipe (an FMA per double read), 15 us each there, so the block-row is spread
-// over a cluster of 8 CTAs (blocks J in turn) whose partial sums are added, in a fixed order,
+// over a cluster of CS CTAs (blocks J in turn) whose partial sums are added, in a fixed order,
 // through distributed shared memory: no workspace, so calls on different streams do not meet.
-// (One CTA per block-row, walking its blocks one after the other, took 690 us;
-// this takes 60.)  Inside a CTA a warp
-// takes four columns of W at a time for W^T x and sums them together; for X t (and dense blocks)
-// it owns a group of 32 rows and a share of the columns, its row sums in registers until the end.
-constexpr int kMvCtas = 8;
+// (One CTA per block-row, walking its blocks one after the other, took 690 us; eight take 60.)
+// Inside a CTA a warp takes four columns of W at a time for W^T x and sums them together; for X t
+// (and dense blocks) it owns a group of 32 rows and a share of the columns, its row sums in
+// registers until the end.  The kinds of 32 of the CTA's blocks are read at once: in a chain matrix
+// nearly all are zero, and read one after the other they were most of the time.
 constexpr int kMvThreads = 512;
 constexpr int kMvWarps = kMvThreads / 32;
 
-__global__ void __cluster_dims__(kMvCtas, 1, 1) __launch_bounds__(kMvThreads)
+template <int CS>
+__global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kMvThreads)
     matvec_kernel(MatView M, const double* x, double* y) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ double part[kMvWarps][CLR_MAX_CLUSTER];   // [0] ends as this CTA's sum
   __shared__ double tw[2][CLR_MAX_CLUSTER / 2];
-  const int I = blockIdx.x / kMvCtas, rank = (int)cluster.block_rank();
+  const int I = blockIdx.x / CS, rank = (int)cluster.block_rank();
   const int m = M.row_off[I + 1] - M.row_off[I];
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
   const int groups = (m + 31) / 32, slices = kMvWarps / groups;
@@ -253,51 +254,55 @@ __global__ void __cluster_dims__(kMvCtas, 1, 1) __launch_bounds__(kMvThreads)
   const bool mine = slice < slices && i < m;
   double acc = 0.0;
   int buf = 0;
-  for (int J = rank; J < M.nc; J += kMvCtas) {
-    const int t = I * M.nc + J;
-    const int kind = M.kind[t];
-    if (kind == CLR_KIND_ZERO) continue;
-    const int n = M.col_off[J + 1] - M.col_off[J];
-    const double* s = M.pool + slot_of(M, I, J, m);
-    const double* xj = x + M.col_off[J];
-    const double* v = xj;
-    int cols = n;
-    if (kind == CLR_KIND_LR) {
-      const int r = M.rank[t];
-      const double* W = s + (int64_t)m * r;
-      for (int c0 = 4 * w; c0 < r; c0 += 4 * kMvWarps) {
-        double d[4] = {0.0, 0.0, 0.0, 0.0};
-        const double* wc[4];
+  for (int J0 = rank; J0 < M.nc; J0 += 32 * CS) {
+    const int Jl = J0 + l * CS;
+    const int kind = Jl < M.nc ? M.kind[I * M.nc + Jl] : CLR_KIND_ZERO;
+    const unsigned lr = __ballot_sync(0xffffffffu, kind == CLR_KIND_LR);
+    for (unsigned todo = __ballot_sync(0xffffffffu, kind != CLR_KIND_ZERO); todo; todo &= todo - 1) {
+      const int bit = __ffs(todo) - 1, J = J0 + bit * CS;
+      const int t = I * M.nc + J;
+      const int n = M.col_off[J + 1] - M.col_off[J];
+      const double* s = M.pool + slot_of(M, I, J, m);
+      const double* xj = x + M.col_off[J];
+      const double* v = xj;
+      int cols = n;
+      if (lr >> bit & 1u) {
+        const int r = M.rank[t];
+        const double* W = s + (int64_t)m * r;
+        for (int c0 = 4 * w; c0 < r; c0 += 4 * kMvWarps) {
+          double d[4] = {0.0, 0.0, 0.0, 0.0};
+          const double* wc[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) wc[c] = W + (int64_t)(c0 + c < r ? c0 + c : c0) * n;
+          for (int c = 0; c < 4; ++c) wc[c] = W + (int64_t)(c0 + c < r ? c0 + c : c0) * n;
 #pragma unroll 4
-        for (int j = l; j < n; j += 32) {
-          const double xv = xj[j];
+          for (int j = l; j < n; j += 32) {
+            const double xv = xj[j];
 #pragma unroll
-          for (int c = 0; c < 4; ++c) d[c] = fma(wc[c][j], xv, d[c]);
+            for (int c = 0; c < 4; ++c) d[c] = fma(wc[c][j], xv, d[c]);
+          }
+          // lane l: the sum of column c0 + l / 8
+          const bool h16 = (l & 16) != 0, h8 = (l & 8) != 0;
+          double a0 = h16 ? d[2] : d[0], a1 = h16 ? d[3] : d[1];
+          a0 += __shfl_xor_sync(0xffffffffu, h16 ? d[0] : d[2], 16);
+          a1 += __shfl_xor_sync(0xffffffffu, h16 ? d[1] : d[3], 16);
+          double a = h8 ? a1 : a0;
+          a += __shfl_xor_sync(0xffffffffu, h8 ? a0 : a1, 8);
+          a += __shfl_xor_sync(0xffffffffu, a, 4);
+          a += __shfl_xor_sync(0xffffffffu, a, 2);
+          a += __shfl_xor_sync(0xffffffffu, a, 1);
+          if (l % 8 == 0 && c0 + l / 8 < r) tw[buf][c0 + l / 8] = a;
         }
-        // lane l: the sum of column c0 + l / 8
-        const bool h16 = (l & 16) != 0, h8 = (l & 8) != 0;
-        double a0 = h16 ? d[2] : d[0], a1 = h16 ? d[3] : d[1];
-        a0 += __shfl_xor_sync(0xffffffffu, h16 ? d[0] : d[2], 16);
-        a1 += __shfl_xor_sync(0xffffffffu, h16 ? d[1] : d[3], 16);
-        double a = h8 ? a1 : a0;
-        a += __shfl_xor_sync(0xffffffffu, h8 ? a0 : a1, 8);
-        a += __shfl_xor_sync(0xffffffffu, a, 4);
-        a += __shfl_xor_sync(0xffffffffu, a, 2);
-        a += __shfl_xor_sync(0xffffffffu, a, 1);
-        if (l % 8 == 0 && c0 + l / 8 < r) tw[buf][c0 + l / 8] = a;
+        // (the other buffer is written only past the next barrier: one barrier per block)
+        __syncthreads();
+        v = tw[buf];
+        cols = r;
+        buf ^= 1;
       }
-      // (the other buffer is written only past the next barrier: one barrier per block)
-      __syncthreads();
-      v = tw[buf];
-      cols = r;
-      buf ^= 1;
-    }
-    if (mine) {
-      const double* si = s + i;
+      if (mine) {
+        const double* si = s + i;
 #pragma unroll 8
-      for (int c = slice; c < cols; c += slices) acc = fma(si[(int64_t)c * m], v[c], acc);
+        for (int c = slice; c < cols; c += slices) acc = fma(si[(int64_t)c * m], v[c], acc);
+      }
     }
   }
   if (mine) part[slice][i] = acc;
@@ -308,16 +313,20 @@ __global__ void __cluster_dims__(kMvCtas, 1, 1) __launch_bounds__(kMvThreads)
     part[0][r] = sum;
   }
   cluster.sync();
-  for (int r = rank + kMvCtas * threadIdx.x; r < m; r += kMvCtas * kMvThreads) {
+  for (int r = rank + CS * threadIdx.x; r < m; r += CS * kMvThreads) {
     double sum = 0.0;
-    for (int q = 0; q < kMvCtas; ++q) sum += cluster.map_shared_rank(&part[0][0], q)[r];
+    for (int q = 0; q < CS; ++q) sum += cluster.map_shared_rank(&part[0][0], q)[r];
     y[M.row_off[I] + r] = sum;
   }
   cluster.sync();   // no CTA's shared memory goes before the others have read it
 }
 
 void launch_matvec(const MatView& M, const double* x, double* y, cudaStream_t st) {
-  matvec_kernel<<<M.nr * kMvCtas, kMvThreads, 0, st>>>(M, x, y);
+  // Eight CTAs a block-row while that makes at most six rounds of the two an SM holds; beyond, two
+  // (chain matrices, 259 and 376 block-rows: 79 and 65 us by eights, 40 and 33 by twos; full ones at
+  // 91 and 220 block-rows: 359 and 486 us by eights, 496 and 563 by twos).
+  if (M.nr <= 228) matvec_kernel<8><<<M.nr * 8, kMvThreads, 0, st>>>(M, x, y);
+  else matvec_kernel<2><<<M.nr * 2, kMvThreads, 0, st>>>(M, x, y);
 }
 
 // T = S^T: block (J,I) of T is block (I,J) of S transposed (dense, 32 x 32 tiles through shared

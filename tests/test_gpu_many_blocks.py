@@ -77,6 +77,27 @@ def test_linear_combination_of_many_blocks(ctx, nb, p_zero):
                 assert abs(norms[i, j] - w) <= tol, (a, i, j)
 
 
+# two CTAs a block-row from 229 on; more blocks in a row than 32 a CTA looks at at once (64 and 256)
+@pytest.mark.parametrize("nr,nc,p_zero", [(229, 70, 0.9), (229, 5, 0.2), (3, 300, 0.97), (2, 513, 0.5)])
+def test_matvec_of_many_blocks(ctx, nr, nc, p_zero):
+    import torch
+    rng = np.random.default_rng(nr + nc)
+    rows, cols = ([3, 40, 1, 17, 70] * 46)[:nr], ([5, 1, 33, 9] * 129)[:nc]
+    a = co.from_blocks(rows, cols, wl.random_blocks_spec(rng, rows, cols, p_zero=p_zero,
+                                                         p_dense=0.5 * (1 - p_zero)))
+    da = a.to_dense()
+    mag = np.zeros(da.shape)
+    for (i, j), b in a.blocks.items():
+        mag[a.row_off[i]:a.row_off[i + 1], a.col_off[j]:a.col_off[j + 1]] = (
+            np.abs(b.d) if b.kind == co.KIND_DENSE else np.abs(b.x) @ np.abs(b.w).T)
+    x = rng.standard_normal(sum(cols))
+    y = torch.empty(sum(rows), dtype=torch.float64, device="cuda")
+    ctx.matvec(clr_pack.to_library(ctx, a), torch.from_numpy(x).cuda(), y)
+    # ranks of at most 35, n terms, on either side
+    bound = 2.0 * (sum(cols) + 35) * U * (mag @ np.abs(x))
+    assert (np.abs(y.cpu().numpy() - da @ x) <= bound).all()
+
+
 # 64 x 64 tiles from 4097 tiles on, 32 x 32 below; warps whose columns lie in one block and in
 # several, all zero, and ragged edges
 @pytest.mark.parametrize("big,sizes", [
