@@ -330,44 +330,65 @@ void launch_matvec(const MatView& M, const double* x, double* y, cudaStream_t st
 }
 
 // T = S^T: block (J,I) of T is block (I,J) of S transposed (dense, 32 x 32 tiles through shared
-// memory so that both sides are accessed along their columns) or with X and W swapped.  Several
-// CTAs per block (lr_parts).
-__global__ void __launch_bounds__(256) transpose_kernel(MatView S, MatView T) {
+// memory so that both sides are accessed along their columns) or with X and W swapped.  Bound by
+// HBM; several parts per block where blocks alone are too few or too large to spread evenly.  A CTA
+// looks at 32 of its (block, part) items at once, as in a chain matrix nearly all are zero (67081
+// blocks, 775 not zero: 129 us with the allocation, 208 with a CTA per block).
+constexpr unsigned kTransposeCtas = 9728;   // eight rounds of what 152 SMs hold
+
+__global__ void __launch_bounds__(256) transpose_kernel(MatView S, MatView T, unsigned parts) {
   __shared__ double tile[32][33];
-  const int t = blockIdx.x;
-  const int I = t / S.nc, J = t % S.nc;
-  const int m = S.row_off[I + 1] - S.row_off[I];
-  const int n = S.col_off[J + 1] - S.col_off[J];
-  const int kind = S.kind[t], r = S.rank[t];
-  const double* s = S.pool + slot_of(S, I, J, m);
-  const int tt = J * T.nc + I;
-  double* d = T.pool + slot_of(T, J, I, n);
-  if (kind == CLR_KIND_DENSE) {
-    const int ti = (m + 31) / 32, tj = (n + 31) / 32, x = threadIdx.x % 32, y = threadIdx.x / 32;
-    for (int q = blockIdx.y; q < ti * tj; q += gridDim.y) {
-      const int i0 = (q % ti) * 32, j0 = (q / ti) * 32;
-      for (int c = y; c < 32; c += 8)
-        if (i0 + x < m && j0 + c < n) tile[c][x] = s[i0 + x + (int64_t)(j0 + c) * m];
-      __syncthreads();
-      for (int c = y; c < 32; c += 8)
-        if (j0 + x < n && i0 + c < m) d[j0 + x + (int64_t)(i0 + c) * n] = tile[x][c];
-      __syncthreads();
+  const int l = threadIdx.x % 32, w = threadIdx.x / 32;
+  const unsigned items = (unsigned)(S.nr * S.nc) * parts;
+  for (unsigned it0 = blockIdx.x; it0 < items; it0 += 32 * gridDim.x) {
+    const unsigned own = it0 + l * gridDim.x;
+    int kind = CLR_KIND_ZERO;
+    if (own < items) {
+      const int t = (int)(own / parts);
+      kind = S.kind[t];
+      if (w == 0 && own % parts == 0) {
+        const int tt = t % S.nc * T.nc + t / S.nc;
+        T.kind[tt] = kind;
+        T.rank[tt] = S.rank[t];
+        T.norm[tt] = S.norm[t];
+      }
     }
-  } else if (kind == CLR_KIND_LR) {
-    const int e0 = threadIdx.x + blockDim.x * blockIdx.y, step = blockDim.x * gridDim.y;
-    for (int e = e0; e < n * r; e += step) d[e] = s[(int64_t)m * r + e];
-    for (int e = e0; e < m * r; e += step) d[(int64_t)n * r + e] = s[e];
-  }
-  if (threadIdx.x == 0 && blockIdx.y == 0) {
-    T.kind[tt] = kind;
-    T.rank[tt] = r;
-    T.norm[tt] = S.norm[t];
+    const unsigned dense = __ballot_sync(0xffffffffu, kind == CLR_KIND_DENSE);
+    for (unsigned todo = __ballot_sync(0xffffffffu, kind != CLR_KIND_ZERO); todo; todo &= todo - 1) {
+      const unsigned bit = __ffs(todo) - 1, it = it0 + bit * gridDim.x;
+      const int t = (int)(it / parts), part = (int)(it % parts), np = (int)parts;
+      const int I = t / S.nc, J = t % S.nc;
+      const int m = S.row_off[I + 1] - S.row_off[I];
+      const int n = S.col_off[J + 1] - S.col_off[J];
+      const double* s = S.pool + slot_of(S, I, J, m);
+      double* d = T.pool + slot_of(T, J, I, n);
+      if (dense >> bit & 1u) {
+        const int ti = (m + 31) / 32, tj = (n + 31) / 32;
+        for (int q = part; q < ti * tj; q += np) {
+          const int i0 = (q % ti) * 32, j0 = (q / ti) * 32;
+          for (int c = w; c < 32; c += 8)
+            if (i0 + l < m && j0 + c < n) tile[c][l] = s[i0 + l + (int64_t)(j0 + c) * m];
+          __syncthreads();
+          for (int c = w; c < 32; c += 8)
+            if (j0 + l < n && i0 + c < m) d[j0 + l + (int64_t)(i0 + c) * n] = tile[l][c];
+          __syncthreads();
+        }
+      } else {
+        const int r = S.rank[t], e0 = threadIdx.x + 256 * part, step = 256 * np;
+        for (int e = e0; e < n * r; e += step) d[e] = s[(int64_t)m * r + e];
+        for (int e = e0; e < m * r; e += step) d[(int64_t)n * r + e] = s[e];
+      }
+    }
   }
 }
 
 void launch_transpose(const MatView& S, const MatView& T, cudaStream_t st) {
-  transpose_kernel<<<dim3((unsigned)(S.nr * S.nc), (unsigned)lr_parts(S.nr * S.nc)), 256, 0,
-                     st>>>(S, T);
+  const int64_t nb = (int64_t)S.nr * S.nc, area = S.n_rows * S.n_cols / nb;
+  // (3D lattice, 4624 and 8281 blocks of 180^2: 337 and 430 us with one part, 249 and 327 with four,
+  // as fast as with eight; 48400 blocks of 37^2: 229 with one, 337 with four)
+  const unsigned parts = nb <= 1024 ? 8 : area >= 8192 ? 4 : area >= 4096 ? 2 : 1;
+  const unsigned items = (unsigned)nb * parts;
+  transpose_kernel<<<items < kTransposeCtas ? items : kTransposeCtas, 256, 0, st>>>(S, T, parts);
 }
 
 }  // namespace clr

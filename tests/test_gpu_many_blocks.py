@@ -98,6 +98,22 @@ def test_matvec_of_many_blocks(ctx, nr, nc, p_zero):
     assert (np.abs(y.cpu().numpy() - da @ x) <= bound).all()
 
 
+# one part a block and more blocks than CTAs; two, four and eight parts; mostly zero
+@pytest.mark.parametrize("sizes,p_zero", [
+    ([1, 20, 7] * 34, 0.3), ([70, 61, 66] * 11, 0.3), ([100, 93, 130] * 11, 0.6), ([256, 40] * 3, 0.1),
+    ([1, 20, 7] * 110, 0.999),
+])
+def test_transposes_of_many_blocks(ctx, sizes, p_zero):
+    rng = np.random.default_rng(len(sizes))
+    a = co.from_blocks(sizes, sizes, wl.random_blocks_spec(rng, sizes, sizes, p_zero=p_zero,
+                                                           p_dense=0.5 * (1 - p_zero)))
+    ga = clr_pack.to_library(ctx, a)
+    gt = ctx.transpose(ga)
+    assert np.array_equal(gt.to_dense(), ga.to_dense().T)
+    for x, y in zip(ga.get_blocks(pool=False)[:3], gt.get_blocks(pool=False)[:3]):
+        assert np.array_equal(x.T, y)
+
+
 # 64 x 64 tiles from 4097 tiles on, 32 x 32 below; warps whose columns lie in one block and in
 # several, all zero, and ragged edges
 @pytest.mark.parametrize("big,sizes", [
