@@ -460,14 +460,15 @@ __device__ __forceinline__ void rotation(double al, double be, double g, double&
   // zeta in FP64 (the operands may lie far outside the FP32 range).  For a large angle
   // (|cos| > 1e-3: the first sweeps of a fresh start, nearly parallel columns) the tangent in
   // FP64, since a rotation that is off by u32 there leaves a leak that is large relative to the
-  // smaller column; for the small angles of a refinement in FP32 where |zeta| < 2^40, else its
-  // asymptote 1 / (2 zeta).
+  // smaller column; for the small angles of a refinement in FP32 where |zeta| < 2^100 (from 2^40 on,
+  // where its square may overflow, by the asymptote 1 / (2 zeta)), else the asymptote in FP64.
   const double zeta = (be - al) / (2.0 * g);
   if (g * g > 1e-6 * (al * be)) {
     t = copysign(1.0 / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0))), zeta);
-  } else if (fabs(zeta) < 0x1p40) {
-    const float z = (float)zeta;
-    t = (double)copysignf(__fdividef(1.f, fabsf(z) + sqrtf(1.f + z * z)), z);
+  } else if (fabs(zeta) < 0x1p100) {
+    const float z = (float)zeta, az = fabsf(z), w = fmaf(z, z, 1.f);
+    t = (double)(az > 0x1p40f ? __fdividef(0.5f, z)
+                              : copysignf(__fdividef(1.f, az + w * rsqrtf(w)), z));
   } else {
     t = 0.5 / zeta;
   }
@@ -485,22 +486,21 @@ struct JacobiShared {
   int rotated, sweeps;
 };
 
-// One-sided Jacobi in FP64 on the q columns of g (p x q, ld p); v (q x q, element (i, c) at
-// v[i v_r + c v_c]) accumulates the rotations, from I when reset is set.  On return g = U S and the
-// input equals g v^T (times the initial v^T when v is not reset).  Pairs whose
+// One-sided Jacobi in FP64 on the q columns of g (p x q, ld p); v (q x q) accumulates the rotations:
+// kOnto: onto its contents, row-major, else from I, column-major.  On return g = U S and the
+// input equals g v^T (times the initial v^T where v is not reset).  Pairs whose
 // inner product is below floor2, or below the FP64 epsilon times sqrt(p) relative to the norms,
 // are left alone.  Returns the number of sweeps.  jac: its norms' place holds the column norms
 // squared, recomputed exactly at every sweep start and refreshed (fused into the rotation pass) for
 // the two columns of every rotated pair, so a pair costs one inner product unless it is rotated.
-__device__ __noinline__ int jacobi_svd(double* g, int p, int q, double* v, int64_t v_r, int64_t v_c,
-                                       bool reset, int max_sweeps, int* sh_flag, double floor2,
-                                       JacobiShared& jac) {
+template <bool kOnto>
+__device__ __noinline__ int jacobi_svd(double* g, int p, int q, double* v, int max_sweeps,
+                                       int* sh_flag, double floor2, JacobiShared& jac) {
   double* nrm2 = reinterpret_cast<double*>(jac.nrm);
   int* last_rot = jac.last_rot;   // the step (sweep * (qq - 1) + round) of its last rotation, -1
   const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  if (reset)
-    for (int e = threadIdx.x; e < q * q; e += kThreads)
-      v[e % q * v_r + e / q * v_c] = (e % q == e / q) ? 1.0 : 0.0;
+  if (!kOnto)
+    for (int e = threadIdx.x; e < q * q; e += kThreads) v[e] = (e % q == e / q) ? 1.0 : 0.0;
   const int qq = q + (q & 1);  // even number of slots; slot q is a dummy when q is odd
   const double tol = DBL_EPSILON * sqrt((double)p);
   for (int c = threadIdx.x; c < q; c += kThreads) last_rot[c] = -1;
@@ -533,6 +533,7 @@ __device__ __noinline__ int jacobi_svd(double* g, int p, int q, double* v, int64
         double xa[kRowsPerLane], xb[kRowsPerLane], d = 0;
 #pragma unroll
         for (int j = 0; j < kRowsPerLane; ++j) {
+          if (32 * j >= p) break;
           const int i = l + 32 * j;
           xa[j] = i < p ? ga[i] : 0.0;
           xb[j] = i < p ? gb[i] : 0.0;
@@ -544,6 +545,7 @@ __device__ __noinline__ int jacobi_svd(double* g, int p, int q, double* v, int64
         rotation(al, be, d, c, sn, t);
 #pragma unroll
         for (int j = 0; j < kRowsPerLane; ++j) {
+          if (32 * j >= p) break;
           const int i = l + 32 * j;
           if (i < p) {
             ga[i] = c * xa[j] - sn * xb[j];
@@ -563,8 +565,9 @@ __device__ __noinline__ int jacobi_svd(double* g, int p, int q, double* v, int64
           na = warp_sum(sa);
           nb = warp_sum(sb);
         }
-        double* va = v + a * v_c;
-        double* vb = v + b * v_c;
+        double* va = v + (kOnto ? a : a * q);
+        double* vb = v + (kOnto ? b : b * q);
+        const int v_r = kOnto ? q : 1;
         for (int i = l; i < q; i += 32) {
           const double x = va[i * v_r], y = vb[i * v_r];
           va[i * v_r] = c * x - sn * y;
@@ -1520,7 +1523,7 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
   // cycles of the lattice product's recompression at N = 4096, of graded factors.)
   int sw64 = 0;
   if (track_v && !lower)   // (one CTA: teams have graded factors)
-    sw64 = jacobi_svd(g, p, q, v, q, 1, false, max_sweeps, &sh.flag, floor64 * floor64, sh.jac);
+    sw64 = jacobi_svd<true>(g, p, q, v, max_sweeps, &sh.flag, floor64 * floor64, sh.jac);
   mark(5);
   if (threadIdx.x == 0) sh.ls_recover = track_v ? 0 : 1;
   if (jstats && tm.tid == 0) {
@@ -2608,7 +2611,7 @@ __global__ void __launch_bounds__(kThreads) compress_block_noalloc_kernel(
   // from ever converging
   const double floor64 = (double)p * DBL_EPSILON * sqrt(nsq);
   const int sweeps =
-      jacobi_svd(G, p, q, V, 1, q, true, max_sweeps, &sh.flag, floor64 * floor64, sh.jac);
+      jacobi_svd<false>(G, p, q, V, max_sweeps, &sh.flag, floor64 * floor64, sh.jac);
   // every sweep still rotated a pair: the column norms the truncation uses may be inexact
   if (sweeps >= max_sweeps && threadIdx.x == 0) status[2] = 4;
   sort_and_truncate(G, p, q, p, eps, sh);
