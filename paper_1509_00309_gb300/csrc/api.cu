@@ -427,6 +427,11 @@ int make_plan(clr_ctx_t ctx, int nI, int nJ, int nK, Plan* p) {
   return CLR_OK;
 }
 
+int max_cluster(clr_mat_t m) {
+  return std::max(*std::max_element(m->row_sizes.begin(), m->row_sizes.end()),
+                  *std::max_element(m->col_sizes.begin(), m->col_sizes.end()));
+}
+
 int grid_of(clr_ctx_t ctx, int per_sm) { return std::max(1, ctx->n_sm * per_sm); }
 
 // A side stream (and a second workspace set) ordered after `s`: work issued on ctx->side
@@ -748,7 +753,7 @@ extern "C" int clr_mat_from_dense(clr_ctx_t ctx, const double* a, int64_t lda, i
     launch_compress_dense(m->view(), nullptr, nullptr, (const int*)ctx->cur->order.p, src, lda,
                           (double*)ctx->cur->ws.p, (double*)ctx->cur->scratch.p,
                           eps_lr, drop_norm, 0, ctx->opts.build_rrqr ? 1 : 0,
-                          ctx->opts.svd_no_prereduce ? 0 : 1,
+                          ctx->opts.svd_no_prereduce ? 0 : 1, max_cluster(m),
                           ctx->opts.jacobi_max_sweeps, grid_of(ctx, 2), &pc->err, &pc->sched[2],
                           nullptr, jst(ctx), s);
   }
@@ -1183,8 +1188,8 @@ int multiply_into(clr_ctx_t ctx, clr_mat_t a, clr_mat_t b, clr_mat_t c, double a
   prof_mark(ctx, s, PH_COMPRESS_QR);
   launch_compress_dense(cv, p.l_dcomp_s, &p.counters->n_dcomp, nullptr, nullptr, 0,
                         (double*)ctx->cur->ws.p, (double*)ctx->cur->scratch.p,
-                        eps_lr, 0.0, 0, 0, o.svd_no_prereduce ? 0 : 1, o.jacobi_max_sweeps,
-                        lr_grid, &p.counters->err,
+                        eps_lr, 0.0, 0, 0, o.svd_no_prereduce ? 0 : 1, max_cluster(c),
+                        o.jacobi_max_sweeps, lr_grid, &p.counters->err,
                         &p.counters->sched[2], &p.counters->n_team, jst(ctx), s);
   CLR_CHECK_LAUNCH("recompression");
   prof_launches(ctx, 2);
@@ -1404,8 +1409,8 @@ extern "C" int clr_lincomb(clr_ctx_t ctx, double a, clr_mat_t x, double b, clr_m
                      jst(ctx, 1), s);
   launch_compress_dense(ov, p.l_dcomp_s, &p.counters->n_dcomp, nullptr, nullptr, 0,
                         (double*)ctx->cur->ws.p, (double*)ctx->cur->scratch.p,
-                        o.eps_lr, 0.0, 0, 0, o.svd_no_prereduce ? 0 : 1, o.jacobi_max_sweeps,
-                        grid, &p.counters->err,
+                        o.eps_lr, 0.0, 0, 0, o.svd_no_prereduce ? 0 : 1, max_cluster(out),
+                        o.jacobi_max_sweeps, grid, &p.counters->err,
                         &p.counters->sched[2], &p.counters->n_team, jst(ctx), s);
   CLR_CHECK_LAUNCH("lincomb");
   return CLR_OK;

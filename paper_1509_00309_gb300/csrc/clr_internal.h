@@ -245,6 +245,7 @@ void launch_compress_qr(const MatView& C, const int* list, const int* count, con
 // prereduce: reduce every block by a column-pivoted QR (stopped at eps/16) before the SVD of
 // its k x q factor R, unless the QR's triangles certify it dense; without it every block takes
 // the full SVD.
+// max_side: the largest cluster of C.
 // n_team (may be null): how many leading tiles of the list take a team of kTeamCtas CTAs each.
 constexpr int kTeamCtas = 4;
 // jstats (7 counters): SVD blocks, FP32 sweeps, FP64 sweeps, early dense exits, FP64 flops,
@@ -252,9 +253,9 @@ constexpr int kTeamCtas = 4;
 void launch_compress_dense(const MatView& C, const int* list, const int* count,
                            const int* order, const double* src, int64_t lds, double* ws,
                            double* svd_scratch, double eps, double drop_norm,
-                           int dense_only, int rrqr, int prereduce, int max_sweeps, int grid,
-                           int* err, int* sched, const int* n_team, unsigned long long* jstats,
-                           cudaStream_t st);
+                           int dense_only, int rrqr, int prereduce, int max_side, int max_sweeps,
+                           int grid, int* err, int* sched, const int* n_team,
+                           unsigned long long* jstats, cudaStream_t st);
 void launch_block_norms(const MatView& M, cudaStream_t st);
 void launch_block_norms_dense(const MatView& M, cudaStream_t st);
 void launch_scale_blocks(const MatView& M, double alpha, cudaStream_t st);

@@ -815,6 +815,12 @@ struct Work32 {
 // Dynamic shared memory of the recompression kernels: with their static part (34 KB) nearly all
 // that a CTA can have, enough for a 256 x 133 pair of copies or a 156 x 156 one.
 constexpr int kSvdSmemBytes = 192 * 1024;
+// Of this launch: none where L1 is to cache the copies in the scratch (launch_compress_dense).
+__device__ __forceinline__ int svd_smem_bytes() {
+  int b;
+  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(b));
+  return b;
+}
 
 // Lanes and packed rows per lane for columns of p rows: 16 lanes a pair put up to 32 pairs into one
 // pass over the CTA's 16 warps, 32 lanes up to 16; one packed row a lane while the rows are few.
@@ -829,7 +835,7 @@ __device__ __forceinline__ Work32 work32(int p, int q, double* sc) {
   extern __shared__ __align__(16) float svd_smem[];
   Work32 k;
   split32(k, p, q);
-  const bool fits = (int64_t)(k.ldg + k.ldv) * q * (int)sizeof(float) <= kSvdSmemBytes;
+  const bool fits = (int64_t)(k.ldg + k.ldv) * q * (int)sizeof(float) <= svd_smem_bytes();
   k.g = fits ? svd_smem : reinterpret_cast<float*>(sc);
   k.v = k.g + k.ldg * q;
   return k;
@@ -840,7 +846,7 @@ __device__ __forceinline__ Work32 work32(int p, int q, double* sc) {
 // each column's error relative to its own norm, as the grading needs.  The QR works in shared
 // memory (p q floats).
 __device__ __forceinline__ bool use_qr32(int p, int q) {
-  return 8 * p >= 9 * q && (int64_t)((p + 1) & ~1) * q * (int)sizeof(float) <= kSvdSmemBytes;
+  return 8 * p >= 9 * q && (int64_t)((p + 1) & ~1) * q * (int)sizeof(float) <= svd_smem_bytes();
 }
 
 // k.g (p x q, ld k.ldg, in shared memory) <- its triangular factor (q x q, zero below the diagonal),
@@ -903,7 +909,7 @@ __device__ __noinline__ void qr32(Work32& k, int p, int q, double* sc) {
     __syncthreads();
     if (i < n.ldg) n.g[c * n.ldg + i] = v;
   }
-  const bool fits = (int64_t)2 * n.ldg * q * (int)sizeof(float) <= kSvdSmemBytes;
+  const bool fits = (int64_t)2 * n.ldg * q * (int)sizeof(float) <= svd_smem_bytes();
   n.v = fits ? n.g + n.ldg * q : reinterpret_cast<float*>(sc);
   k = n;
   __syncthreads();
@@ -916,7 +922,7 @@ __device__ __forceinline__ int run_jacobi32(const TM& tm, const Work32& k, int q
   extern __shared__ __align__(16) float svd_smem[];
 #define CLR_JACOBI32(LP, VEC, SH) \
   return jacobi32<LP, VEC, SH>(tm, k.g, q, k.ldg, k.v, k.ldv, max_sweeps, tol, floor2, sh)
-  const float* end = svd_smem + kSvdSmemBytes / sizeof(float);
+  const float* end = svd_smem + svd_smem_bytes() / (int)sizeof(float);
   if (!(k.g >= svd_smem && k.g < end && k.v >= svd_smem && k.v < end)) {
     if (k.vec <= 3) CLR_JACOBI32(32, 3, false);   // (columns of more than 128 rows only)
     CLR_JACOBI32(32, 4, false);
@@ -945,7 +951,7 @@ __device__ __forceinline__ int run_jacobi32(const TM& tm, const Work32& k, int q
 // orthonormalisation has read by then.
 __device__ __forceinline__ float* series_f32(int q, double* sc) {
   extern __shared__ __align__(16) float svd_smem[];
-  return (int64_t)2 * q * q * (int)sizeof(float) <= kSvdSmemBytes ? svd_smem
+  return (int64_t)2 * q * q * (int)sizeof(float) <= svd_smem_bytes() ? svd_smem
                                                                  : reinterpret_cast<float*>(sc);
 }
 
@@ -1056,28 +1062,47 @@ struct SrcView {
   }
 };
 
+// How the FP32 matrices at f (series_f32) are written: in its own shared memory by every CTA of the
+// team for itself, in the team's one global scratch (more than ~156 columns) dealt over the team.
+struct FloatShare {
+  bool own;
+  int t0, step;
+  template <class TM>
+  __device__ __forceinline__ FloatShare(const TM& tm, const float* f) {
+    extern __shared__ __align__(16) float svd_smem[];
+    own = tm.size == 1 || f == svd_smem;
+    t0 = own ? (int)threadIdx.x : tm.tid;
+    step = own ? kThreads : tm.nt;
+  }
+};
+
 // The matrix function of a small symmetric E (q x q) that both uses below need, in place:
 //   e <- c1 E + c2 E^2 + c3 E^3.
-// The powers are taken in FP32 (f: 2 q^2 floats): E is at most a few 1e-4, so their error is
-// below 1e-16.  Returns ||E||_F^2.
+// The powers are taken in FP32 (f: 2 q^2 floats): their error is 6e-8 c2 ||E||_F^2, 1e-15 at the
+// ||E||_F = 2e-4 (kSeriesFro) that its callers take for the last time; not at all where E^2 is below
+// 1e-18 (kTinyFro).  Returns ||E||_F^2.
+constexpr double kTinyFro = 1e-9;
+
 template <class TM>
 __device__ __noinline__ double small_series(const TM& tm, double* e, int q, double c1, float c2,
                                             float c3, float* f, SvdShared& sh) {
-  // Where the powers lie in the CTA's shared memory every CTA of the team takes them itself; in the
-  // team's one global scratch (more than ~156 columns) they are dealt over the team.
-  extern __shared__ __align__(16) float svd_smem[];
-  const bool own = tm.size == 1 || f == svd_smem;
-  const int t0 = own ? (int)threadIdx.x : tm.tid, step = own ? kThreads : tm.nt;
+  const FloatShare fs(tm, f);
   float* t = f + q * q;
   float part = 0.f;
   for (int x = threadIdx.x; x < q * q; x += kThreads) {
     const float v = (float)e[x];
     part = fmaf(v, v, part);
   }
-  for (int x = t0; x < q * q; x += step) f[x] = (float)e[x];
   const double fro2 = block_sum((double)part, sh.red);
-  if (!own) tm.sync();
-  cta_gemm_auto(t0, step, q, q, q, f, 1, q, f, 1, q, t, q);
+  if (fro2 <= kTinyFro * kTinyFro) {
+    tm.sync();   // (every CTA has read E)
+    for (int x = tm.tid; x < q * q; x += tm.nt) e[x] *= c1;
+    tm.sync();
+    return fro2;
+  }
+  for (int x = fs.t0; x < q * q; x += fs.step) f[x] = (float)e[x];
+  if (fs.own) __syncthreads(); else tm.sync();
+  cta_gemm_auto(fs.t0, fs.step, q, q, q, f, 1, q, f, 1, q, t, q);
   tm.sync();
   // E^3 = F T an output at a time, added to the rest of the series
   for (int x = tm.tid; x < q * q; x += tm.nt) {
@@ -1177,9 +1202,11 @@ constexpr double kRefineFro = 0.05;   // up to this, by refinement (ls_solve)
 // about 1e-5; repeated until ||E||_F has been below kSeriesFro.  Two products of q^3 FMAs (one of
 // them symmetric) that fill the CTA, against Gram-Schmidt's q^3 FMAs in q dependent steps of
 // reductions.  Measured (q = 16, with the product that follows): 218k -> 25k SM cycles; 3D lattice
-// product at N = 4096, both stages over all blocks: 3.1 -> 2.1 G cycles.  v32 is
-// the team's first CTA's; e: q^2 doubles, f: 2 q^2 floats, not overlapping v32's matrix until it
-// has been read.
+// product at N = 4096, both stages over all blocks: 3.1 -> 2.1 G cycles.  From ~200 columns on a
+// second pass is needed; its E is below kTinyFro (a few 1e-13), so that V E / 2 taken in FP32 is
+// exact to 1e-19 (with FP64 products that pass made whole blocks of 256 columns slower than
+// Gram-Schmidt).  v32 is the team's first CTA's; e: q^2 doubles, f: 2 q^2 floats, not overlapping
+// v32's matrix until it has been read.
 template <class TM>
 __device__ __noinline__ void orthonormalise_fp64(const TM& tm, const float* v32, int ldv,
                                                  double* v, int q, double* e, float* f,
@@ -1193,6 +1220,21 @@ __device__ __noinline__ void orthonormalise_fp64(const TM& tm, const float* v32,
   for (int pass = 0; pass < 4; ++pass) {
     gram_minus_identity(tm, v, q, q, nullptr, e);
     const double fro2 = small_series(tm, e, q, -0.5, 0.375f, -0.3125f, f, sh);
+    if (fro2 <= kTinyFro * kTinyFro) {
+      float* w = f + q * q;
+      float* d = reinterpret_cast<float*>(e);   // V (-E / 2), in E's place
+      const FloatShare fs(tm, f);
+      for (int x = fs.t0; x < q * q; x += fs.step) {
+        f[x] = (float)v[x];
+        w[x] = (float)e[x];
+      }
+      tm.sync();
+      cta_gemm_auto(tm.tid, tm.nt, q, q, q, w, 1, q, f, 1, q, d, q);
+      tm.sync();
+      for (int x = tm.tid; x < q * q; x += tm.nt) v[x] += (double)d[x];
+      tm.sync();
+      break;
+    }
     right_multiply_fp64(tm, v, q, q, 1, q, e, true);
     if (!(fro2 > kSeriesFro * kSeriesFro)) break;
   }
@@ -1389,7 +1431,7 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
   const int q_even = (q + 1) & ~1;
   const bool spread1 =
       tm.size > 1 && (tri32 ? 2 * q_even * q : (wk.ldg + wk.ldv) * q) * (int)sizeof(float) >
-                         kSvdSmemBytes;
+                         svd_smem_bytes();
   constexpr int64_t kSq = (int64_t)CLR_MAX_CLUSTER * CLR_MAX_CLUSTER;
   double* v2 = sc + kSq;       // after p q + q^2 floats
   double* e = sc + 4 * kSq;    // the orthonormalisations' E, and their FP32 powers
@@ -1477,7 +1519,7 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
   wk = work32(p, q, sc);
   const float tol_g = lower ? 16.f * tol32 : tol32;
   int sw32b = 0;
-  if (tm.size > 1 && (wk.ldg + wk.ldv) * q * (int)sizeof(float) > kSvdSmemBytes) {
+  if (tm.size > 1 && (wk.ldg + wk.ldv) * q * (int)sizeof(float) > svd_smem_bytes()) {
     for (int e = tm.tid; e < wk.ldg * q; e += tm.nt) {
       const int i = e % wk.ldg;
       wk.g[e] = i < p ? (float)(g[i + (int64_t)(e / wk.ldg) * p] * sc32) : 0.f;
@@ -1679,6 +1721,8 @@ int svd_launch_grid(K kernel, int grid_max, bool* attr_done) {
   // set once per device (outside any stream capture the first time a product runs)
   if (dev >= 0 && dev < 64 && !attr_done[dev]) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSvdSmemBytes);
+    // (as much L1 as a launch's shared memory leaves)
+    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
     attr_done[dev] = true;
   }
   int grid = n_sm;
@@ -2177,7 +2221,7 @@ __device__ __noinline__ int compress_by_pivoted_qr(const TM& tm, const SrcView& 
   }
   __syncthreads();
   // the reflectors in shared memory where they fit
-  if ((int64_t)p * k * (int64_t)sizeof(double) <= kSvdSmemBytes) {
+  if ((int64_t)p * k * (int64_t)sizeof(double) <= svd_smem_bytes()) {
     extern __shared__ __align__(16) float svd_smem[];
     double* st = reinterpret_cast<double*>(svd_smem);
     for (int c = w; c < k; c += kWarps)
@@ -2467,9 +2511,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 void launch_compress_dense(const MatView& C, const int* list, const int* count,
                            const int* order, const double* src, int64_t lds, double* ws,
                            double* svd_scratch, double eps, double drop_norm,
-                           int dense_only, int rrqr, int prereduce, int max_sweeps, int grid,
-                           int* err, int* sched, const int* n_team, unsigned long long* jstats,
-                           cudaStream_t st) {
+                           int dense_only, int rrqr, int prereduce, int max_side, int max_sweeps,
+                           int grid, int* err, int* sched, const int* n_team,
+                           unsigned long long* jstats, cudaStream_t st) {
   static bool attr_done[64] = {false}, attr_done_team[64] = {false};
   const int g = svd_launch_grid(compress_dense_kernel, grid, attr_done);
   const int gt =
@@ -2481,7 +2525,11 @@ void launch_compress_dense(const MatView& C, const int* list, const int* count,
         C, list, count, order, src, lds, ws, svd_scratch, eps, drop_norm, dense_only, rrqr,
         prereduce, max_sweeps, err, sched, n_team, jstats);
   else
-    compress_dense_kernel<<<g, kThreads, kSvdSmemBytes, st>>>(
+    // Without the pivoted QR a 256 x 256 block's sweeps run on 512 KB in the scratch; they are bound
+    // by what L1 holds of it, and shared memory would take that (build of the 3D lattice, N = 1024
+    // and 2048, clusters of up to 256: 87 and 76 ms, now 84 and 72).
+    compress_dense_kernel<<<g, kThreads, !prereduce && 8 * max_side * max_side > kSvdSmemBytes
+                                             ? 0 : kSvdSmemBytes, st>>>(
         C, list, count, order, src, lds, ws, svd_scratch, eps, drop_norm, dense_only, rrqr,
         prereduce, max_sweeps, err, sched, jstats);
 }

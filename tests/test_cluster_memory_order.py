@@ -39,9 +39,12 @@ def test_a_cluster_barrier_precedes_the_first_access_to_a_peer(file, kernel, bar
 def test_the_series_powers_in_a_teams_scratch_are_dealt_over_the_team():
     # F and F^2 lie in one global scratch for all CTAs of a team where they do not fit shared
     # memory: each entry is then written by one thread of the team, and read behind its barrier
-    body = _function("k_svd.cu", "small_series")
-    assert re.search(r"own \? \(int\)threadIdx\.x : tm\.tid, step = own \? kThreads : tm\.nt", body)
-    stores = re.findall(r"for \(int x = (\S+); x < q \* q; x \+= (\S+)\)[ \n]*f\[x\] =", body)
-    assert stores == [("t0", "step")] and body.count("f[x] =") == 1
-    square = body.index("cta_gemm_auto(t0, step,")
-    assert body.index("f[x] =") < body.index("if (!own) tm.sync();") < square
+    share = _function("k_svd.cu", "FloatShare")
+    assert "t0 = own ? (int)threadIdx.x : tm.tid" in share and "own ? kThreads : tm.nt" in share
+    for name, stores in (("small_series", ["f"]), ("orthonormalise_fp64", ["f", "w"])):
+        body = _function("k_svd.cu", name)
+        loop = body.index("for (int x = fs.t0; x < q * q; x += fs.step)")
+        for m in stores:
+            assert body.count(m + "[x] =") == 1 and body.index(m + "[x] =") > loop
+        sync = re.search(r"(?:if \(fs\.own\) __syncthreads\(\); else )?tm\.sync\(\);", body[loop:])
+        assert loop + sync.start() < body.index("cta_gemm_auto(")

@@ -48,15 +48,17 @@ def test_rank_of_sums_near_the_noise_floor(ctx, eps, spread):
             <= 3 * eps * (1 + 1e-6) + 3e-14)
 
 
-# the SVD of whole blocks, without the pivoted QR in front
+# the SVD of whole blocks, without the pivoted QR in front: FP32 copies cached by L1 (a cluster above
+# 156) or in shared memory, one pass of the orthonormalisation or two
+@pytest.mark.parametrize("m,n", [(256, 240), (157, 90), (156, 130)])
 @pytest.mark.parametrize("eps", [1e-13, 1e-12, 1e-11])
-def test_rank_of_whole_blocks_near_the_noise_floor(ctx, eps):
+def test_rank_of_whole_blocks_near_the_noise_floor(ctx, eps, m, n):
     rng = np.random.default_rng(5)
     decay = 0.985
-    a = _slow_tail(rng, 256, 240, 20, decay, 0.9 * eps * np.sqrt(1.0 - decay ** 2))
+    a = _slow_tail(rng, m, n, 20, decay, 0.9 * eps * np.sqrt(1.0 - decay ** 2))
     ctx.set_opts(svd_no_prereduce=1)
     try:
-        m = ctx.from_dense(a, [256], [240], eps_lr=eps)
+        m = ctx.from_dense(a, [m], [n], eps_lr=eps)
     finally:
         ctx.set_opts(svd_no_prereduce=0)
     kinds, ranks = m.get_blocks()[:2]
