@@ -122,8 +122,12 @@ __device__ __forceinline__ void cta_gemm_micro(int tid, int nt, int P, int Q, in
 
 // CTAs per block of the kernels that form the low-rank blocks' values, by the number of blocks
 // (how many of them are low rank is not known on the host): 8 where a CTA per block could not
-// fill 152 SMs evenly, 1 where the blocks alone do.
-inline int lr_parts(int n_blocks) { return n_blocks <= 1024 ? 8 : n_blocks <= 4096 ? 4 : 1; }
+// fill 152 SMs evenly (4 where the blocks are below 64^2 on average: starting eight for each took
+// longer than their work), 1 where the blocks alone do.
+inline int lr_parts(const MatView& M) {
+  const int64_t nb = (int64_t)M.nr * M.nc;
+  return nb <= 1024 && M.n_rows * M.n_cols >= 4096 * nb ? 8 : nb <= 4096 ? 4 : 1;
+}
 
 // The micro-tile by the size of the output: 4 x 2 from four rounds of the threads on
 // (less than a quarter of a round idle at the end), 2 x 2 from one, else an entry per thread.

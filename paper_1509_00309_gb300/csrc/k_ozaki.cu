@@ -845,7 +845,7 @@ void launch_ozaki_stage(const MatView& M, const int* row_idx, const int* col_idx
     const dim3 ne((unsigned)rows_pad, (unsigned)n_seg);
     oz_exp_b_kernel<<<ne, 256, 0, st>>>(M, row_idx, col_idx, exps, rows_pad, cols_pad);
   }
-  const dim3 nl(nb, (unsigned)lr_parts((int)nb));
+  const dim3 nl(nb, (unsigned)lr_parts(M));
   if (!recon_formed) oz_lr_recon_kernel<<<nl, 256, 0, st>>>(M, recon);
   oz_exp_lr_kernel<<<nl, 256, 0, st>>>(M, recon, exps, rows_pad, a_mode);
   if (a_mode) {

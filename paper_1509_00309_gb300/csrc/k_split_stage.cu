@@ -183,7 +183,7 @@ void launch_split_stage(const MatView& M, const int* row_idx, const int* col_idx
     else
       split_stage_b_kernel<3><<<n, 256, 0, st>>>(M, row_idx, col_idx, pn, rows_pad, cols_pad);
   }
-  const dim3 nb((unsigned)(M.nr * M.nc), (unsigned)lr_parts(M.nr * M.nc));
+  const dim3 nb((unsigned)(M.nr * M.nc), (unsigned)lr_parts(M));
   if (terms == 2)
     split_stage_lr_kernel<2><<<nb, 256, 0, st>>>(M, pn, rows_pad, cols_pad, a_mode);
   else

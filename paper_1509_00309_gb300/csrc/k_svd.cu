@@ -2604,7 +2604,7 @@ __global__ void scale_blocks_kernel(MatView M, double alpha) {
 }
 
 void launch_scale_blocks(const MatView& M, double alpha, cudaStream_t st) {
-  scale_blocks_kernel<<<dim3((unsigned)(M.nr * M.nc), (unsigned)lr_parts(M.nr * M.nc)), 256, 0,
+  scale_blocks_kernel<<<dim3((unsigned)(M.nr * M.nc), (unsigned)lr_parts(M)), 256, 0,
                         st>>>(M, alpha);
 }
 
