@@ -208,10 +208,11 @@ void launch_set_route_kinds(const MatView& C, const Plan& p, cudaStream_t st) {
 // CTAs per tile, its parts added in a fixed order (with one CTA a tile's loads took 20 us), while
 // the tiles are few (kNormFew a cluster: 512); beyond, CTAs fill the SMs with a tile each and a
 // cluster would only wait at its barriers (48400 tiles of at most 48^2: 2350 us by clusters, 330 by
-// CTAs).
+// CTAs).  Nor has a small tile (kNormSmall on average) loads to share: 169 tiles of 39^2 16 and 8 us.
 constexpr int kNormCtas = 8;
 constexpr int kNormGrid = 1024;
 constexpr int kNormFew = 4;
+constexpr int kNormSmall = 4096;
 __global__ void __cluster_dims__(kNormCtas, 1, 1) __launch_bounds__(256)
     dense_tile_norms_kernel(MatView C, Plan p) {
   namespace cg = cooperative_groups;
@@ -219,7 +220,8 @@ __global__ void __cluster_dims__(kNormCtas, 1, 1) __launch_bounds__(256)
   __shared__ double red[8];
   __shared__ double part;
   const int n_items = p.counters->n_dense;
-  const bool alone = n_items > kNormFew * (int)(gridDim.x / kNormCtas);
+  const bool alone = n_items > kNormFew * (int)(gridDim.x / kNormCtas) ||
+                     C.n_rows * C.n_cols <= (int64_t)kNormSmall * p.nI * p.nJ;
   const int rank = alone ? 0 : (int)cluster.block_rank(), ctas = alone ? 1 : kNormCtas;
   for (int it = blockIdx.x / ctas; it < n_items; it += gridDim.x / ctas) {
     const int t = p.l_dense[it];
