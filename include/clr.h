@@ -391,6 +391,10 @@ typedef struct clr_profile {
 } clr_profile;
 int clr_profile_enable(clr_ctx_t ctx, int on);
 int clr_profile_read(clr_ctx_t ctx, clr_profile* out);
+/* How many tiles compress_dense_kernel has given to teams of CTAs (several CTAs on one tile, where
+ * few or a few expensive tiles would leave SMs idle) since profiling was enabled.  Synchronises the
+ * device. */
+int clr_profile_team_tiles(clr_ctx_t ctx, int64_t* tiles);
 /* FP64 FMA throughput of `device` measured by a short kernel of independent FMA chains on every
  * SM (the roofline of the FP64 arithmetic in recompression): *tflops = 2 x FMAs / second.
  * Synchronises the device. */

@@ -127,6 +127,7 @@ _SIGNATURES = {
     "clr_mem_cached": (C.c_int64, []),
     "clr_profile_enable": (C.c_int, [_VP, C.c_int]),
     "clr_profile_read": (C.c_int, [_VP, C.POINTER(ClrProfile)]),
+    "clr_profile_team_tiles": (C.c_int, [_VP, C.POINTER(C.c_int64)]),
     "clr_probe_fp64_rate": (C.c_int, [C.c_int, C.POINTER(C.c_double)]),
     "clr_split_bf16": (C.c_int, [_VP, C.c_int64, C.c_int, _VP, _VP]),
     "clr_multiply_host_stream": (C.c_int, [_VP, _VP, C.c_int64, _VP, C.c_int64, _VP, C.c_int64,
@@ -320,6 +321,12 @@ class Context:
         for f in ("svd_path_cycles", "svd_path_blocks", "svd_full_cycles", "svd_pre_cycles"):
             out[f] = list(out[f])
         return out
+
+    def profile_team_tiles(self) -> int:
+        """Tiles recompressed by teams of CTAs since profiling was enabled."""
+        n = C.c_int64()
+        self._check(load().clr_profile_team_tiles(self.handle, C.byref(n)))
+        return n.value
 
     # matrices ------------------------------------------------------------------------------
     def zeros(self, row_sizes, col_sizes=None) -> Matrix:

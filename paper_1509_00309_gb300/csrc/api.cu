@@ -470,13 +470,11 @@ const double* host_device_ptr(const void* p) {
 }
 
 
-// SVD counters while profiling (not inside a graph capture), else null.  Three blocks of 8:
-// [0, 8) for dense truncated SVDs (compress_dense_kernel), [8, 16) for the QR route
-// (compress_qr_kernel), [16, 24) SM cycles and counts of compress_dense_kernel's paths.
+// SVD counters while profiling (not inside a graph capture), else null, in blocks of 8:
 constexpr int kJstatsBlock = 8;
 // counter blocks: 0 compress_dense_kernel, 1 compress_qr_kernel, 2 per-path cycles of
-// compress_dense_kernel, 3 its full-SVD stages, 4 its pre-reduced path's stages
-constexpr int kJstatsBlocks = 5;
+// compress_dense_kernel, 3 its full-SVD stages, 4 its pre-reduced path's stages, 5 its tiles by teams
+constexpr int kJstatsBlocks = 6;
 unsigned long long* jst(clr_ctx_t ctx, int block = 0) {
   return (ctx->prof_on && !ctx->capturing && ctx->jstats.p)
              ? (unsigned long long*)ctx->jstats.p + block * kJstatsBlock : nullptr;
@@ -1296,6 +1294,19 @@ extern "C" int clr_profile_read(clr_ctx_t ctx, clr_profile* out) {
     ctx->prof.svd_pre_blocks = (int64_t)rc[7];
   }
   *out = ctx->prof;
+  return CLR_OK;
+}
+
+extern "C" int clr_profile_team_tiles(clr_ctx_t ctx, int64_t* tiles) {
+  if (!ctx || !tiles) return CLR_EINVAL;
+  *tiles = 0;
+  if (!ctx->jstats.p) return CLR_OK;
+  cudaSetDevice(ctx->device);
+  CLR_CUDA(cudaDeviceSynchronize());
+  unsigned long long n = 0;
+  CLR_CUDA(cudaMemcpy(&n, (unsigned long long*)ctx->jstats.p + 5 * kJstatsBlock, sizeof(n),
+                      cudaMemcpyDeviceToHost));
+  *tiles = (int64_t)n;
   return CLR_OK;
 }
 

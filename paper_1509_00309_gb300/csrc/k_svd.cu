@@ -36,6 +36,8 @@ constexpr int kFullStageCounters = 24;
 // the same for the pre-reduced path (block 4): the QR, the five stages of svd_mixed on R^T,
 // truncation, recovery and the factors' stores; then the count
 constexpr int kPreStageCounters = 32;
+// tiles taken by a team of CTAs (block 5)
+constexpr int kTeamTileCounter = 40;
 constexpr int kWarps = kThreads / 32;
 
 template <typename T>
@@ -2322,6 +2324,7 @@ __device__ __forceinline__ void compress_dense_body(
     prev_t = tm.rank == 0 ? t : -1;
     prev_c = now;
     prev_x = tm.size > 1 ? 2 : 1;
+    if (jstats && tm.size > 1 && tm.tid == 0) atomicAdd(&jstats[kTeamTileCounter], 1ull);
     const int I = t / C.nc, J = t % C.nc;
     const int m = C.row_off[I + 1] - C.row_off[I];
     const int n = C.col_off[J + 1] - C.col_off[J];
