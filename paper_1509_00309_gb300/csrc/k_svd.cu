@@ -7,7 +7,8 @@
 // singular values on the left factor (X' = Q_X U_r S_r, W' = Q_W V_r).  A block whose rank
 // exceeds floor(min(m,n)/2) is stored dense.
 //
-// One CTA (16 warps) handles one tile at a time, taking tiles from a launch-wide counter:
+// A CTA (16 warps), or a team of CTAs (compress_dense_body, compress_qr_kernel's pairs), handles one
+// tile at a time, taking tiles from a launch-wide counter:
 //   Householder QR         LAPACK-style reflectors H = I - tau v v^T, v_0 = 1;
 //   one-sided Jacobi SVD   Hestenes rotations on column pairs, round-robin ordering so a
 //                          round's pairs are disjoint (one warp per pair), until no pair has
@@ -31,7 +32,8 @@ constexpr int kThreads = 512;
 // index of the per-path cycle counters in the profiling counters (third block of 8)
 constexpr int kPathCounters = 16;
 // compress_dense_kernel's full-SVD stages while profiling (block 3 of the counters): cycles of
-// the pivoted QR attempt, the five stages of svd_mixed, truncation and stores; then the count
+// the pivoted QR attempt, the five stages of svd_mixed (the fifth: FP64 sweeps, near the noise
+// floor only), truncation and stores; then the count
 constexpr int kFullStageCounters = 24;
 // the same for the pre-reduced path (block 4): the QR, the five stages of svd_mixed on R^T,
 // truncation, recovery and the factors' stores; then the count
@@ -1065,7 +1067,8 @@ struct SrcView {
 };
 
 // How the FP32 matrices at f (series_f32) are written: in its own shared memory by every CTA of the
-// team for itself, in the team's one global scratch (more than ~156 columns) dealt over the team.
+// team for itself, in the team's one global scratch (more than ~156 columns) dealt over the team
+// (3D lattice iterates, N = 2048: orthonormalisation and projection 1870 -> 1750 M SM cycles).
 struct FloatShare {
   bool own;
   int t0, step;
@@ -1195,7 +1198,10 @@ __device__ void right_multiply_fp64(const TM& tm, double* m, int rows, int64_t m
 }
 
 // Above this ||E||_F the series in small_series, cut after E^3 and with FP32 powers, is not FP64
-// accurate (the first term left out is 35/128 E^4, the powers' error 4e-8 E^2).
+// accurate (at it the first term left out, 35/128 E^4, is 4e-16 and the powers' error 1e-15).
+// ||V^T V - I||_F afterwards, against extended precision, and that of Gram-Schmidt: 16 columns 1.2e-15
+// and 7e-16 at this limit (6e-16 at the usual ||E||_F of 1e-5), 100 columns 3.3e-15 and 3.4e-15, 240
+// columns 8.0e-15 and 7.4e-15, after two passes 7.4e-15.
 constexpr double kSeriesFro = 2e-4;
 constexpr double kRefineFro = 0.05;   // up to this, by refinement (ls_solve)
 
@@ -1325,46 +1331,44 @@ __device__ __noinline__ bool ls_solve(const TM& tm, double* y, int q, int r, dou
     return true;
   }
   if (tm.rank == 0) {   // (by the first CTA alone)
-  if (threadIdx.x == 0) sh.flag = 1;
-  for (int x = threadIdx.x; x < r; x += kThreads) mw[x + (int64_t)x * r] += 1.0;
-  __syncthreads();
-  for (int j = 0; j < r; ++j) {  // lower Cholesky, column by column
-    if (threadIdx.x == 0) {
-      double a = mw[j + (int64_t)j * r];
-      for (int k = 0; k < j; ++k) a -= mw[j + (int64_t)k * r] * mw[j + (int64_t)k * r];
-      if (!(a > 0.0) || !isfinite(a)) {
-        sh.flag = 0;
-        a = 1.0;
+    if (threadIdx.x == 0) sh.flag = 1;
+    for (int x = threadIdx.x; x < r; x += kThreads) mw[x + (int64_t)x * r] += 1.0;
+    __syncthreads();
+    for (int j = 0; j < r; ++j) {  // lower Cholesky, column by column
+      if (threadIdx.x == 0) {
+        double a = mw[j + (int64_t)j * r];
+        for (int k = 0; k < j; ++k) a -= mw[j + (int64_t)k * r] * mw[j + (int64_t)k * r];
+        if (!(a > 0.0) || !isfinite(a)) {
+          sh.flag = 0;
+          a = 1.0;
+        }
+        mw[j + (int64_t)j * r] = sqrt(a);
       }
-      mw[j + (int64_t)j * r] = sqrt(a);
+      __syncthreads();
+      const double ljj = mw[j + (int64_t)j * r];
+      for (int i = j + 1 + threadIdx.x; i < r; i += kThreads) {
+        double a = mw[i + (int64_t)j * r];
+        for (int k = 0; k < j; ++k) a -= mw[i + (int64_t)k * r] * mw[j + (int64_t)k * r];
+        mw[i + (int64_t)j * r] = a / ljj;
+      }
+      __syncthreads();
     }
-    __syncthreads();
-    const double ljj = mw[j + (int64_t)j * r];
-    for (int i = j + 1 + threadIdx.x; i < r; i += kThreads) {
-      double a = mw[i + (int64_t)j * r];
-      for (int k = 0; k < j; ++k) a -= mw[i + (int64_t)k * r] * mw[j + (int64_t)k * r];
-      mw[i + (int64_t)j * r] = a / ljj;
+    // each row t: x = (y_t D^-1) (L L^T)^-1 D^-1 (no row when a pivot failed)
+    for (int t = sh.flag ? threadIdx.x : q; t < q; t += kThreads) {
+      double* yt = y + (int64_t)t * r;
+      for (int i = 0; i < r; ++i) {  // forward: L u = (y_t D^-1)^T
+        double a = yt[i] / d[i];
+        for (int k = 0; k < i; ++k) a -= mw[i + (int64_t)k * r] * yt[k];
+        yt[i] = a / mw[i + (int64_t)i * r];
+      }
+      for (int i = r - 1; i >= 0; --i) {  // back: L^T x = u
+        double a = yt[i];
+        for (int k = i + 1; k < r; ++k) a -= mw[k + (int64_t)i * r] * yt[k];
+        yt[i] = a / mw[i + (int64_t)i * r];
+      }
+      for (int i = 0; i < r; ++i) yt[i] /= d[i];
     }
-    __syncthreads();
-  }
-  __syncthreads();
-  if (sh.flag)
-  // each row t: x = (y_t D^-1) (L L^T)^-1 D^-1
-  for (int t = threadIdx.x; t < q; t += kThreads) {
-    double* yt = y + (int64_t)t * r;
-    for (int i = 0; i < r; ++i) {  // forward: L u = (y_t D^-1)^T
-      double a = yt[i] / d[i];
-      for (int k = 0; k < i; ++k) a -= mw[i + (int64_t)k * r] * yt[k];
-      yt[i] = a / mw[i + (int64_t)i * r];
-    }
-    for (int i = r - 1; i >= 0; --i) {  // back: L^T x = u
-      double a = yt[i];
-      for (int k = i + 1; k < r; ++k) a -= mw[k + (int64_t)i * r] * yt[k];
-      yt[i] = a / mw[i + (int64_t)i * r];
-    }
-    for (int i = 0; i < r; ++i) yt[i] /= d[i];
-  }
-  if (threadIdx.x == 0) tm.put(&sh.flag, sh.flag);
+    if (threadIdx.x == 0) tm.put(&sh.flag, sh.flag);
   }
   tm.sync();
   return sh.flag != 0;
@@ -2257,13 +2261,14 @@ __device__ __noinline__ int compress_by_pivoted_qr(const TM& tm, const SrcView& 
 // up to 45 where its QR rank is ~240), so with few tiles the launch takes what its largest tile takes
 // while most SMs idle.  With few tiles the CTAs come in clusters of four, and a cluster can work on
 // one tile as a team (the columns of the QR, the rows and blocks of the products, the pairs of
-// FP32 sweeps that leave shared memory).  A team takes a 256 x 240 tile in 9.8 M SM cycles, one CTA
-// in 21, so that half of its SMs' time is lost.  Teams take all tiles while these are at most half
+// FP32 sweeps that leave shared memory).  A team takes a 256 x 240 tile of QR rank ~235 in 45 M SM
+// cycles, one CTA in 100 (of QR rank ~60 in 5.1 and 9.3), so that about half of its SMs' time is
+// lost.  Teams take all tiles while these are at most half
 // the CTAs (64 tiles, gradient of the 1D chain at N = 1024: 3.6 ms against 5.1), else the leading
 // n_team ones of the list (team_tiles, by their costs), after which each CTA takes its own: with
 // 144 tiles on 152 SMs all by teams were no faster than none (Coulomb-like lattice at N = 2048,
 // 6.2 ms against 5.8), the largest few are (3D lattice iterates at N = 2048, 29 launches: 247 ->
-// 197 ms, the longest 43 -> 20).  Either way a tile's arithmetic is the same to the bit.
+// 192 ms, the longest 43 -> 18).  Either way a tile's arithmetic is the same to the bit.
 // ---------------------------------------------------------------------------------------------
 template <bool kTeams>
 __device__ __forceinline__ void compress_dense_body(
