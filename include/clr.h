@@ -357,7 +357,8 @@ typedef struct clr_profile {
   double ms_finalize;          /* norms and scaling */
   int64_t svd_blocks;          /* truncated SVDs (one-sided Jacobi) run by recompression */
   int64_t svd_sweeps_fp32;     /* FP32 sweeps, summed over those SVDs */
-  int64_t svd_sweeps_fp64;     /* FP64 sweeps, summed */
+  int64_t svd_sweeps_fp64;     /* FP64 sweeps, summed (near the noise floor, blocks without the
+                                  pivoted QR and cores of low-rank sums) */
   int64_t svd_early_dense;     /* SVDs stopped after the FP32 phase (certified dense) */
   double svd_flops_fp64;       /* algorithmic FP64 flops of recompression: QR 2(m+n)R^2, core
                                   products, orthonormalisations 2q^3, projections 2pq^2, Jacobi
