@@ -234,8 +234,8 @@ void launch_identity_distance(const MatView& X, double* out_sq, cudaStream_t st)
 // (One CTA per block-row, walking its blocks one after the other, took 690 us; eight take 60.)
 // Inside a CTA a warp takes four columns of W at a time for W^T x and sums them together; for X t
 // (and dense blocks) it owns a group of 32 rows and a share of the columns, its row sums in
-// registers until the end.  The kinds of 32 of the CTA's blocks are read at once: in a chain matrix
-// nearly all are zero, and read one after the other they were most of the time.
+// registers until the end.  The kinds, ranks and places of 32 of the CTA's blocks are read at once: in
+// a chain matrix nearly all are zero, and read one after the other they were most of the time.
 constexpr int kMvThreads = 512;
 constexpr int kMvWarps = kMvThreads / 32;
 
@@ -256,18 +256,21 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kMvThreads)
   int buf = 0;
   for (int J0 = rank; J0 < M.nc; J0 += 32 * CS) {
     const int Jl = J0 + l * CS;
-    const int kind = Jl < M.nc ? M.kind[I * M.nc + Jl] : CLR_KIND_ZERO;
+    const bool in = Jl < M.nc;
+    const int kind = in ? M.kind[I * M.nc + Jl] : CLR_KIND_ZERO;
+    const int rank_l = in ? M.rank[I * M.nc + Jl] : 0;
+    const int off_l = in ? M.col_off[Jl] : 0, end_l = in ? M.col_off[Jl + 1] : 0;
     const unsigned lr = __ballot_sync(0xffffffffu, kind == CLR_KIND_LR);
     for (unsigned todo = __ballot_sync(0xffffffffu, kind != CLR_KIND_ZERO); todo; todo &= todo - 1) {
-      const int bit = __ffs(todo) - 1, J = J0 + bit * CS;
-      const int t = I * M.nc + J;
-      const int n = M.col_off[J + 1] - M.col_off[J];
-      const double* s = M.pool + slot_of(M, I, J, m);
-      const double* xj = x + M.col_off[J];
+      const int bit = __ffs(todo) - 1;
+      const int off = __shfl_sync(0xffffffffu, off_l, bit);
+      const int n = __shfl_sync(0xffffffffu, end_l, bit) - off;
+      const double* s = M.pool + (int64_t)M.row_off[I] * M.n_cols + (int64_t)m * off;
+      const double* xj = x + off;
       const double* v = xj;
       int cols = n;
       if (lr >> bit & 1u) {
-        const int r = M.rank[t];
+        const int r = __shfl_sync(0xffffffffu, rank_l, bit);
         const double* W = s + (int64_t)m * r;
         for (int c0 = 4 * w; c0 < r; c0 += 4 * kMvWarps) {
           double d[4] = {0.0, 0.0, 0.0, 0.0};
