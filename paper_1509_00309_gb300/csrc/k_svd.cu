@@ -533,27 +533,44 @@ __device__ __noinline__ int jacobi_svd(double* g, int p, int q, double* v, int m
         if (ab == 0.0 || ab <= floor2 * floor2) continue;
         double* ga = g + (int64_t)a * p;
         double* gb = g + (int64_t)b * p;
-        // the two columns stay in registers between the inner product and the rotation
-        double xa[kRowsPerLane], xb[kRowsPerLane], d = 0;
+        // kOnto: the two columns are read again for the rotation (in a kernel with all its registers
+        // in use the callee's are spilled by every caller: compress_qr_kernel 210 -> 216 us where no
+        // such sweep runs); else they stay in registers in between
+        constexpr int kHold = kOnto ? 1 : kRowsPerLane;
+        double xa[kHold], xb[kHold], d = 0;
+        if constexpr (kOnto) {
+#pragma unroll 2
+          for (int i = l; i < p; i += 32) d = fma(ga[i], gb[i], d);
+        } else {
 #pragma unroll
-        for (int j = 0; j < kRowsPerLane; ++j) {
-          if (32 * j >= p) break;
-          const int i = l + 32 * j;
-          xa[j] = i < p ? ga[i] : 0.0;
-          xb[j] = i < p ? gb[i] : 0.0;
-          d = fma(xa[j], xb[j], d);
+          for (int j = 0; j < kHold; ++j) {
+            if (32 * j >= p) break;
+            const int i = l + 32 * j;
+            xa[j] = i < p ? ga[i] : 0.0;
+            xb[j] = i < p ? gb[i] : 0.0;
+            d = fma(xa[j], xb[j], d);
+          }
         }
         d = warp_sum(d);
         if (d * d <= tol * tol * ab || d * d <= floor2 * floor2) continue;
         double c, sn, t;
         rotation(al, be, d, c, sn, t);
+        if constexpr (kOnto) {
+#pragma unroll 2
+          for (int i = l; i < p; i += 32) {
+            const double x = ga[i], y = gb[i];
+            ga[i] = c * x - sn * y;
+            gb[i] = sn * x + c * y;
+          }
+        } else {
 #pragma unroll
-        for (int j = 0; j < kRowsPerLane; ++j) {
-          if (32 * j >= p) break;
-          const int i = l + 32 * j;
-          if (i < p) {
-            ga[i] = c * xa[j] - sn * xb[j];
-            gb[i] = sn * xa[j] + c * xb[j];
+          for (int j = 0; j < kHold; ++j) {
+            if (32 * j >= p) break;
+            const int i = l + 32 * j;
+            if (i < p) {
+              ga[i] = c * xa[j] - sn * xb[j];
+              gb[i] = sn * xa[j] + c * xb[j];
+            }
           }
         }
         // new squared norms: a - t g and b + t g exactly; recomputed from the rotated columns
@@ -1096,6 +1113,7 @@ __device__ __noinline__ double small_series(const TM& tm, double* e, int q, doub
   float part = 0.f;
   for (int x = threadIdx.x; x < q * q; x += kThreads) {
     const float v = (float)e[x];
+    if (fs.own) f[x] = v;
     part = fmaf(v, v, part);
   }
   const double fro2 = block_sum((double)part, sh.red);
@@ -1105,8 +1123,10 @@ __device__ __noinline__ double small_series(const TM& tm, double* e, int q, doub
     tm.sync();
     return fro2;
   }
-  for (int x = fs.t0; x < q * q; x += fs.step) f[x] = (float)e[x];
-  if (fs.own) __syncthreads(); else tm.sync();
+  if (!fs.own) {
+    for (int x = fs.t0; x < q * q; x += fs.step) f[x] = (float)e[x];
+    tm.sync();
+  }
   cta_gemm_auto(fs.t0, fs.step, q, q, q, f, 1, q, f, 1, q, t, q);
   tm.sync();
   // E^3 = F T an output at a time, added to the rest of the series
@@ -1374,6 +1394,17 @@ __device__ __noinline__ bool ls_solve(const TM& tm, double* y, int q, int r, dou
   return sh.flag != 0;
 }
 
+// x 2^k by integer arithmetic on the exponent (an FP64 multiplication holds the pipe for 64 cycles a
+// warp): zero where the exponent leaves the range below; the caller keeps it in range above.
+__device__ __forceinline__ int double_exponent(double x) {
+  return __double2hiint(x) >> 20 & 0x7ff;
+}
+__device__ __forceinline__ double scaled(double x, int k) {
+  const int e = double_exponent(x);
+  return e > 0 && e + k > 0 ? __hiloint2double(__double2hiint(x) + (k << 20), __double2loint(x))
+                            : 0.0;
+}
+
 // Mixed-precision one-sided Jacobi SVD of the p x q (p >= q) matrix A given by `a`.  FP64 runs
 // at a small fraction of the FP32 rate on this part, so the rotations are found in FP32 and only
 // applied, once per stage, in FP64:
@@ -1452,24 +1483,24 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
   // the block's norm is, and V does not depend on the scale.  (Unscaled, no pair of columns was
   // rotated in blocks of norm below ~1e-18 or above 1.8e19, and their ranks were those of the
   // columns as they came.)
-  const double sc32 = fro > 0.0 && isfinite(fro) ? scalbn(1.0, -ilogb(fro)) : 1.0;
-  const float floor_g = (float)(floor64 * sc32);
+  const int fro_exp = double_exponent(fro), shift = fro_exp < 0x7ff ? 0x3ff - fro_exp : 0;
+  const float floor_g = (float)scaled(floor64, shift);
   const float tol32 = 4.f * FLT_EPSILON * sqrtf((float)p);
-  const float floor32 = lower ? floor_g : (float)((double)p * FLT_EPSILON * fro * sc32);
+  const float floor32 = lower ? floor_g : (float)((double)p * FLT_EPSILON * scaled(fro, shift));
   // (else the FP32 stages are the first CTA's)
   int sw32 = 0;
   const One solo;
   if (spread1 && !tri32) {
     for (int e = tm.tid; e < wk.ldg * q; e += tm.nt) {
       const int i = e % wk.ldg;
-      wk.g[e] = i < p ? (float)(a.at(i, e / wk.ldg) * sc32) : 0.f;
+      wk.g[e] = i < p ? (float)scaled(a.at(i, e / wk.ldg), shift) : 0.f;
     }
     tm.sync();
     sw32 = run_jacobi32(tm, wk, q, max_sweeps, tol32, floor32 * floor32, sh.jac);
   } else if (tm.rank == 0) {
     for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
       const int i = e % wk.ldg;
-      wk.g[e] = i < p ? (float)(a.at(i, e / wk.ldg) * sc32) : 0.f;
+      wk.g[e] = i < p ? (float)scaled(a.at(i, e / wk.ldg), shift) : 0.f;
     }
     __syncthreads();
     if (tri32) qr32(wk, p, q, sc);
@@ -1493,7 +1524,7 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
       double s2 = 0.0;
       for (int i = l; i < p; i += 32) s2 = fma((double)gc[i], (double)gc[i], s2);
       s2 = warp_sum(s2);
-      if (l == 0) sh.sigma[c] = sqrt(s2) / sc32;
+      if (l == 0) sh.sigma[c] = scaled(sqrt(s2), -shift);
     }
     __syncthreads();
     double part = 0.0;
@@ -1528,7 +1559,7 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
   if (tm.size > 1 && (wk.ldg + wk.ldv) * q * (int)sizeof(float) > svd_smem_bytes()) {
     for (int e = tm.tid; e < wk.ldg * q; e += tm.nt) {
       const int i = e % wk.ldg;
-      wk.g[e] = i < p ? (float)(g[i + (int64_t)(e / wk.ldg) * p] * sc32) : 0.f;
+      wk.g[e] = i < p ? (float)scaled(g[i + (int64_t)(e / wk.ldg) * p], shift) : 0.f;
     }
     tm.sync();
     sw32b = run_jacobi32(tm, wk, q, max_sweeps, tol_g, floor_g * floor_g, sh.jac);
@@ -1536,7 +1567,7 @@ __device__ __noinline__ int svd_mixed(const TM& tm, const SrcView& a, int p, int
     if (tm.rank == 0) {
       for (int e = threadIdx.x; e < wk.ldg * q; e += kThreads) {
         const int i = e % wk.ldg;
-        wk.g[e] = i < p ? (float)(g[i + (int64_t)(e / wk.ldg) * p] * sc32) : 0.f;
+        wk.g[e] = i < p ? (float)scaled(g[i + (int64_t)(e / wk.ldg) * p], shift) : 0.f;
       }
       __syncthreads();
       const int sw = run_jacobi32(solo, wk, q, max_sweeps, tol_g, floor_g * floor_g, sh.jac);
